@@ -26,7 +26,7 @@
  *     before anything is launched.  No call synchronises the stream except
  *     vidkv_cache_status and vidkv_set_token_mask with n_protected == -1.  The first key
  *     quantization or decode call on each device fills the tables of DFT coefficients inside
- *     the library (56 KB) with one extra small kernel on the caller's stream and records an
+ *     the library (60 KB) with one extra small kernel on the caller's stream and records an
  *     event that later calls make their streams wait for; make that first call outside any
  *     stream capture.
  *   - Fixed in this library: D = 128, G = 32, R = 128, H_q a multiple of H_kv with

@@ -49,12 +49,17 @@ cudaError_t launch_encode_keys(int dtype, const KSrc& src, int64_t T_tokens, con
 cudaError_t launch_encode_keys_general(int dtype, const KSrc& src, int64_t T_tokens, const CacheView& cv, int layer0,
                                        int n_slabs, int slabs_per_layer, int chunk, int64_t kgroup0, cudaStream_t stream);
 
-// Device address of the 64-point DFT matrix in MMA B-fragment order: word
+// Device addresses of the DFT tables.  frag: the 64-point matrix in MMA B-fragment order: word
 // ((ks * 8 + nt) * 32 + lane) * 4 + {0, 1} = leading binary16 pairs, + {2, 3} = remainders, for
 // rows 16 ks + 2 r (+1; +8, +9) and column 16 (n / 2) + 2 nt + (n % 2), lane = 4 n + r; column f
 // holds 1/8, (-1)^c / 8, cos(2 pi k c / 64) / 8 (f = 2k) or -sin(2 pi k c / 64) / 8 (f = 2k + 1).
+// w32: the 32-point matrix [channel][column] in float32, orthonormal, columns from 2 on doubled.
 // Filled on first use on each device by one small kernel; later calls order their stream after it with an event.
-cudaError_t dft_fragments(const uint32_t** table, cudaStream_t stream);
+struct DftTables {
+  const uint32_t* frag;
+  const float* w32;
+};
+cudaError_t dft_tables(DftTables* tables, cudaStream_t stream);
 
 // Algorithm 2 on the prefill tokens of n_layers layers (source slabs run over layers, then b, then h).  T_q (multiple of 32) tokens; the
 // unprotected ones go to ternary stream positions 0.., the protected ones to 2-bit groups.
@@ -123,7 +128,7 @@ struct DecodeArgs {
   void* out;
   float* partials;     // [n_slabs][parts_stride][8 heads][kRecordFloats]
   uint32_t* prep;      // per (slab, chunk) query images of the tensor-core path (decode_prep_bytes)
-  const uint32_t* dft; // DFT matrix fragments (dft_fragments), set by launch_decode_prep
+  DftTables dft;       // set by launch_decode_prep
   int32_t append_row;  // >= 0: the preparation kernel also writes k_new / v_new into this residual row
   int32_t layer0, n_layers;
   int32_t in_dtype, out_dtype;

@@ -24,6 +24,7 @@
 
 #include "common.cuh"
 #include "kernels.cuh"
+#include "quant_common.cuh"
 
 namespace vidkv {
 
@@ -41,6 +42,10 @@ __device__ __align__(16) uint32_t g_dft_frag[kDftWords];
 constexpr int kWParts = 5;
 __device__ __align__(16) uint16_t g_dft_w[kWParts * 64 * 64];
 
+// [channel position c][spectrum column f]: the weight with which column f of a 32-point Hermitian half spectrum
+// enters channel c under the inverse orthonormal transform (the query preparation of the k = 0.75 Eq. 5 format).
+__device__ __align__(16) float g_dft_w32[32 * 32];
+
 // Byte offset of element (row, k) of a K-major operand with 64 binary16 per row under the
 // 128-byte swizzle: 8-row atoms of 1024 bytes, 16-byte pieces XORed with the row within the atom.
 __host__ __device__ constexpr int sw128_offset(int row, int k) {
@@ -51,56 +56,6 @@ __device__ __forceinline__ void cp_async16(void* smem_dst, const void* gmem_src)
   const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(smem_dst));
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(gmem_src) : "memory");
 }
-__device__ __forceinline__ __half2 as_h2(uint32_t v) { return *reinterpret_cast<const __half2*>(&v); }
-__device__ __forceinline__ uint32_t as_u32(__half2 v) { return *reinterpret_cast<const uint32_t*>(&v); }
-
-// Element-type helpers: raw 16-bit patterns in, binary16 1.0 / 0.0 pairs out of the comparison.
-template <typename T> struct Ops;
-template <> struct Ops<__half> {
-  static __device__ __forceinline__ float to_float(uint16_t b) { return __half2float(__ushort_as_half(b)); }
-  static __device__ __forceinline__ uint16_t from_float_rn(float f) { return __half_as_ushort(__float2half_rn(f)); }
-  static __device__ __forceinline__ uint16_t vmin(uint16_t a, uint16_t b) { return __half_as_ushort(__hmin(__ushort_as_half(a), __ushort_as_half(b))); }
-  static __device__ __forceinline__ uint16_t vmax(uint16_t a, uint16_t b) { return __half_as_ushort(__hmax(__ushort_as_half(a), __ushort_as_half(b))); }
-  static __device__ __forceinline__ uint32_t ge(uint32_t a, uint32_t b) { return as_u32(__hge2(as_h2(a), as_h2(b))); }
-  static __device__ __forceinline__ uint32_t to_half_pair(uint32_t raw) { return raw; }
-  static constexpr uint16_t kInf = 0x7c00u;
-};
-template <> struct Ops<__nv_bfloat16> {
-  static __device__ __forceinline__ float to_float(uint16_t b) { return __uint_as_float(static_cast<uint32_t>(b) << 16); }
-  static __device__ __forceinline__ uint16_t from_float_rn(float f) { return __bfloat16_as_ushort(__float2bfloat16_rn(f)); }
-  static __device__ __forceinline__ uint16_t vmin(uint16_t a, uint16_t b) { return to_float(a) <= to_float(b) ? a : b; }
-  static __device__ __forceinline__ uint16_t vmax(uint16_t a, uint16_t b) { return to_float(a) >= to_float(b) ? a : b; }
-  static __device__ __forceinline__ uint32_t ge(uint32_t a, uint32_t b) {
-    const __nv_bfloat162 r = __hge2(*reinterpret_cast<const __nv_bfloat162*>(&a), *reinterpret_cast<const __nv_bfloat162*>(&b));
-    return *reinterpret_cast<const uint32_t*>(&r) & 0x3c003c00u;   // bfloat16 1.0 -> binary16 1.0
-  }
-  static __device__ __forceinline__ uint32_t to_half_pair(uint32_t raw) {
-    const __half2 h = __floats2half2_rn(__uint_as_float(raw << 16), __uint_as_float(raw & 0xffff0000u));
-    return as_u32(h);
-  }
-  static constexpr uint16_t kInf = 0x7f80u;
-};
-
-// Value order of 16-bit sign-magnitude patterns as integers (both zeros map to 0).
-__device__ __forceinline__ int ord_of(uint16_t b) { return (b & 0x8000u) ? -static_cast<int>(b & 0x7fffu) : static_cast<int>(b); }
-__device__ __forceinline__ uint16_t bits_of(int o) { return o >= 0 ? static_cast<uint16_t>(o) : static_cast<uint16_t>(0x8000u | static_cast<uint32_t>(-o)); }
-
-// Eq. 4 for one element: is clamp(rint(RN(RN(x - z) / s)), 0, 3) >= k for the element with value
-// order o (k = 1..3, s > 0)?  Decided without the division.  rint(q) >= k holds from q = 0.5 + 2^-24,
-// 1.5 and 2.5 + 2^-22 on (round half to even), and the rounded quotient reaches that float exactly
-// when the real quotient passes the midpoint below it: d / s > 0.5 + 2^-25, >= 1.5 - 2^-24,
-// > 2.5 + 2^-23 (ties go to the even neighbour 0.5, 1.5, 2.5).  With c = k - 0.5 the sign of
-// d - (c + delta) s is that of u - delta s, u = fma(-c, s, d): c s is exact, u is exact whenever
-// d is within a factor two of c s (the only case where delta matters), delta s is a power of two times s.
-template <typename T>
-__device__ __forceinline__ bool code_at_least(int o, float z, float s, int k) {
-  const float d = __fsub_rn(Ops<T>::to_float(bits_of(o)), z);
-  const float u = fmaf(0.5f - static_cast<float>(k), s, d);
-  if (k == 1) return u > 0x1p-25f * s;
-  if (k == 2) return u >= -0x1p-24f * s;
-  return u > 0x1p-23f * s;
-}
-
 }  // namespace
 
 // Column f of the DFT matrix at channel position c: f = 0: 1/8; f = 1: (-1)^c / 8;
@@ -144,6 +99,12 @@ __global__ void dft_table_kernel() {
     g_dft_w[2 * 4096 + i] = __bfloat16_as_ushort(b0);
     g_dft_w[3 * 4096 + i] = __bfloat16_as_ushort(b1);
     g_dft_w[4 * 4096 + i] = __bfloat16_as_ushort(__float2bfloat16_rn(r2));
+  }
+  for (int i = threadIdx.x; i < 32 * 32; i += blockDim.x) {
+    const int c = i >> 5, f = i & 31, k = f < 2 ? 16 * f : f >> 1;
+    double sn, cs;
+    sincospi(static_cast<double>((k * c) & 31) / 16.0, &sn, &cs);
+    g_dft_w32[i] = static_cast<float>((f < 2 ? cs : 2.0 * ((f & 1) ? -sn : cs)) / sqrt(32.0));
   }
 }
 
@@ -406,25 +367,7 @@ __global__ void __launch_bounds__(256, 2) k_encode_kernel(KSrc src, int64_t T_to
         uint32_t thr[3];
 #pragma unroll
         for (int k = 1; k <= 3; ++k) {
-          uint16_t X = Ops<T>::kInf;                     // s == 0: every code is 0
-          if (sc != 0.0f) {
-            int o = ord_of(Ops<T>::from_float_rn(fmaf(static_cast<float>(k) - 0.5f, sc, z)));
-            // the threshold is almost always the candidate or its upper neighbour: two evaluations
-            const bool p0 = code_at_least<T>(o, z, sc, k);
-            const bool p1 = code_at_least<T>(p0 ? o - 1 : o + 1, z, sc, k);
-            if (p0 != p1) {
-              o += p0 ? 0 : 1;
-            } else if (p0) {
-              o -= 1;
-#pragma unroll 1
-              for (int it = 0; it < 4 && code_at_least<T>(o - 1, z, sc, k); ++it) --o;
-            } else {
-              o += 2;
-#pragma unroll 1
-              for (int it = 0; it < 4 && !code_at_least<T>(o, z, sc, k); ++it) ++o;
-            }
-            X = bits_of(o);
-          }
+          const uint16_t X = code_cut<T>(z, sc, k);
           thr[k - 1] = static_cast<uint32_t>(X) * 0x10001u;
         }
         // codes of token pairs as 1024 + code * 4^pos per 16-bit lane: the low byte of a lane is the
@@ -528,32 +471,34 @@ __global__ void __launch_bounds__(256, 2) k_encode_kernel(KSrc src, int64_t T_to
 // ---------------------------------------------------------------------------------
 // Host launcher of the encode pass
 // ---------------------------------------------------------------------------------
-// The DFT fragments are written once per device by a small kernel on the stream of the first
+// The DFT tables are written once per device by a small kernel on the stream of the first
 // call that needs them, followed by an event; every call makes its stream wait for that event
 // (free once it has completed), so uses on other streams are ordered after the fill without a
 // host-side synchronisation.
-cudaError_t dft_fragments(const uint32_t** table, cudaStream_t stream) {
+cudaError_t dft_tables(DftTables* tables, cudaStream_t stream) {
   static bool done[64] = {};
-  static const uint32_t* addr[64] = {};
+  static DftTables addr[64] = {};
   static cudaEvent_t ready[64] = {};
   cudaError_t e;
   int dev = 0;
   if ((e = cudaGetDevice(&dev))) return e;
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   if (!done[dev]) {
-    void* p = nullptr;
+    void *p = nullptr, *p32 = nullptr;
     if ((e = cudaGetSymbolAddress(&p, g_dft_frag))) return e;
+    if ((e = cudaGetSymbolAddress(&p32, g_dft_w32))) return e;
     if ((e = cudaEventCreateWithFlags(&ready[dev], cudaEventDisableTiming))) return e;
     dft_table_kernel<<<1, 256, 0, stream>>>();
     if ((e = cudaGetLastError())) return e;
     if ((e = cudaEventRecord(ready[dev], stream))) return e;
-    addr[dev] = static_cast<const uint32_t*>(p);
+    addr[dev].frag = static_cast<const uint32_t*>(p);
+    addr[dev].w32 = static_cast<const float*>(p32);
     done[dev] = true;
     count_launches(1);
   } else if ((e = cudaStreamWaitEvent(stream, ready[dev], 0))) {
     return e;
   }
-  *table = addr[dev];
+  *tables = addr[dev];
   return cudaSuccess;
 }
 
@@ -561,8 +506,8 @@ template <typename T>
 static cudaError_t launch_encode_t(const KSrc& src, int64_t T_tokens, const CacheView& cv, int layer0, int n_slabs,
                                    int slabs_per_layer, int chunk, int64_t kgroup0, cudaStream_t stream) {
   cudaError_t e;
-  const uint32_t* table = nullptr;
-  if ((e = dft_fragments(&table, stream))) return e;
+  DftTables tables;
+  if ((e = dft_tables(&tables, stream))) return e;
   static int n_sms[64] = {};   // per device; 0 = the kernel's attributes are not set there yet
   constexpr int smem = enc_sm_bytes<T>();
   int dev = 0;

@@ -107,6 +107,18 @@ def test_prefill_codes_and_dequantized_keys(fmt, name, T, B):
 
 
 @pytest.mark.parametrize("fmt", FORMATS, ids=_fmt_id)
+@pytest.mark.parametrize("name,T", [("tiny", 9728), ("qwen", 32)])
+def test_encoder_blocks_of_several_groups(fmt, name, T):
+    """4 slabs x 304 groups are more than the encoder's resident blocks (1184 and 592 on 148 multiprocessors), so
+    blocks walk several groups and cross slabs; 32 tokens are its smallest call.  Bit-exact, as every prefill."""
+    pair = Pair(CONFIGS[name], T, B=1, L=1, max_new=4, k_ratio=fmt[0], one_bit=fmt[1])
+    pair.flushed_chunks = {}
+    pair.prefill()
+    assert pair.cache.status() == 0
+    _check_layer(pair)
+
+
+@pytest.mark.parametrize("fmt", FORMATS, ids=_fmt_id)
 @pytest.mark.parametrize("p", [0.0, 0.2])
 def test_decode_across_a_flush(fmt, p):
     T = 200
