@@ -186,8 +186,8 @@ typedef struct vidkv_cache vidkv_cache_t;
 /* Sizes (host only).  cache_bytes / workspace_bytes are what vidkv_cache_init wants.
  * The workspace holds partial attention results, prepared queries, channel ranges and
  * the gather lists of the token selection.  Between calls it carries the gather lists,
- * which vidkv_quantize_values reads, and the armed channel-range accumulators that
- * vidkv_cache_init sets up: it belongs to one handle and must not be overwritten while
+ * which vidkv_quantize_values reads, and the armed channel-range accumulators and cleared
+ * arrival counters that vidkv_cache_init sets up: it belongs to one handle and must not be overwritten while
  * that handle is in use. */
 vidkv_status_t vidkv_cache_bytes(const vidkv_config_t* cfg, size_t* cache_bytes, size_t* workspace_bytes);
 
@@ -383,9 +383,10 @@ vidkv_status_t vidkv_attend_noalloc(const vidkv_config_t* cfg, const void* cache
  * Eq. 3 open; the library cuts a decode call into work like this: the quantized tokens of all
  * slabs of the call form one sequence of 160-token units, and every warp of the launch walks a
  * run of `run_units` consecutive units (crossing slab boundaries where its run does) and leaves
- * one partial result per slab it touches.
- * vidkv_debug_set_decode_plan forces run_units (>= 1) for later vidkv_decode_attention calls on
- * this handle; 0 leaves the choice to the library.  A forced plan that needs more partial records
+ * one partial result per slab it touches; calls of a few thousand units at most take another
+ * kernel, whose blocks walk stretches of units together.
+ * vidkv_debug_set_decode_plan forces run_units (>= 1), and with it the first of the two kernels, for later
+ * vidkv_decode_attention calls on this handle; 0 leaves the choice to the library.  A forced plan that needs more partial records
  * than the workspace holds makes the decode call return VIDKV_ERR_CAPACITY.
  * vidkv_debug_decode_plan (host only) reports the plan for given token counts on a device with
  * sm_count multiprocessors: plan_out[8] = { units per slab, run_units, runs (= warps),
@@ -397,17 +398,17 @@ vidkv_status_t vidkv_debug_decode_plan(const vidkv_config_t* cfg, int64_t n_pref
                                        int32_t run_units, int64_t* plan_out);
 
 /* Test hook for the two bounded device-side waits (no counterpart in the paper).  The key encoder
- * waits on the barrier its tensor-core products commit to, the stream kernel of the decode call
+ * waits on the barrier its tensor-core products commit to, the attention kernel of the decode call
  * on the barriers of its bulk copies; both waits give up after a fixed number of polls, record
  * VIDKV_ERR_TIMEOUT in the cache's status word and leave in order (copies drained, tensor memory
  * freed).  what = 1 makes the next key quantization withhold the products of every block's first
- * tile, what = 2 makes the next decode call (on a cache without protected tokens) withhold every warp's first
+ * tile, what = 2 makes the next decode call (on a cache without protected tokens) withhold every warp's (block's) first
  * value copy, so that the waits run out with nothing outstanding; the affected call's results
  * are garbage by design, the flag clears itself, and later calls are normal.  0 switches it off. */
 vidkv_status_t vidkv_debug_withhold_once(int32_t what);
 
 /* Profiling aid: record the two CUDA events (cudaEvent_t passed as void*) immediately before
- * and after the attention kernel (the stream kernel) of every later vidkv_decode_attention call on this
+ * and after the attention kernel of every later vidkv_decode_attention call on this
  * handle; NULL, NULL switches it off.  The events are the caller's. */
 vidkv_status_t vidkv_set_profile_events(vidkv_cache_t* handle, void* ev_begin, void* ev_end);
 

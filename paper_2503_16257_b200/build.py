@@ -11,8 +11,8 @@ import sys
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libvidkv.so")
-SOURCES = ["host.cu", "quant_keys.cu", "quant_keys_enc.cu", "quant_keys_general.cu", "quant_values.cu", "decode.cu", "decode_prep.cu", "decode_stream.cu", "dequant.cu", "export.cu", "noalloc.cu", "saliency.cu", "chan_metrics.cu"]
-HEADERS = ["common.cuh", "quant_common.cuh", "kernels.cuh", "decode_common.cuh", os.path.join("..", "..", "include", "vidkv.h")]
+SOURCES = ["host.cu", "quant_keys.cu", "quant_keys_enc.cu", "quant_keys_general.cu", "quant_values.cu", "decode.cu", "decode_prep.cu", "decode_block.cu", "decode_stream.cu", "dequant.cu", "export.cu", "noalloc.cu", "saliency.cu", "chan_metrics.cu"]
+HEADERS = ["common.cuh", "quant_common.cuh", "kernels.cuh", "decode_common.cuh", "decode_device.cuh", os.path.join("..", "..", "include", "vidkv.h")]
 
 
 def _nvcc() -> str:
@@ -35,7 +35,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
     if not force and not needs_build():
         return LIB
     cmd = [_nvcc(), "-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-lineinfo", "-std=c++17",
-           "-shared", "-Xcompiler", "-fPIC", "-o", LIB]
+           "-t", "8", "-shared", "-Xcompiler", "-fPIC", "-o", LIB]
     if verbose:
         cmd += ["-Xptxas", "-v"]
     cmd += [os.path.join(CSRC, s) for s in SOURCES]

@@ -12,6 +12,13 @@ namespace {
 
 constexpr int kMaxSMs = 256;        // multiprocessor count the sizing formulas assume at most
 constexpr int kMinRunUnits = 1;     // with fewer units than warps every unit gets its own warp (shortest critical path)
+// Units per block up to which a call goes to the block kernel.  It has one launch, short parts and a parallel merge
+// where the stream kernel has three launches and a warp per run, but takes half as many instructions again per unit
+// (every warp of the block pays the unit's loop).  Measured (us per call, block / stream kernel): 160 units of 4 slabs
+// 15.8 / 25.1, 2560 units of 16 slabs 33 / 59, 4480 units of 448 slabs (8 a block) 47 / 47, 8960 units of 112 slabs 75 / 77;
+// with protected tokens 160 units 21.9 / 31.2, 1792 units of 448 slabs (4 a block) 37 / 41, 2240 units of 224 slabs 50 / 43.
+constexpr int kMaxBlockUnits = 7;
+constexpr int kMaxBlockUnitsStp = 3;
 
 }  // namespace
 
@@ -27,7 +34,14 @@ int device_sm_count() {
   return sm_of_device[dev];
 }
 
-DecodePlan plan_decode(const LayerState& st, int64_t n_slabs, bool stp, int sm_count, int force_run_units) {
+// Levels of eight-way joins over n parts: how many counters they take.
+static int64_t join_counters(int64_t n) {
+  int64_t c = 0;
+  while (n > 1) { n = (n + kJoin - 1) / kJoin; c += n; }
+  return c;
+}
+
+DecodePlan plan_decode(const LayerState& st, int64_t n_slabs, bool stp, bool general, int sm_count, int force_run_units) {
   DecodePlan p = {};
   const int64_t T_qt = st.T_q0 + st.n_flush * kR;
   p.n_chunks = T_qt > 0 ? 1 + static_cast<int32_t>(st.n_flush) : 0;
@@ -42,7 +56,20 @@ DecodePlan plan_decode(const LayerState& st, int64_t n_slabs, bool stp, int sm_c
   p.n_runs = static_cast<int32_t>((p.n_units + run - 1) / run);
   p.parts_stride = p.units_per_slab > 0 ? static_cast<int32_t>((p.units_per_slab + run - 1) / run) + 1 : 1;
   p.records = n_slabs * p.parts_stride * kMaxRep;
+  const int64_t blocks = static_cast<int64_t>(sms) * (stp && general ? kBlockGenStpPerSM : kBlocksPerSM);
+  const int64_t per_block = (p.n_units + blocks - 1) / blocks;
+  if (p.n_units == 0 || (per_block <= (stp ? kMaxBlockUnitsStp : kMaxBlockUnits) && force_run_units == 0)) {
+    p.block_units = per_block < run ? static_cast<int32_t>(run) : static_cast<int32_t>(per_block);
+    p.n_blocks = static_cast<int32_t>((p.n_units + p.block_units - 1) / p.block_units);
+    p.res_blocks = st.n_res > 0 && (p.n_units == 0 || p.block_units == 1) ? static_cast<int32_t>(n_slabs) : 0;
+    p.counters_per_slab = static_cast<int32_t>(join_counters(p.parts_stride));
+  }
   return p;
+}
+
+int64_t max_decode_counters(int64_t max_slabs, int64_t records) {
+  // the levels over n parts have at most n / 7 nodes and one more per level; ten levels cover 2^30 parts
+  return records / kMaxRep / 7 + 12 * max_slabs + 64;
 }
 
 int64_t max_decode_records(int64_t max_slabs, int64_t max_tokens) {
@@ -284,6 +311,13 @@ cudaError_t launch_merge_partials(const float* parts, int64_t n_parts, int64_t n
 cudaError_t launch_decode(const DecodeArgs& a_in, cudaStream_t stream) {
   DecodeArgs a = a_in;
   cudaError_t e;
+  if ((e = dft_tables(&a.dft, stream))) return e;
+  if (a.plan.n_blocks + a.plan.res_blocks > 0) {
+    if (a.ev_begin) cudaEventRecord(a.ev_begin, stream);
+    e = launch_decode_block(a, stream);
+    if (a.ev_end) cudaEventRecord(a.ev_end, stream);
+    return e;
+  }
   const int n_slabs = a.n_layers * a.cv.B * a.cv.H_kv;
   if (a.plan.n_chunks > 0) {
     if ((e = launch_decode_prep(a, stream)) != cudaSuccess) return e;

@@ -1,4 +1,5 @@
-// Device helpers shared by the decode attention kernels (decode_prep.cu, decode_stream.cu, decode.cu):
+// Device helpers shared by the decode attention kernels (decode_block.cu, decode_prep.cu,
+// decode_stream.cu, decode.cu):
 // mma.sync wrappers, the logic / multiply-add forms of the code expansion, and the query
 // normalisation.
 #pragma once
@@ -8,8 +9,6 @@
 
 namespace vidkv {
 namespace {
-
-constexpr int kThreads = 128;
 
 __device__ __forceinline__ void mma_f16(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
                                         uint32_t b1) {
@@ -46,21 +45,6 @@ template <> __device__ __forceinline__ void mma_in<__nv_bfloat16>(float (&d)[4],
 __device__ __forceinline__ void cp_async16(void* smem_dst, const void* gmem_src) {
   const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(smem_dst));
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(gmem_src) : "memory");
-}
-// Copy n16 16-byte pieces from global to shared memory, pieces interleaved over the CTA's threads;
-// unrolled by four so that the offsets are immediates.
-__device__ __forceinline__ void stage_async(uint8_t* dst, const uint8_t* src, int n16, int tid) {
-  constexpr int kStep = 128 * 16;
-  uint8_t* d = dst + tid * 16;
-  const uint8_t* s = src + tid * 16;
-  int i = tid;
-  for (; i + 3 * 128 < n16; i += 4 * 128, d += 4 * kStep, s += 4 * kStep) {
-    cp_async16(d, s);
-    cp_async16(d + kStep, s + kStep);
-    cp_async16(d + 2 * kStep, s + 2 * kStep);
-    cp_async16(d + 3 * kStep, s + 3 * kStep);
-  }
-  for (; i < n16; i += 128, d += kStep, s += kStep) cp_async16(d, s);
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }

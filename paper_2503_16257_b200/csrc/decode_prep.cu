@@ -11,6 +11,8 @@
 
 namespace vidkv {
 
+constexpr int kPrepThreads = 128;
+
 size_t decode_prep_bytes(int64_t n_slabs, int64_t n_chunks) {
   return static_cast<size_t>(n_slabs) * n_chunks * kPrepWords * 32 * sizeof(uint32_t);
 }
@@ -32,10 +34,10 @@ size_t decode_prep_bytes(int64_t n_slabs, int64_t n_chunks) {
 // on the tensor cores against the same split-precision matrix fragments the encoder uses.
 // ---------------------------------------------------------------------------------
 template <typename T>
-__global__ void __launch_bounds__(kThreads) decode_prep_kernel(DecodeArgs a, int n_chunks, int n_items) {
+__global__ void __launch_bounds__(kPrepThreads) decode_prep_kernel(DecodeArgs a, int n_chunks, int n_items) {
   const CacheView& cv = a.cv;
   const int lane = threadIdx.x & 31;
-  const int item = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5);
+  const int item = blockIdx.x * (kPrepThreads / 32) + (threadIdx.x >> 5);
   pdl_release();                                           // the attention kernel may start its first copies now
   if (item >= n_items) return;
   const int chunk = item % n_chunks, slab = item / n_chunks;
@@ -114,10 +116,10 @@ __global__ void __launch_bounds__(kThreads) decode_prep_kernel(DecodeArgs a, int
 // table: computing sines and cosines here took 49 us of a decode step of 224 slabs, the table takes 13.
 // ---------------------------------------------------------------------------------
 template <typename T>
-__global__ void __launch_bounds__(kThreads) decode_prep_general_kernel(DecodeArgs a, int n_chunks, int n_items) {
+__global__ void __launch_bounds__(kPrepThreads) decode_prep_general_kernel(DecodeArgs a, int n_chunks, int n_items) {
   const CacheView& cv = a.cv;
   const int lane = threadIdx.x & 31;
-  const int item = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5);
+  const int item = blockIdx.x * (kPrepThreads / 32) + (threadIdx.x >> 5);
   pdl_release();                                           // the attention kernel may start its first copies now
   if (item >= n_items) return;
   const int chunk = item % n_chunks, slab = item / n_chunks;
@@ -169,23 +171,20 @@ __global__ void __launch_bounds__(kThreads) decode_prep_general_kernel(DecodeArg
   out[24 * 32] = __float_as_uint(a.scale * 1.4426950408889634f * pow2i(qe + kQShift));
 }
 
-cudaError_t launch_decode_prep(DecodeArgs& a, cudaStream_t stream) {
-  a.dft = DftTables{nullptr, nullptr};
+cudaError_t launch_decode_prep(const DecodeArgs& a, cudaStream_t stream) {
   const int n_slabs = a.n_layers * a.cv.B * a.cv.H_kv;
   const int n_chunks = a.plan.n_chunks;
   if (n_chunks < 1) return cudaSuccess;
-  cudaError_t e;
   const int n_items = n_slabs * n_chunks;
-  const int pgrid = (n_items + kThreads / 32 - 1) / (kThreads / 32);
-  if ((e = dft_tables(&a.dft, stream))) return e;
+  const int pgrid = (n_items + kPrepThreads / 32 - 1) / (kPrepThreads / 32);
   if (a.cv.kf.general) {
-    if (a.in_dtype == VIDKV_F16) decode_prep_general_kernel<__half><<<pgrid, kThreads, 0, stream>>>(a, n_chunks, n_items);
-    else decode_prep_general_kernel<__nv_bfloat16><<<pgrid, kThreads, 0, stream>>>(a, n_chunks, n_items);
+    if (a.in_dtype == VIDKV_F16) decode_prep_general_kernel<__half><<<pgrid, kPrepThreads, 0, stream>>>(a, n_chunks, n_items);
+    else decode_prep_general_kernel<__nv_bfloat16><<<pgrid, kPrepThreads, 0, stream>>>(a, n_chunks, n_items);
     count_launches(1);
     return cudaGetLastError();
   }
-  if (a.in_dtype == VIDKV_F16) decode_prep_kernel<__half><<<pgrid, kThreads, 0, stream>>>(a, n_chunks, n_items);
-  else decode_prep_kernel<__nv_bfloat16><<<pgrid, kThreads, 0, stream>>>(a, n_chunks, n_items);
+  if (a.in_dtype == VIDKV_F16) decode_prep_kernel<__half><<<pgrid, kPrepThreads, 0, stream>>>(a, n_chunks, n_items);
+  else decode_prep_kernel<__nv_bfloat16><<<pgrid, kPrepThreads, 0, stream>>>(a, n_chunks, n_items);
   count_launches(1);
   return cudaGetLastError();
 }

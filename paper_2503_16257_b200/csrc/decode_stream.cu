@@ -26,49 +26,14 @@
 // merge kernel combines them and attends to the FP16 / BF16 residual.
 //
 // Nothing is shared between warps: no block-wide barrier, no shared score matrix.
-#include "decode_common.cuh"
+#include "decode_device.cuh"
 
 namespace vidkv {
 
 namespace {
 
-constexpr int kKBufBytes = kSGGroups * kKGroupBytes;   // 5760: the key groups of one unit
-constexpr int kVBufBytes = kSGBytes;                   // 5376: its ternary supergroup
 constexpr int kTotBytes = 4 * 2 * 32 * 16;             // 4096: the warp's running output (128 channels x 8 heads, float)
 constexpr int kWarpBufBytes = kKBufBytes + kVBufBytes + kTotBytes;   // 15232 per warp
-constexpr int kGenKBufBytes = kSGGroups * kMaxKGroupBytes;           // key buffer of the general key formats
-constexpr uint32_t kWaitLimit = 1u << 19;              // mbarrier polls before a warp gives up (about a second)
-constexpr float kStaleLog2 = 6.0f;                     // the running maximum may lag a unit's maximum by this much
-constexpr uint32_t kMinus5 = 0xc500c500u;              // binary16 pair (-5.0, -5.0)
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
-
-__device__ __forceinline__ void mbar_init(uint64_t* bar, int count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-// One bulk copy global -> shared of `bytes` (multiple of 16, both addresses 16-byte aligned),
-// completion counted on `bar`.
-__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
-  const uint32_t b = smem_u32(bar), d = smem_u32(dst);
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(b), "r"(bytes) : "memory");
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(d),
-               "l"(src), "r"(bytes), "r"(b)
-               : "memory");
-}
-// Bounded wait for the phase with the given parity; false if it never completed.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
-  const uint32_t b = smem_u32(bar);
-  for (uint32_t i = 0; i < kWaitLimit; ++i) {
-    uint32_t ok;
-    asm volatile(
-        "{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
-        : "=r"(ok)
-        : "r"(b), "r"(parity)
-        : "memory");
-    if (ok) return true;
-  }
-  return false;
-}
 
 // Per-lane state of the running softmax of one slab (the running output itself is in shared memory).
 struct Running {
@@ -564,7 +529,6 @@ constexpr int kPRing = 6 * kG;                         // protected ring: an unf
 constexpr int kPRingAt = kTRing * 2;                   // a head's row: 320 ternary entries, then 192 protected ones,
 constexpr int kRingRow = (kTRing + kPRing) * 2 + 48;   // then padding: 1072 bytes, rows start in different banks
 constexpr int kStpWarpBytes = kKBufBytes + kVBufBytes + kPGBytes + kTotBytes + 8 * kRingRow;
-constexpr uint32_t kMinus4 = 0xc400c400u;              // binary16 pair (-4.0, -4.0)
 
 // P V of one protected group (Eq. 4 codes as 4 + code): P4[nt] = probabilities of head hd at
 // the group's tokens 8 nt + 2 r, + 1.  out += s * (sum (4 + code) p - 4 sum p) + z * sum p.

@@ -69,8 +69,8 @@ void compute_layout(const vidkv_config_t& c, Layout* out) {
 }
 
 struct WsPlan {
-  int64_t minmax_off, partials_off, prep_off, idx_prot_off, idx_rest_off, counts_off, total;
-  int64_t partial_entries;
+  int64_t minmax_off, partials_off, prep_off, counters_off, idx_prot_off, idx_rest_off, counts_off, total;
+  int64_t partial_entries, counter_words;
 };
 
 void plan_workspace(const vidkv_config_t& c, const Layout& L, WsPlan* w) {
@@ -83,6 +83,9 @@ void plan_workspace(const vidkv_config_t& c, const Layout& L, WsPlan* w) {
   w->prep_off = off;
   off = round_up(off + static_cast<int64_t>(decode_prep_bytes(static_cast<int64_t>(c.L) * c.B * c.H_kv, L.lay.max_chunks)),
                  kAlign);
+  w->counters_off = off;
+  w->counter_words = max_decode_counters(static_cast<int64_t>(c.L) * c.B * c.H_kv, w->partial_entries);
+  off = round_up(off + w->counter_words * 4, kAlign);
   w->idx_prot_off = off;
   off = round_up(off + static_cast<int64_t>(c.B) * L.max_prot * 4, kAlign);
   w->idx_rest_off = off;
@@ -205,9 +208,11 @@ vidkv_status_t vidkv_cache_init(const vidkv_config_t* cfg, void* cache, size_t c
   h->layers.assign(cfg->L, LayerInfo());
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (cudaMemsetAsync(h->cache, 0, static_cast<size_t>(l.total_bytes), s) != cudaSuccess) { delete h; return VIDKV_ERR_CUDA; }
-  // the kernel that arms the channel-range accumulators also writes the header words
-  if (launch_init_minmax(reinterpret_cast<uint32_t*>(h->workspace + h->ws.minmax_off),
-                         2 * static_cast<int64_t>(cfg->L) * cfg->B * cfg->H_kv * 2 * kD, reinterpret_cast<uint32_t*>(h->cache),
+  // the kernel that arms the channel-range accumulators also clears the decode counters and writes the header words
+  if (launch_init_workspace(reinterpret_cast<uint32_t*>(h->workspace + h->ws.minmax_off),
+                         2 * static_cast<int64_t>(cfg->L) * cfg->B * cfg->H_kv * 2 * kD,
+                         reinterpret_cast<int32_t*>(h->workspace + h->ws.counters_off), h->ws.counter_words,
+                         reinterpret_cast<uint32_t*>(h->cache),
                          static_cast<uint32_t>(vidkv_version()), s) != cudaSuccess) {
     delete h;
     return VIDKV_ERR_CUDA;
@@ -424,17 +429,14 @@ static vidkv_status_t decode_impl(vidkv_cache_t* h, int32_t layer_begin, int32_t
   }
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const int dt = h->cfg.in_dtype;
-  // the append rides on the query-preparation kernel when there is one (some chunk is quantized)
-  const bool has_chunks = first.T_q0 + first.n_flush * kR > 0;
-  if (!append && !has_chunks && first.n_res == 0) return VIDKV_ERR_STATE;       // nothing to attend to
-  if (append && !has_chunks && launch_append(dt, k_new, v_new, h->cv, layer_begin, n_layers, first.n_res, s) != cudaSuccess)
-    return VIDKV_ERR_CUDA;
+  if (!append && first.T_q0 + first.n_flush * kR == 0 && first.n_res == 0) return VIDKV_ERR_STATE;       // nothing to attend to
   DecodeArgs a;
   a.cv = h->cv;
   a.q = q; a.k_new = k_new; a.v_new = v_new; a.out = out;
   a.partials = reinterpret_cast<float*>(h->workspace + h->ws.partials_off);
   a.prep = reinterpret_cast<uint32_t*>(h->workspace + h->ws.prep_off);
-  a.append_row = append && has_chunks ? first.n_res : -1;
+  a.counters = reinterpret_cast<int32_t*>(h->workspace + h->ws.counters_off);
+  a.append_row = append ? first.n_res : -1;
   a.partial_out = partial;
   a.layer0 = layer_begin; a.n_layers = n_layers;
   a.in_dtype = dt; a.out_dtype = h->cfg.out_dtype;
@@ -444,8 +446,8 @@ static vidkv_status_t decode_impl(vidkv_cache_t* h, int32_t layer_begin, int32_t
   a.withhold = 0;
   a.st.T_q0 = first.T_q0; a.st.n_flush = first.n_flush; a.st.n_res = first.n_res + (append ? 1 : 0);
   const int64_t n_slabs = static_cast<int64_t>(n_layers) * h->cfg.B * h->cfg.H_kv;
-  a.plan = plan_decode(a.st, n_slabs, h->n_prot > 0, device_sm_count(), h->dbg_run_units);
-  if (a.plan.records > h->ws.partial_entries) return VIDKV_ERR_CAPACITY;
+  a.plan = plan_decode(a.st, n_slabs, h->n_prot > 0, h->cv.kf.general != 0, device_sm_count(), h->dbg_run_units);
+  if (a.plan.records > h->ws.partial_entries || n_slabs * a.plan.counters_per_slab > h->ws.counter_words) return VIDKV_ERR_CAPACITY;
   if (launch_decode(a, s) != cudaSuccess) return VIDKV_ERR_CUDA;
   if (!append) return VIDKV_OK;
   const bool flush = a.st.n_res == kR;
@@ -529,7 +531,8 @@ vidkv_status_t vidkv_debug_decode_plan(const vidkv_config_t* cfg, int64_t n_pref
   plan_workspace(*cfg, L, &w);
   LayerState ls;
   ls.T_q0 = n_prefill_quantized; ls.n_flush = n_flushed_chunks; ls.n_res = n_residual;
-  const DecodePlan p = plan_decode(ls, static_cast<int64_t>(n_layers) * cfg->B * cfg->H_kv, n_protected > 0, sm_count, run_units);
+  const DecodePlan p = plan_decode(ls, static_cast<int64_t>(n_layers) * cfg->B * cfg->H_kv, n_protected > 0,
+                                   key_fmt_of_config(*cfg).general != 0, sm_count, run_units);
   plan_out[0] = p.units_per_slab; plan_out[1] = p.run_units; plan_out[2] = p.n_runs; plan_out[3] = p.parts_stride;
   plan_out[4] = p.records; plan_out[5] = w.partial_entries; plan_out[6] = p.n_chunks; plan_out[7] = p.n_units;
   return VIDKV_OK;

@@ -31,8 +31,9 @@ struct MinMaxBuffers {
   uint32_t* next;
   int next_dirty_words;
 };
-// Also writes the cache header (magic, version, cleared status word) when `header` is not null.
-cudaError_t launch_init_minmax(uint32_t* minmax, int64_t n_words, uint32_t* header, uint32_t version, cudaStream_t stream);
+// Arms both buffers, clears the decode counters and writes the cache header (magic, version, cleared status word).
+cudaError_t launch_init_workspace(uint32_t* minmax, int64_t n_words, int32_t* counters, int64_t n_counters, uint32_t* header,
+                                  uint32_t version, cudaStream_t stream);
 
 // Algorithm 3 on `T_tokens` tokens (a multiple of 32) of every slab of layers
 // [layer0, layer0 + n_layers): writes chunk `chunk` of the chunk table and the key groups
@@ -96,13 +97,21 @@ constexpr int kStreamUnitTokens = 160;  // one unit of the stream kernel: 5 key 
 constexpr int kStreamWarps = 4;         // warps per CTA of the stream kernel
 constexpr int kStreamCtasPerSM = 3;     // its CTAs per multiprocessor (register bound)
 constexpr int kStreamStpCtasPerSM = 2;  // the same for the variant with protected tokens (shared-memory bound)
-constexpr int kPrepWords = 25;     // 32-bit words per lane per (slab, chunk) of prepared query
+constexpr int kPrepWords = 25;          // 32-bit words per lane per (slab, chunk) of prepared query
+constexpr int kBlocksPerSM = 4;         // blocks of the block kernel per multiprocessor (96 registers x 160 threads;
+                                        // 56 KB of shared memory with protected tokens)
+constexpr int kBlockGenStpPerSM = 3;    // general key formats with protected tokens: 60 KB
 constexpr int kRecordFloats = 130; // one partial record: running maximum (base-2 logits), sum, out[128]
+constexpr int kPartFloats = kMaxRep * kRecordFloats;   // the block kernel's record of a part of a slab: m [8], l [8], out [8][128]
+constexpr int kJoin = 8;           // records joined at a node of the block kernel's merge tree
 
 // How one attention call over n_slabs slabs is cut into work (host side, decode.cu): the
-// quantized tokens of all slabs form one sequence of 160-token units (units_per_slab each); warp
-// number w of the launch walks the units [w * run_units, (w + 1) * run_units) and leaves one
-// partial record per slab it touches, record (slab, w - first warp of the slab).
+// quantized tokens of all slabs form one sequence of 160-token units (units_per_slab each).
+//   stream kernel  warp number w of the launch walks the units [w * run_units, (w + 1) * run_units) and leaves one
+//                  partial record per slab it touches, record (slab, w - first warp of the slab).
+//   block kernel   (n_blocks > 0 or nothing quantized: small calls) block b walks the units [b * block_units,
+//                  (b + 1) * block_units), at least one run; records are numbered the same way, and joined by a tree
+//                  of eight-way nodes.
 // parts_stride = records reserved per slab; the partials buffer holds n_slabs * parts_stride * 8
 // records of kRecordFloats floats.
 struct DecodePlan {
@@ -111,10 +120,16 @@ struct DecodePlan {
   int32_t parts_stride;
   int32_t n_chunks;        // chunk-table entries the query preparation covers (0: nothing quantized)
   int64_t records;         // n_slabs * parts_stride * 8
+  int32_t block_units, n_blocks;
+  int32_t res_blocks;      // blocks that attend to a slab's residual alone: n_slabs or 0 (the slab's last block does it)
+  int32_t counters_per_slab;   // arrival counters of the merge tree
 };
-// stp: the cache holds protected tokens (the kernel for them keeps fewer warps per multiprocessor).
-// force_run_units: 0 = choose; otherwise the test hook's value.
-DecodePlan plan_decode(const LayerState& st, int64_t n_slabs, bool stp, int sm_count, int force_run_units);
+// stp: the cache holds protected tokens (the stream kernel for them keeps fewer warps per multiprocessor).
+// general: a key format other than the default.
+// force_run_units: 0 = choose; otherwise the test hook's value (always the stream kernel).
+DecodePlan plan_decode(const LayerState& st, int64_t n_slabs, bool stp, bool general, int sm_count, int force_run_units);
+// Arrival counters any call that needs at most `records` records on at most max_slabs slabs uses.
+int64_t max_decode_counters(int64_t max_slabs, int64_t records);
 // Largest `records` any call on at most max_slabs slabs and max_tokens tokens can plan.
 int64_t max_decode_records(int64_t max_slabs, int64_t max_tokens);
 // Multiprocessors of the current device (cached per device); 0 on error.
@@ -127,9 +142,10 @@ struct DecodeArgs {
   const void* v_new;
   void* out;
   float* partials;     // [n_slabs][parts_stride][8 heads][kRecordFloats]
-  uint32_t* prep;      // per (slab, chunk) query images of the tensor-core path (decode_prep_bytes)
-  DftTables dft;       // set by launch_decode_prep
-  int32_t append_row;  // >= 0: the preparation kernel also writes k_new / v_new into this residual row
+  uint32_t* prep;      // stream kernel: per (slab, chunk) query images (decode_prep_bytes)
+  int32_t* counters;   // block kernel: [n_slabs][counters_per_slab], zero between calls
+  DftTables dft;       // set by launch_decode
+  int32_t append_row;  // >= 0: k_new / v_new are written into this residual row first
   int32_t layer0, n_layers;
   int32_t in_dtype, out_dtype;
   DecodePlan plan;
@@ -158,21 +174,19 @@ extern int g_debug_withhold;
 extern unsigned long long g_launch_count;
 inline void count_launches(int n) { g_launch_count += static_cast<unsigned long long>(n); }
 
-// Attention over the packed cache + residual: query preparation, the stream kernel, then the merge
-// of the partial records, which also attends to the residual.
+// Attention over the packed cache + residual: the block kernel alone, or the query preparation, the stream kernel and
+// the merge of the partial records, which also attends to the residual.
 cudaError_t launch_decode(const DecodeArgs& a, cudaStream_t stream);
+cudaError_t launch_decode_block(const DecodeArgs& a, cudaStream_t stream);
 // Log-sum-exp merge of n_parts partial sets [n_parts][n_rows][kRecordFloats] into out [n_rows][128].
 cudaError_t launch_merge_partials(const float* parts, int64_t n_parts, int64_t n_rows, void* out, int out_dtype,
                                   cudaStream_t stream);
 // Query preparation (and the step's append) for a.plan.n_chunks chunk-table entries per slab.
-cudaError_t launch_decode_prep(DecodeArgs& a, cudaStream_t stream);
+cudaError_t launch_decode_prep(const DecodeArgs& a, cudaStream_t stream);
 // Persistent warps over 160-token units: caches without / with protected tokens.
 cudaError_t launch_decode_stream(const DecodeArgs& a, cudaStream_t stream);
 cudaError_t launch_decode_stream_stp(const DecodeArgs& a, cudaStream_t stream);
 size_t decode_prep_bytes(int64_t n_slabs, int64_t n_chunks);
-// Write k_new / v_new [n_layers, B, H_kv, D] into row `row` of the residual rings.
-cudaError_t launch_append(int dtype, const void* k_new, const void* v_new, const CacheView& cv, int layer0,
-                          int n_layers, int row, cudaStream_t stream);
 
 // Test-only dequantizers (float32 [B, H_kv, n_quantized, D]).
 cudaError_t launch_dequant_keys(const CacheView& cv, int layer, int64_t T_q0, int64_t n_flush, float* out,

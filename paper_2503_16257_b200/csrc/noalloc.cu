@@ -19,21 +19,31 @@ namespace {
 // that loads this library holds the array until the process exits.
 constexpr size_t kStaticPartialFloats = 4u * 1024u * 1024u;
 static __device__ __align__(256) float g_static_partials[kStaticPartialFloats];
+// Arrival counters of the block kernel's merge tree, cleared by every call.  A slab of n parts has fewer than n
+// join nodes, and the array holds 4032 parts.
+constexpr int kStaticCounters = 4096;
+static __device__ int32_t g_static_counters[kStaticCounters];
 
 constexpr int kMaxDevices = 64;
-float* g_partials_ptr[kMaxDevices] = {};   // device address of the array, per device (set up once)
+struct StaticScratch {
+  float* partials;
+  int32_t* counters;
+};
+StaticScratch g_scratch[kMaxDevices] = {};   // device addresses of the arrays, per device (set up once)
 
-// In host code `g_static_partials` is only a handle for the runtime, not a device address:
-// ask the runtime for the address on the current device and hand that to the kernels.
-vidkv_status_t static_partials(float** out) {
+// In host code the arrays' names are only handles for the runtime, not device addresses:
+// ask the runtime for the addresses on the current device and hand those to the kernel.
+vidkv_status_t static_scratch(StaticScratch* out) {
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return VIDKV_ERR_CUDA;
-  if (!g_partials_ptr[dev]) {
-    void* p = nullptr;
+  if (!g_scratch[dev].partials) {
+    void *p = nullptr, *c = nullptr;
+    if (cudaGetSymbolAddress(&c, g_static_counters) != cudaSuccess || !c) return VIDKV_ERR_CUDA;
     if (cudaGetSymbolAddress(&p, g_static_partials) != cudaSuccess || !p) return VIDKV_ERR_CUDA;
-    g_partials_ptr[dev] = static_cast<float*>(p);
+    g_scratch[dev].counters = static_cast<int32_t*>(c);
+    g_scratch[dev].partials = static_cast<float*>(p);
   }
-  *out = g_partials_ptr[dev];
+  *out = g_scratch[dev];
   return VIDKV_OK;
 }
 
@@ -83,16 +93,27 @@ extern "C" vidkv_status_t vidkv_attend_noalloc(const vidkv_config_t* cfg, const 
   a.partial_out = nullptr;
   const int64_t n_slabs = static_cast<int64_t>(n_layers) * cfg->B * cfg->H_kv;
   a.append_row = -1;
-  a.plan = plan_decode(a.st, n_slabs, n_protected > 0, device_sm_count(), 0);
+  a.plan = plan_decode(a.st, n_slabs, n_protected > 0, cv.kf.general != 0, device_sm_count(), 0);
   // the array holds the partial records, then (256-byte aligned) the per-chunk query images
   const int64_t prep_at = (a.plan.records * kRecordFloats * 4 + 255) / 256 * 256;
   const int64_t prep_bytes = static_cast<int64_t>(decode_prep_bytes(n_slabs, a.plan.n_chunks));
-  if (prep_at + prep_bytes > static_cast<int64_t>(kStaticPartialFloats * sizeof(float))) return VIDKV_ERR_CAPACITY;
-  const vidkv_status_t sp = static_partials(&a.partials);
+  if (prep_at + prep_bytes > static_cast<int64_t>(kStaticPartialFloats * sizeof(float)) ||
+      n_slabs * a.plan.counters_per_slab > kStaticCounters)
+    return VIDKV_ERR_CAPACITY;
+  StaticScratch scratch;
+  const vidkv_status_t sp = static_scratch(&scratch);
   if (sp != VIDKV_OK) return sp;
+  a.partials = scratch.partials;
+  a.counters = scratch.counters;
   a.prep = reinterpret_cast<uint32_t*>(reinterpret_cast<uint8_t*>(a.partials) + prep_at);
+  // every kernel leaves the counters zero; clearing them first keeps a call independent of whatever two calls that
+  // overlapped against the rules may have left behind
+  if (a.plan.counters_per_slab > 0 &&
+      cudaMemsetAsync(a.counters, 0, static_cast<size_t>(n_slabs) * a.plan.counters_per_slab * sizeof(int32_t),
+                      static_cast<cudaStream_t>(stream)) != cudaSuccess)
+    return VIDKV_ERR_CUDA;
   // Every record the merge reads is written by the attention kernel of this same call, so
-  // nothing in the array has to be cleared between calls.
+  // nothing else has to be cleared between calls.
   if (launch_decode(a, static_cast<cudaStream_t>(stream)) != cudaSuccess) return VIDKV_ERR_CUDA;
   return VIDKV_OK;
 }

@@ -152,14 +152,19 @@ static cudaError_t launch_keys_t(const KSrc& src, int64_t T_tokens, const CacheV
   return cudaGetLastError();
 }
 
-__global__ void init_min_kernel(uint32_t* minmax, int n_words, uint32_t* header, uint32_t version) {
+__global__ void init_workspace_kernel(uint32_t* minmax, int n_words, int32_t* counters, int n_counters, uint32_t* header,
+                                      uint32_t version) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n_counters) counters[i] = 0;
   if (i < n_words) minmax[i] = (i & (2 * kD - 1)) < kD ? 0xffffffffu : 0u;
   if (header && i == 0) { header[0] = kMagic; header[1] = version; header[2] = 0u; }
 }
 
-cudaError_t launch_init_minmax(uint32_t* minmax, int64_t n_words, uint32_t* header, uint32_t version, cudaStream_t stream) {
-  init_min_kernel<<<static_cast<unsigned>((n_words + 255) / 256), 256, 0, stream>>>(minmax, static_cast<int>(n_words), header, version);
+cudaError_t launch_init_workspace(uint32_t* minmax, int64_t n_words, int32_t* counters, int64_t n_counters, uint32_t* header,
+                                  uint32_t version, cudaStream_t stream) {
+  const int64_t n = n_words > n_counters ? n_words : n_counters;
+  init_workspace_kernel<<<static_cast<unsigned>((n + 255) / 256), 256, 0, stream>>>(minmax, static_cast<int>(n_words), counters,
+                                                                                   static_cast<int>(n_counters), header, version);
   count_launches(1);
   return cudaGetLastError();
 }

@@ -360,7 +360,7 @@ __global__ void __launch_bounds__(kD) v_flush_kernel(KSrc src, CacheView cv, int
 }
 
 // ---------------------------------------------------------------------------------
-// Residual copies (Algorithm 1: X_r = X[l - r:], and the per-step append).
+// Residual copies (Algorithm 1: X_r = X[l - r:]).
 // ---------------------------------------------------------------------------------
 template <typename T>
 __global__ void copy_to_residual_kernel(KSrc src, int64_t t_begin, int n_tok, CacheView cv, int layer0,
@@ -374,20 +374,6 @@ __global__ void copy_to_residual_kernel(KSrc src, int64_t t_begin, int n_tok, Ca
     const int r = i >> 4, l = i & 15;
     dst[(r0 + r) * 16 + l] = __ldg(reinterpret_cast<const uint4*>(base + (t_begin + r) * src.stride_t) + l);
   }
-}
-
-// One block of 32 threads per (layer, b, h): lanes 0-15 copy the key row, 16-31 the value row.
-__global__ void append_kernel(const uint4* __restrict__ k_new, const uint4* __restrict__ v_new, CacheView cv,
-                              int layer0, int slabs_per_layer, int row) {
-  const int slab = blockIdx.x;
-  const int layer = layer0 + slab / slabs_per_layer;
-  const int bh = slab % slabs_per_layer;
-  uint8_t* sp = cv.slab(layer, bh / cv.H_kv, bh % cv.H_kv);
-  const int l = threadIdx.x & 15;
-  if (threadIdx.x < 16)
-    reinterpret_cast<uint4*>(sp + cv.kres_offset)[row * 16 + l] = __ldg(k_new + static_cast<int64_t>(slab) * 16 + l);
-  else
-    reinterpret_cast<uint4*>(sp + cv.vres_offset)[row * 16 + l] = __ldg(v_new + static_cast<int64_t>(slab) * 16 + l);
 }
 
 // ---------------------------------------------------------------------------------
@@ -580,16 +566,6 @@ cudaError_t launch_copy_to_residual(int dtype, const KSrc& src, int64_t t_begin,
   // 16-bit elements either way: the copy is type-agnostic
   (void)dtype;
   copy_to_residual_kernel<__half><<<n_layers * cv.B * cv.H_kv, 256, 0, stream>>>(src, t_begin, n_tok, cv, layer, off, r0);
-  count_launches(1);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_append(int dtype, const void* k_new, const void* v_new, const CacheView& cv, int layer0,
-                          int n_layers, int row, cudaStream_t stream) {
-  (void)dtype;
-  const int spl = cv.B * cv.H_kv;
-  append_kernel<<<spl * n_layers, 32, 0, stream>>>(static_cast<const uint4*>(k_new), static_cast<const uint4*>(v_new),
-                                                   cv, layer0, spl, row);
   count_launches(1);
   return cudaGetLastError();
 }

@@ -216,6 +216,26 @@ def test_seeded_random_shapes_and_run_lengths(name, T, B, L, p, run_units, steps
     assert pair.cache.status() == 0
 
 
+# ------------------------------------------------------------------ the one-launch kernel of small calls
+@pytest.mark.parametrize("name,L,B,T,p,steps,check_from", [
+    ("tiny", 1, 1, 160, 0.0, 2, 0),          # one unit and a residual block per slab
+    ("qwen", 1, 1, 36000, 0.0, 2, 0),        # 900 units: two to a block, 113 parts and three levels of joins per slab
+    ("tiny", 12, 4, 2029, 0.0, 100, 96),     # 13 units per slab, five to a block, slabs shared by blocks; across a flush
+    ("tiny", 28, 4, 330, 0.0, 3, 0),         # slabs of three units, the last one a single group
+    ("qwen", 1, 1, 163, 0.5, 2, 0),          # protected tokens: one unit per slab
+    ("tiny", 8, 4, 2029, 0.2, 100, 96),      # three units to a block; across a flush
+    ("llava", 1, 2, 26000, 0.93, 2, 0),      # long protected stream, 1304 units
+])
+def test_small_calls_in_one_launch(name, L, B, T, p, steps, check_from):
+    """Calls of up to seven units (three with protected tokens) per block: block and slab boundaries inside and on unit
+    boundaries, the residual with a block of its own and with the slab's last block, every depth of the merge tree."""
+    samples = sorted({(0, 0, 0), (L - 1, B - 1, 3), (L // 2, B // 2, 1)})
+    run = SampledRun(name, L, B, T, p, steps, samples)
+    for s in range(steps):
+        run.decode(check=s >= check_from)
+    assert run.cache.status() == 0
+
+
 # ------------------------------------------------------------------ prompts shorter than one group
 @pytest.mark.parametrize("T", [31, 0])
 def test_flushes_after_a_prompt_with_nothing_to_quantize(T):
