@@ -382,7 +382,7 @@ vidkv_status_t vidkv_attend_noalloc(const vidkv_config_t* cfg, const void* cache
  * beyond floating-point summation order).  Algorithm 1 "Decoding" leaves the evaluation order of
  * Eq. 3 open; the library cuts a decode call into work like this: the quantized tokens of all
  * slabs of the call form one sequence of 160-token units, and every warp of the launch walks a
- * run of `run_units` consecutive units (crossing slab boundaries where its run does) and leaves
+ * run of at most `run_units` consecutive units (crossing slab boundaries where its run does) and leaves
  * one partial result per slab it touches; calls of a few thousand units at most take another
  * kernel, whose blocks walk stretches of units together.
  * vidkv_debug_set_decode_plan forces run_units (>= 1), and with it the first of the two kernels, for later
@@ -390,7 +390,7 @@ vidkv_status_t vidkv_attend_noalloc(const vidkv_config_t* cfg, const void* cache
  * than the workspace holds makes the decode call return VIDKV_ERR_CAPACITY.
  * vidkv_debug_decode_plan (host only) reports the plan for given token counts on a device with
  * sm_count multiprocessors: plan_out[8] = { units per slab, run_units, runs (= warps),
- * records per slab, records needed, records the workspace of `cfg` holds, chunk-table entries,
+ * most runs that touch one slab, records needed, records the workspace of `cfg` holds, chunk-table entries,
  * units in all }. */
 vidkv_status_t vidkv_debug_set_decode_plan(vidkv_cache_t* handle, int32_t run_units);
 vidkv_status_t vidkv_debug_decode_plan(const vidkv_config_t* cfg, int64_t n_prefill_quantized, int64_t n_flushed_chunks,

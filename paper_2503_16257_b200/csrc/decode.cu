@@ -53,16 +53,20 @@ DecodePlan plan_decode(const LayerState& st, int64_t n_slabs, bool stp, bool gen
   if (run < kMinRunUnits) run = kMinRunUnits;
   if (force_run_units > 0) run = force_run_units;
   p.run_units = static_cast<int32_t>(run);
-  p.n_runs = static_cast<int32_t>((p.n_units + run - 1) / run);
-  p.parts_stride = p.units_per_slab > 0 ? static_cast<int32_t>((p.units_per_slab + run - 1) / run) + 1 : 1;
-  p.records = n_slabs * p.parts_stride * kMaxRep;
+  p.n_runs = static_cast<int32_t>(force_run_units > 0 ? (p.n_units + run - 1) / run : (p.n_units < warps ? p.n_units : warps));
+  // a run is n_units / n_runs units long or one more
+  const auto most_parts = [&](int64_t runs) -> int64_t {
+    const int64_t shortest = runs > 0 ? p.n_units / runs : 1;
+    return p.units_per_slab > 0 ? (p.units_per_slab + shortest - 1) / shortest + 1 : 1;
+  };
+  p.slab_parts = static_cast<int32_t>(most_parts(p.n_runs));
+  p.records = (p.n_runs + n_slabs) * kMaxRep;
   const int64_t blocks = static_cast<int64_t>(sms) * (stp && general ? kBlockGenStpPerSM : kBlocksPerSM);
   const int64_t per_block = (p.n_units + blocks - 1) / blocks;
   if (p.n_units == 0 || (per_block <= (stp ? kMaxBlockUnitsStp : kMaxBlockUnits) && force_run_units == 0)) {
-    p.block_units = per_block < run ? static_cast<int32_t>(run) : static_cast<int32_t>(per_block);
-    p.n_blocks = static_cast<int32_t>((p.n_units + p.block_units - 1) / p.block_units);
-    p.res_blocks = st.n_res > 0 && (p.n_units == 0 || p.block_units == 1) ? static_cast<int32_t>(n_slabs) : 0;
-    p.counters_per_slab = static_cast<int32_t>(join_counters(p.parts_stride));
+    p.n_blocks = static_cast<int32_t>(p.n_units < blocks ? p.n_units : blocks);
+    p.res_blocks = st.n_res > 0 && per_block <= 1 ? static_cast<int32_t>(n_slabs) : 0;
+    p.counters_per_slab = static_cast<int32_t>(join_counters(most_parts(p.n_blocks) + (p.res_blocks > 0)));
   }
   return p;
 }
@@ -74,9 +78,8 @@ int64_t max_decode_counters(int64_t max_slabs, int64_t records) {
 
 int64_t max_decode_records(int64_t max_slabs, int64_t max_tokens) {
   if (max_tokens < 1) max_tokens = 1;
-  // parts per slab = ceil(S / run) + 1 with run >= max(1, n_units / warps) (the chooser never goes
-  // below kMinRunUnits, the test hook may force 1), warps >= 8 per multiprocessor, so
-  // slabs * parts <= min(slabs * S, warps + slabs) + slabs for every S.
+  // a call has at most min(units, warps) runs (the test hook may force one unit per run) and leaves fewer than
+  // runs + slabs records; units <= slabs * S.
   const int64_t S = (max_tokens + kStreamUnitTokens - 1) / kStreamUnitTokens;
   const int64_t warps = static_cast<int64_t>(kMaxSMs) * kStreamCtasPerSM * kStreamWarps;
   int64_t parts = max_slabs * S;
@@ -118,15 +121,17 @@ __global__ void __launch_bounds__(kD) decode_merge_kernel(DecodeArgs a, int n_re
   const int h = slab % cv.H_kv, lb = slab / cv.H_kv, rep = cv.rep;
   const uint8_t* slab_ptr = cv.base + cv.slab_offset + (static_cast<int64_t>(a.layer0) * cv.B * cv.H_kv + slab) * cv.slab_stride;
   int n_parts;
+  int64_t first_run = 0;
   {
     const DecodePlan& pl = a.plan;
     if (pl.units_per_slab == 0) n_parts = 0;
     else {
       const int64_t u0 = static_cast<int64_t>(slab) * pl.units_per_slab;
-      n_parts = static_cast<int>((u0 + pl.units_per_slab - 1) / pl.run_units - u0 / pl.run_units) + 1;
+      first_run = pl.run_of(u0);
+      n_parts = static_cast<int>(pl.run_of(u0 + pl.units_per_slab - 1) - first_run) + 1;
     }
   }
-  const float* rec = a.partials + static_cast<int64_t>(slab) * a.plan.parts_stride * (kMaxRep * kRecordFloats);
+  const float* rec = a.partials + (slab + first_run) * (kMaxRep * kRecordFloats);
   pdl_wait();                                              // the partial records come from the attention kernel before
   const int64_t q0 = (static_cast<int64_t>(lb) * cv.H_q + h * rep) * kD;
   // ---- the records' maxima, sums and this lane's output fragments are fetched first, so that their

@@ -70,8 +70,7 @@ template <bool GEN, bool STP> struct Smem {
 // units of the normalised query.  Consecutive products go to different accumulators (the four
 // 8-token tiles, and the chain of the constants in between), so that no product waits for the
 // one issued just before it.
-__device__ __forceinline__ void score_group(const uint8_t* kg, int lane, int hd, int r, const uint4* img, uint32_t m_field,
-                                            uint32_t c_four, uint32_t m_sign, uint32_t c_neg1, float (&sc)[4][2], float& cst) {
+__device__ __forceinline__ void score_group(const uint8_t* kg, int lane, int hd, int r, const uint4* img, float (&sc)[4][2], float& cst) {
   uint32_t s2[8], z2[8], s1[8];
   {
     const uint4 x0 = *reinterpret_cast<const uint4*>(kg + kKG_S2 + 32 * r);
@@ -110,8 +109,8 @@ __device__ __forceinline__ void score_group(const uint8_t* kg, int lane, int hd,
         // fields 2 ks and 2 ks + 1 of the word: shifts by 8 - 4 ks and 6 - 4 ks bits
         const uint32_t f0 = ks == 0 ? w2[nt] << 8 : ks == 1 ? w2[nt] << 4 : ks == 2 ? w2[nt] : wh[nt] << 2;
         const uint32_t f1 = ks == 0 ? w2[nt] << 6 : ks == 1 ? w2[nt] << 2 : ks == 2 ? wh[nt] << 4 : wh[nt];
-        mma_f16(acc[nt], h0, l0, h1, l1, and_or(f0, m_field, c_four),
-                and_or(f1, m_field, c_four));
+        mma_f16(acc[nt], h0, l0, h1, l1, field_or(f0, kFour),
+                field_or(f1, kFour));
       }
     }
   }
@@ -125,7 +124,7 @@ __device__ __forceinline__ void score_group(const uint8_t* kg, int lane, int hd,
 #pragma unroll
       for (int nt = 0; nt < 4; ++nt)
         mma_f16(acc[nt], qv.x, qv.y, qv.z, qv.w,
-                nand_xor(X[nt] << (4 * ks), m_sign, s1[2 * ks]), nand_xor(X[nt] << (4 * ks + 2), m_sign, s1[2 * ks + 1]));
+                signed_by(X[nt] << (4 * ks), s1[2 * ks]), signed_by(X[nt] << (4 * ks + 2), s1[2 * ks + 1]));
     }
   }
   cst = cz[0] - 4.0f * cz[1];
@@ -142,8 +141,7 @@ __device__ __forceinline__ void score_group(const uint8_t* kg, int lane, int hd,
 // with the transformed query; in plain mode the value is code s + z = (+-1) s / 2 + (z + s / 2), so q s
 // (hi + lo) meets +-1, the products are halved at the end and the constant takes sum q z + sum q s / 2.
 __device__ __forceinline__ void score_group_general(const uint8_t* kg, const KeyFmt& kf, int lane, int hd, int r,
-                                                    const uint4* img, uint32_t m_field, uint32_t c_four, uint32_t m_sign,
-                                                    uint32_t c_neg1, float (&sc)[4][2], float& cst) {
+                                                    const uint4* img, float (&sc)[4][2], float& cst) {
   float acc[4][4], acc1[4][4];
 #pragma unroll
   for (int nt = 0; nt < 4; ++nt) {
@@ -174,8 +172,8 @@ __device__ __forceinline__ void score_group_general(const uint8_t* kg, const Key
       mma_f16(cz, qa[2 * kp], 0u, qa[2 * kp + 1], 0u, zw[2 * kp], zw[2 * kp + 1]);
 #pragma unroll
       for (int nt = 0; nt < 4; ++nt)
-        mma_f16(acc[nt], hi[2 * kp], lo[2 * kp], hi[2 * kp + 1], lo[2 * kp + 1], and_or(W[nt] >> (4 * kp), m_field, c_four),
-                and_or(W[nt] >> (4 * kp + 2), m_field, c_four));
+        mma_f16(acc[nt], hi[2 * kp], lo[2 * kp], hi[2 * kp + 1], lo[2 * kp + 1], field_or(W[nt] >> (4 * kp), kFour),
+                field_or(W[nt] >> (4 * kp + 2), kFour));
     }
   }
   const uint4* img1 = img + n2b * 32;
@@ -203,8 +201,8 @@ __device__ __forceinline__ void score_group_general(const uint8_t* kg, const Key
       const uint32_t X = ((cw >> (8 * nt)) & 0xffu) * 0x02000100u;   // low lane: bit 7 at the sign, high lane: bit 6
 #pragma unroll
       for (int kp = 0; kp < 2; ++kp)
-        mma_f16(acc1[nt], ah[2 * kp], al[2 * kp], ah[2 * kp + 1], al[2 * kp + 1], nand_xor(X << (4 * kp), m_sign, sw[2 * kp]),
-                nand_xor(X << (4 * kp + 2), m_sign, sw[2 * kp + 1]));
+        mma_f16(acc1[nt], ah[2 * kp], al[2 * kp], ah[2 * kp + 1], al[2 * kp + 1], signed_by(X << (4 * kp), sw[2 * kp]),
+                signed_by(X << (4 * kp + 2), sw[2 * kp + 1]));
     }
   }
   const float f1 = kf.plain ? 0.5f : 1.0f;
@@ -322,7 +320,7 @@ struct Running {
 // the accumulator fragment P V starts from.
 template <typename PFrag>
 __device__ __forceinline__ void pv_ternary(const uint8_t* vbuf, int w, PFrag P, const float4 (&ps)[kSGGroups], Running& run, int hd,
-                                           int r, uint32_t m_field, uint32_t c_four) {
+                                           int r) {
   uint32_t W[2][8];
 #pragma unroll
   for (int kt = 0; kt < 2; ++kt) {
@@ -347,7 +345,7 @@ __device__ __forceinline__ void pv_ternary(const uint8_t* vbuf, int w, PFrag P, 
         // Next W = 3 * (W - digit << 8) = 3 W - 3 A + 3 * 0x4400 (no lane ever borrows).
         // Half of the lanes take that route (two multiply-adds), the other half mask the digit
         // away and multiply (one logic, one multiply-add): the two pipes share the work.
-        A[k] = and_or(W[kt][k], m_field, c_four);
+        A[k] = field_or(W[kt][k], kFour);
         if (g + 1 < kSGGroups) {
           if (k & 1) W[kt][k] = mad_u32(A[k], 0xfffffffdu, mad_u32(W[kt][k], 3u, 0xcc00cc00u));
           else W[kt][k] = mad_u32(W[kt][k] & 0x00ff00ffu, 3u, 0u);
@@ -376,8 +374,7 @@ __device__ __forceinline__ void pv_ternary(const uint8_t* vbuf, int w, PFrag P, 
 
 // P V of one protected group (Eq. 4 codes as 4 + code) for the 32 channels of warp w: P4[nt] = probabilities of
 // head hd at the group's tokens 8 nt + 2 r, + 1.  out += s * (sum (4 + code) p - 4 sum p) + z * sum p.
-__device__ __forceinline__ void pv_protected(const uint8_t* pg, int w, const uint32_t (&P4)[4], Running& run, int hd, int r,
-                                             uint32_t m_field, uint32_t c_four) {
+__device__ __forceinline__ void pv_protected(const uint8_t* pg, int w, const uint32_t (&P4)[4], Running& run, int hd, int r) {
   float cq[4] = {0.0f, 0.0f, 0.0f, 0.0f};               // -4 * (sum of the probabilities) of heads 2 r, 2 r + 1
   mma_f16(cq, kMinus4, kMinus4, kMinus4, kMinus4, P4[0], P4[1]);
   mma_f16(cq, kMinus4, kMinus4, kMinus4, kMinus4, P4[2], P4[3]);
@@ -392,14 +389,14 @@ __device__ __forceinline__ void pv_protected(const uint8_t* pg, int w, const uin
   for (int kt = 0; kt < 2; ++kt) {
     const uint32_t wd = wk[kt], wh = wd >> 6;
     uint32_t x[8];
-    x[0] = and_or(wd << 8, m_field, c_four);
-    x[1] = and_or(wd << 6, m_field, c_four);
-    x[2] = and_or(wd << 4, m_field, c_four);
-    x[3] = and_or(wd << 2, m_field, c_four);
-    x[4] = and_or(wd, m_field, c_four);
-    x[5] = and_or(wh << 4, m_field, c_four);
-    x[6] = and_or(wh << 2, m_field, c_four);
-    x[7] = and_or(wh, m_field, c_four);
+    x[0] = field_or(wd << 8, kFour);
+    x[1] = field_or(wd << 6, kFour);
+    x[2] = field_or(wd << 4, kFour);
+    x[3] = field_or(wd << 2, kFour);
+    x[4] = field_or(wd, kFour);
+    x[5] = field_or(wh << 4, kFour);
+    x[6] = field_or(wh << 2, kFour);
+    x[7] = field_or(wh, kFour);
     const uint32_t b0 = P4[2 * kt], b1 = P4[2 * kt + 1];
     if (kt == 0) {
       mma_f16_c(acc[0], x[0], x[1], x[4], x[5], b0, b1, cq[0], cq[1], cq[2], cq[3]);
@@ -590,10 +587,10 @@ __device__ __forceinline__ void store_result(const DecodeArgs& a, int slab, cons
     }
   }
 }
-// One part of a slab is done.  The only part writes the result; otherwise it leaves its record and arrives at its
+// Part `part` of a slab is done; block `first` has part 0.  The only part writes the result; otherwise it leaves its record and arrives at its
 // node of the join tree, and the last to arrive goes on with the joined record.  Whole block; `flag` is a shared word.
 // The counters are zero between calls (the last arrival clears its node's).
-__device__ __forceinline__ void finish_part(const DecodeArgs& a, int slab, int part, int n_parts, const Running& run, volatile int* flag,
+__device__ __forceinline__ void finish_part(const DecodeArgs& a, int slab, int first, int part, int n_parts, const Running& run, volatile int* flag,
                                             int warp, int lane) {
   const int hd = lane >> 2, r = lane & 3;
   Part p;
@@ -602,7 +599,7 @@ __device__ __forceinline__ void finish_part(const DecodeArgs& a, int slab, int p
   p.l[0] = run.l[0]; p.l[1] = run.l[1];
 #pragma unroll
   for (int j = 0; j < 8; ++j) p.o[j] = run.o[j];
-  float* rec = a.partials + static_cast<int64_t>(slab) * a.plan.parts_stride * kPartFloats;
+  float* rec = a.partials + static_cast<int64_t>(slab + first) * kPartFloats;
   int32_t* cnt = a.counters + static_cast<int64_t>(slab) * a.plan.counters_per_slab;
   int64_t stride = kPartFloats;
   while (n_parts > 1) {
@@ -653,22 +650,23 @@ __global__ void __launch_bounds__(kUnitThreads, GEN && STP ? kBlockGenStpPerSM :
   uint8_t* const slab0 = cv.base + cv.slab_offset + static_cast<int64_t>(a.layer0) * cv.B * cv.H_kv * cv.slab_stride;
   const bool live = hd < cv.rep;
   auto query_row = [&](int slab) { return reinterpret_cast<const T*>(a.q) + (static_cast<int64_t>(slab / cv.H_kv) * cv.H_q + (slab % cv.H_kv) * cv.rep + hd) * kD; };
-  auto unit_parts = [&](int slab) { return static_cast<int>(((slab + 1u) * n_slab_units - 1u) / pl.block_units - static_cast<unsigned>(slab) * n_slab_units / pl.block_units) + 1; };
+  // block b owns the units [b * units / blocks, (b + 1) * units / blocks)
+  const uint32_t n_units = static_cast<uint32_t>(pl.n_units), n_blocks = static_cast<uint32_t>(pl.n_blocks);
+  auto block_of = [&](uint32_t u) { return static_cast<int>(((u + 1u) * n_blocks - 1u) / n_units); };
   Running run;
   // everything below may depend on the kernel before this one in the stream
   pdl_wait();
   pdl_release();
   if (static_cast<int>(blockIdx.x) >= pl.n_blocks) {
     // a residual of its own (blocks that own one unit each, or nothing quantized yet)
-    const int slab = blockIdx.x - pl.n_blocks, parts = n_slab_units ? unit_parts(slab) : 0;
+    const int slab = blockIdx.x - pl.n_blocks, first = slab * n_slab_units;   // one unit per block
     run.reset();
     add_residual<T>(a, slab, slab0 + static_cast<int64_t>(slab) * cv.slab_stride, query_row(slab), live, sm + S::prob_at, warp, lane, run);
-    finish_part(a, slab, parts, parts + 1, run, &flag, warp, lane);
+    finish_part(a, slab, first, n_slab_units, n_slab_units + 1, run, &flag, warp, lane);
     return;
   }
-  const uint32_t m_field = kExpand[0], c_four = kExpand[1], m_sign = kExpand[2], c_neg1 = kExpand[3];
-  const int u_begin = static_cast<int>(blockIdx.x) * pl.block_units;
-  const int n_local = min(pl.block_units, static_cast<int>(pl.n_units) - u_begin);
+  const int u_begin = static_cast<int>(blockIdx.x * n_units / n_blocks);
+  const int n_local = static_cast<int>((blockIdx.x + 1u) * n_units / n_blocks) - u_begin;
   // token and stream positions fit 32 bits (the layout's group counts do)
   const int T_q0 = static_cast<int>(a.st.T_q0), T_qt = T_q0 + static_cast<int>(a.st.n_flush) * kR;
   const int n_groups = T_qt / kG, g0n = T_q0 / kG;
@@ -772,7 +770,7 @@ __global__ void __launch_bounds__(kUnitThreads, GEN && STP ? kBlockGenStpPerSM :
 #pragma unroll
         for (int g = 0; g < kSGGroups; ++g) ps[g] = psum[unit & 1][g][r];
         pv_ternary(sm + S::v_at + (unit & 1) * kVBufBytes, warp,
-                   [&](int g, int nt) { return *reinterpret_cast<const uint32_t*>(prow + g * (kG * 2) + nt * 16); }, ps, run, hd, r, m_field, c_four);
+                   [&](int g, int nt) { return *reinterpret_cast<const uint32_t*>(prow + g * (kG * 2) + nt * 16); }, ps, run, hd, r);
       };
       auto multiply_streams = [&](int u_done, int p_done) {
         const uint8_t* trow = sm + S::prob_at + hd * kRingRow + 4 * r;
@@ -791,7 +789,7 @@ __global__ void __launch_bounds__(kUnitThreads, GEN && STP ? kBlockGenStpPerSM :
                 mma_f16(c, kMinus5, kMinus5, kMinus5, kMinus5, P(g, 2), P(g, 3));
                 ps[g] = make_float4(c[0], c[1], c[2], c[3]);
               }
-              pv_ternary(sm + S::v_at + (vcnt & 1) * kVBufBytes, warp, P, ps, run, hd, r, m_field, c_four);
+              pv_ternary(sm + S::v_at + (vcnt & 1) * kVBufBytes, warp, P, ps, run, hd, r);
             }
           }
           ++sg_next; ++vcnt;
@@ -805,7 +803,7 @@ __global__ void __launch_bounds__(kUnitThreads, GEN && STP ? kBlockGenStpPerSM :
 #pragma unroll
               for (int nt = 0; nt < 4; ++nt)
                 P4[nt] = *reinterpret_cast<const uint32_t*>(trow + (kTRing + ((pg_next * kG) & (kPRing - 1))) * 2 + nt * 16);
-              pv_protected(sm + S::p_at + pslot * kPGBytes, warp, P4, run, hd, r, m_field, c_four);
+              pv_protected(sm + S::p_at + pslot * kPGBytes, warp, P4, run, hd, r);
             }
           }
           ++pg_next;
@@ -848,8 +846,8 @@ __global__ void __launch_bounds__(kUnitThreads, GEN && STP ? kBlockGenStpPerSM :
           if (warp < ng) {
             const uint8_t* kg = sm + S::k_at + (i & 1) * S::kKBuf + warp * kgb;
             const uint4* img = reinterpret_cast<const uint4*>(sm + S::img_at + (chunk_of(g_first + warp) & 1) * kImgBytes) + lane;
-            if (GEN) score_group_general(kg, kf, lane, hd, r, img, m_field, c_four, m_sign, c_neg1, sc, cst);
-            else score_group(kg, lane, hd, r, img, m_field, c_four, m_sign, c_neg1, sc, cst);
+            if (GEN) score_group_general(kg, kf, lane, hd, r, img, sc, cst);
+            else score_group(kg, lane, hd, r, img, sc, cst);
             gm = fmaxf(fmaxf(fmaxf(sc[0][0], sc[0][1]), fmaxf(sc[1][0], sc[1][1])), fmaxf(fmaxf(sc[2][0], sc[2][1]), fmaxf(sc[3][0], sc[3][1])));
             gm = fmaxf(gm, __shfl_xor_sync(0xffffffffu, gm, 1));
             gm = fmaxf(gm, __shfl_xor_sync(0xffffffffu, gm, 2)) + cst;
@@ -958,8 +956,8 @@ __global__ void __launch_bounds__(kUnitThreads, GEN && STP ? kBlockGenStpPerSM :
     } else {
       i += k_end - k;
     }
-    const int first = static_cast<int>(static_cast<unsigned>(slab) * n_slab_units / pl.block_units);
-    finish_part(a, slab, static_cast<int>(blockIdx.x) - first, unit_parts(slab) + (pl.res_blocks ? 1 : 0), run, &flag, warp, lane);
+    const int first = block_of(static_cast<uint32_t>(slab) * n_slab_units), last = block_of((slab + 1u) * n_slab_units - 1u);
+    finish_part(a, slab, first, static_cast<int>(blockIdx.x) - first, last - first + 1 + (pl.res_blocks ? 1 : 0), run, &flag, warp, lane);
     k = 0;
     ++slab;
   }

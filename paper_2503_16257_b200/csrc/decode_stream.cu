@@ -47,8 +47,7 @@ struct Running {
 // 8-token tiles, and the chain of the constants in between), so that no product waits for the
 // one issued just before it.
 __device__ __forceinline__ void score_group(const uint8_t* kg, int lane, int hd, int r, const uint32_t (&qa)[8],
-                                            const uint32_t (&qha)[8], const uint32_t (&qhb)[8], uint32_t m_field,
-                                            uint32_t c_four, uint32_t m_sign, uint32_t c_neg1, float (&sc)[4][2],
+                                            const uint32_t (&qha)[8], const uint32_t (&qhb)[8], float (&sc)[4][2],
                                             float& cst) {
   uint32_t s2[8], z2[8], s1[8];
   {
@@ -91,8 +90,8 @@ __device__ __forceinline__ void score_group(const uint8_t* kg, int lane, int hd,
         // fields 2 ks and 2 ks + 1 of the word: shifts by 8 - 4 ks and 6 - 4 ks bits
         const uint32_t f0 = ks == 0 ? w2[nt] << 8 : ks == 1 ? w2[nt] << 4 : ks == 2 ? w2[nt] : wh[nt] << 2;
         const uint32_t f1 = ks == 0 ? w2[nt] << 6 : ks == 1 ? w2[nt] << 2 : ks == 2 ? wh[nt] << 4 : wh[nt];
-        mma_f16(acc[nt], hi2[2 * ks], lo2[2 * ks], hi2[2 * ks + 1], lo2[2 * ks + 1], and_or(f0, m_field, c_four),
-                and_or(f1, m_field, c_four));
+        mma_f16(acc[nt], hi2[2 * ks], lo2[2 * ks], hi2[2 * ks + 1], lo2[2 * ks + 1], field_or(f0, kFour),
+                field_or(f1, kFour));
       }
     }
   }
@@ -105,7 +104,7 @@ __device__ __forceinline__ void score_group(const uint8_t* kg, int lane, int hd,
 #pragma unroll
       for (int nt = 0; nt < 4; ++nt)
         mma_f16(acc[nt], qha[2 * ks], qhb[2 * ks], qha[2 * ks + 1], qhb[2 * ks + 1],
-                nand_xor(X[nt] << (4 * ks), m_sign, s1[2 * ks]), nand_xor(X[nt] << (4 * ks + 2), m_sign, s1[2 * ks + 1]));
+                signed_by(X[nt] << (4 * ks), s1[2 * ks]), signed_by(X[nt] << (4 * ks + 2), s1[2 * ks + 1]));
     }
   }
   cst = cz[0] - 4.0f * cz[1];
@@ -122,8 +121,7 @@ __device__ __forceinline__ void score_group(const uint8_t* kg, int lane, int hd,
 // with the transformed query; in plain mode the value is code s + z = (+-1) s / 2 + (z + s / 2), so q s
 // (hi + lo) meets +-1, the products are halved at the end and the constant takes sum q z + sum q s / 2.
 __device__ __forceinline__ void score_group_general(const uint8_t* kg, const KeyFmt& kf, int lane, int hd, int r,
-                                                    const uint32_t* pp, uint32_t m_field, uint32_t c_four, uint32_t m_sign,
-                                                    uint32_t c_neg1, float (&sc)[4][2], float& cst) {
+                                                    const uint32_t* pp, float (&sc)[4][2], float& cst) {
   float acc[4][4], acc1[4][4];
 #pragma unroll
   for (int nt = 0; nt < 4; ++nt) {
@@ -153,8 +151,8 @@ __device__ __forceinline__ void score_group_general(const uint8_t* kg, const Key
       mma_f16(cz, qa[2 * kp], 0u, qa[2 * kp + 1], 0u, zw[2 * kp], zw[2 * kp + 1]);
 #pragma unroll
       for (int nt = 0; nt < 4; ++nt)
-        mma_f16(acc[nt], hi[2 * kp], lo[2 * kp], hi[2 * kp + 1], lo[2 * kp + 1], and_or(W[nt] >> (4 * kp), m_field, c_four),
-                and_or(W[nt] >> (4 * kp + 2), m_field, c_four));
+        mma_f16(acc[nt], hi[2 * kp], lo[2 * kp], hi[2 * kp + 1], lo[2 * kp + 1], field_or(W[nt] >> (4 * kp), kFour),
+                field_or(W[nt] >> (4 * kp + 2), kFour));
     }
   }
   const int w1 = kf.n2 >> 3, nw1 = (kD - kf.n2) >> 3;
@@ -188,8 +186,8 @@ __device__ __forceinline__ void score_group_general(const uint8_t* kg, const Key
       const uint32_t X = ((cw >> (8 * nt)) & 0xffu) * 0x02000100u;   // low lane: bit 7 at the sign, high lane: bit 6
 #pragma unroll
       for (int kp = 0; kp < 2; ++kp)
-        mma_f16(acc1[nt], ah[2 * kp], al[2 * kp], ah[2 * kp + 1], al[2 * kp + 1], nand_xor(X << (4 * kp), m_sign, sw[2 * kp]),
-                nand_xor(X << (4 * kp + 2), m_sign, sw[2 * kp + 1]));
+        mma_f16(acc1[nt], ah[2 * kp], al[2 * kp], ah[2 * kp + 1], al[2 * kp + 1], signed_by(X << (4 * kp), sw[2 * kp]),
+                signed_by(X << (4 * kp + 2), sw[2 * kp + 1]));
     }
   }
   const float f1 = kf.plain ? 0.5f : 1.0f;
@@ -211,8 +209,7 @@ __device__ __forceinline__ void score_group_general(const uint8_t* kg, const Key
 // hd + 8.  Adds into the warp's running output.
 template <int NG>
 __device__ __forceinline__ void pv_ternary(const uint8_t* vbuf, float* totbuf, const uint32_t (&P)[NG][4],
-                                           const float (&ps)[NG][4], int lane, int hd, int r, uint32_t m_field,
-                                           uint32_t c_four) {
+                                           const float (&ps)[NG][4], int lane, int hd, int r) {
 #pragma unroll 1
   for (int w = 0; w < 4; ++w) {
     float acc[NG][2][4];
@@ -236,7 +233,7 @@ __device__ __forceinline__ void pv_ternary(const uint8_t* vbuf, float* totbuf, c
           // Next W = 3 * (W - digit << 8) = 3 W - 3 A + 3 * 0x4400 (no lane ever borrows).
           // Half of the lanes take that route (two multiply-adds), the other half mask the digit
           // away and multiply (one logic, one multiply-add): the two pipes share the work.
-          A[k] = and_or(W[k], m_field, c_four);
+          A[k] = field_or(W[k], kFour);
           if (g + 1 < NG) {
             if (k & 1) W[k] = mad_u32(A[k], 0xfffffffdu, mad_u32(W[k], 3u, 0xcc00cc00u));
             else W[k] = mad_u32(W[k] & 0x00ff00ffu, 3u, 0u);
@@ -278,7 +275,6 @@ __device__ __forceinline__ bool process_unit(const KeyFmt& kf, const uint32_t*& 
                                              uint32_t (&qa)[8], uint32_t (&qha)[8], uint32_t (&qhb)[8], float sl2,
                                              Running& run, bool more, const uint8_t* next_k, uint32_t next_k_bytes,
                                              const uint8_t* next_v) {
-  const uint32_t m_field = kExpand[0], c_four = kExpand[1], m_sign = kExpand[2], c_neg1 = kExpand[3];
   const int kgb = GEN ? kf.group_bytes : kKGroupBytes;      // bytes of one key group
   if (!mbar_wait(kbar, kpar)) return false;
   kpar ^= 1u;
@@ -305,8 +301,8 @@ __device__ __forceinline__ bool process_unit(const KeyFmt& kf, const uint32_t*& 
     }
     float sc[4][2], cst;
     uint8_t* kg = kbuf + g * kgb;
-    if (GEN) score_group_general(kg, kf, lane, hd, r, ppc, m_field, c_four, m_sign, c_neg1, sc, cst);
-    else score_group(kg, lane, hd, r, qa, qha, qhb, m_field, c_four, m_sign, c_neg1, sc, cst);
+    if (GEN) score_group_general(kg, kf, lane, hd, r, ppc, sc, cst);
+    else score_group(kg, lane, hd, r, qa, qha, qhb, sc, cst);
     __syncwarp();                                           // every lane has read the group's bytes
     float gm = fmaxf(sc[0][0], sc[0][1]);
 #pragma unroll
@@ -369,7 +365,7 @@ __device__ __forceinline__ bool process_unit(const KeyFmt& kf, const uint32_t*& 
     return false;
   }
   vpar ^= 1u;
-  pv_ternary<NG>(vbuf, totbuf, P, ps, lane, hd, r, m_field, c_four);
+  pv_ternary<NG>(vbuf, totbuf, P, ps, lane, hd, r);
   __syncwarp();
   if (more && lane == 0) {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -380,10 +376,8 @@ __device__ __forceinline__ bool process_unit(const KeyFmt& kf, const uint32_t*& 
 
 __device__ __forceinline__ void write_record(const DecodeArgs& a, int slab, int run_id, int lane, int hd, int r,
                                              const Running& run, const float* totbuf) {
-  const DecodePlan& pl = a.plan;
   const int rep = a.cv.rep;
-  const int first = static_cast<int>(static_cast<int64_t>(slab) * pl.units_per_slab / pl.run_units);
-  float* rec = a.partials + (static_cast<int64_t>(slab) * pl.parts_stride + (run_id - first)) * (kMaxRep * kRecordFloats);
+  float* rec = a.partials + static_cast<int64_t>(slab + run_id) * (kMaxRep * kRecordFloats);
 #pragma unroll
   for (int w = 0; w < 4; ++w)
 #pragma unroll
@@ -416,8 +410,8 @@ __global__ void __launch_bounds__(kStreamWarps * 32, kStreamCtasPerSM) decode_st
   const DecodePlan& pl = a.plan;
   const CacheView& cv = a.cv;
   const int run_id = blockIdx.x * kStreamWarps + warp;
-  const int64_t u_begin = static_cast<int64_t>(run_id) * pl.run_units;
-  const int64_t u_end = min(u_begin + pl.run_units, pl.n_units);
+  const int64_t u_begin = pl.run_begin(run_id);
+  const int64_t u_end = run_id < pl.n_runs ? pl.run_begin(run_id + 1) : u_begin;
   if (u_begin >= u_end) return;                            // warps do not wait on one another
   const KeyFmt& kf = a.cv.kf;
   const int kgb = GEN ? kf.group_bytes : kKGroupBytes;
@@ -533,7 +527,7 @@ constexpr int kStpWarpBytes = kKBufBytes + kVBufBytes + kPGBytes + kTotBytes + 8
 // P V of one protected group (Eq. 4 codes as 4 + code): P4[nt] = probabilities of head hd at
 // the group's tokens 8 nt + 2 r, + 1.  out += s * (sum (4 + code) p - 4 sum p) + z * sum p.
 __device__ __forceinline__ void pv_protected(const uint8_t* pg, float* totbuf, const uint32_t (&P4)[4], float (&l)[2],
-                                             int lane, int hd, int r, uint32_t m_field, uint32_t c_four) {
+                                             int lane, int hd, int r) {
   float cq[4] = {0.0f, 0.0f, 0.0f, 0.0f};               // -4 * (sum of the probabilities) of heads 2 r, 2 r + 1
   mma_f16(cq, kMinus4, kMinus4, kMinus4, kMinus4, P4[0], P4[1]);
   mma_f16(cq, kMinus4, kMinus4, kMinus4, kMinus4, P4[2], P4[3]);
@@ -550,14 +544,14 @@ __device__ __forceinline__ void pv_protected(const uint8_t* pg, float* totbuf, c
     for (int kt = 0; kt < 2; ++kt) {
       const uint32_t wd = wk[kt], wh = wd >> 6;
       uint32_t x[8];
-      x[0] = and_or(wd << 8, m_field, c_four);
-      x[1] = and_or(wd << 6, m_field, c_four);
-      x[2] = and_or(wd << 4, m_field, c_four);
-      x[3] = and_or(wd << 2, m_field, c_four);
-      x[4] = and_or(wd, m_field, c_four);
-      x[5] = and_or(wh << 4, m_field, c_four);
-      x[6] = and_or(wh << 2, m_field, c_four);
-      x[7] = and_or(wh, m_field, c_four);
+      x[0] = field_or(wd << 8, kFour);
+      x[1] = field_or(wd << 6, kFour);
+      x[2] = field_or(wd << 4, kFour);
+      x[3] = field_or(wd << 2, kFour);
+      x[4] = field_or(wd, kFour);
+      x[5] = field_or(wh << 4, kFour);
+      x[6] = field_or(wh << 2, kFour);
+      x[7] = field_or(wh, kFour);
       const uint32_t b0 = P4[2 * kt], b1 = P4[2 * kt + 1];
       if (kt == 0) {
         mma_f16_c(acc[0], x[0], x[1], x[4], x[5], b0, b1, cq[0], cq[1], cq[2], cq[3]);
@@ -602,8 +596,8 @@ __global__ void __launch_bounds__(kStreamWarps * 32, kStreamStpCtasPerSM) decode
   const DecodePlan& pl = a.plan;
   const CacheView& cv = a.cv;
   const int run_id = blockIdx.x * kStreamWarps + warp;
-  const int64_t u_begin = static_cast<int64_t>(run_id) * pl.run_units;
-  const int64_t u_end = min(u_begin + pl.run_units, pl.n_units);
+  const int64_t u_begin = pl.run_begin(run_id);
+  const int64_t u_end = run_id < pl.n_runs ? pl.run_begin(run_id + 1) : u_begin;
   if (u_begin >= u_end) return;
   const KeyFmt& kf = a.cv.kf;
   const int kgb = GEN ? kf.group_bytes : kKGroupBytes;
@@ -624,7 +618,6 @@ __global__ void __launch_bounds__(kStreamWarps * 32, kStreamStpCtasPerSM) decode
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncwarp();
-  const uint32_t m_field = kExpand[0], c_four = kExpand[1], m_sign = kExpand[2], c_neg1 = kExpand[3];
   const int S = pl.units_per_slab;
   // token and stream positions fit 32 bits (the layout's group counts do)
   const int T_q0 = static_cast<int>(a.st.T_q0), T_qt = T_q0 + static_cast<int>(a.st.n_flush) * kR;
@@ -734,8 +727,8 @@ __global__ void __launch_bounds__(kStreamWarps * 32, kStreamStpCtasPerSM) decode
       }
       float sc[4][2], cst;
       uint8_t* kg = kbuf + g * kgb;
-      if (GEN) score_group_general(kg, kf, lane, hd, r, ppc, m_field, c_four, m_sign, c_neg1, sc, cst);
-      else score_group(kg, lane, hd, r, qa, qha, qhb, m_field, c_four, m_sign, c_neg1, sc, cst);
+      if (GEN) score_group_general(kg, kf, lane, hd, r, ppc, sc, cst);
+      else score_group(kg, lane, hd, r, qa, qha, qhb, sc, cst);
       __syncwarp();
       float gm = fmaxf(sc[0][0], sc[0][1]);
 #pragma unroll
@@ -845,7 +838,7 @@ __global__ void __launch_bounds__(kStreamWarps * 32, kStreamStpCtasPerSM) decode
         run.l[0] = fmaf(-0.2f, ps[g][0], run.l[0]);
         run.l[1] = fmaf(-0.2f, ps[g][1], run.l[1]);
       }
-      pv_ternary<kSGGroups>(vbuf, totbuf, P, ps, lane, hd, r, m_field, c_four);
+      pv_ternary<kSGGroups>(vbuf, totbuf, P, ps, lane, hd, r);
       ++sg_next;
       __syncwarp();
       if (sg_next < sg_total) {
@@ -865,7 +858,7 @@ __global__ void __launch_bounds__(kStreamWarps * 32, kStreamStpCtasPerSM) decode
       const uint8_t* rp = myrow + kPRingAt + ((pg_next % 6) * kG + 2 * r) * 2;
 #pragma unroll
       for (int nt = 0; nt < 4; ++nt) P4[nt] = *reinterpret_cast<const uint32_t*>(rp + 8 * nt * 2);
-      pv_protected(pbuf, totbuf, P4, run.l, lane, hd, r, m_field, c_four);
+      pv_protected(pbuf, totbuf, P4, run.l, lane, hd, r);
       ++pg_next;
       __syncwarp();
       if (pg_next < pg_total) {

@@ -107,22 +107,26 @@ constexpr int kJoin = 8;           // records joined at a node of the block kern
 
 // How one attention call over n_slabs slabs is cut into work (host side, decode.cu): the
 // quantized tokens of all slabs form one sequence of 160-token units (units_per_slab each).
-//   stream kernel  warp number w of the launch walks the units [w * run_units, (w + 1) * run_units) and leaves one
-//                  partial record per slab it touches, record (slab, w - first warp of the slab).
-//   block kernel   (n_blocks > 0 or nothing quantized: small calls) block b walks the units [b * block_units,
-//                  (b + 1) * block_units), at least one run; records are numbered the same way, and joined by a tree
-//                  of eight-way nodes.
-// parts_stride = records reserved per slab; the partials buffer holds n_slabs * parts_stride * 8
-// records of kRecordFloats floats.
+//   stream kernel  warp number w of the launch walks the units [w * units / runs, (w + 1) * units / runs), all
+//                  warps that fit the device taking part: runs of equal length, rounded up, left some multiprocessors a
+//                  whole block short (8960 units on 1776 warps as 1494 runs of 6: 76.5 us a step, now 70).  It leaves
+//                  one partial record per slab it touches, record slab + w: from one record to the next the slab or
+//                  the warp number goes up, so the records need no more room than there are runs and slabs.
+//   block kernel   (small calls: n_blocks > 0 or res_blocks > 0) the same with blocks in place of warps; the records
+//                  of a slab are joined by a tree of eight-way nodes.
 struct DecodePlan {
-  int32_t units_per_slab, run_units, n_runs;
+  int32_t units_per_slab;
+  int32_t run_units;       // units of the longest run
+  int32_t n_runs;
   int64_t n_units;
-  int32_t parts_stride;
+  int32_t slab_parts;      // most runs that can touch one slab
   int32_t n_chunks;        // chunk-table entries the query preparation covers (0: nothing quantized)
-  int64_t records;         // n_slabs * parts_stride * 8
-  int32_t block_units, n_blocks;
+  int64_t records;         // records of one query head: (n_runs + n_slabs) * 8
+  int32_t n_blocks;
   int32_t res_blocks;      // blocks that attend to a slab's residual alone: n_slabs or 0 (the slab's last block does it)
   int32_t counters_per_slab;   // arrival counters of the merge tree
+  __host__ __device__ int64_t run_begin(int64_t w) const { return w * n_units / n_runs; }
+  __host__ __device__ int64_t run_of(int64_t u) const { return ((u + 1) * n_runs - 1) / n_units; }
 };
 // stp: the cache holds protected tokens (the stream kernel for them keeps fewer warps per multiprocessor).
 // general: a key format other than the default.
@@ -141,7 +145,7 @@ struct DecodeArgs {
   const void* k_new;
   const void* v_new;
   void* out;
-  float* partials;     // [n_slabs][parts_stride][8 heads][kRecordFloats]
+  float* partials;     // [n_runs + n_slabs][8 heads][kRecordFloats]
   uint32_t* prep;      // stream kernel: per (slab, chunk) query images (decode_prep_bytes)
   int32_t* counters;   // block kernel: [n_slabs][counters_per_slab], zero between calls
   DftTables dft;       // set by launch_decode
