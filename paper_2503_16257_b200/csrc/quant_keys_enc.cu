@@ -117,14 +117,23 @@ __device__ __forceinline__ uint64_t umma_desc_sw128(uint32_t smem_addr) {
   return static_cast<uint64_t>((smem_addr >> 4) & 0x3fffu) | (static_cast<uint64_t>(1u) << 16) |
          (static_cast<uint64_t>(1024u >> 4) << 32) | (static_cast<uint64_t>(1u) << 46) | (static_cast<uint64_t>(2u) << 61);
 }
-constexpr int kTmemCols = 256;        // two float32 accumulators of 128 x 128
+constexpr int kTmemCols = 256;        // two tiles' float32 accumulators of 128 x 128
 constexpr int kWaitLimit = 1 << 14;
 
-__device__ __forceinline__ void umma_f16(uint32_t tmem_d, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
+// One lane of a converged warp.  Issued behind this in a warp-uniform branch an MMA takes the tensor pipe's own time
+// (66 clocks at N = 128); behind "if (threadIdx.x == 0)" its operands take a slower way: 49 clocks and more for any N.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{ .reg .pred q; elect.sync _|q, 0xffffffff; selp.u32 %0, 1, 0, q; }" : "=r"(p));
+  return p != 0;
+}
+// off_lo / off_hi: all ones keeps the accumulator rows 0 .. 63 / 64 .. 127 as they are.
+__device__ __forceinline__ void umma_f16(uint32_t tmem_d, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate,
+                                         uint32_t off_lo, uint32_t off_hi) {
   asm volatile(
       "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, {%5, %5, %5, %5}, p;\n\t}"
-      ::"r"(tmem_d), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(0u)
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, {%5, %5, %6, %6}, p;\n\t}"
+      ::"r"(tmem_d), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(off_lo), "r"(off_hi)
       : "memory");
 }
 // 32 consecutive accumulator columns of the calling warp's 32 lanes of tensor memory.
@@ -200,7 +209,7 @@ __global__ void __launch_bounds__(256, 2) k_encode_kernel(KSrc src, int64_t T_to
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(perm + kD + 8);
   volatile uint32_t* fault = reinterpret_cast<volatile uint32_t*>(perm + kD + 12);
 
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
   const int quad = warp & 3, half = warp >> 2;
   // Row arrangement of the A operand: 0 puts the anomalous slots in rows 0 .. 63 and the DFT
   // columns in rows 64 .. 127, 1 the other way round.  The two blocks that share an SM (b and
@@ -252,8 +261,56 @@ __global__ void __launch_bounds__(256, 2) k_encode_kernel(KSrc src, int64_t T_to
     if (++lti == tiles_per_slab) { lti = 0; ++lslab; }
   };
 
+  // ---- D[128 rows x 128 tokens] = the smaller parts of the DFT rows x tile^T (the 64 rows those parts do not have read
+  // neighbouring shared memory and are masked out of the accumulator), then A (leading) x tile^T on top: small terms first,
+  // which keeps the sums as close to exact as two accumulators that are added at the end
+  const int issuer = arr ? 0 : 2;                            // one of the loading warps
+  auto issue = [&](int buf) {
+    if (elect_one()) {
+      constexpr uint32_t idesc = (1u << 4) | (static_cast<uint32_t>(Enc<T>::kFmt) << 7) | (static_cast<uint32_t>(Enc<T>::kFmt) << 10) |
+                                 ((128u >> 3) << 17) | ((128u >> 4) << 24);
+      const uint32_t d = tmem + static_cast<uint32_t>(buf * 128);
+      const uint32_t off_lo = arr ? 0u : 0xffffffffu, off_hi = ~off_lo;   // the selector rows / (off_hi, off_lo): the DFT rows
+#pragma unroll
+      for (int part = Enc<T>::kParts - 1; part >= 1; --part) {
+#pragma unroll
+        for (int kb = 0; kb < 2; ++kb) {
+          // the part's 64 rows are rows 64 .. 127 of arrangement 0 (start 8192 bytes early), rows 0 .. 63 of arrangement 1
+          const uint64_t da = umma_desc_sw128(smem_u32(a_ex + (part - 1) * 16384 + kb * 8192 - (arr ? 0 : 8192)));
+          const uint64_t db = umma_desc_sw128(smem_u32(tile + kb * 16384));
+#pragma unroll
+          for (int ks = 0; ks < 4; ++ks)   // 16 elements = 32 bytes along K per step; the address field counts 16 bytes
+            umma_f16(d, da + static_cast<uint64_t>(2 * ks), db + static_cast<uint64_t>(2 * ks), idesc,
+                     part < Enc<T>::kParts - 1 || (kb | ks) != 0 ? 1u : 0u, off_lo, off_hi);
+        }
+      }
+#pragma unroll
+      for (int kb = 0; kb < 2; ++kb) {
+        const uint64_t da = umma_desc_sw128(smem_u32(a_hi + kb * 16384)), db = umma_desc_sw128(smem_u32(tile + kb * 16384));
+        // the first step starts the selector rows and goes on top of the small parts in the DFT rows
+        if (kb == 0) umma_f16(d, da, db, idesc, 0u, off_hi, off_lo);
+        if (kb == 0) umma_f16(d, da, db, idesc, 1u, off_lo, off_hi);
+#pragma unroll
+        for (int ks = kb == 0 ? 1 : 0; ks < 4; ++ks)
+          umma_f16(d, da + static_cast<uint64_t>(2 * ks), db + static_cast<uint64_t>(2 * ks), idesc, 1u, 0u, 0u);
+      }
+      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(mbar)) : "memory");
+    }
+    __syncwarp();
+  };
+  auto accumulators_ready = [&](uint32_t parity) -> bool {
+    uint32_t done = 0;
+    for (int it = 0; it < kWaitLimit && !done; ++it) {
+      asm volatile(
+          "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+          : "=r"(done) : "r"(smem_u32(mbar)), "r"(parity) : "memory");
+    }
+    return __all_sync(0xffffffffu, done != 0);
+  };
+
   int cur_slab = -1;
   uint32_t phase = 0;
+  bool ahead = false;                                        // this tile's products are issued already
   uint8_t* slab_ptr = nullptr;
   if (loader && tile_begin < tile_end) load_next_tile();
   for (int t = tile_begin; t < tile_end; ++t, ti = (ti + 1 == tiles_per_slab) ? 0 : ti + 1, slab += (ti == 0) ? 1 : 0) {
@@ -270,80 +327,69 @@ __global__ void __launch_bounds__(256, 2) k_encode_kernel(KSrc src, int64_t T_to
     // ---- a new slab: its channel order and the A operand built from it
     if (slab != cur_slab) {
       cur_slab = slab;
+      // eight entries of the matrix per load, all in flight before anything else (one by one they cost the block 16 memory
+      // latencies, as long as a tile)
+      uint4 wv[Enc<T>::kParts][2];
+#pragma unroll
+      for (int part = 0; part < Enc<T>::kParts; ++part)
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+          wv[part][j] = __ldg(reinterpret_cast<const uint4*>(g_dft_w + (Enc<T>::kTab + part) * 4096) + tid + 256 * j);
       if (tid < kD) perm[tid] = slab_ptr[cv.chunk_table_offset + static_cast<int64_t>(chunk) * kChunkBytes + tid];
       constexpr int kAVec = (32768 + 16384 * (Enc<T>::kParts - 1)) / 16;
+#pragma unroll 4
       for (int i = tid; i < kAVec; i += 256) reinterpret_cast<uint4*>(a_ex)[i] = make_uint4(0u, 0u, 0u, 0u);
       __syncthreads();
       if (tid < kNA) {
         const int c = perm[tid];
         *reinterpret_cast<uint16_t*>(a_hi + (c >> 6) * 16384 + sw128_offset(64 * arr + tid, c & 63)) = Enc<T>::kOne;
       }
-      for (int i = tid; i < 64 * 64; i += 256) {
-        const int f = i >> 6, c = perm[kNA + (i & 63)];
-        *reinterpret_cast<uint16_t*>(a_hi + (c >> 6) * 16384 + sw128_offset(64 - 64 * arr + f, c & 63)) = g_dft_w[Enc<T>::kTab * 4096 + i];
 #pragma unroll
-        for (int part = 1; part < Enc<T>::kParts; ++part)
-          *reinterpret_cast<uint16_t*>(a_ex + (part - 1) * 16384 + (c >> 6) * 8192 + sw128_offset(f, c & 63)) =
-              g_dft_w[(Enc<T>::kTab + part) * 4096 + i];
-      }
-    }
-
-    // ---- the tile has landed; the accumulators of the previous tile have been read
-    if (loader) asm volatile("cp.async.wait_group 0;" ::: "memory");
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (*fault) break;
-
-    // ---- D[128 rows x 128 tokens] = A (leading) x tile^T; D'[.. x ..] = A (remaining parts) x tile^T
-    // (withhold_first, a test hook: the block's first tile gets neither products nor a commit, so the
-    // wait below runs out with nothing outstanding)
-    if (tid == 0 && !(withhold_first && t == tile_begin)) {
-      constexpr uint32_t idesc = (1u << 4) | (static_cast<uint32_t>(Enc<T>::kFmt) << 7) | (static_cast<uint32_t>(Enc<T>::kFmt) << 10) |
-                                 ((128u >> 3) << 17) | ((128u >> 4) << 24);
+      for (int j = 0; j < 2; ++j) {
+        const int v = tid + 256 * j, f = v >> 3;               // entries 8 (v % 8) .. + 7 of column f
+        const uint2 pc = *reinterpret_cast<const uint2*>(perm + kNA + 8 * (v & 7));
 #pragma unroll
-      for (int kb = 0; kb < 2; ++kb) {
-        const uint64_t da = umma_desc_sw128(smem_u32(a_hi + kb * 16384)), db = umma_desc_sw128(smem_u32(tile + kb * 16384));
+        for (int x = 0; x < 8; ++x) {
+          const int c = ((x < 4 ? pc.x : pc.y) >> (8 * (x & 3))) & 0xff;
+          const int hi_at = (c >> 6) * 16384 + sw128_offset(64 - 64 * arr + f, c & 63), ex_at = (c >> 6) * 8192 + sw128_offset(f, c & 63);
 #pragma unroll
-        for (int ks = 0; ks < 4; ++ks)   // 16 elements = 32 bytes along K per step; the address field counts 16 bytes
-          umma_f16(tmem, da + static_cast<uint64_t>(2 * ks), db + static_cast<uint64_t>(2 * ks), idesc, (kb | ks) != 0 ? 1u : 0u);
-      }
-#pragma unroll
-      for (int part = 1; part < Enc<T>::kParts; ++part) {
-#pragma unroll
-        for (int kb = 0; kb < 2; ++kb) {
-          // the part's 64 rows are rows 64 .. 127 of arrangement 0 (start 8192 bytes early), rows 0 .. 63 of arrangement 1
-          const uint64_t da = umma_desc_sw128(smem_u32(a_ex + (part - 1) * 16384 + kb * 8192 - (arr ? 0 : 8192)));
-          const uint64_t db = umma_desc_sw128(smem_u32(tile + kb * 16384));
-#pragma unroll
-          for (int ks = 0; ks < 4; ++ks)
-            umma_f16(tmem + 128u, da + static_cast<uint64_t>(2 * ks), db + static_cast<uint64_t>(2 * ks), idesc,
-                     (part - 1) | kb | ks ? 1u : 0u);
+          for (int part = 0; part < Enc<T>::kParts; ++part) {
+            const uint4& q = wv[part][j];
+            const uint32_t word = x < 2 ? q.x : x < 4 ? q.y : x < 6 ? q.z : q.w;
+            const uint16_t val = static_cast<uint16_t>((x & 1) ? word >> 16 : word);
+            if (part == 0) *reinterpret_cast<uint16_t*>(a_hi + hi_at) = val;
+            else *reinterpret_cast<uint16_t*>(a_ex + (part - 1) * 16384 + ex_at) = val;
+          }
         }
       }
-      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(mbar)) : "memory");
     }
+
+    // ---- this tile's products were issued behind the epilogue of the tile before, unless its operand A is new
+    if (!ahead && loader) asm volatile("cp.async.wait_group 0;" ::: "memory");
+    if (!ahead) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();                                           // and everyone has read the accumulators of the tile before
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (*fault) break;
+    // (withhold_first, a test hook: the block's first tile gets neither products nor a commit, so the
+    // wait below runs out with nothing outstanding)
+    if (!ahead && warp == issuer && !(withhold_first && t == tile_begin)) issue((t - tile_begin) & 1);
     // every thread waits for the accumulators; the wait is bounded, a timeout is reported in the status word
-    uint32_t done = 0;
-    for (int it = 0; it < kWaitLimit && !done; ++it) {
-      asm volatile(
-          "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-          : "=r"(done) : "r"(smem_u32(mbar)), "r"(phase) : "memory");
-    }
+    const bool done = accumulators_ready(phase);
     phase ^= 1u;
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    done = __all_sync(0xffffffffu, done != 0);
-    if (!done) {
-      if (lane == 0) {
-        *fault = 1u;
-        atomicCAS(reinterpret_cast<int*>(cv.base + kHdrStatus), 0, static_cast<int>(VIDKV_ERR_TIMEOUT));
-      }
-      continue;
+    if (!done && lane == 0) {
+      *fault = 1u;
+      atomicCAS(reinterpret_cast<int*>(cv.base + kHdrStatus), 0, static_cast<int>(VIDKV_ERR_TIMEOUT));
     }
     // the products are done with shared memory: fetch the next tile behind the epilogue
-    if (loader && t + 1 < tile_end) load_next_tile();
-
+    const bool more = t + 1 < tile_end;
+    if (loader && more) load_next_tile();
+    ahead = more && ti + 1 < tiles_per_slab;                   // the next tile has the same operand A
+    const uint32_t acc = tmem + static_cast<uint32_t>(((t - tile_begin) & 1) * 128);
+    if (!done) {
+      // nothing to encode; the loading warps still meet below
+    } else
     if (!loader) {
       // ---- Eq. 4: lane = anomalous slot j, the accumulator row holds its 128 tokens (exact values)
       const int j = (quad & 1) * 32 + lane, wg = j >> 4;
@@ -354,7 +400,7 @@ __global__ void __launch_bounds__(256, 2) k_encode_kernel(KSrc src, int64_t T_to
 #pragma unroll 1
       for (int g = 2 * half; g < 2 * half + 2 && g < n_groups; ++g) {
         uint32_t x[32];
-        tmem_ld32(tmem + (static_cast<uint32_t>(quad * 32) << 16) + static_cast<uint32_t>(g * 32), x);
+        tmem_ld32(acc + (static_cast<uint32_t>(quad * 32) << 16) + static_cast<uint32_t>(g * 32), x);
         float fmn = __uint_as_float(x[0]), fmx = fmn;
 #pragma unroll
         for (int i = 1; i < 32; ++i) { fmn = fminf(fmn, __uint_as_float(x[i])); fmx = fmaxf(fmx, __uint_as_float(x[i])); }
@@ -426,16 +472,14 @@ __global__ void __launch_bounds__(256, 2) k_encode_kernel(KSrc src, int64_t T_to
       const int hq = quad & 1, f = hq * 32 + lane;
 #pragma unroll 1
       for (int g = 2 * half; g < 2 * half + 2 && g < n_groups; ++g) {
-        uint32_t xa[32], xb[32];
-        tmem_ld32(tmem + (static_cast<uint32_t>(quad * 32) << 16) + static_cast<uint32_t>(g * 32), xa);
-        tmem_ld32(tmem + (static_cast<uint32_t>(quad * 32) << 16) + static_cast<uint32_t>(128 + g * 32), xb);
+        uint32_t xa[32];
+        tmem_ld32(acc + (static_cast<uint32_t>(quad * 32) << 16) + static_cast<uint32_t>(g * 32), xa);
         float sum = 0.0f;
         uint32_t bits = 0u;   // bit i = sign bit of the column's coefficient of token i
 #pragma unroll
         for (int i = 31; i >= 0; --i) {
-          const float X = __uint_as_float(xa[i]) + __uint_as_float(xb[i]);
-          sum += fabsf(X);
-          bits = __funnelshift_l(__float_as_uint(X), bits, 1);
+          sum += fabsf(__uint_as_float(xa[i]));
+          bits = __funnelshift_l(xa[i], bits, 1);
         }
         uint8_t* kg = kg_base + g * kKGroupBytes;
         reinterpret_cast<uint16_t*>(kg + kKG_S1)[f] = f2h_bits(sum * (1.0f / 32.0f));
@@ -458,8 +502,16 @@ __global__ void __launch_bounds__(256, 2) k_encode_kernel(KSrc src, int64_t T_to
         hw[hidx + 4] = static_cast<uint16_t>(mine);
       }
     }
+    if (loader && ahead) {
+      // the next tile has landed: its products run while the anomalous warps are still at this one's codes
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      asm volatile("bar.sync 1, 128;" ::: "memory");           // the four loading warps
+      if (warp == issuer) issue((t + 1 - tile_begin) & 1);
+    }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   }
+  if (ahead) accumulators_ready(phase);                        // left early: the products that are under way land first
   if (loader) asm volatile("cp.async.wait_group 0;" ::: "memory");
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
