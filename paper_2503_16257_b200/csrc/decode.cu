@@ -41,7 +41,7 @@ static int64_t join_counters(int64_t n) {
   return c;
 }
 
-DecodePlan plan_decode(const LayerState& st, int64_t n_slabs, bool stp, bool general, int sm_count, int force_run_units) {
+DecodePlan plan_decode(const LayerState& st, int64_t n_slabs, bool stp, bool general, int sm_count, int force_run_units, bool partial) {
   DecodePlan p = {};
   const int64_t T_qt = st.T_q0 + st.n_flush * kR;
   p.n_chunks = T_qt > 0 ? 1 + static_cast<int32_t>(st.n_flush) : 0;
@@ -53,17 +53,18 @@ DecodePlan plan_decode(const LayerState& st, int64_t n_slabs, bool stp, bool gen
   if (run < kMinRunUnits) run = kMinRunUnits;
   if (force_run_units > 0) run = force_run_units;
   p.run_units = static_cast<int32_t>(run);
-  p.n_runs = static_cast<int32_t>(force_run_units > 0 ? (p.n_units + run - 1) / run : (p.n_units < warps ? p.n_units : warps));
+  if (partial) p.equal_units = p.run_units;
+  p.n_runs = static_cast<int32_t>(force_run_units > 0 || partial ? (p.n_units + run - 1) / run : (p.n_units < warps ? p.n_units : warps));
   // a run is n_units / n_runs units long or one more
   const auto most_parts = [&](int64_t runs) -> int64_t {
-    const int64_t shortest = runs > 0 ? p.n_units / runs : 1;
+    const int64_t shortest = p.equal_units > 0 ? p.equal_units : runs > 0 ? p.n_units / runs : 1;
     return p.units_per_slab > 0 ? (p.units_per_slab + shortest - 1) / shortest + 1 : 1;
   };
   p.slab_parts = static_cast<int32_t>(most_parts(p.n_runs));
   p.records = (p.n_runs + n_slabs) * kMaxRep;
   const int64_t blocks = static_cast<int64_t>(sms) * (stp && general ? kBlockGenStpPerSM : kBlocksPerSM);
   const int64_t per_block = (p.n_units + blocks - 1) / blocks;
-  if (p.n_units == 0 || (per_block <= (stp ? kMaxBlockUnitsStp : kMaxBlockUnits) && force_run_units == 0)) {
+  if (p.n_units == 0 || (per_block <= (stp ? kMaxBlockUnitsStp : kMaxBlockUnits) && force_run_units == 0 && (!partial || run == 1))) {
     p.n_blocks = static_cast<int32_t>(p.n_units < blocks ? p.n_units : blocks);
     p.res_blocks = st.n_res > 0 && per_block <= 1 ? static_cast<int32_t>(n_slabs) : 0;
     p.counters_per_slab = static_cast<int32_t>(join_counters(most_parts(p.n_blocks) + (p.res_blocks > 0)));

@@ -300,10 +300,11 @@ __device__ __forceinline__ void make_images(uint32_t* img, const KeyFmt& kf, con
 // to warps 0-3: o[4 i + c] = channel 32 w + 4 (lane / 4) + 2 i + c / 2, head 2 (lane % 4) + c % 2.
 struct Running {
   float m;
+  float exact;         // what m would be if it followed every unit's maximum (for the triples of a token shard)
   float l[2];
   float o[8];
   __device__ __forceinline__ void reset() {
-    m = -INFINITY; l[0] = 0.0f; l[1] = 0.0f;
+    m = -INFINITY; exact = -INFINITY; l[0] = 0.0f; l[1] = 0.0f;
 #pragma unroll
     for (int j = 0; j < 8; ++j) o[j] = 0.0f;
   }
@@ -471,6 +472,7 @@ __device__ __forceinline__ void add_residual(const DecodeArgs& a, int slab, uint
   mu = fmaxf(mu, __shfl_xor_sync(0xffffffffu, mu, 1));
   mu = fmaxf(mu, __shfl_xor_sync(0xffffffffu, mu, 2));
   float fa, fb, f;
+  run.exact = fmaxf(run.exact, mu);
   if (move_maximum(mu, false, r, run.m, fa, fb, f)) run.scale(fa, fb);
   const int n_pad = (n_res + 15) & ~15;
   for (int t = 8 * r + 32 * warp; warp < 4 && t < n_pad; t += kR) {
@@ -590,9 +592,14 @@ __device__ __forceinline__ void store_result(const DecodeArgs& a, int slab, cons
 // Part `part` of a slab is done; block `first` has part 0.  The only part writes the result; otherwise it leaves its record and arrives at its
 // node of the join tree, and the last to arrive goes on with the joined record.  Whole block; `flag` is a shared word.
 // The counters are zero between calls (the last arrival clears its node's).
-__device__ __forceinline__ void finish_part(const DecodeArgs& a, int slab, int first, int part, int n_parts, const Running& run, volatile int* flag,
+__device__ __forceinline__ void finish_part(const DecodeArgs& a, int slab, int first, int part, int n_parts, Running& run, volatile int* flag,
                                             int warp, int lane) {
   const int hd = lane >> 2, r = lane & 3;
+  if (a.partial_out) {
+    const float f = exp2f(run.m - run.exact);
+    run.scale(__shfl_sync(0xffffffffu, f, 8 * r), __shfl_sync(0xffffffffu, f, 8 * r + 4));
+    run.m = run.exact;
+  }
   Part p;
   p.m[0] = __shfl_sync(0xffffffffu, run.m, 8 * r);
   p.m[1] = __shfl_sync(0xffffffffu, run.m, 8 * r + 4);
@@ -867,6 +874,7 @@ __global__ void __launch_bounds__(kUnitThreads, GEN && STP ? kBlockGenStpPerSM :
         float fa, fb, f;
         const float4 ga = *reinterpret_cast<const float4*>(&gmax[i & 1][hd][0]);
         const float mu = fmaxf(fmaxf(fmaxf(ga.x, ga.y), fmaxf(ga.z, ga.w)), gmax[i & 1][hd][4]) * sl2;   // sl2 > 0
+        run.exact = fmaxf(run.exact, STP ? ceilf(mu) : mu);
         const bool moved = move_maximum(mu, STP, r, run.m, fa, fb, f);
         const float off = fmaf(cst, sl2, -run.m);
         if (!STP) {

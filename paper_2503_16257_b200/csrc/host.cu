@@ -446,7 +446,7 @@ static vidkv_status_t decode_impl(vidkv_cache_t* h, int32_t layer_begin, int32_t
   a.withhold = 0;
   a.st.T_q0 = first.T_q0; a.st.n_flush = first.n_flush; a.st.n_res = first.n_res + (append ? 1 : 0);
   const int64_t n_slabs = static_cast<int64_t>(n_layers) * h->cfg.B * h->cfg.H_kv;
-  a.plan = plan_decode(a.st, n_slabs, h->n_prot > 0, h->cv.kf.general != 0, device_sm_count(), h->dbg_run_units);
+  a.plan = plan_decode(a.st, n_slabs, h->n_prot > 0, h->cv.kf.general != 0, device_sm_count(), h->dbg_run_units, partial != nullptr);
   if (a.plan.records > h->ws.partial_entries || n_slabs * a.plan.counters_per_slab > h->ws.counter_words) return VIDKV_ERR_CAPACITY;
   if (launch_decode(a, s) != cudaSuccess) return VIDKV_ERR_CUDA;
   if (!append) return VIDKV_OK;

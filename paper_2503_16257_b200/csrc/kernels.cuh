@@ -125,13 +125,21 @@ struct DecodePlan {
   int32_t n_blocks;
   int32_t res_blocks;      // blocks that attend to a slab's residual alone: n_slabs or 0 (the slab's last block does it)
   int32_t counters_per_slab;   // arrival counters of the merge tree
-  __host__ __device__ int64_t run_begin(int64_t w) const { return w * n_units / n_runs; }
-  __host__ __device__ int64_t run_of(int64_t u) const { return ((u + 1) * n_runs - 1) / n_units; }
+  int32_t equal_units;     // > 0: runs of exactly this many units (the last one shorter) instead of a proportional share
+  __host__ __device__ int64_t run_begin(int64_t w) const {
+    if (equal_units > 0) return w * equal_units < n_units ? w * equal_units : n_units;
+    return w * n_units / n_runs;
+  }
+  __host__ __device__ int64_t run_of(int64_t u) const { return equal_units > 0 ? u / equal_units : ((u + 1) * n_runs - 1) / n_units; }
 };
 // stp: the cache holds protected tokens (the stream kernel for them keeps fewer warps per multiprocessor).
 // general: a key format other than the default.
 // force_run_units: 0 = choose; otherwise the test hook's value (always the stream kernel).
-DecodePlan plan_decode(const LayerState& st, int64_t n_slabs, bool stp, bool general, int sm_count, int force_run_units);
+// partial: the call leaves (maximum, sum, unnormalised output) triples.  Their maximum is the one the walk has kept, which
+// need not be the largest logit, so it depends on how the units are cut: such calls keep runs of equal length, and take the
+// block kernel only where every run is one unit (its maximum is then exact however blocks share the units).
+DecodePlan plan_decode(const LayerState& st, int64_t n_slabs, bool stp, bool general, int sm_count, int force_run_units,
+                       bool partial = false);
 // Arrival counters any call that needs at most `records` records on at most max_slabs slabs uses.
 int64_t max_decode_counters(int64_t max_slabs, int64_t records);
 // Largest `records` any call on at most max_slabs slabs and max_tokens tokens can plan.
