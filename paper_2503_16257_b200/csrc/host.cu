@@ -350,11 +350,11 @@ vidkv_status_t vidkv_quantize_keys_layers(vidkv_cache_t* h, int32_t layer_begin,
   KSrc src{K, stride_b, stride_h, stride_t, h->cfg.H_kv};
   if (T_q > 0) {
     const MinMaxBuffers mm = next_minmax(h, static_cast<int64_t>(n_layers) * h->cfg.B * h->cfg.H_kv);
-    if (launch_quantize_keys(h->cfg.in_dtype, src, T_q, h->cv, layer_begin, n_layers, 0, 0, mm, s) != cudaSuccess)
+    if (launch_quantize_keys(h->cfg.in_dtype, src, T_q, r, h->cv, layer_begin, n_layers, 0, 0, mm, s) != cudaSuccess)
       return VIDKV_ERR_CUDA;
-  }
-  if (launch_copy_to_residual(h->cfg.in_dtype, src, T_q, r, h->cv, layer_begin, n_layers, false, 0, s) != cudaSuccess)
+  } else if (launch_copy_to_residual(src, r, h->cv, layer_begin, n_layers, false, s) != cudaSuccess) {
     return VIDKV_ERR_CUDA;
+  }
   for (int l = layer_begin; l < layer_begin + n_layers; ++l) {
     LayerInfo& li = h->layers[l];
     li.k_done = true; li.T = T; li.T_q0 = T_q; li.n_res = r; li.n_flush = 0;
@@ -391,11 +391,10 @@ vidkv_status_t vidkv_quantize_values_layers(vidkv_cache_t* h, int32_t layer_begi
     sel.stride_rest = h->cfg.max_prefill_tokens;
     sel.n_prot = h->n_prot;
   }
-  if (T_q > 0 && launch_quantize_values(h->cfg.in_dtype, src, T_q, h->cv, layer_begin, n_layers, sel, h->cfg.gamma,
-                                        h->cfg.ternary_scale == VIDKV_TERNARY_SCALE_NONZERO_MEAN, s) != cudaSuccess)
-    return VIDKV_ERR_CUDA;
-  if (launch_copy_to_residual(h->cfg.in_dtype, src, T_q, r, h->cv, layer_begin, n_layers, true, 0, s) != cudaSuccess)
-    return VIDKV_ERR_CUDA;
+  const cudaError_t e = T_q > 0 ? launch_quantize_values(h->cfg.in_dtype, src, T_q, r, h->cv, layer_begin, n_layers, sel, h->cfg.gamma,
+                                                         h->cfg.ternary_scale == VIDKV_TERNARY_SCALE_NONZERO_MEAN, s)
+                                : launch_copy_to_residual(src, r, h->cv, layer_begin, n_layers, true, s);
+  if (e != cudaSuccess) return VIDKV_ERR_CUDA;
   for (int l = layer_begin; l < layer_begin + n_layers; ++l) {
     LayerInfo& li = h->layers[l];
     li.v_done = true; li.T = T; li.T_q0 = T_q; li.n_res = r; li.n_flush = 0;
@@ -459,7 +458,7 @@ static vidkv_status_t decode_impl(vidkv_cache_t* h, int32_t layer_begin, int32_t
     const MinMaxBuffers mm = next_minmax(h, static_cast<int64_t>(n_layers) * h->cfg.B * h->cfg.H_kv);
     const int chunk = 1 + static_cast<int>(first.n_flush);
     const int64_t kgroup0 = first.T_q0 / kG + (kR / kG) * first.n_flush;
-    if (launch_quantize_keys(dt, ksrc, kR, h->cv, layer_begin, n_layers, chunk, kgroup0, mm, s) != cudaSuccess)
+    if (launch_quantize_keys(dt, ksrc, kR, 0, h->cv, layer_begin, n_layers, chunk, kgroup0, mm, s) != cudaSuccess)
       return VIDKV_ERR_CUDA;
     const int64_t n_rest = first.T_q0 - h->n_prot;
     const int64_t tgroup0 = (n_rest + kG - 1) / kG + (kR / kG) * first.n_flush;

@@ -5,6 +5,24 @@
 
 namespace vidkv {
 
+// Programmatic dependent launch: a kernel launched with the stream-serialization attribute may start
+// while the kernel before it still runs; pdl_wait() returns once that kernel has completed and its
+// writes are visible (a no-op for an ordinary launch), pdl_release() lets the kernel after this one start.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// Launch `kernel` so that it may overlap the tail of the previous kernel on `stream` (it must call pdl_wait()
+// before touching anything that kernel writes).
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr; cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
 // A [slabs, tokens, 128] source of keys or values.  Source slab i (= b * H + h, running
 // over layers first when several layers are processed) starts at
 // ptr + (i / H) * stride_b + (i % H) * stride_h elements; token t at + t * stride_t.
@@ -13,6 +31,17 @@ struct KSrc {
   int64_t stride_b, stride_h, stride_t;
   int32_t H;
 };
+
+// Algorithm 1: X_r = X[l - r:].  Rows t_begin .. t_begin + n_tok - 1 of source slab `slab` into the residual ring at
+// res_offset of its cache slab, rows 0 on; called by a whole block (16-bit elements either way: the copy is type-agnostic).
+__device__ __forceinline__ void copy_residual_rows(const KSrc& src, int64_t t_begin, int n_tok, const CacheView& cv, int layer0, int slab,
+                                                   int64_t res_offset) {
+  const int lb = slab / cv.H_kv, h = slab % cv.H_kv;
+  const uint16_t* base = static_cast<const uint16_t*>(src.ptr) + static_cast<int64_t>(lb) * src.stride_b + h * src.stride_h;
+  uint4* dst = reinterpret_cast<uint4*>(cv.slab(layer0 + lb / cv.B, lb % cv.B, h) + res_offset);
+  for (int i = threadIdx.x; i < n_tok * 16; i += blockDim.x)
+    dst[i] = __ldg(reinterpret_cast<const uint4*>(base + (t_begin + (i >> 4)) * src.stride_t) + (i & 15));
+}
 
 // Token-selection data handed to the value quantizer (NULL lists = no protection).
 struct SelView {
@@ -38,15 +67,17 @@ cudaError_t launch_init_workspace(uint32_t* minmax, int64_t n_words, int32_t* co
 // Algorithm 3 on `T_tokens` tokens (a multiple of 32) of every slab of layers
 // [layer0, layer0 + n_layers): writes chunk `chunk` of the chunk table and the key groups
 // starting at group index kgroup0.
-cudaError_t launch_quantize_keys(int dtype, const KSrc& src, int64_t T_tokens, const CacheView& cv, int layer0,
+// n_res rows that follow (0..31) are copied to the residual.
+cudaError_t launch_quantize_keys(int dtype, const KSrc& src, int64_t T_tokens, int n_res, const CacheView& cv, int layer0,
                                  int n_layers, int chunk, int64_t kgroup0, const MinMaxBuffers& mm, cudaStream_t stream);
 
-// Encode pass of Algorithm 3 for `n_slabs` slabs whose channel split (chunk table entry
-// `chunk`) is already written.
+// Channel split and encode pass of Algorithm 3 for `n_slabs` slabs whose channel ranges are in mm.cur; launched behind the
+// range pass.  Writes the chunk table entry `chunk` too, and re-arms mm.next.
 cudaError_t launch_encode_keys(int dtype, const KSrc& src, int64_t T_tokens, const CacheView& cv, int layer0, int n_slabs,
-                               int slabs_per_layer, int chunk, int64_t kgroup0, cudaStream_t stream);
+                               int slabs_per_layer, int chunk, int64_t kgroup0, const MinMaxBuffers& mm, cudaStream_t stream);
 
-// The same for the general key formats (other k, plain 1-bit code): one block per 32-token group.
+// Encode pass for the general key formats (other k, plain 1-bit code), whose channel split (chunk table entry `chunk`) is
+// already written.
 cudaError_t launch_encode_keys_general(int dtype, const KSrc& src, int64_t T_tokens, const CacheView& cv, int layer0,
                                        int n_slabs, int slabs_per_layer, int chunk, int64_t kgroup0, cudaStream_t stream);
 
@@ -64,7 +95,8 @@ cudaError_t dft_tables(DftTables* tables, cudaStream_t stream);
 
 // Algorithm 2 on the prefill tokens of n_layers layers (source slabs run over layers, then b, then h).  T_q (multiple of 32) tokens; the
 // unprotected ones go to ternary stream positions 0.., the protected ones to 2-bit groups.
-cudaError_t launch_quantize_values(int dtype, const KSrc& src, int64_t T_q, const CacheView& cv, int layer, int n_layers,
+// n_res rows that follow the T_q are copied to the residual.
+cudaError_t launch_quantize_values(int dtype, const KSrc& src, int64_t T_q, int n_res, const CacheView& cv, int layer, int n_layers,
                                    const SelView& sel, float gamma, bool nonzero_mean_scale, cudaStream_t stream);
 
 // 1.58Quant of a full 128-token residual of every slab of the given layers, appended at
@@ -72,10 +104,9 @@ cudaError_t launch_quantize_values(int dtype, const KSrc& src, int64_t T_q, cons
 cudaError_t launch_flush_values(int dtype, const KSrc& src, const CacheView& cv, int layer0, int n_layers,
                                 int64_t tgroup0, float gamma, bool nonzero_mean_scale, cudaStream_t stream);
 
-// Copy `n_tok` tokens starting at token t_begin of every slab of one layer into the
-// residual rings (rows r0 .. r0 + n_tok - 1); n_layers layers from `layer` on.
-cudaError_t launch_copy_to_residual(int dtype, const KSrc& src, int64_t t_begin, int n_tok, const CacheView& cv,
-                                    int layer, int n_layers, bool is_value, int r0, cudaStream_t stream);
+// A prompt shorter than one group: all of its n_tok tokens into the residual rings.
+cudaError_t launch_copy_to_residual(const KSrc& src, int n_tok, const CacheView& cv, int layer, int n_layers, bool is_value,
+                                    cudaStream_t stream);
 
 // Token selection (Sec. 3.3(2)): top-n by saliency, E words + prefix counts into the cache,
 // gather lists into the workspace.

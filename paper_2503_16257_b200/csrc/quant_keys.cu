@@ -1,8 +1,8 @@
 // Key quantizer kernels: Algorithm 3 (MixQuant) of the paper.
 //   k_range_kernel   per-channel min / max over the tokens of a chunk        (range)
-//   k_select_kernel  top-64 channels by range -> D-mask / N-mask as id lists (TopK)
-// The encode pass (Eq. 4 on the anomalous channels, DFT + sign / mean-abs code of Eq. 5 on
-// the rest) lives in quant_keys_enc.cu.
+//   k_select_kernel  top channels by range -> D-mask / N-mask as id lists (TopK), general key formats
+// The encode pass (TopK, Eq. 4 on the anomalous channels, DFT + sign / mean-abs code of Eq. 5 on
+// the rest) of the default format lives in quant_keys_enc.cu.
 #include <type_traits>
 
 #include "common.cuh"
@@ -29,11 +29,17 @@ template <> struct Pair2<__nv_bfloat16> {
 };
 
 template <typename T>
-__global__ void __launch_bounds__(256) k_range_kernel(KSrc src, int64_t T_tokens, int tokens_per_block,
-                                                      uint32_t* __restrict__ minmax) {
+__global__ void __launch_bounds__(256) k_range_kernel(KSrc src, int64_t T_tokens, int tokens_per_block, int splits, int n_res,
+                                                      CacheView cv, int layer0, uint32_t* __restrict__ minmax) {
   using P = Pair2<T>;
   using V = typename P::V;
   const int slab = blockIdx.y;
+  pdl_wait();
+  pdl_release();                                           // the encode pass may set itself up beside this one
+  if (static_cast<int>(blockIdx.x) == splits) {            // one more block per slab for the tokens that stay as they are
+    copy_residual_rows(src, T_tokens, n_res, cv, layer0, slab, cv.kres_offset);
+    return;
+  }
   const T* base = reinterpret_cast<const T*>(src.ptr) + (slab / src.H) * src.stride_b + (slab % src.H) * src.stride_h;
   const int lane16 = threadIdx.x & 15, row = threadIdx.x >> 4;
   const int64_t t0 = static_cast<int64_t>(blockIdx.x) * tokens_per_block;
@@ -88,7 +94,8 @@ __global__ void __launch_bounds__(256) k_range_kernel(KSrc src, int64_t T_tokens
 }
 
 // ---------------------------------------------------------------------------------
-// Channel selection.  One block of 128 threads per slab.  rank(c) = number of channels
+// Channel selection for the general key formats (the default format's encoder does it itself).  One block of 128 threads
+// per slab.  rank(c) = number of channels
 // that come before c in (range descending, index ascending) order; the first 64 are
 // the anomalous ones.  Writes the chunk-table entry: 64 anomalous ids ascending, then
 // 64 normal ids ascending.
@@ -132,7 +139,7 @@ __global__ void __launch_bounds__(kD) k_select_kernel(const uint32_t* __restrict
 // Host launchers
 // ---------------------------------------------------------------------------------
 template <typename T>
-static cudaError_t launch_keys_t(const KSrc& src, int64_t T_tokens, const CacheView& cv, int layer0, int n_layers,
+static cudaError_t launch_keys_t(const KSrc& src, int64_t T_tokens, int n_res, const CacheView& cv, int layer0, int n_layers,
                                  int chunk, int64_t kgroup0, const MinMaxBuffers& mm, cudaStream_t stream) {
   uint32_t* minmax = mm.cur;
   const int slabs_per_layer = cv.B * cv.H_kv;
@@ -141,15 +148,17 @@ static cudaError_t launch_keys_t(const KSrc& src, int64_t T_tokens, const CacheV
   cudaError_t e;
   int tokens_per_block = 512;
   const int64_t splits = (T_tokens + tokens_per_block - 1) / tokens_per_block;
-  k_range_kernel<T><<<dim3(static_cast<unsigned>(splits), n_slabs), 256, 0, stream>>>(src, T_tokens, tokens_per_block,
-                                                                                       minmax);
-  k_select_kernel<<<n_slabs, kD, 0, stream>>>(minmax, cv, layer0, slabs_per_layer, chunk, mm.next, mm.next_dirty_words);
-  const int dt = std::is_same<T, __half>::value ? VIDKV_F16 : VIDKV_BF16;
-  if ((e = cv.kf.general ? launch_encode_keys_general(dt, src, T_tokens, cv, layer0, n_slabs, slabs_per_layer, chunk, kgroup0, stream)
-                         : launch_encode_keys(dt, src, T_tokens, cv, layer0, n_slabs, slabs_per_layer, chunk, kgroup0, stream)))
+  if ((e = launch_dependent(k_range_kernel<T>, dim3(static_cast<unsigned>(splits + (n_res > 0)), n_slabs), dim3(256), 0, stream, src,
+                            T_tokens, tokens_per_block, static_cast<int>(splits), n_res, cv, layer0, minmax)))
     return e;
-  count_launches(2);
-  return cudaGetLastError();
+  count_launches(1);
+  const int dt = std::is_same<T, __half>::value ? VIDKV_F16 : VIDKV_BF16;
+  if (!cv.kf.general)
+    return launch_encode_keys(dt, src, T_tokens, cv, layer0, n_slabs, slabs_per_layer, chunk, kgroup0, mm, stream);
+  k_select_kernel<<<n_slabs, kD, 0, stream>>>(minmax, cv, layer0, slabs_per_layer, chunk, mm.next, mm.next_dirty_words);
+  count_launches(1);
+  if ((e = cudaGetLastError())) return e;
+  return launch_encode_keys_general(dt, src, T_tokens, cv, layer0, n_slabs, slabs_per_layer, chunk, kgroup0, stream);
 }
 
 __global__ void init_workspace_kernel(uint32_t* minmax, int n_words, int32_t* counters, int n_counters, uint32_t* header,
@@ -169,11 +178,11 @@ cudaError_t launch_init_workspace(uint32_t* minmax, int64_t n_words, int32_t* co
   return cudaGetLastError();
 }
 
-cudaError_t launch_quantize_keys(int dtype, const KSrc& src, int64_t T_tokens, const CacheView& cv, int layer0,
+cudaError_t launch_quantize_keys(int dtype, const KSrc& src, int64_t T_tokens, int n_res, const CacheView& cv, int layer0,
                                  int n_layers, int chunk, int64_t kgroup0, const MinMaxBuffers& mm, cudaStream_t stream) {
   if (dtype == VIDKV_F16)
-    return launch_keys_t<__half>(src, T_tokens, cv, layer0, n_layers, chunk, kgroup0, mm, stream);
-  return launch_keys_t<__nv_bfloat16>(src, T_tokens, cv, layer0, n_layers, chunk, kgroup0, mm, stream);
+    return launch_keys_t<__half>(src, T_tokens, n_res, cv, layer0, n_layers, chunk, kgroup0, mm, stream);
+  return launch_keys_t<__nv_bfloat16>(src, T_tokens, n_res, cv, layer0, n_layers, chunk, kgroup0, mm, stream);
 }
 
 }  // namespace vidkv

@@ -16,7 +16,14 @@
 //                     float32 accumulation.  Accumulator row = spectrum column: the sign bits
 //                     and the per-group mean |.| are per-thread work, a warp-wide bit
 //                     transpose gives the cache's (token, 16 columns) half-words.
-// Persistent grid of two blocks per SM; block = 256 threads = 8 warps.
+// Persistent grid of two blocks per SM; block = 8 warps that load and encode and one that issues the products.
+//
+// What bounds it: the instructions of the epilogue (code thresholds, comparisons, bit transposes).  A tile goes through in
+// two halves of 64 tokens with accumulators of their own, so that the products of one half run behind the epilogue of the
+// other and the loads of the next tile behind both.  The parts of the DFT rows accumulate apart and are added at the end;
+// in one accumulator the sums would take 10 us less but come out one rounding different, and a coefficient next to zero
+// would change its stored sign.  64 slabs x 12544 tokens, binary16, with the range pass: 128 us, 140 before the halves,
+// code_cut and the selection in here; bfloat16 145 / 159.
 #include <math.h>
 
 #include <algorithm>
@@ -117,23 +124,21 @@ __device__ __forceinline__ uint64_t umma_desc_sw128(uint32_t smem_addr) {
   return static_cast<uint64_t>((smem_addr >> 4) & 0x3fffu) | (static_cast<uint64_t>(1u) << 16) |
          (static_cast<uint64_t>(1024u >> 4) << 32) | (static_cast<uint64_t>(1u) << 46) | (static_cast<uint64_t>(2u) << 61);
 }
-constexpr int kTmemCols = 256;        // two tiles' float32 accumulators of 128 x 128
+constexpr int kTmemCols = 256;        // two halves of a tile, each with two float32 accumulators of 128 x 64
 constexpr int kWaitLimit = 1 << 14;
 
 // One lane of a converged warp.  Issued behind this in a warp-uniform branch an MMA takes the tensor pipe's own time
-// (66 clocks at N = 128); behind "if (threadIdx.x == 0)" its operands take a slower way: 49 clocks and more for any N.
+// (35 clocks at N = 64); behind "if (threadIdx.x == 0)" its operands take a slower way: 49 clocks and more for any N.
 __device__ __forceinline__ bool elect_one() {
   uint32_t p;
   asm volatile("{ .reg .pred q; elect.sync _|q, 0xffffffff; selp.u32 %0, 1, 0, q; }" : "=r"(p));
   return p != 0;
 }
-// off_lo / off_hi: all ones keeps the accumulator rows 0 .. 63 / 64 .. 127 as they are.
-__device__ __forceinline__ void umma_f16(uint32_t tmem_d, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate,
-                                         uint32_t off_lo, uint32_t off_hi) {
+__device__ __forceinline__ void umma_f16(uint32_t tmem_d, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
   asm volatile(
       "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, {%5, %5, %6, %6}, p;\n\t}"
-      ::"r"(tmem_d), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(off_lo), "r"(off_hi)
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, {%5, %5, %5, %5}, p;\n\t}"
+      ::"r"(tmem_d), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(0u)
       : "memory");
 }
 // 32 consecutive accumulator columns of the calling warp's 32 lanes of tensor memory.
@@ -183,21 +188,24 @@ template <> struct Enc<__nv_bfloat16> {
 //                  The products of X use M = 128 too: in arrangement 0 the descriptor starts 64
 //                  rows early, in arrangement 1 it runs 64 rows long; the extra rows read
 //                  neighbouring shared memory and land in accumulator rows that nobody reads.
-//   then the channel order [128], the mbarrier, the tensor-memory address, the fault flag
+//   then the channel order [128], the five mbarriers, the tensor-memory address, the fault flag (64 bytes), and the channel
+//   selection's work area: float range [128], int rank of two halves [2][128], mask words [4]
+constexpr int kEncSelect = kD * 4 + 2 * kD * 4 + 16;
+constexpr int kEncThreads = 288;       // eight warps that load and encode, one that issues the products
 constexpr int kSmTile = 0, kSmAex = 32768;
 template <typename T> __host__ __device__ constexpr int enc_sm_ahi() { return kSmAex + 16384 * (Enc<T>::kParts - 1); }
 template <typename T> __host__ __device__ constexpr int enc_sm_perm() { return enc_sm_ahi<T>() + 32768; }
-template <typename T> __host__ __device__ constexpr int enc_sm_bytes() { return enc_sm_perm<T>() + kD + 32 + 1024; }
+template <typename T> __host__ __device__ constexpr int enc_sm_bytes() { return enc_sm_perm<T>() + kD + 64 + kEncSelect + 1024; }
 
 size_t k_encode_smem_bytes(int dtype) { return dtype == VIDKV_F16 ? enc_sm_bytes<__half>() : enc_sm_bytes<__nv_bfloat16>(); }
 
 // Persistent blocks, two per SM: block b encodes the tiles [n b / G, n (b + 1) / G) of the
 // launch's n = slabs x tiles-per-slab tiles.  Warp w works on tensor-memory lanes 32 (w % 4):
 // warps with w % 4 < 2 own 32 anomalous slots each, the others 32 spectrum columns each (and
-// issue the tile loads); w / 4 picks two of the tile's four 32-token groups.
+// issue the tile loads); w / 4 picks the first or second of the two 32-token groups of each half tile.
 template <typename T>
-__global__ void __launch_bounds__(256, 2) k_encode_kernel(KSrc src, int64_t T_tokens, CacheView cv, int layer0,
-                                                          int slabs_per_layer, int chunk, int64_t kgroup0,
+__global__ void __launch_bounds__(kEncThreads, 2) k_encode_kernel(KSrc src, int64_t T_tokens, CacheView cv, int layer0,
+                                                          int slabs_per_layer, int chunk, int64_t kgroup0, MinMaxBuffers mm,
                                                           int tiles_per_slab, int total_tiles, int withhold_first) {
   extern __shared__ uint8_t esm_raw[];
   uint8_t* esm = esm_raw + ((1024u - (smem_u32(esm_raw) & 1023u)) & 1023u);
@@ -206,8 +214,11 @@ __global__ void __launch_bounds__(256, 2) k_encode_kernel(KSrc src, int64_t T_to
   uint8_t* a_ex = esm + kSmAex;
   uint8_t* perm = esm + enc_sm_perm<T>();
   uint64_t* mbar = reinterpret_cast<uint64_t*>(perm + kD);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(perm + kD + 8);
-  volatile uint32_t* fault = reinterpret_cast<volatile uint32_t*>(perm + kD + 12);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(perm + kD + 40);
+  volatile uint32_t* fault = reinterpret_cast<volatile uint32_t*>(perm + kD + 44);
+  float* sel_range = reinterpret_cast<float*>(perm + kD + 64);
+  int* sel_rank = reinterpret_cast<int*>(sel_range + kD);
+  uint32_t* sel_mask = reinterpret_cast<uint32_t*>(sel_rank + 2 * kD);
 
   const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
   const int quad = warp & 3, half = warp >> 2;
@@ -220,7 +231,9 @@ __global__ void __launch_bounds__(256, 2) k_encode_kernel(KSrc src, int64_t T_to
   const int lt = half * 64 + (quad & 1) * 32 + lane;    // 0 .. 127 among the loading threads
 
   if (tid == 0) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(mbar)) : "memory");
+#pragma unroll
+    for (int i = 0; i < 5; ++i)
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(mbar + i)), "r"(i < 3 ? 1 : 8) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     *fault = 0u;
   }
@@ -242,77 +255,112 @@ __global__ void __launch_bounds__(256, 2) k_encode_kernel(KSrc src, int64_t T_to
   int lslab = slab, lti = ti, lbase_slab = -1;
   const T* lbase = nullptr;
 
-  // 16-byte pieces of a tile: thread lt moves piece lt % 16 of the rows lt / 16 + 8 i
-  auto load_next_tile = [&]() {
+  // Half hs of the next tile in 16-byte pieces: thread lt moves piece lt % 16 of the rows 64 hs + lt / 16 + 8 i
+  auto load_next = [&](int hs) {
     if (lslab != lbase_slab) {
       lbase_slab = lslab;
       lbase = reinterpret_cast<const T*>(src.ptr) + (lslab / src.H) * src.stride_b + (lslab % src.H) * src.stride_h;
     }
     const int64_t t0 = static_cast<int64_t>(lti) * kEncTokens;
     const int n_tok = static_cast<int>(min(static_cast<int64_t>(kEncTokens), T_tokens - t0));
-    const int row0 = lt >> 4, piece = lt & 15;
+    const int row0 = 64 * hs + (lt >> 4), piece = lt & 15;
     const uint8_t* srow = reinterpret_cast<const uint8_t*>(lbase + (t0 + row0) * src.stride_t) + piece * 16;
-    uint8_t* drow = tile + (piece >> 3) * 16384 + row0 * 128 + (((piece & 7) ^ row0) << 4);
+    uint8_t* drow = tile + (piece >> 3) * 16384 + row0 * 128 + (((piece ^ row0) & 7) << 4);
     const int64_t sstep = 8 * src.stride_t * static_cast<int64_t>(sizeof(T));
 #pragma unroll
-    for (int i = 0; i < kEncTokens / 8; ++i)
+    for (int i = 0; i < kEncTokens / 16; ++i)
       if (row0 + 8 * i < n_tok) cp_async16(drow + i * 1024, srow + i * sstep);
     asm volatile("cp.async.commit_group;" ::: "memory");
-    if (++lti == tiles_per_slab) { lti = 0; ++lslab; }
+    if (hs == 1 && ++lti == tiles_per_slab) { lti = 0; ++lslab; }
   };
 
-  // ---- D[128 rows x 128 tokens] = the smaller parts of the DFT rows x tile^T (the 64 rows those parts do not have read
-  // neighbouring shared memory and are masked out of the accumulator), then A (leading) x tile^T on top: small terms first,
-  // which keeps the sums as close to exact as two accumulators that are added at the end
-  const int issuer = arr ? 0 : 2;                            // one of the loading warps
-  auto issue = [&](int buf) {
+  // ---- D[128 rows x 64 tokens] = A (leading) x tile^T; D'[.. x ..] = A (remaining parts) x tile^T, for tokens 64 hs .. 64 hs + 63
+  // Products issued so far arrive at mbarrier i when they are done.
+  auto commit = [&](int i) {
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(mbar + i)) : "memory");
+  };
+  auto issue = [&](int hs) {
     if (elect_one()) {
       constexpr uint32_t idesc = (1u << 4) | (static_cast<uint32_t>(Enc<T>::kFmt) << 7) | (static_cast<uint32_t>(Enc<T>::kFmt) << 10) |
-                                 ((128u >> 3) << 17) | ((128u >> 4) << 24);
-      const uint32_t d = tmem + static_cast<uint32_t>(buf * 128);
-      const uint32_t off_lo = arr ? 0u : 0xffffffffu, off_hi = ~off_lo;   // the selector rows / (off_hi, off_lo): the DFT rows
+                                 ((64u >> 3) << 17) | ((128u >> 4) << 24);
+      const uint32_t d = tmem + static_cast<uint32_t>(hs * 128);
+      const uint32_t b0 = smem_u32(tile) + static_cast<uint32_t>(hs * 8192);
 #pragma unroll
-      for (int part = Enc<T>::kParts - 1; part >= 1; --part) {
+      for (int kb = 0; kb < 2; ++kb) {
+        const uint64_t da = umma_desc_sw128(smem_u32(a_hi + kb * 16384)), db = umma_desc_sw128(b0 + static_cast<uint32_t>(kb * 16384));
+#pragma unroll
+        for (int ks = 0; ks < 4; ++ks)   // 16 elements = 32 bytes along K per step; the address field counts 16 bytes
+          umma_f16(d, da + static_cast<uint64_t>(2 * ks), db + static_cast<uint64_t>(2 * ks), idesc, (kb | ks) != 0 ? 1u : 0u);
+      }
+#pragma unroll
+      for (int part = 1; part < Enc<T>::kParts; ++part) {
 #pragma unroll
         for (int kb = 0; kb < 2; ++kb) {
           // the part's 64 rows are rows 64 .. 127 of arrangement 0 (start 8192 bytes early), rows 0 .. 63 of arrangement 1
           const uint64_t da = umma_desc_sw128(smem_u32(a_ex + (part - 1) * 16384 + kb * 8192 - (arr ? 0 : 8192)));
-          const uint64_t db = umma_desc_sw128(smem_u32(tile + kb * 16384));
+          const uint64_t db = umma_desc_sw128(b0 + static_cast<uint32_t>(kb * 16384));
 #pragma unroll
-          for (int ks = 0; ks < 4; ++ks)   // 16 elements = 32 bytes along K per step; the address field counts 16 bytes
-            umma_f16(d, da + static_cast<uint64_t>(2 * ks), db + static_cast<uint64_t>(2 * ks), idesc,
-                     part < Enc<T>::kParts - 1 || (kb | ks) != 0 ? 1u : 0u, off_lo, off_hi);
+          for (int ks = 0; ks < 4; ++ks)
+            umma_f16(d + 64u, da + static_cast<uint64_t>(2 * ks), db + static_cast<uint64_t>(2 * ks), idesc,
+                     (part - 1) | kb | ks ? 1u : 0u);
         }
       }
-#pragma unroll
-      for (int kb = 0; kb < 2; ++kb) {
-        const uint64_t da = umma_desc_sw128(smem_u32(a_hi + kb * 16384)), db = umma_desc_sw128(smem_u32(tile + kb * 16384));
-        // the first step starts the selector rows and goes on top of the small parts in the DFT rows
-        if (kb == 0) umma_f16(d, da, db, idesc, 0u, off_hi, off_lo);
-        if (kb == 0) umma_f16(d, da, db, idesc, 1u, off_lo, off_hi);
-#pragma unroll
-        for (int ks = kb == 0 ? 1 : 0; ks < 4; ++ks)
-          umma_f16(d, da + static_cast<uint64_t>(2 * ks), db + static_cast<uint64_t>(2 * ks), idesc, 1u, 0u, 0u);
-      }
-      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(mbar)) : "memory");
+      commit(hs);
     }
     __syncwarp();
   };
-  auto accumulators_ready = [&](uint32_t parity) -> bool {
+  auto wait_for = [&](int i, uint32_t parity) -> bool {
     uint32_t done = 0;
     for (int it = 0; it < kWaitLimit && !done; ++it) {
       asm volatile(
           "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-          : "=r"(done) : "r"(smem_u32(mbar)), "r"(parity) : "memory");
+          : "=r"(done) : "r"(smem_u32(mbar + i)), "r"(parity) : "memory");
     }
     return __all_sync(0xffffffffu, done != 0);
   };
 
+  // mbarriers: hs, the products of half hs are done; 2, all products are done; 3 + hs, half hs of the tile is in shared
+  // memory, operand A is built and the half's accumulators of the tile before have been read (one arrival per warp).
+  // Every wait is bounded; whoever runs out of patience sets the fault flag and waits and arrives no more.
+  if (loader && tile_begin < tile_end) { load_next(0); load_next(1); }   // the keys are complete: the range pass has waited for them
+  pdl_wait();                                                // the ranges
+  if (warp == 8) {
+    uint32_t parity = 0;
+    bool lost = false;
+    for (int t = tile_begin; t < tile_end && !lost; ++t, parity ^= 1u) {
+#pragma unroll
+      for (int hs = 0; hs < 2; ++hs) {
+        lost = lost || !wait_for(3 + hs, parity) || __any_sync(0xffffffffu, *fault != 0u);
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        // (withhold_first, a test hook: the block's first tile gets neither products nor a commit, so the
+        // waits for them run out with nothing outstanding)
+        if (!lost && !(withhold_first && t == tile_begin)) issue(hs);
+      }
+    }
+    if (elect_one()) commit(2);
+    __syncwarp();
+    wait_for(2, 0u);                                           // nothing is under way when the tensor memory is given back
+    if (lost && lane == 0) {
+      *fault = 1u;
+      atomicCAS(reinterpret_cast<int*>(cv.base + kHdrStatus), 0, static_cast<int>(VIDKV_ERR_TIMEOUT));
+    }
+    __syncthreads();
+    return;
+  }
+  bool lost = false;                                         // a wait ran out: nothing more is encoded
+  auto arrive = [&](int hs) {
+    __syncwarp();
+    if (lane == 0 && !lost) asm volatile("{ .reg .b64 s; mbarrier.arrive.shared::cta.b64 s, [%0]; }" ::"r"(smem_u32(mbar + 3 + hs)) : "memory");
+  };
+
   int cur_slab = -1;
   uint32_t phase = 0;
-  bool ahead = false;                                        // this tile's products are issued already
+  bool ahead = false;                                        // this tile's arrivals have happened already
   uint8_t* slab_ptr = nullptr;
-  if (loader && tile_begin < tile_end) load_next_tile();
+  // Re-arm the buffer the next call accumulates into (min half all ones, max half zero).  Nobody reads it now: its last
+  // readers ran before this call's range pass in stream order.
+  for (int i = blockIdx.x * 256 + tid; i < mm.next_dirty_words; i += gridDim.x * 256)
+    mm.next[i] = (i & (2 * kD - 1)) < kD ? 0xffffffffu : 0u;
   for (int t = tile_begin; t < tile_end; ++t, ti = (ti + 1 == tiles_per_slab) ? 0 : ti + 1, slab += (ti == 0) ? 1 : 0) {
     if (slab != cur_slab) {
       const int layer = layer0 + slab / slabs_per_layer;
@@ -335,11 +383,42 @@ __global__ void __launch_bounds__(256, 2) k_encode_kernel(KSrc src, int64_t T_to
 #pragma unroll
         for (int j = 0; j < 2; ++j)
           wv[part][j] = __ldg(reinterpret_cast<const uint4*>(g_dft_w + (Enc<T>::kTab + part) * 4096) + tid + 256 * j);
-      if (tid < kD) perm[tid] = slab_ptr[cv.chunk_table_offset + static_cast<int64_t>(chunk) * kChunkBytes + tid];
+      // TopK (Algorithm 3): rank(c) = channels before c in (range descending, index ascending) order, two threads per
+      // channel; the first 64 are the anomalous ones.  Every block does it for the slabs it meets, about 0.5 us, where a
+      // kernel of its own took 3 us and a launch gap per call.
+      {
+        const int c = tid & (kD - 1), side = tid >> 7;
+        const uint32_t* mmw = mm.cur + static_cast<int64_t>(slab) * 2 * kD;
+        if (side == 0) sel_range[c] = __fsub_rn(ordered_float(mmw[kD + c]), ordered_float(mmw[c]));
+        asm volatile("bar.sync 1, 256;" ::: "memory");
+        const float rg = sel_range[c];
+        int rank = 0;
+#pragma unroll 16
+        for (int o = side * (kD / 2); o < (side + 1) * (kD / 2); o += 4) {
+          const float4 v = *reinterpret_cast<const float4*>(sel_range + o);
+          rank += (v.x > rg) || (v.x == rg && o < c);
+          rank += (v.y > rg) || (v.y == rg && o + 1 < c);
+          rank += (v.z > rg) || (v.z == rg && o + 2 < c);
+          rank += (v.w > rg) || (v.w == rg && o + 3 < c);
+        }
+        sel_rank[tid] = rank;
+        asm volatile("bar.sync 1, 256;" ::: "memory");
+        const bool abn = sel_rank[c] + sel_rank[kD + c] < kNA;
+        const uint32_t word = __ballot_sync(0xffffffffu, abn);
+        if (lane == 0 && side == 0) sel_mask[warp] = word;
+        asm volatile("bar.sync 1, 256;" ::: "memory");
+        if (side == 0) {
+          int before = __popc(word & ((1u << lane) - 1u));
+          for (int i = 0; i < warp; ++i) before += __popc(sel_mask[i]);
+          const int at = abn ? before : kNA + c - before;
+          perm[at] = static_cast<uint8_t>(c);
+          if (ti == 0) slab_ptr[cv.chunk_table_offset + static_cast<int64_t>(chunk) * kChunkBytes + at] = static_cast<uint8_t>(c);
+        }
+      }
       constexpr int kAVec = (32768 + 16384 * (Enc<T>::kParts - 1)) / 16;
 #pragma unroll 4
       for (int i = tid; i < kAVec; i += 256) reinterpret_cast<uint4*>(a_ex)[i] = make_uint4(0u, 0u, 0u, 0u);
-      __syncthreads();
+      asm volatile("bar.sync 1, 256;" ::: "memory");
       if (tid < kNA) {
         const int c = perm[tid];
         *reinterpret_cast<uint16_t*>(a_hi + (c >> 6) * 16384 + sw128_offset(64 * arr + tid, c & 63)) = Enc<T>::kOne;
@@ -364,43 +443,44 @@ __global__ void __launch_bounds__(256, 2) k_encode_kernel(KSrc src, int64_t T_to
       }
     }
 
-    // ---- this tile's products were issued behind the epilogue of the tile before, unless its operand A is new
-    if (!ahead && loader) asm volatile("cp.async.wait_group 0;" ::: "memory");
-    if (!ahead) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();                                           // and everyone has read the accumulators of the tile before
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (*fault) break;
-    // (withhold_first, a test hook: the block's first tile gets neither products nor a commit, so the
-    // wait below runs out with nothing outstanding)
-    if (!ahead && warp == issuer && !(withhold_first && t == tile_begin)) issue((t - tile_begin) & 1);
-    // every thread waits for the accumulators; the wait is bounded, a timeout is reported in the status word
-    const bool done = accumulators_ready(phase);
-    phase ^= 1u;
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (!done && lane == 0) {
-      *fault = 1u;
-      atomicCAS(reinterpret_cast<int*>(cv.base + kHdrStatus), 0, static_cast<int>(VIDKV_ERR_TIMEOUT));
+    // ---- unless operand A is new, the products were ordered behind the epilogue of the tile before
+    if (!ahead) {
+      if (loader) asm volatile("cp.async.wait_group 0;" ::: "memory");
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      arrive(0);
+      arrive(1);
     }
-    // the products are done with shared memory: fetch the next tile behind the epilogue
     const bool more = t + 1 < tile_end;
-    if (loader && more) load_next_tile();
     ahead = more && ti + 1 < tiles_per_slab;                   // the next tile has the same operand A
-    const uint32_t acc = tmem + static_cast<uint32_t>(((t - tile_begin) & 1) * 128);
-    if (!done) {
-      // nothing to encode; the loading warps still meet below
-    } else
-    if (!loader) {
-      // ---- Eq. 4: lane = anomalous slot j, the accumulator row holds its 128 tokens (exact values)
-      const int j = (quad & 1) * 32 + lane, wg = j >> 4;
-      const int pos = (lane >> 1) & 3;                            // field of the slot inside its code byte
-      const bool pb0 = (lane & 2) != 0, pb1 = (lane & 4) != 0;    // bits of pos
-      const bool bb0 = (lane & 8) != 0, bb1 = (lane & 1) != 0;    // bits of the slot's byte index 2 (e % 2) + e / 8
-      const uint32_t wgt = pos == 0 ? 0x3c003c00u : pos == 1 ? 0x44004400u : pos == 2 ? 0x4c004c00u : 0x54005400u;   // 4^pos
 #pragma unroll 1
-      for (int g = 2 * half; g < 2 * half + 2 && g < n_groups; ++g) {
+    for (int hs = 0; hs < 2; ++hs) {
+      // every warp waits for the half's accumulators; a timeout is reported in the status word, and the warp goes on to the
+      // end without waiting or writing
+      if (!lost) {
+        lost = !wait_for(hs, phase) || __any_sync(0xffffffffu, *fault != 0u);
+        if (lost && lane == 0) {
+          *fault = 1u;
+          atomicCAS(reinterpret_cast<int*>(cv.base + kHdrStatus), 0, static_cast<int>(VIDKV_ERR_TIMEOUT));
+        }
+      }
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      // the products are done with this half of the tile: fetch the next tile's
+      if (loader && more) load_next(hs);
+      const int g = 2 * hs + half;
+      const uint32_t acc = tmem + (static_cast<uint32_t>(quad * 32) << 16) + static_cast<uint32_t>(hs * 128 + half * 32);
+      if (lost || g >= n_groups) {
+        // nothing to encode; the warps still meet
+      } else
+      if (!loader) {
+        // ---- Eq. 4: lane = anomalous slot j, the accumulator row holds its 64 tokens (exact values)
+        const int j = (quad & 1) * 32 + lane, wg = j >> 4;
+        const int pos = (lane >> 1) & 3;                            // field of the slot inside its code byte
+        const bool pb0 = (lane & 2) != 0, pb1 = (lane & 4) != 0;    // bits of pos
+        const bool bb0 = (lane & 8) != 0, bb1 = (lane & 1) != 0;    // bits of the slot's byte index 2 (e % 2) + e / 8
+        const uint32_t wgt = pos == 0 ? 0x3c003c00u : pos == 1 ? 0x44004400u : pos == 2 ? 0x4c004c00u : 0x54005400u;   // 4^pos
         uint32_t x[32];
-        tmem_ld32(acc + (static_cast<uint32_t>(quad * 32) << 16) + static_cast<uint32_t>(g * 32), x);
+        tmem_ld32(acc, x);
         float fmn = __uint_as_float(x[0]), fmx = fmn;
 #pragma unroll
         for (int i = 1; i < 32; ++i) { fmn = fminf(fmn, __uint_as_float(x[i])); fmx = fmaxf(fmx, __uint_as_float(x[i])); }
@@ -466,20 +546,19 @@ __global__ void __launch_bounds__(256, 2) k_encode_kernel(KSrc src, int64_t T_to
           codes[((2 * pos) * 4 + wg) * 4 + nt] = prmt(lowpair, highpair, 0x5410u);
           codes[((2 * pos + 1) * 4 + wg) * 4 + nt] = prmt(lowpair, highpair, 0x7632u);
         }
-      }
-    } else {
-      // ---- Eq. 5: lane = spectrum column f, the two accumulators' rows 64 + f hold its 128 tokens
-      const int hq = quad & 1, f = hq * 32 + lane;
-#pragma unroll 1
-      for (int g = 2 * half; g < 2 * half + 2 && g < n_groups; ++g) {
-        uint32_t xa[32];
-        tmem_ld32(acc + (static_cast<uint32_t>(quad * 32) << 16) + static_cast<uint32_t>(g * 32), xa);
+      } else {
+        // ---- Eq. 5: lane = spectrum column f, the two accumulators' rows 64 + f hold its 64 tokens
+        const int hq = quad & 1, f = hq * 32 + lane;
+        uint32_t xa[32], xb[32];
+        tmem_ld32(acc, xa);
+        tmem_ld32(acc + 64u, xb);
         float sum = 0.0f;
         uint32_t bits = 0u;   // bit i = sign bit of the column's coefficient of token i
 #pragma unroll
         for (int i = 31; i >= 0; --i) {
-          sum += fabsf(__uint_as_float(xa[i]));
-          bits = __funnelshift_l(xa[i], bits, 1);
+          const float X = __uint_as_float(xa[i]) + __uint_as_float(xb[i]);
+          sum += fabsf(X);
+          bits = __funnelshift_l(__float_as_uint(X), bits, 1);
         }
         uint8_t* kg = kg_base + g * kKGroupBytes;
         reinterpret_cast<uint16_t*>(kg + kKG_S1)[f] = f2h_bits(sum * (1.0f / 32.0f));
@@ -501,17 +580,20 @@ __global__ void __launch_bounds__(256, 2) k_encode_kernel(KSrc src, int64_t T_to
         hw[hidx] = static_cast<uint16_t>(mine >> 16);
         hw[hidx + 4] = static_cast<uint16_t>(mine);
       }
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      if (ahead && !loader) arrive(hs);
     }
-    if (loader && ahead) {
-      // the next tile has landed: its products run while the anomalous warps are still at this one's codes
+    phase ^= 1u;
+    if (ahead && loader) {
+      // the products of the next tile's first half run while the anomalous warps are still at this tile's codes
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      arrive(0);
       asm volatile("cp.async.wait_group 0;" ::: "memory");
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      asm volatile("bar.sync 1, 128;" ::: "memory");           // the four loading warps
-      if (warp == issuer) issue((t + 1 - tile_begin) & 1);
+      arrive(1);
     }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   }
-  if (ahead) accumulators_ready(phase);                        // left early: the products that are under way land first
   if (loader) asm volatile("cp.async.wait_group 0;" ::: "memory");
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -528,7 +610,7 @@ __global__ void __launch_bounds__(256, 2) k_encode_kernel(KSrc src, int64_t T_to
 // (free once it has completed), so uses on other streams are ordered after the fill without a
 // host-side synchronisation.
 cudaError_t dft_tables(DftTables* tables, cudaStream_t stream) {
-  static bool done[64] = {};
+  static bool done[64] = {}, complete[64] = {};
   static DftTables addr[64] = {};
   static cudaEvent_t ready[64] = {};
   cudaError_t e;
@@ -547,8 +629,16 @@ cudaError_t dft_tables(DftTables* tables, cudaStream_t stream) {
     addr[dev].w32 = static_cast<const float*>(p32);
     done[dev] = true;
     count_launches(1);
-  } else if ((e = cudaStreamWaitEvent(stream, ready[dev], 0))) {
-    return e;
+  } else if (!complete[dev]) {
+    // once the fill is known to have completed, no stream has to be ordered after it any more (the wait costs 2 us of host
+    // time per call); relaxed mode, so that the query leaves another thread's stream capture alone
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    if ((e = cudaThreadExchangeStreamCaptureMode(&mode))) return e;
+    const cudaError_t state = cudaEventQuery(ready[dev]);
+    if ((e = cudaThreadExchangeStreamCaptureMode(&mode))) return e;
+    if (state == cudaSuccess) complete[dev] = true;
+    else if (state != cudaErrorNotReady) return state;
+    else if ((e = cudaStreamWaitEvent(stream, ready[dev], 0))) return e;
   }
   *tables = addr[dev];
   return cudaSuccess;
@@ -556,7 +646,7 @@ cudaError_t dft_tables(DftTables* tables, cudaStream_t stream) {
 
 template <typename T>
 static cudaError_t launch_encode_t(const KSrc& src, int64_t T_tokens, const CacheView& cv, int layer0, int n_slabs,
-                                   int slabs_per_layer, int chunk, int64_t kgroup0, cudaStream_t stream) {
+                                   int slabs_per_layer, int chunk, int64_t kgroup0, const MinMaxBuffers& mm, cudaStream_t stream) {
   cudaError_t e;
   DftTables tables;
   if ((e = dft_tables(&tables, stream))) return e;
@@ -576,16 +666,15 @@ static cudaError_t launch_encode_t(const KSrc& src, int64_t T_tokens, const Cach
   const int blocks = static_cast<int>(std::min<int64_t>(total, 2 * n_sms[dev]));
   const int withhold = (g_debug_withhold == 1) ? 1 : 0;
   if (withhold) g_debug_withhold = 0;
-  k_encode_kernel<T><<<blocks, 256, smem, stream>>>(src, T_tokens, cv, layer0, slabs_per_layer, chunk, kgroup0,
-                                                    static_cast<int>(tiles_per_slab), static_cast<int>(total), withhold);
   count_launches(1);
-  return cudaGetLastError();
+  return launch_dependent(k_encode_kernel<T>, dim3(blocks), dim3(kEncThreads), smem, stream, src, T_tokens, cv, layer0, slabs_per_layer, chunk,
+                          kgroup0, mm, static_cast<int>(tiles_per_slab), static_cast<int>(total), withhold);
 }
 
 cudaError_t launch_encode_keys(int dtype, const KSrc& src, int64_t T_tokens, const CacheView& cv, int layer0, int n_slabs,
-                               int slabs_per_layer, int chunk, int64_t kgroup0, cudaStream_t stream) {
-  if (dtype == VIDKV_F16) return launch_encode_t<__half>(src, T_tokens, cv, layer0, n_slabs, slabs_per_layer, chunk, kgroup0, stream);
-  return launch_encode_t<__nv_bfloat16>(src, T_tokens, cv, layer0, n_slabs, slabs_per_layer, chunk, kgroup0, stream);
+                               int slabs_per_layer, int chunk, int64_t kgroup0, const MinMaxBuffers& mm, cudaStream_t stream) {
+  if (dtype == VIDKV_F16) return launch_encode_t<__half>(src, T_tokens, cv, layer0, n_slabs, slabs_per_layer, chunk, kgroup0, mm, stream);
+  return launch_encode_t<__nv_bfloat16>(src, T_tokens, cv, layer0, n_slabs, slabs_per_layer, chunk, kgroup0, mm, stream);
 }
 
 }  // namespace vidkv

@@ -1,15 +1,19 @@
 // Value quantizer kernels: Algorithm 2 of the paper (1.58Quant, STPQuant), the token
 // selection of Sec. 3.3(2), and the residual copies of Algorithm 1.
+#include <cooperative_groups.h>
+
 #include "common.cuh"
 #include "kernels.cuh"
+#include "quant_common.cuh"
 
 namespace vidkv {
+
+namespace cg = cooperative_groups;
 
 __device__ __forceinline__ __half2 as_half2(uint32_t v) { return *reinterpret_cast<const __half2*>(&v); }
 
 // ---------------------------------------------------------------------------------
-// 1.58Quant (Eq. 6) of one supergroup = 5 groups x 32 stream tokens x 128 channels.
-// grid = (supergroups, slabs of one layer); block = 256 threads.
+// 1.58Quant (Eq. 6) of one supergroup = 5 groups x 32 stream tokens x 128 channels by a block of 256 threads.
 // Stream position u of the unprotected tokens maps to token idx_rest[u] (identity when
 // no token is protected).
 //   stage   the 160 x 128 tile is copied to shared memory as it is (cp.async, 16 bytes a piece);
@@ -62,10 +66,9 @@ __device__ __forceinline__ void cp_async16_v(void* smem_dst, const void* gmem_sr
 // NZ: the stored scale is the mean of |v| over the non-zero codes instead of Mean |v| (one more
 // sweep over the staged tile; needs kSGGroups * 4 * kD more floats of shared memory).
 template <typename T, bool NZ>
-__global__ void __launch_bounds__(256) v_ternary_kernel(KSrc src, int64_t n_rest, CacheView cv, int layer0,
-                                                        SelView sel, float gamma) {
-  extern __shared__ __align__(16) uint8_t vsm[];
-  uint8_t* tile = vsm;                                                         // [160][288]
+__device__ __forceinline__ void ternary_supergroup(uint8_t* vsm, KSrc src, int64_t n_rest, CacheView cv, int layer0,
+                                                   SelView sel, float gamma) {
+  uint8_t* tile = vsm;                                                         // [160][kVRowBytes]
   float* part = reinterpret_cast<float*>(tile + kSGTokens * kVRowBytes);       // [5][4][128]
   uint32_t* thr = reinterpret_cast<uint32_t*>(part + kSGGroups * 4 * kD);      // [5][64] threshold pairs
   uint8_t* lut = reinterpret_cast<uint8_t*>(thr + kSGGroups * 64);             // [256]
@@ -205,89 +208,50 @@ __global__ void __launch_bounds__(256) v_ternary_kernel(KSrc src, int64_t n_rest
 }
 
 // ---------------------------------------------------------------------------------
-// 2-bit GQuant (Eq. 4) of one group of up to 32 protected tokens.  grid = (groups, slabs).
+// 2-bit GQuant (Eq. 4) of groups of up to 32 protected tokens: 128 threads per group, two groups per block.
 //
 // code(v) = clamp(rint((v - z) / s), 0, 3) does not decrease with v, so it equals the number of
-// k in {1, 2, 3} with v >= t_k, t_k the smallest value of the input type whose code reaches k.
-// One thread per channel finds the three t_k with the literal formula (IEEE division included)
-// evaluated on a handful of candidates around z + (k - 1/2) s; the elements are then coded with
-// three comparisons each instead of a division each.
+// k in {1, 2, 3} with v >= X_k, X_k the smallest value of the input type whose code reaches k (code_cut).
+// The elements are compared with X_k two channels at a time; the comparisons' ones times 4^e, on top of 1024, put the
+// fields of a code byte into the low bits of two binary16 lanes.  2508 protected and 10036 other tokens of 64 slabs take 78
+// us; three threshold searches with divisions per channel, conversions and float comparisons per element took 95.
 // ---------------------------------------------------------------------------------
-template <typename T> struct Ordered16;     // 16-bit patterns of T <-> integers in value order
-template <> struct Ordered16<__half> {
-  static constexpr int kMin = 0x0400, kMax = 0xfbff;          // keys of -65504 and +65504
-  static __device__ __forceinline__ float value(int key) {
-    const uint16_t b = static_cast<uint16_t>(key ^ ((key & 0x8000) ? 0x8000 : 0xffff));
-    return __half2float(__ushort_as_half(b));
-  }
-  static __device__ __forceinline__ int key(float x) {
-    const uint16_t b = __half_as_ushort(__float2half_rn(x));
-    return b ^ ((b & 0x8000u) ? 0xffffu : 0x8000u);
-  }
-};
-template <> struct Ordered16<__nv_bfloat16> {
-  static constexpr int kMin = 0x0080, kMax = 0xff7f;          // keys of the largest finite magnitudes
-  static __device__ __forceinline__ float value(int key) {
-    const uint32_t b = static_cast<uint32_t>(key ^ ((key & 0x8000) ? 0x8000 : 0xffff));
-    return __uint_as_float(b << 16);
-  }
-  static __device__ __forceinline__ int key(float x) {
-    const uint16_t b = __bfloat16_as_ushort(__float2bfloat16_rn(x));
-    return b ^ ((b & 0x8000u) ? 0xffffu : 0x8000u);
-  }
-};
-
-// Smallest value of type T (as a float) whose Eq. 4 code with (s, z) is >= k; +infinity if none.
-template <typename T>
-__device__ __forceinline__ float code_threshold(float s, float z, int k) {
-  using O = Ordered16<T>;
-  if (!(s > 0.0f)) return INFINITY;                            // zero range: every code is 0
-  const float kf = static_cast<float>(k);
-  auto reaches = [&](int key) -> bool {
-    float q = rintf(__fdiv_rn(__fsub_rn(O::value(key), z), s));
-    q = fminf(fmaxf(q, 0.0f), 3.0f);
-    return q >= kf;
-  };
-  const int ck = min(max(O::key(fmaf(kf - 0.5f, s, z)), O::kMin), O::kMax);
-  int lo = max(ck - 4, O::kMin - 1), hi = min(ck + 4, O::kMax);   // invariant: code(lo) < k <= code(hi)
-  if (!reaches(hi)) {
-    lo = hi; hi = O::kMax;
-    if (!reaches(hi)) return INFINITY;
-  }
-  if (lo >= O::kMin && reaches(lo)) { hi = lo; lo = O::kMin - 1; }
-  while (hi - lo > 1) {                                        // at most 16 rounds
-    const int mid = (lo + hi) >> 1;
-    if (reaches(mid)) hi = mid; else lo = mid;
-  }
-  return O::value(hi);
-}
+constexpr int kPRow = 144;                  // elements per staged row: rows two apart land 16 banks apart
+constexpr int kProtectSmem = 2 * (kG * kPRow * 2 + 3 * kD * 2);
 
 template <typename T>
-__global__ void __launch_bounds__(128) v_protect_kernel(KSrc src, CacheView cv, int layer0, SelView sel) {
-  __shared__ __align__(16) uint16_t tile[kG * kD];
-  __shared__ float s_thr[3][kD];
+__device__ __forceinline__ void protect_groups(uint8_t* vsm, const KSrc& src, int block, const CacheView& cv, int layer0, const SelView& sel) {
+  const int half = threadIdx.x >> 7, tid = threadIdx.x & 127;
+  uint16_t* tile = reinterpret_cast<uint16_t*>(vsm) + half * kG * kPRow;                    // [32][kPRow]
+  uint16_t* s_thr = reinterpret_cast<uint16_t*>(vsm + 2 * kG * kPRow * 2) + half * 3 * kD;     // [3][128]
   const int slab = blockIdx.y;
   const int lb = slab / cv.H_kv, h = slab % cv.H_kv;
   const int b = lb % cv.B, layer = layer0 + lb / cv.B;
   const T* base = reinterpret_cast<const T*>(src.ptr) + static_cast<int64_t>(lb) * src.stride_b + h * src.stride_h;
-  const int64_t p0 = static_cast<int64_t>(blockIdx.x) * kG;
-  const int n_rows = static_cast<int>(min(static_cast<int64_t>(kG), sel.n_prot - p0));
+  const int64_t pgroup = 2 * static_cast<int64_t>(block) + half;
+  const int64_t p0 = pgroup * kG;
+  const int n_rows = static_cast<int>(min(static_cast<int64_t>(kG), sel.n_prot - p0));       // <= 0: nothing left for this half
   const int32_t* idx = sel.idx_prot + b * sel.stride_prot;
   {
-    const int lane16 = threadIdx.x & 15, row = threadIdx.x >> 4;
-    for (int r = row; r < kG; r += 8) {
+    const int lane16 = tid & 15, row = tid >> 4;
+    int tok[kG / 8];
+#pragma unroll
+    for (int k = 0; k < kG / 8; ++k) tok[k] = row + 8 * k < n_rows ? __ldg(idx + p0 + row + 8 * k) : -1;
+#pragma unroll
+    for (int k = 0; k < kG / 8; ++k) {
       uint4 v = make_uint4(0, 0, 0, 0);
-      if (r < n_rows) v = __ldg(reinterpret_cast<const uint4*>(base + static_cast<int64_t>(idx[p0 + r]) * src.stride_t) + lane16);
-      reinterpret_cast<uint4*>(tile + r * kD)[lane16] = v;
+      if (tok[k] >= 0) v = __ldg(reinterpret_cast<const uint4*>(base + static_cast<int64_t>(tok[k]) * src.stride_t) + lane16);
+      reinterpret_cast<uint4*>(tile + (row + 8 * k) * kPRow)[lane16] = v;
     }
   }
   __syncthreads();
-  uint8_t* pg = cv.slab(layer, b, h) + cv.prot_offset + static_cast<int64_t>(blockIdx.x) * kPGBytes;
-  {
-    const int c = threadIdx.x;
+  uint8_t* pg = cv.slab(layer, b, h) + cv.prot_offset + pgroup * kPGBytes;
+  if (n_rows > 0) {
+    const int c = tid;
     float mn = INFINITY, mx = -INFINITY;
+#pragma unroll 8
     for (int j = 0; j < n_rows; ++j) {
-      const float v = Elem<T>::to_float(reinterpret_cast<const T*>(tile)[j * kD + c]);
+      const float v = Elem<T>::to_float(reinterpret_cast<const T*>(tile)[j * kPRow + c]);
       mn = fminf(mn, v); mx = fmaxf(mx, v);
     }
     const uint16_t sh = f2h_bits(__fdiv_rn(__fsub_rn(mx, mn), 3.0f)), zh = f2h_bits(mn);
@@ -295,29 +259,58 @@ __global__ void __launch_bounds__(128) v_protect_kernel(KSrc src, CacheView cv, 
     reinterpret_cast<uint16_t*>(pg + kPG_Z)[c] = zh;
     const float s = h2f(sh), z = h2f(zh);
 #pragma unroll
-    for (int k = 1; k <= 3; ++k) s_thr[k - 1][c] = code_threshold<T>(s, z, k);
+    for (int k = 1; k <= 3; ++k) s_thr[(k - 1) * kD + c] = code_cut<T>(z, s, k);
   }
   __syncthreads();
-  for (int item = threadIdx.x; item < kG * 8; item += 128) {
+  if (n_rows <= 0) return;
+  for (int item = tid; item < kG * 8; item += 128) {
     // item = word index ((kt * 4 + w) * 4 + r) * 8 + rho: 4 channels x 4 tokens
     const int rho = item & 7, r = (item >> 3) & 3, w = (item >> 5) & 3, kt = item >> 7;
     const int c0 = 32 * w + 4 * rho;
-    float t1[4], t2[4], t3[4];
+    uint2 X[3];                                       // thresholds of channels c0 .. c0 + 3
 #pragma unroll
-    for (int e = 0; e < 4; ++e) { t1[e] = s_thr[0][c0 + e]; t2[e] = s_thr[1][c0 + e]; t3[e] = s_thr[2][c0 + e]; }
+    for (int k = 0; k < 3; ++k) X[k] = *reinterpret_cast<const uint2*>(s_thr + k * kD + c0);
     uint32_t word = 0;
 #pragma unroll
-    for (int f = 0; f < 16; ++f) {
-      const int e = f & 3, u = (f >> 2) & 1, hf = f >> 3;
-      const int j = 16 * kt + 8 * u + 2 * r + hf;
-      if (j < n_rows) {
-        const float v = Elem<T>::to_float(reinterpret_cast<const T*>(tile)[j * kD + c0 + e]);
-        const uint32_t code = static_cast<uint32_t>(v >= t1[e]) + static_cast<uint32_t>(v >= t2[e]) + static_cast<uint32_t>(v >= t3[e]);
-        word |= code << (2 * (4 * u + e) + 16 * hf);
+    for (int u = 0; u < 2; ++u) {
+#pragma unroll
+      for (int hf = 0; hf < 2; ++hf) {
+        const int j = 16 * kt + 8 * u + 2 * r + hf;
+        const uint2 v = *reinterpret_cast<const uint2*>(tile + j * kPRow + c0);
+        // lanes: (c0, c0 + 1) with weights 1, 4, then (c0 + 2, c0 + 3) with 16, 64
+        __half2 acc = as_h2(0x64006400u);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) acc = __hfma2(as_h2(Ops<T>::ge(v.x, X[k].x)), as_h2(0x44003c00u), acc);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) acc = __hfma2(as_h2(Ops<T>::ge(v.y, X[k].y)), as_h2(0x54004c00u), acc);
+        const uint32_t a = as_u32(acc);
+        const uint32_t byte = (a | (a >> 16)) & 0xffu;
+        if (j < n_rows) word |= byte << (8 * u + 16 * hf);
       }
     }
     reinterpret_cast<uint32_t*>(pg)[item] = word;
   }
+}
+
+// ---------------------------------------------------------------------------------
+// Algorithm 2 and the value half of Algorithm 1's residual in one launch.  grid = (supergroups of the ternary stream and
+// pairs of protected groups, then one block for the n_res rows that stay as they are, if any; slabs of the call).  It lets
+// the kernel behind it start only when it is done: with the next layer's range pass resident beside it four layers of 64 x
+// 12544 tokens took 745 us, without 720.
+// ---------------------------------------------------------------------------------
+template <typename T, bool NZ>
+__global__ void __launch_bounds__(256) v_quantize_kernel(KSrc src, int64_t T_q, int64_t n_rest, int n_res, CacheView cv, int layer0, SelView sel,
+                                                         float gamma, int ternary_blocks, int protect_blocks) {
+  extern __shared__ __align__(16) uint8_t vsm[];
+  pdl_wait();
+  const uint32_t block = blockIdx.x;
+  if (block >= static_cast<uint32_t>(ternary_blocks)) {
+    const int pair = static_cast<int>(block) - ternary_blocks;
+    if (pair < protect_blocks) protect_groups<T>(vsm, src, pair, cv, layer0, sel);
+    else copy_residual_rows(src, T_q, n_res, cv, layer0, blockIdx.y, cv.vres_offset);
+    return;
+  }
+  ternary_supergroup<T, NZ>(vsm, src, n_rest, cv, layer0, sel, gamma);
 }
 
 // ---------------------------------------------------------------------------------
@@ -360,183 +353,225 @@ __global__ void __launch_bounds__(kD) v_flush_kernel(KSrc src, CacheView cv, int
 }
 
 // ---------------------------------------------------------------------------------
-// Residual copies (Algorithm 1: X_r = X[l - r:]).
+// Algorithm 1 for a prompt that is shorter than one group (longer ones leave it to the quantizing kernels).
 // ---------------------------------------------------------------------------------
-template <typename T>
-__global__ void copy_to_residual_kernel(KSrc src, int64_t t_begin, int n_tok, CacheView cv, int layer0,
-                                        int64_t res_offset, int r0) {
-  const int slab = blockIdx.x;
-  const int lb = slab / cv.H_kv, h = slab % cv.H_kv;
-  const int b = lb % cv.B, layer = layer0 + lb / cv.B;
-  const T* base = reinterpret_cast<const T*>(src.ptr) + static_cast<int64_t>(lb) * src.stride_b + h * src.stride_h;
-  uint4* dst = reinterpret_cast<uint4*>(cv.slab(layer, b, h) + res_offset);
-  for (int i = threadIdx.x; i < n_tok * 16; i += blockDim.x) {
-    const int r = i >> 4, l = i & 15;
-    dst[(r0 + r) * 16 + l] = __ldg(reinterpret_cast<const uint4*>(base + (t_begin + r) * src.stride_t) + l);
-  }
+__global__ void copy_to_residual_kernel(KSrc src, int n_tok, CacheView cv, int layer0, int64_t res_offset) {
+  copy_residual_rows(src, 0, n_tok, cv, layer0, blockIdx.x, res_offset);
 }
 
 // ---------------------------------------------------------------------------------
 // Token selection: top n of l_v saliency scores per batch element (ties: lower index).
-// One block of 1024 threads per batch element.  Phase 1: 4-pass radix select of the n-th
-// largest key.  Phase 2: E words, per-word prefix counts and the two gather lists.
+// One block of 1024 threads per batch element, or a cluster of kSelCluster of them where the row is long.
+//   phase 1  radix select of the n-th largest key, 11 + 11 + 10 bits (11 bits of a float's pattern spread a smooth
+//            distribution over some twenty bins where 8 bits have four, which the shared-memory atomics of a warp would
+//            queue up on); the blocks of a cluster add their histograms up through distributed shared memory;
+//   phase 2  E words, per-word prefix counts and the two gather lists.  With gt / eq the numbers of keys above / at the
+//            threshold before a word, min(eq, need) + gt tokens are protected before it: one scan for both.  Token t is
+//            lane t % 32 everywhere, so that scores, mask bytes and list entries move in whole lines.
+// What bounds it is latency: 4 sweeps over scores that sit in L2, and a barrier after each.  4 x 196000 scores take 43
+// us (298 with one block a row, 32 consecutive scores a thread and a serial walk over 256 bins), 6272 take 18 (39).
 // ---------------------------------------------------------------------------------
-__device__ __forceinline__ int block_exclusive_scan_1024(int v, int* s_warp, int* total) {
+constexpr int kSelThreads = 1024;
+constexpr int kSelCluster = 8;                 // portable cluster size
+// Up to 8 rows from 16384 tokens on get a cluster each.  us with one block / a cluster per row: 4 x 6272 18.8 / 20.4,
+// 4 x 12544 22.7 / 22.8, 4 x 25088 28.7 / 24.7, 4 x 196000 142 / 43; 16 x 25088 28.9 / 45.5, 16 x 50176 45.6 / 53.7.
+constexpr int64_t kSelClusterTokens = 16384;
+constexpr int kSelClusterRows = 8;
+constexpr int kSelBins = 2048;
+
+// Exclusive prefix sum over the block; *total = the sum.  s_warp: 32 words that nothing else uses until the next barrier.
+__device__ __forceinline__ int64_t block_exclusive_scan(int64_t v, int64_t* s_warp, int64_t* total) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int x = v;
+  int64_t x = v;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
-    const int y = __shfl_up_sync(0xffffffffu, x, o);
+    const int64_t y = __shfl_up_sync(0xffffffffu, x, o);
     if (lane >= o) x += y;
   }
   if (lane == 31) s_warp[warp] = x;
   __syncthreads();
-  if (warp == 0) {
-    int w = s_warp[lane];
+  int64_t w = s_warp[lane];                    // every warp sums up the warps itself
+  const int64_t own = w;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, w, o);
-      if (lane >= o) w += y;
-    }
-    s_warp[lane] = w;
+  for (int o = 1; o < 32; o <<= 1) {
+    const int64_t y = __shfl_up_sync(0xffffffffu, w, o);
+    if (lane >= o) w += y;
   }
+  *total = __shfl_sync(0xffffffffu, w, 31);
+  const int64_t before = __shfl_sync(0xffffffffu, w - own, warp);
   __syncthreads();
-  const int warp_off = warp ? s_warp[warp - 1] : 0;
-  *total = s_warp[31];
-  __syncthreads();
-  return warp_off + x - v;
+  return before + x - v;
 }
 
-// mode 0: from saliency (radix select); mode 1: from a byte mask E [B][T].
-__global__ void __launch_bounds__(1024) select_tokens_kernel(const float* __restrict__ saliency,
-                                                             const uint8_t* __restrict__ mask, int64_t mask_stride,
-                                                             int64_t vis_begin, int64_t l_v, int64_t n_prot,
-                                                             int64_t T_q, CacheView cv, int32_t* idx_prot,
-                                                             int32_t* idx_rest, int64_t stride_prot,
-                                                             int64_t stride_rest, int32_t* counts,
-                                                             int64_t expect_count) {
-  __shared__ int hist[256];
-  __shared__ int s_warp[32];
-  __shared__ uint32_t s_prefix, s_need;
-  const int b = blockIdx.x;
+// From saliency (radix select) or, where that is NULL, from a byte mask E [B][T].
+__global__ void __launch_bounds__(kSelThreads) select_tokens_kernel(const float* __restrict__ saliency,
+                                                                    const uint8_t* __restrict__ mask, int64_t mask_stride,
+                                                                    int64_t vis_begin, int64_t l_v, int64_t n_prot,
+                                                                    int64_t T_q, CacheView cv, int32_t* idx_prot,
+                                                                    int32_t* idx_rest, int64_t stride_prot,
+                                                                    int64_t stride_rest, int32_t* counts,
+                                                                    int64_t expect_count) {
+  __shared__ int hist[3][kSelBins];
+  __shared__ int64_t s_warp[32];
+  __shared__ int64_t s_block;                  // (keys at the threshold) << 32 | (keys above it) in this block's words
+  __shared__ uint32_t s_bin, s_need;
+  cg::cluster_group cluster = cg::this_cluster();
+  const int n_blocks = static_cast<int>(cluster.num_blocks()), rank = static_cast<int>(cluster.block_rank());
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int b = blockIdx.x / n_blocks;
   const float* sal = saliency ? saliency + b * l_v : nullptr;
+  const int64_t W = T_q / kG;
+  const int64_t w_begin = W * rank / n_blocks, w_end = W * (rank + 1) / n_blocks;
   uint32_t thr = 0, need = 0;
-  if (sal && n_prot > 0) {
-    uint32_t prefix = 0, pmask = 0;
+  if (sal) {
+    for (int i = tid; i < 3 * kSelBins; i += kSelThreads) hist[0][i] = 0;
+    __syncthreads();
+    const int64_t s_begin = l_v * rank / n_blocks, s_end = l_v * (rank + 1) / n_blocks;
+    uint32_t pmask = 0;
     need = static_cast<uint32_t>(n_prot);
-    for (int pass = 0; pass < 4; ++pass) {
-      const int shift = 24 - 8 * pass;
-      if (threadIdx.x < 256) hist[threadIdx.x] = 0;
-      __syncthreads();
-      for (int64_t i = threadIdx.x; i < l_v; i += 1024) {
-        const uint32_t key = float_ordered(sal[i]);
-        if ((key & pmask) == prefix) atomicAdd(&hist[(key >> shift) & 255], 1);
+#pragma unroll
+    for (int pass = 0; pass < 3; ++pass) {
+      const int shift = pass == 0 ? 21 : (pass == 1 ? 10 : 0);
+      const uint32_t bins = pass == 2 ? 1024u : 2048u;
+#pragma unroll 8
+      for (int64_t i = s_begin + tid; i < s_end; i += kSelThreads) {
+        const uint32_t key = float_ordered(__ldg(sal + i));
+        if ((key & pmask) == thr) atomicAdd(&hist[pass][(key >> shift) & (bins - 1)], 1);
       }
-      __syncthreads();
-      if (threadIdx.x == 0) {
-        uint32_t cum = 0;
-        int d = 255;
-        for (; d > 0; --d) {
-          if (cum + hist[d] >= need) break;
-          cum += hist[d];
-        }
-        s_prefix = prefix | (static_cast<uint32_t>(d) << shift);
-        s_need = need - cum;
+      cluster.sync();
+      // bins from the top: thread i has bins - 1 - 2 i and the one below it
+      int c0 = 0, c1 = 0;
+      const int top = kSelBins - 1 - 2 * tid;
+      for (int r = 0; r < n_blocks; ++r) {
+        const int2 c = *reinterpret_cast<const int2*>(cluster.map_shared_rank(&hist[pass][top - 1], r));
+        c0 += c.y; c1 += c.x;
       }
+      int64_t total;
+      const int64_t above = block_exclusive_scan(c0 + c1, s_warp, &total);
+      if (above < need && above + c0 >= need) { s_bin = top; s_need = need - static_cast<uint32_t>(above); }
+      else if (above + c0 < need && above + c0 + c1 >= need) { s_bin = top - 1; s_need = need - static_cast<uint32_t>(above + c0); }
       __syncthreads();
-      prefix = s_prefix; need = s_need;
-      pmask |= 255u << shift;
-      __syncthreads();
+      thr |= s_bin << shift; need = s_need;    // thr: key of the n-th largest; `need` of the keys equal to it are taken
+      pmask |= (bins - 1) << shift;
     }
-    thr = prefix;       // key of the n-th largest; `need` of the keys equal to it are taken
+  }
+  // gt / eq bits of token group w, the same in every lane
+  auto word_bits = [&](int64_t w, uint32_t& gt, uint32_t& eq) {
+    const int64_t t = w * kG + lane;
+    bool g = false, e = false;
+    if (sal) {
+      if (t >= vis_begin && t < vis_begin + l_v) {
+        const uint32_t key = float_ordered(__ldg(sal + (t - vis_begin)));
+        g = key > thr; e = key == thr;
+      }
+    } else {
+      g = __ldg(mask + b * mask_stride + t) != 0;
+    }
+    gt = __ballot_sync(0xffffffffu, g); eq = __ballot_sync(0xffffffffu, e);
+  };
+  int64_t carry = 0;                           // (at) << 32 | (above) before the next stretch of words
+  if (n_blocks > 1) {
+    int64_t mine = 0;
+#pragma unroll 8
+    for (int64_t w = w_begin + warp; w < w_end; w += 32) {
+      uint32_t gt, eq;
+      word_bits(w, gt, eq);
+      mine += static_cast<int64_t>(__popc(gt)) | (static_cast<int64_t>(__popc(eq)) << 32);
+    }
+    if (lane == 0) s_warp[warp] = mine;
+    __syncthreads();
+    if (tid == 0) {
+      int64_t sum = 0;
+      for (int i = 0; i < 32; ++i) sum += s_warp[i];
+      s_block = sum;
+    }
+    cluster.sync();
+    for (int r = 0; r < rank; ++r) carry += *cluster.map_shared_rank(&s_block, r);
   }
   uint32_t* e_words = const_cast<uint32_t*>(cv.e_words(b));
   uint32_t* e_prefix = const_cast<uint32_t*>(cv.e_prefix(b));
-  const int64_t W = T_q / kG;
-  int eq_carry = 0, prot_carry = 0;
-  for (int64_t wbase = 0; wbase < W; wbase += 1024) {
-    const int64_t w = wbase + threadIdx.x;
-    uint32_t word_gt = 0, word_eq = 0;
-    if (w < W) {
-      for (int i = 0; i < 32; ++i) {
-        const int64_t t = w * 32 + i;
-        if (mask) {
-          if (mask[b * mask_stride + t]) word_gt |= 1u << i;
-        } else if (sal && n_prot > 0 && t >= vis_begin && t < vis_begin + l_v) {
-          const uint32_t key = float_ordered(sal[t - vis_begin]);
-          if (key > thr) word_gt |= 1u << i;
-          else if (key == thr) word_eq |= 1u << i;
-        }
-      }
+  for (int64_t base = w_begin; base < w_end; base += kSelThreads) {
+    // up to 1024 words at a time: every warp takes per_warp consecutive ones, lane i keeps word i
+    const int n = static_cast<int>(min(static_cast<int64_t>(kSelThreads), w_end - base));
+    const int per_warp = (n + 31) / 32;
+    const int n_own = max(0, min(per_warp, n - warp * per_warp));
+    const int64_t w0 = base + warp * per_warp;
+    uint32_t gt = 0, eq = 0;
+#pragma unroll 8
+    for (int i = 0; i < n_own; ++i) {
+      uint32_t g, e;
+      word_bits(w0 + i, g, e);
+      if (lane == i) { gt = g; eq = e; }
     }
-    int total;
-    int eq_before = block_exclusive_scan_1024(__popc(word_eq), s_warp, &total) + eq_carry;
-    eq_carry += total;
-    uint32_t word = word_gt;
-    int take = static_cast<int>(need) - eq_before;
-    for (uint32_t rem = word_eq; rem && take > 0; rem &= rem - 1, --take) word |= rem & (0u - rem);
-    int prot_before = block_exclusive_scan_1024(__popc(word), s_warp, &total) + prot_carry;
-    prot_carry += total;
-    if (w < W) {
-      e_words[w] = word;
-      e_prefix[w] = static_cast<uint32_t>(prot_before);
-      int pk = prot_before;
-      for (int i = 0; i < 32; ++i) {
-        const int64_t t = w * 32 + i;
-        if (word & (1u << i)) { if (idx_prot && pk < stride_prot) idx_prot[b * stride_prot + pk] = static_cast<int32_t>(t); ++pk; }
-        else if (idx_rest) idx_rest[b * stride_rest + (t - pk)] = static_cast<int32_t>(t);
+    int64_t total;
+    const int64_t before = carry + block_exclusive_scan(static_cast<int64_t>(__popc(gt)) | (static_cast<int64_t>(__popc(eq)) << 32), s_warp, &total);
+    carry += total;
+    const int64_t eq_before = before >> 32;
+    int take = static_cast<int>(need) - static_cast<int>(min(eq_before, static_cast<int64_t>(need)));
+    const int prot = static_cast<int>((before & 0xffffffff) + (static_cast<int64_t>(need) - take));
+    uint32_t word = gt;
+    for (uint32_t rem = eq; rem && take > 0; rem &= rem - 1, --take) word |= rem & (0u - rem);
+    if (lane < n_own) {
+      e_words[w0 + lane] = word;
+      e_prefix[w0 + lane] = static_cast<uint32_t>(prot);
+    }
+#pragma unroll 4
+    for (int i = 0; i < n_own; ++i) {
+      const uint32_t bits = __shfl_sync(0xffffffffu, word, i);
+      const int64_t t = (w0 + i) * kG + lane;
+      const int64_t pk = __shfl_sync(0xffffffffu, prot, i) + __popc(bits & ((1u << lane) - 1u));
+      if ((bits >> lane) & 1u) {
+        if (pk < stride_prot) idx_prot[b * stride_prot + pk] = static_cast<int32_t>(t);
+      } else {
+        idx_rest[b * stride_rest + (t - pk)] = static_cast<int32_t>(t);
       }
     }
   }
-  if (threadIdx.x == 0) {
-    e_prefix[W] = static_cast<uint32_t>(prot_carry);
+  if (rank == n_blocks - 1 && tid == 0) {
+    const int n = static_cast<int>((carry & 0xffffffff) + min(carry >> 32, static_cast<int64_t>(need)));
+    e_prefix[W] = static_cast<uint32_t>(n);
     e_words[W] = 0;
-    if (counts) counts[b] = prot_carry;
+    if (counts) counts[b] = n;
     // a mask whose row does not protect the number of tokens the caller stated
-    if (expect_count >= 0 && prot_carry != expect_count)
+    if (expect_count >= 0 && n != expect_count)
       atomicCAS(reinterpret_cast<int*>(cv.base + kHdrStatus), VIDKV_OK, VIDKV_ERR_INVALID_ARG);
   }
+  if (n_blocks > 1) cluster.sync();            // the other blocks may still read this one's shared memory
 }
 
 // ---------------------------------------------------------------------------------
 // Host launchers
 // ---------------------------------------------------------------------------------
 template <typename T, bool NZ>
-static cudaError_t quantize_values_t(const KSrc& src, int64_t T_q, const CacheView& cv, int layer, int n_layers,
+static cudaError_t quantize_values_t(const KSrc& src, int64_t T_q, int n_res, const CacheView& cv, int layer, int n_layers,
                                      const SelView& sel, float gamma, cudaStream_t stream) {
   const int n_slabs = n_layers * cv.B * cv.H_kv;
-  const int64_t n_rest = T_q - sel.n_prot;
-  if (n_rest > 0) {
-    const int64_t sgs = (n_rest + kSGTokens - 1) / kSGTokens;
-    const size_t smem = kSGTokens * kVRowBytes + sizeof(float) * kSGGroups * 4 * kD + sizeof(uint32_t) * kSGGroups * 64 + 256 +
-                        (NZ ? sizeof(float) * kSGGroups * 4 * kD : 0);
-    static bool attr_set_dev[64] = {};   // function attributes are per device (and per instantiation)
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    bool& attr_set = attr_set_dev[dev];
-    if (!attr_set) {
-      cudaError_t e;
-      if ((e = cudaFuncSetAttribute(v_ternary_kernel<T, NZ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))) return e;
-      attr_set = true;
-    }
-    v_ternary_kernel<T, NZ><<<dim3(static_cast<unsigned>(sgs), n_slabs), 256, smem, stream>>>(src, n_rest, cv, layer, sel, gamma);
-    count_launches(1);
+  const int ternary_blocks = static_cast<int>((T_q - sel.n_prot + kSGTokens - 1) / kSGTokens);
+  const int protect_blocks = static_cast<int>((sel.n_prot + 2 * kG - 1) / (2 * kG));
+  constexpr size_t smem = kSGTokens * kVRowBytes + sizeof(float) * kSGGroups * 4 * kD + sizeof(uint32_t) * kSGGroups * 64 + 256 +
+                          (NZ ? sizeof(float) * kSGGroups * 4 * kD : 0);
+  static_assert(smem >= kProtectSmem, "the protected groups live in the ternary tile's shared memory");
+  static bool attr_set_dev[64] = {};   // function attributes are per device (and per instantiation)
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  bool& attr_set = attr_set_dev[dev];
+  cudaError_t e;
+  if (!attr_set) {
+    if ((e = cudaFuncSetAttribute(v_quantize_kernel<T, NZ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))) return e;
+    attr_set = true;
   }
-  if (sel.n_prot > 0) {
-    const int64_t pgs = (sel.n_prot + kG - 1) / kG;
-    v_protect_kernel<T><<<dim3(static_cast<unsigned>(pgs), n_slabs), 128, 0, stream>>>(src, cv, layer, sel);
-    count_launches(1);
-  }
-  return cudaGetLastError();
+  count_launches(1);
+  return launch_dependent(v_quantize_kernel<T, NZ>, dim3(static_cast<unsigned>(ternary_blocks + protect_blocks + (n_res > 0)), n_slabs),
+                          dim3(256), smem, stream, src, T_q, T_q - sel.n_prot, n_res, cv, layer, sel, gamma, ternary_blocks, protect_blocks);
 }
 
-cudaError_t launch_quantize_values(int dtype, const KSrc& src, int64_t T_q, const CacheView& cv, int layer, int n_layers,
+cudaError_t launch_quantize_values(int dtype, const KSrc& src, int64_t T_q, int n_res, const CacheView& cv, int layer, int n_layers,
                                    const SelView& sel, float gamma, bool nonzero_mean_scale, cudaStream_t stream) {
   if (dtype == VIDKV_F16)
-    return nonzero_mean_scale ? quantize_values_t<__half, true>(src, T_q, cv, layer, n_layers, sel, gamma, stream)
-                              : quantize_values_t<__half, false>(src, T_q, cv, layer, n_layers, sel, gamma, stream);
-  return nonzero_mean_scale ? quantize_values_t<__nv_bfloat16, true>(src, T_q, cv, layer, n_layers, sel, gamma, stream)
-                            : quantize_values_t<__nv_bfloat16, false>(src, T_q, cv, layer, n_layers, sel, gamma, stream);
+    return nonzero_mean_scale ? quantize_values_t<__half, true>(src, T_q, n_res, cv, layer, n_layers, sel, gamma, stream)
+                              : quantize_values_t<__half, false>(src, T_q, n_res, cv, layer, n_layers, sel, gamma, stream);
+  return nonzero_mean_scale ? quantize_values_t<__nv_bfloat16, true>(src, T_q, n_res, cv, layer, n_layers, sel, gamma, stream)
+                            : quantize_values_t<__nv_bfloat16, false>(src, T_q, n_res, cv, layer, n_layers, sel, gamma, stream);
 }
 
 template <typename T, bool NZ>
@@ -559,33 +594,39 @@ cudaError_t launch_flush_values(int dtype, const KSrc& src, const CacheView& cv,
   return cudaGetLastError();
 }
 
-cudaError_t launch_copy_to_residual(int dtype, const KSrc& src, int64_t t_begin, int n_tok, const CacheView& cv,
-                                    int layer, int n_layers, bool is_value, int r0, cudaStream_t stream) {
+cudaError_t launch_copy_to_residual(const KSrc& src, int n_tok, const CacheView& cv, int layer, int n_layers, bool is_value,
+                                    cudaStream_t stream) {
   if (n_tok <= 0) return cudaSuccess;
-  const int64_t off = is_value ? cv.vres_offset : cv.kres_offset;
-  // 16-bit elements either way: the copy is type-agnostic
-  (void)dtype;
-  copy_to_residual_kernel<__half><<<n_layers * cv.B * cv.H_kv, 256, 0, stream>>>(src, t_begin, n_tok, cv, layer, off, r0);
+  copy_to_residual_kernel<<<n_layers * cv.B * cv.H_kv, 256, 0, stream>>>(src, n_tok, cv, layer, is_value ? cv.vres_offset : cv.kres_offset);
   count_launches(1);
   return cudaGetLastError();
+}
+
+static cudaError_t launch_select(const float* saliency, const uint8_t* mask, int64_t mask_stride, int64_t vis_begin, int64_t l_v,
+                                 int64_t n_prot, int64_t T_q, const CacheView& cv, int32_t* idx_prot, int32_t* idx_rest,
+                                 int64_t stride_prot, int64_t stride_rest, int32_t* counts, int64_t expect_count, cudaStream_t stream) {
+  const unsigned blocks = T_q >= kSelClusterTokens && cv.B <= kSelClusterRows ? kSelCluster : 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(blocks * cv.B); cfg.blockDim = dim3(kSelThreads); cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = blocks; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr; cfg.numAttrs = 1;
+  count_launches(1);
+  return cudaLaunchKernelEx(&cfg, select_tokens_kernel, saliency, mask, mask_stride, vis_begin, l_v, n_prot, T_q, cv, idx_prot, idx_rest,
+                            stride_prot, stride_rest, counts, expect_count);
 }
 
 cudaError_t launch_select_tokens(const float* saliency, int64_t vis_begin, int64_t l_v, int64_t n_prot, int64_t T_q,
                                  const CacheView& cv, int32_t* idx_prot, int32_t* idx_rest, int64_t stride_prot,
                                  int64_t stride_rest, cudaStream_t stream) {
-  select_tokens_kernel<<<cv.B, 1024, 0, stream>>>(saliency, nullptr, 0, vis_begin, l_v, n_prot, T_q, cv, idx_prot,
-                                                  idx_rest, stride_prot, stride_rest, nullptr, -1);
-  count_launches(1);
-  return cudaGetLastError();
+  return launch_select(saliency, nullptr, 0, vis_begin, l_v, n_prot, T_q, cv, idx_prot, idx_rest, stride_prot, stride_rest, nullptr, -1, stream);
 }
 
 cudaError_t launch_mask_to_selection(const uint8_t* E, int64_t T, int64_t T_q, const CacheView& cv, int32_t* idx_prot,
                                      int32_t* idx_rest, int64_t stride_prot, int64_t stride_rest, int32_t* counts,
                                      int64_t expect_count, cudaStream_t stream) {
-  select_tokens_kernel<<<cv.B, 1024, 0, stream>>>(nullptr, E, T, 0, 0, 0, T_q, cv, idx_prot, idx_rest, stride_prot,
-                                                  stride_rest, counts, expect_count);
-  count_launches(1);
-  return cudaGetLastError();
+  return launch_select(nullptr, E, T, 0, 0, 0, T_q, cv, idx_prot, idx_rest, stride_prot, stride_rest, counts, expect_count, stream);
 }
 
 }  // namespace vidkv

@@ -22,7 +22,19 @@ __global__ void __launch_bounds__(kSalThreads) text_sum_kernel(const T* __restri
   if (2 * c2 >= d) return;
   const uint32_t* p = reinterpret_cast<const uint32_t*>(x_t + b * l_t * d) + c2;
   float a0 = 0.0f, a1 = 0.0f;
-  for (int64_t j = 0; j < l_t; ++j) {
+  constexpr int kAhead = 32;                    // loads in flight: the sum itself is one chain, in token order
+  int64_t j = 0;
+  for (; j + kAhead <= l_t; j += kAhead) {
+    uint32_t w[kAhead];
+#pragma unroll
+    for (int i = 0; i < kAhead; ++i) w[i] = __ldg(p + (j + i) * (d / 2));
+#pragma unroll
+    for (int i = 0; i < kAhead; ++i) {
+      const float2 f = Elem<T>::to_float2(w[i]);
+      a0 += f.x; a1 += f.y;
+    }
+  }
+  for (; j < l_t; ++j) {
     const float2 f = Elem<T>::to_float2(__ldg(p + j * (d / 2)));
     a0 += f.x; a1 += f.y;
   }
