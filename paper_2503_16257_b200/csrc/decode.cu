@@ -19,6 +19,9 @@ constexpr int kMinRunUnits = 1;     // with fewer units than warps every unit ge
 // with protected tokens 160 units 21.9 / 31.2, 1792 units of 448 slabs (4 a block) 37 / 41, 2240 units of 224 slabs 50 / 43.
 constexpr int kMaxBlockUnits = 7;
 constexpr int kMaxBlockUnitsStp = 3;
+// A token shard's call with protected tokens (exact maxima, see DecodePlan::equal_units): 1152 units of 64 slabs, two a block,
+// took 275 us for eight calls against 269 with runs.
+constexpr int kMaxBlockUnitsStpPartial = 1;
 
 }  // namespace
 
@@ -54,17 +57,32 @@ DecodePlan plan_decode(const LayerState& st, int64_t n_slabs, bool stp, bool gen
   if (force_run_units > 0) run = force_run_units;
   p.run_units = static_cast<int32_t>(run);
   if (partial) p.equal_units = p.run_units;
-  p.n_runs = static_cast<int32_t>(force_run_units > 0 || partial ? (p.n_units + run - 1) / run : (p.n_units < warps ? p.n_units : warps));
+  int64_t runs = p.n_units < warps ? p.n_units : warps;
+  if (force_run_units > 0 || partial) {
+    runs = (p.n_units + run - 1) / run;
+  } else if (stp && n_slabs > 0 && warps >= n_slabs) {
+    // With protected tokens a run pays for every slab that it enters and for the supergroup and the protected group that it
+    // shares with its neighbour at a cut inside a slab.  Where a slab divides evenly into its share of the warps (at most half
+    // a key group per run left over), every slab gets that many runs and none straddles two.  us per step, all warps /
+    // evenly: 112 slabs of 6400 tokens 59.5 / 59.0, of 16000 109.1 / 107.2, 168 of 9000 98.3 / 92.4, 224 of 6400 (k = 0.75)
+    // 117.4 / 112.3; uneven shares lose: 64 slabs of 12544 (4.4 units a run) 64.8 / 69.2, 112 of 12544 (7.8) 90.4 / 92.9.
+    // Without protected tokens they lose too: 112 slabs of 12819 70.3 / 77.0.
+    const int64_t share = warps / n_slabs, groups = T_qt / kG;
+    if (groups >= share * kSGGroups && groups % (share * kSGGroups) <= share / 2 && n_slabs * share * run >= p.n_units)
+      runs = n_slabs * share;
+  }
+  p.n_runs = static_cast<int32_t>(runs);
   // a run is n_units / n_runs units long or one more
-  const auto most_parts = [&](int64_t runs) -> int64_t {
-    const int64_t shortest = p.equal_units > 0 ? p.equal_units : runs > 0 ? p.n_units / runs : 1;
+  const auto most_parts = [&](int64_t n) -> int64_t {
+    const int64_t shortest = p.equal_units > 0 ? p.equal_units : n > 0 ? p.n_units / n : 1;
     return p.units_per_slab > 0 ? (p.units_per_slab + shortest - 1) / shortest + 1 : 1;
   };
   p.slab_parts = static_cast<int32_t>(most_parts(p.n_runs));
   p.records = (p.n_runs + n_slabs) * kMaxRep;
   const int64_t blocks = static_cast<int64_t>(sms) * (stp && general ? kBlockGenStpPerSM : kBlocksPerSM);
   const int64_t per_block = (p.n_units + blocks - 1) / blocks;
-  if (p.n_units == 0 || (per_block <= (stp ? kMaxBlockUnitsStp : kMaxBlockUnits) && force_run_units == 0 && (!partial || run == 1))) {
+  const int64_t most = !stp ? kMaxBlockUnits : partial ? kMaxBlockUnitsStpPartial : kMaxBlockUnitsStp;
+  if (p.n_units == 0 || (per_block <= most && force_run_units == 0 && (!partial || run == 1))) {
     p.n_blocks = static_cast<int32_t>(p.n_units < blocks ? p.n_units : blocks);
     p.res_blocks = st.n_res > 0 && per_block <= 1 ? static_cast<int32_t>(n_slabs) : 0;
     p.counters_per_slab = static_cast<int32_t>(join_counters(most_parts(p.n_blocks) + (p.res_blocks > 0)));
