@@ -1,4 +1,4 @@
-// Device helpers of the key quantizers: 16-bit element operations and the exact decision of Eq. 4 codes
+// Device helpers of the quantizers: 16-bit element operations and the exact decision of Eq. 4 codes
 // without a division per element.
 #pragma once
 

@@ -22,7 +22,7 @@ __global__ void __launch_bounds__(kSalThreads) text_sum_kernel(const T* __restri
   if (2 * c2 >= d) return;
   const uint32_t* p = reinterpret_cast<const uint32_t*>(x_t + b * l_t * d) + c2;
   float a0 = 0.0f, a1 = 0.0f;
-  constexpr int kAhead = 32;                    // loads in flight: the sum itself is one chain, in token order
+  constexpr int kAhead = 32;                    // loads in flight: the sum itself is one chain, in token order (128 tokens: 20 -> 10 us)
   int64_t j = 0;
   for (; j + kAhead <= l_t; j += kAhead) {
     uint32_t w[kAhead];

@@ -733,6 +733,38 @@ def test_saliency_ties_take_lower_index():
     assert (E == ref).all() and E.sum() == 12 and E[0] and not E[2]
 
 
+@pytest.mark.parametrize("B,T,vis_begin,l_v", [
+    (2, 16383, 0, 16352),           # the longest rows with one block each
+    (2, 16384 + 77, 35, 16384),     # a cluster per row; the scored tokens start and end inside words
+    (8, 16384, 0, 16384), (9, 16384, 0, 16384),
+    (1, 33000, 5, 40),              # most of the cluster's blocks see no score
+    (1, 20000, 31, 4)])             # fewer scores than blocks
+def test_token_selection_by_blocks_and_by_clusters(B, T, vis_begin, l_v):
+    """One block or a cluster of blocks per row of scores: the same tokens as the oracle's (whole numbers, no
+    tolerance), with ties across the blocks' borders (scores in steps of 1/8), and the same gather lists as the mask
+    entry point gives."""
+    import paper_2503_16257_b200 as P
+    p = 0.3125
+    sal = (torch.randn((B, l_v), generator=torch.Generator().manual_seed(T + B)) * 8).round() / 8
+    V = torch.randn((B, 1, T, 128), generator=torch.Generator().manual_seed(1)).to(torch.float16).cuda()
+    cfg = P.VidKVConfig(B=B, L=1, H_kv=1, H_q=1, max_prefill_tokens=T, max_new_tokens=1, p_ratio=p)
+    a, b = P.VidKVCache(cfg), P.VidKVCache(cfg)
+    a.select_tokens(sal.cuda(), vis_begin, l_v, T)
+    a.quantize_values(0, V)
+    Tq = T - T % 32
+    want = np.stack([O.select_tokens(sal[i].numpy(), p, vis_begin, Tq) for i in range(B)])
+    E = np.zeros((B, T), dtype=np.uint8)
+    E[:, :Tq] = want
+    b.set_token_mask(torch.from_numpy(E).cuda(), T)
+    b.quantize_values(0, V)
+    torch.cuda.synchronize()
+    host = a.cache.cpu().numpy()
+    for i in range(B):
+        got, _ = U.selection_mask(host, a.layout, i, Tq)
+        assert (got == want[i]).all()
+    assert torch.equal(a.cache, b.cache) and a.status() == 0 and b.status() == 0
+
+
 @pytest.mark.parametrize("name,p", [("tiny", 0.2), ("qwen", 0.0)])
 def test_values_quantized_on_a_second_stream_give_the_same_cache(name, p):
     """The key and the value quantizer write disjoint parts of the cache and workspace: with the values on a
