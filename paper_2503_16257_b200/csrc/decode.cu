@@ -118,11 +118,12 @@ int64_t max_decode_records(int64_t max_slabs, int64_t max_tokens) {
 // Shared memory for n_pad staged rows (n_res rounded up to 16):
 //   Ks, Vs  n_pad rows of 272 bytes (256 + 16 of padding: conflict-free fragment loads)
 //   S       [8][n_pad] float scores        Ph  [8][n_pad + 8] binary16 probabilities
-//   Mh, Lh  [8] maxima and denominators
+//   Mh, Lh, Wh  [8] maxima, denominators and the weight of the residual's sums, whose probabilities are
+//           taken against the residual's own maximum
 // ---------------------------------------------------------------------------------
 constexpr int kMergeRow = kD * 2 + 16;
 size_t merge_smem_bytes(int n_pad) {
-  return static_cast<size_t>(2) * n_pad * kMergeRow + sizeof(float) * 8 * n_pad + sizeof(__half) * 8 * (n_pad + 8) + 64;
+  return static_cast<size_t>(2) * n_pad * kMergeRow + sizeof(float) * 8 * n_pad + sizeof(__half) * 8 * (n_pad + 8) + 3 * 8 * sizeof(float);
 }
 
 template <typename T>
@@ -135,6 +136,7 @@ __global__ void __launch_bounds__(kD) decode_merge_kernel(DecodeArgs a, int n_re
   const int PS = n_pad + 8;
   float* Mh = reinterpret_cast<float*>(Ph + 8 * PS);
   float* Lh = Mh + 8;
+  float* Wh = Lh + 8;
   const CacheView& cv = a.cv;
   const int slab = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, hd = lane >> 2, r = lane & 3;
   const int h = slab % cv.H_kv, lb = slab / cv.H_kv, rep = cv.rep;
@@ -224,20 +226,26 @@ __global__ void __launch_bounds__(kD) decode_merge_kernel(DecodeArgs a, int n_re
   }
   // ---- maxima and denominators: warp w takes heads w and w + 4
   for (int k = warp; k < kMaxRep; k += kD / 32) {
-    float m = -INFINITY;
+    float m = -INFINITY, m_res = -INFINITY;
     if (k < rep) {
-      for (int t = lane; t < n_res; t += 32) m = fmaxf(m, S[k * n_pad + t]);
+      for (int t = lane; t < n_res; t += 32) m_res = fmaxf(m_res, S[k * n_pad + t]);
       for (int j = lane; j < n_parts; j += 32) m = fmaxf(m, __ldg(rec + (j * kMaxRep + k) * kRecordFloats));
     }
 #pragma unroll
-    for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    for (int o = 16; o; o >>= 1) {
+      m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+      m_res = fmaxf(m_res, __shfl_xor_sync(0xffffffffu, m_res, o));
+    }
+    m = fmaxf(m, m_res);
+    const float w_res = k < rep && n_res > 0 ? exp2f(m_res - m) : 0.0f;
     float l = 0.0f;
     for (int t = lane; t < n_pad; t += 32) {
       __half ph = __float2half_rn(0.0f);
-      if (k < rep && t < n_res) ph = __float2half_rn(exp2f(S[k * n_pad + t] - m));
+      if (k < rep && t < n_res) ph = __float2half_rn(exp2f(S[k * n_pad + t] - m_res));
       Ph[k * PS + t] = ph;
       l += __half2float(ph);
     }
+    l *= w_res;
     if (k < rep)
       for (int j = lane; j < n_parts; j += 32) {
         const float* pr = rec + (j * kMaxRep + k) * kRecordFloats;
@@ -245,7 +253,7 @@ __global__ void __launch_bounds__(kD) decode_merge_kernel(DecodeArgs a, int n_re
       }
 #pragma unroll
     for (int o = 16; o; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
-    if (lane == 0) { Mh[k] = m; Lh[k] = l; }
+    if (lane == 0) { Mh[k] = m; Lh[k] = l; Wh[k] = w_res; }
   }
   __syncthreads();
   // ---- P V_r: warp w owns channels 32 w .. 32 w + 31 as four 8-channel tiles
@@ -265,7 +273,9 @@ __global__ void __launch_bounds__(kD) decode_merge_kernel(DecodeArgs a, int n_re
   }
   // ---- join the records: lane (hd, r) holds head hd, channels 32 w + 8 j + 2 r, + 1
   if (hd < rep) {
-    const float M = Mh[hd], inv = 1.0f / Lh[hd];
+    const float M = Mh[hd], inv = 1.0f / Lh[hd], w_res = Wh[hd];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) { acc[j][0] *= w_res; acc[j][1] *= w_res; }
 #pragma unroll
     for (int jp = 0; jp < kRecAhead; ++jp) {
       const float wgt = exp2f(rec_m[jp] - M);                // 0 for a record that does not exist

@@ -206,10 +206,10 @@ __device__ __forceinline__ void score_group_general(const uint8_t* kg, const Key
 // head hd at stream tokens 32 g + 8 nt + 2 r, + 1 (binary16 pairs) and ps[g] the accumulator
 // fragment -5 * (sum of those probabilities) of heads 2 r, 2 r + 1.  32 channels (two MMA row
 // blocks) at a time: fragment i of block w covers channels 32 w + 4 hd + 2 i + {0, 1} in rows hd,
-// hd + 8.  Adds into the warp's running output.
-template <int NG>
+// hd + 8.  Adds into the warp's running output; WEIGHTED: times wa (heads 2 r) and wb (heads 2 r + 1).
+template <int NG, bool WEIGHTED>
 __device__ __forceinline__ void pv_ternary(const uint8_t* vbuf, float* totbuf, const uint32_t (&P)[NG][4],
-                                           const float (&ps)[NG][4], int lane, int hd, int r) {
+                                           const float (&ps)[NG][4], float wa, float wb, int lane, int hd, int r) {
 #pragma unroll 1
   for (int w = 0; w < 4; ++w) {
     float acc[NG][2][4];
@@ -250,7 +250,8 @@ __device__ __forceinline__ void pv_ternary(const uint8_t* vbuf, float* totbuf, c
       }
     }
     float4* tp = reinterpret_cast<float4*>(totbuf) + (2 * w) * 32 + lane;
-    float4 t0 = tp[0], t1 = tp[32];
+    float4 t0 = make_float4(0.0f, 0.0f, 0.0f, 0.0f), t1 = t0;
+    if (!WEIGHTED) { t0 = tp[0]; t1 = tp[32]; }
 #pragma unroll
     for (int g = 0; g < NG; ++g) {
       const uint2 sc2 = *reinterpret_cast<const uint2*>(vbuf + kSG_Scales + g * (kD * 2) + (32 * w + 4 * hd) * 2);
@@ -261,6 +262,11 @@ __device__ __forceinline__ void pv_ternary(const uint8_t* vbuf, float* totbuf, c
       t1.x += sb.x * acc[g][1][0]; t1.y += sb.x * acc[g][1][1];
       t1.z += sb.y * acc[g][1][2]; t1.w += sb.y * acc[g][1][3];
     }
+    if (WEIGHTED) {
+      const float4 u0 = tp[0], u1 = tp[32];
+      t0.x = fmaf(wa, t0.x, u0.x); t0.y = fmaf(wb, t0.y, u0.y); t0.z = fmaf(wa, t0.z, u0.z); t0.w = fmaf(wb, t0.w, u0.w);
+      t1.x = fmaf(wa, t1.x, u1.x); t1.y = fmaf(wb, t1.y, u1.y); t1.z = fmaf(wa, t1.z, u1.z); t1.w = fmaf(wb, t1.w, u1.w);
+    }
     tp[0] = t0;
     tp[32] = t1;
   }
@@ -268,7 +274,12 @@ __device__ __forceinline__ void pv_ternary(const uint8_t* vbuf, float* totbuf, c
 
 // One unit of NG (1..5) groups: scores, probabilities, P V into the running state.
 // Returns false if a copy never arrived.
-template <int NG, bool GEN>
+// SHARD (the call leaves triples): the probabilities are taken against the running maximum, which is part of the result
+// and fixes the cut.  Otherwise against the unit's own maximum: where their binary16 rounding falls depends on the unit
+// alone, not on where the warp's run began, and the largest one is exact; the unit's sums join the running ones with the
+// weight 2^(mu - m).  Off by 3.3e-5 of the outputs' norm on 64 slabs x 12544 tokens, where the running maximum gives
+// 1.14e-4 and another cut moves the outputs by 1.5e-4.  The weights cost 1.3 % of a step (a token shard's 2 %).
+template <int NG, bool GEN, bool SHARD>
 __device__ __forceinline__ bool process_unit(const KeyFmt& kf, const uint32_t*& ppc, uint8_t* kbuf, uint8_t* vbuf, float* totbuf, uint64_t* kbar, uint64_t* vbar,
                                              uint32_t& kpar, uint32_t& vpar, int lane, int hd, int r,
                                              const uint32_t* prep_slab, int64_t g_first, int64_t g0n, int& cur_chunk,
@@ -313,11 +324,11 @@ __device__ __forceinline__ bool process_unit(const KeyFmt& kf, const uint32_t*& 
     reinterpret_cast<float*>(kg)[256 + lane] = cst;         // the group's constant joins in the exponent
     mx = fmaxf(mx, gm + cst);
   }
-  // ---- probabilities against the running maximum
+  // ---- maximum of the unit, running maximum, probabilities
   mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
   mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+  const float mu = mx * sl2;                                // sl2 > 0
   {
-    const float mu = mx * sl2;                              // sl2 > 0
     const bool up = mu > run.m + kStaleLog2;                // always true for the first unit (run.m = -inf)
     if (__any_sync(0xffffffffu, up)) {
       const float m_new = up ? mu : run.m;
@@ -334,11 +345,19 @@ __device__ __forceinline__ bool process_unit(const KeyFmt& kf, const uint32_t*& 
       run.l[0] *= fa; run.l[1] *= fb;
     }
   }
+  const float ref = SHARD ? run.m : mu;
+  float wa = 1.0f, wb = 1.0f;
+  if (!SHARD) {
+    const float wgt = ex2_approx(mu - run.m);
+    wa = __shfl_sync(0xffffffffu, wgt, 8 * r);
+    wb = __shfl_sync(0xffffffffu, wgt, 8 * r + 4);
+  }
   uint32_t P[NG][4];
   float ps[NG][4];
+  float sum0 = 0.0f, sum1 = 0.0f;
 #pragma unroll
   for (int g = 0; g < NG; ++g) {
-    const float off = fmaf(reinterpret_cast<const float*>(kbuf + g * kgb)[256 + lane], sl2, -run.m);
+    const float off = fmaf(reinterpret_cast<const float*>(kbuf + g * kgb)[256 + lane], sl2, -ref);
 #pragma unroll
     for (int nt = 0; nt < 4; ++nt) {
       const float2 v = reinterpret_cast<const float2*>(kbuf + g * kgb)[nt * 32 + lane];
@@ -350,8 +369,16 @@ __device__ __forceinline__ bool process_unit(const KeyFmt& kf, const uint32_t*& 
     ps[g][0] = 0.0f; ps[g][1] = 0.0f; ps[g][2] = 0.0f; ps[g][3] = 0.0f;
     mma_f16(ps[g], kMinus5, kMinus5, kMinus5, kMinus5, P[g][0], P[g][1]);
     mma_f16(ps[g], kMinus5, kMinus5, kMinus5, kMinus5, P[g][2], P[g][3]);
-    run.l[0] = fmaf(-0.2f, ps[g][0], run.l[0]);
-    run.l[1] = fmaf(-0.2f, ps[g][1], run.l[1]);
+    if (SHARD) {
+      run.l[0] = fmaf(-0.2f, ps[g][0], run.l[0]);
+      run.l[1] = fmaf(-0.2f, ps[g][1], run.l[1]);
+    } else {
+      sum0 += ps[g][0]; sum1 += ps[g][1];
+    }
+  }
+  if (!SHARD) {
+    run.l[0] = fmaf(-0.2f * wa, sum0, run.l[0]);
+    run.l[1] = fmaf(-0.2f * wb, sum1, run.l[1]);
   }
   __syncwarp();                                             // the scores are in registers: the key buffer is free
   if (more && lane == 0) {
@@ -365,7 +392,7 @@ __device__ __forceinline__ bool process_unit(const KeyFmt& kf, const uint32_t*& 
     return false;
   }
   vpar ^= 1u;
-  pv_ternary<NG>(vbuf, totbuf, P, ps, lane, hd, r);
+  pv_ternary<NG, !SHARD>(vbuf, totbuf, P, ps, wa, wb, lane, hd, r);
   __syncwarp();
   if (more && lane == 0) {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -402,7 +429,7 @@ __device__ __forceinline__ void write_record(const DecodeArgs& a, int slab, int 
 
 }  // namespace
 
-template <bool GEN>
+template <bool GEN, bool SHARD>
 __global__ void __launch_bounds__(kStreamWarps * 32, kStreamCtasPerSM) decode_stream_kernel(DecodeArgs a) {
   extern __shared__ __align__(128) uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t bars[kStreamWarps][2];
@@ -481,7 +508,7 @@ __global__ void __launch_bounds__(kStreamWarps * 32, kStreamCtasPerSM) decode_st
     const uint32_t next_k_bytes = more ? static_cast<uint32_t>(groups_of(nk) * kgb) : 0u;
     const uint8_t* next_v = more ? val_src(nslab, nk) : nullptr;
 #define VIDKV_UNIT(N)                                                                                                \
-  ok = process_unit<N, GEN>(kf, ppc, kbuf, vbuf, totbuf, kbar, vbar, kpar, vpar, lane, hd, r, prep_slab,                           \
+  ok = process_unit<N, GEN, SHARD>(kf, ppc, kbuf, vbuf, totbuf, kbar, vbar, kpar, vpar, lane, hd, r, prep_slab,                           \
                        static_cast<int64_t>(k) * kSGGroups, g0n, cur_chunk, qa, qha, qhb, sl2, run, more, next_k,      \
                        next_k_bytes, next_v)
     if (ng == 5) VIDKV_UNIT(5);
@@ -838,7 +865,7 @@ __global__ void __launch_bounds__(kStreamWarps * 32, kStreamStpCtasPerSM) decode
         run.l[0] = fmaf(-0.2f, ps[g][0], run.l[0]);
         run.l[1] = fmaf(-0.2f, ps[g][1], run.l[1]);
       }
-      pv_ternary<kSGGroups>(vbuf, totbuf, P, ps, lane, hd, r);
+      pv_ternary<kSGGroups, false>(vbuf, totbuf, P, ps, 1.0f, 1.0f, lane, hd, r);
       ++sg_next;
       __syncwarp();
       if (sg_next < sg_total) {
@@ -911,33 +938,30 @@ cudaError_t launch_decode_stream_stp(const DecodeArgs& a, cudaStream_t stream) {
   return le;
 }
 
-cudaError_t launch_decode_stream(const DecodeArgs& a_in, cudaStream_t stream) {
-  DecodeArgs a = a_in;
-  if (g_debug_withhold == 2) { a.withhold = 1; g_debug_withhold = 0; }
-  const bool gen = a.cv.kf.general != 0;
-  const size_t smem = static_cast<size_t>(kStreamWarps) * (kWarpBufBytes + (gen ? kGenKBufBytes - kKBufBytes : 0));
-  static bool attr_set[64][2] = {};
+template <bool GEN, bool SHARD>
+static cudaError_t launch_stream_t(const DecodeArgs& a, cudaStream_t stream) {
+  constexpr int smem = kStreamWarps * (kWarpBufBytes + (GEN ? kGenKBufBytes - kKBufBytes : 0));
+  static bool attr_set[64] = {};
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-  if (!attr_set[dev][gen]) {
-    const cudaError_t e = gen ? cudaFuncSetAttribute(decode_stream_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
-                              : cudaFuncSetAttribute(decode_stream_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (!attr_set[dev]) {
+    const cudaError_t e = cudaFuncSetAttribute(decode_stream_kernel<GEN, SHARD>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    attr_set[dev][gen] = true;
+    attr_set[dev] = true;
   }
   const int grid = (a.plan.n_runs + kStreamWarps - 1) / kStreamWarps;
   if (grid < 1) return cudaSuccess;
-  cudaError_t le;
-  if (a.ev_begin) {
-    if (gen) decode_stream_kernel<true><<<grid, kStreamWarps * 32, smem, stream>>>(a);
-    else decode_stream_kernel<false><<<grid, kStreamWarps * 32, smem, stream>>>(a);
-    le = cudaGetLastError();
-  } else {
-    le = gen ? launch_dependent(decode_stream_kernel<true>, dim3(grid), dim3(kStreamWarps * 32), smem, stream, a)
-             : launch_dependent(decode_stream_kernel<false>, dim3(grid), dim3(kStreamWarps * 32), smem, stream, a);
-  }
   count_launches(1);
-  return le;
+  if (!a.ev_begin) return launch_dependent(decode_stream_kernel<GEN, SHARD>, dim3(grid), dim3(kStreamWarps * 32), smem, stream, a);
+  decode_stream_kernel<GEN, SHARD><<<grid, kStreamWarps * 32, smem, stream>>>(a);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_decode_stream(const DecodeArgs& a_in, cudaStream_t stream) {
+  DecodeArgs a = a_in;
+  if (g_debug_withhold == 2) { a.withhold = 1; g_debug_withhold = 0; }
+  if (a.cv.kf.general) return a.partial_out ? launch_stream_t<true, true>(a, stream) : launch_stream_t<true, false>(a, stream);
+  return a.partial_out ? launch_stream_t<false, true>(a, stream) : launch_stream_t<false, false>(a, stream);
 }
 
 }  // namespace vidkv

@@ -236,6 +236,40 @@ def test_small_calls_in_one_launch(name, L, B, T, p, steps, check_from):
     assert run.cache.status() == 0
 
 
+# ------------------------------------------------------------------ one call, cut in different ways
+@pytest.mark.parametrize("name,T,B,L,p,k_ratio,one_bit", [
+    ("tiny", 2029, 2, 2, 0.0, 0.5, "fft"), ("qwen", 2003, 2, 1, 0.0, 0.5, "fft"), ("tiny", 2029, 2, 2, 0.2, 0.5, "fft"),
+    ("tiny", 2029, 2, 1, 0.0, 0.75, "minmax")])
+def test_outputs_do_not_depend_on_the_cut(name, T, B, L, p, k_ratio, one_bit):
+    """Runs of 1, 3 and 40 units and the small-call kernel over the same cache: the rounding of a probability to
+    binary16 must not depend on where a run began.  What is left is the order of the float32 sums, chains of at most
+    about 100 additions (13 units of 5 groups, 13 records, the residual): 100 x 2^-24 = 6e-6 of the norm."""
+    import paper_2503_16257_b200 as P
+    wl = CONFIGS[name]
+    cfg = P.VidKVConfig(B=B, L=L, max_prefill_tokens=T, max_new_tokens=4, p_ratio=p, k_ratio=k_ratio,
+                        key_1bit_mode=P.VIDKV_KEY1BIT_PLAIN_MINMAX if one_bit == "minmax" else P.VIDKV_KEY1BIT_FFT_SIGN,
+                        in_dtype=P.VIDKV_F16 if wl.dtype == "fp16" else P.VIDKV_BF16, out_dtype=P.VIDKV_F32)
+    kv = [make_layer_kv(wl, layer, "cuda", T=T, B=B) for layer in range(L)]
+    outs = {}
+    for run_units in (0, 1, 3, 40):
+        c = P.VidKVCache(cfg)
+        if p > 0:
+            l_v = min(wl.l_v, T - T % 32)
+            c.select_tokens(make_saliency(wl, "cpu", l_v=l_v, B=B).cuda(), 0, l_v, T)
+        for layer, (K, V) in enumerate(kv):
+            c.quantize_keys(layer, K)
+            c.quantize_values(layer, V)
+        c.debug_set_decode_plan(run_units=run_units)
+        out = torch.empty((3, L, B, 28, 128), dtype=torch.float32, device="cuda")
+        for s in range(3):
+            q, k, v = (torch.stack(t) for t in zip(*[make_step_inputs(wl, layer, s, "cuda", T=T, B=B) for layer in range(L)]))
+            c.decode_attention(0, L, q, k, v, out[s])
+        assert c.status() == 0
+        outs[run_units] = out.double()
+    for run_units in (1, 3, 40):
+        assert float((outs[run_units] - outs[0]).norm() / outs[0].norm()) <= 6e-6, run_units
+
+
 # ------------------------------------------------------------------ prompts shorter than one group
 @pytest.mark.parametrize("T", [31, 0])
 def test_flushes_after_a_prompt_with_nothing_to_quantize(T):
