@@ -985,15 +985,15 @@ __global__ void __launch_bounds__(kUnitThreads, GEN && STP ? kBlockGenStpPerSM :
   if (__syncthreads_or(fault) && producer) {
     // a copy never arrived: report it, and let the others that are in flight land before the block leaves
     atomicCAS(reinterpret_cast<int*>(cv.base + kHdrStatus), VIDKV_OK, VIDKV_ERR_TIMEOUT);
-    for (int j = max(0, ks - 2); j < ks; ++j) mbar_wait(kbar + (j & 1), (j >> 1) & 1);
+    for (int j = max(0, ks - 2); j < ks; ++j) mbar_wait_lane(kbar + (j & 1), (j >> 1) & 1);
     if (STP) {
-      for (int j = max(0, vreq - 2); j < vreq; ++j) mbar_wait(vbar + (j & 1), (j >> 1) & 1);
+      for (int j = max(0, vreq - 2); j < vreq; ++j) mbar_wait_lane(vbar + (j & 1), (j >> 1) & 1);
       for (; pg_next < pg_req; ++pg_next) {
-        mbar_wait(pbar + pslot, pphase);
+        mbar_wait_lane(pbar + pslot, pphase);
         if (++pslot == kPBufs) { pslot = 0; pphase ^= 1u; }
       }
     } else {
-      for (int j = max(a.withhold ? 1 : 0, vs - 2); j < vs; ++j) mbar_wait(vbar + (j & 1), (j >> 1) & 1);
+      for (int j = max(a.withhold ? 1 : 0, vs - 2); j < vs; ++j) mbar_wait_lane(vbar + (j & 1), (j >> 1) & 1);
     }
   }
 }

@@ -29,8 +29,8 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t b
                "l"(src), "r"(bytes), "r"(b)
                : "memory");
 }
-// Bounded wait for the phase with the given parity; false if it never completed.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
+// Bounded wait of one lane for the phase with the given parity; false if it never completed.
+__device__ __forceinline__ bool mbar_wait_lane(uint64_t* bar, uint32_t parity) {
   const uint32_t b = smem_u32(bar);
   for (uint32_t i = 0; i < kWaitLimit; ++i) {
     uint32_t ok;
@@ -43,6 +43,9 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
   }
   return false;
 }
+// The same by a whole warp, with one answer for all lanes: a copy that lands just as the polls run out may be seen by some
+// of them only, and what follows a wait (matrix products, shuffles) needs the warp together.
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) { return __all_sync(0xffffffffu, mbar_wait_lane(bar, parity)); }
 
 }  // namespace
 }  // namespace vidkv

@@ -32,19 +32,29 @@ def test_key_encoder_wait_runs_out_and_reports_timeout():
     _fresh_run_is_fine()
 
 
-def test_stream_kernel_wait_runs_out_and_reports_timeout():
+@pytest.mark.parametrize("L,B,T,run_units", [
+    (1, 1, 640, 1),      # stream kernel, nothing else in flight
+    (1, 1, 640, 3),      # stream kernel, runs that cross slabs: the next unit's keys are in flight when the wait runs out
+    (1, 1, 640, 0),      # small-call kernel, a unit per block: the wait behind the last unit
+    (12, 4, 2029, 0),    # small-call kernel, four or five units per block, slabs of 13: the exit inside the walk
+])
+def test_decode_wait_runs_out_and_reports_timeout(L, B, T, run_units):
     import paper_2503_16257_b200 as P
     from workloads import CONFIGS, make_layer_kv, make_step_inputs
     wl = CONFIGS["tiny"]
-    cfg = P.VidKVConfig(B=1, L=1, max_prefill_tokens=640, max_new_tokens=2)
+    cfg = P.VidKVConfig(B=B, L=L, max_prefill_tokens=T, max_new_tokens=2)
     cache = P.VidKVCache(cfg)
-    K, V = make_layer_kv(wl, 0, "cuda", T=640, B=1)
-    cache.quantize_keys(0, K)
-    cache.quantize_values(0, V)
+    for layer in range(L):
+        K, V = make_layer_kv(wl, layer, "cuda", T=T, B=B)
+        cache.quantize_keys(layer, K)
+        cache.quantize_values(layer, V)
     assert cache.status() == 0
-    q, k, v = make_step_inputs(wl, 0, 0, "cuda", T=640, B=1)
-    out = torch.empty((1, 1, 28, 128), dtype=torch.float32, device="cuda")
+    cache.debug_set_decode_plan(run_units=run_units)
+    q, k, v = (torch.stack(t) for t in zip(*[make_step_inputs(wl, layer, 0, "cuda", T=T, B=B) for layer in range(L)]))
+    out = torch.empty((L, B, 28, 128), dtype=torch.float32, device="cuda")
+    before = P.vidkv_launch_count()
     P.vidkv_debug_withhold_once(2)
-    cache.decode_attention(0, 1, q[None], k[None], v[None], out)
+    cache.decode_attention(0, L, q, k, v, out)
+    assert P.vidkv_launch_count() - before == (3 if run_units else 1)      # the kernel that the case is about
     assert cache.status() == -7
     _fresh_run_is_fine()
