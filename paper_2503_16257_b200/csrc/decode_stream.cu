@@ -287,7 +287,10 @@ __device__ __forceinline__ bool process_unit(const KeyFmt& kf, const uint32_t*& 
                                              Running& run, bool more, const uint8_t* next_k, uint32_t next_k_bytes,
                                              const uint8_t* next_v) {
   const int kgb = GEN ? kf.group_bytes : kKGroupBytes;      // bytes of one key group
-  if (!mbar_wait(kbar, kpar)) return false;
+  if (!mbar_wait(kbar, kpar)) {
+    mbar_wait(vbar, vpar);                                  // the unit's value copy is under way: let it land before leaving
+    return false;
+  }
   kpar ^= 1u;
   // ---- scores, group by group; a group's scores replace its (spent) bytes in the key buffer:
   // float2 (tokens 8 nt + 2 r, + 1 of head hd) at word pair (nt * 32 + lane) of the group, the
@@ -521,8 +524,7 @@ __global__ void __launch_bounds__(kStreamWarps * 32, kStreamCtasPerSM) decode_st
     slab = nslab; k = nk;
   }
   if (!ok) {
-    // a copy never arrived: report it and leave (the wait already ran its full course, so nothing
-    // this warp issued can still be expected)
+    // a copy never arrived: report it and leave (process_unit has waited for the other one that was in flight)
     if (lane == 0) atomicCAS(reinterpret_cast<int*>(cv.base + kHdrStatus), VIDKV_OK, VIDKV_ERR_TIMEOUT);
     return;
   }
@@ -669,7 +671,7 @@ __global__ void __launch_bounds__(kStreamWarps * 32, kStreamStpCtasPerSM) decode
   pdl_release();
   const uint32_t lt_mask = (1u << lane) - 1u;              // lanes (= tokens of a group) before this one
   uint32_t kpar = 0u, vpar = 0u, ppar = 0u;
-  bool v_pending = false, p_pending = false;               // a copy into vbuf / pbuf has been issued and not yet waited for
+  bool k_pending = true, v_pending = false, p_pending = false;   // a copy into kbuf / vbuf / pbuf has been issued and not yet waited for
   Running run;
   run.l[0] = 0.0f; run.l[1] = 0.0f; run.m = -INFINITY;
   uint32_t qa[8], qha[8], qhb[8];
@@ -734,6 +736,7 @@ __global__ void __launch_bounds__(kStreamWarps * 32, kStreamStpCtasPerSM) decode
     // ---- scores of the unit's groups into the key buffer (raw scores, then the group's constant)
     if (!mbar_wait(kbar, kpar)) { ok = false; break; }
     kpar ^= 1u;
+    k_pending = more;                                       // the next unit's is issued below, before anything else can fail
     float mx = -INFINITY;
 #pragma unroll 1
     for (int g = 0; g < ng; ++g) {
@@ -904,7 +907,11 @@ __global__ void __launch_bounds__(kStreamWarps * 32, kStreamStpCtasPerSM) decode
     slab = nslab; k = nk;
   }
   if (!ok) {
+    // a copy never arrived: report it, and let the others that are in flight land before the warp leaves
     if (lane == 0) atomicCAS(reinterpret_cast<int*>(cv.base + kHdrStatus), VIDKV_OK, VIDKV_ERR_TIMEOUT);
+    if (k_pending) mbar_wait(kbar, kpar);
+    if (v_pending) mbar_wait(vbar, vpar);
+    if (p_pending) mbar_wait(pbar, ppar);
     return;
   }
   write_record(a, cur_slab, run_id, lane, hd, r, run, totbuf);
