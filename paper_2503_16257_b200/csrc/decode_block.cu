@@ -437,23 +437,25 @@ __device__ __forceinline__ bool move_maximum(float mu, bool integral, int r, flo
   return true;
 }
 
-// The slab's residual rows (n_res of them, the step's new row among them) in the input type: scores on the tensor
+// Algorithm 1, Decoding: the step's new key / value row joins the residual (lanes 0-15 copy the key row, 16-31 the value
+// row).  One warp.
+__device__ __forceinline__ void append_row(const DecodeArgs& a, int slab, uint8_t* slab_ptr, int lane) {
+  if (a.append_row < 0) return;
+  const uint4* srcp = reinterpret_cast<const uint4*>(lane < 16 ? a.k_new : a.v_new) + static_cast<int64_t>(slab) * 16 + (lane & 15);
+  reinterpret_cast<uint4*>(slab_ptr + (lane < 16 ? a.cv.kres_offset : a.cv.vres_offset))[a.append_row * 16 + (lane & 15)] = __ldg(srcp);
+}
+
+// The slab's residual rows (n_res of them, the step's new row among them: append_row by warp 0 first) in the input type: scores on the tensor
 // cores straight from global memory (the contraction may take the channels in any order: lane (token hd, r) reads
 // 16-byte pieces, two k steps each), probabilities through `scratch`, P V with the two tokens of an operand register
 // brought together from two rows.  Whole block; scratch as large as kResScratch.
 template <typename T>
-__device__ __forceinline__ void add_residual(const DecodeArgs& a, int slab, uint8_t* slab_ptr, const T* qrow, bool live, uint8_t* scratch,
-                                             int warp, int lane, Running& run) {
+__device__ __forceinline__ void add_residual(const DecodeArgs& a, const uint8_t* slab_ptr, const T* qrow, bool live, uint8_t* scratch, int warp,
+                                             int lane, Running& run) {
   const CacheView& cv = a.cv;
   const int hd = lane >> 2, r = lane & 3, n_res = a.st.n_res;
   float* Sx = reinterpret_cast<float*>(scratch);
   __half* Px = reinterpret_cast<__half*>(scratch + 8 * kResS * 4);
-  if (a.append_row >= 0 && warp == 0) {
-    // Algorithm 1, Decoding: the step's new key / value row joins the residual (lanes 0-15 copy
-    // the key row, 16-31 the value row)
-    const uint4* srcp = reinterpret_cast<const uint4*>(lane < 16 ? a.k_new : a.v_new) + static_cast<int64_t>(slab) * 16 + (lane & 15);
-    reinterpret_cast<uint4*>(slab_ptr + (lane < 16 ? cv.kres_offset : cv.vres_offset))[a.append_row * 16 + (lane & 15)] = __ldg(srcp);
-  }
   uint4 qn[4];
 #pragma unroll
   for (int j = 0; j < 4; ++j) qn[j] = live ? __ldg(reinterpret_cast<const uint4*>(qrow + 32 * j + 8 * r)) : make_uint4(0u, 0u, 0u, 0u);
@@ -674,8 +676,10 @@ __global__ void __launch_bounds__(kUnitThreads, GEN && STP ? kBlockGenStpPerSM :
   if (static_cast<int>(blockIdx.x) >= pl.n_blocks) {
     // a residual of its own (blocks that own one unit each, or nothing quantized yet)
     const int slab = blockIdx.x - pl.n_blocks, first = slab * n_slab_units;   // one unit per block
+    uint8_t* const slab_ptr = slab0 + static_cast<int64_t>(slab) * cv.slab_stride;
     run.reset();
-    add_residual<T>(a, slab, slab0 + static_cast<int64_t>(slab) * cv.slab_stride, query_row(slab), live, sm + S::prob_at, warp, lane, run);
+    if (warp == 0) append_row(a, slab, slab_ptr, lane);
+    add_residual<T>(a, slab_ptr, query_row(slab), live, sm + S::prob_at, warp, lane, run);
     finish_part(a, slab, first, n_slab_units, n_slab_units + 1, run, &flag, warp, lane);
     return;
   }
@@ -970,12 +974,14 @@ __global__ void __launch_bounds__(kUnitThreads, GEN && STP ? kBlockGenStpPerSM :
             __syncthreads();
             multiply_streams(sg_end * kStreamUnitTokens, pg_end * kG);
           }
-          if (k_end == n_slab_units && a.st.n_res > 0 && pl.res_blocks == 0)
-            add_residual<T>(a, slab, slab_ptr, qrow, live, sm + S::prob_at, warp, lane, run);
         }
       }
     } else {
       i += k_end - k;
+    }
+    if (k_end == n_slab_units && a.st.n_res > 0 && pl.res_blocks == 0) {
+      if (warp == 0) append_row(a, slab, slab_ptr, lane);    // also where a copy never arrived: later calls find the row
+      if (!dead) add_residual<T>(a, slab_ptr, qrow, live, sm + S::prob_at, warp, lane, run);
     }
     const int first = block_of(static_cast<uint32_t>(slab) * n_slab_units), last = block_of((slab + 1u) * n_slab_units - 1u);
     finish_part(a, slab, first, static_cast<int>(blockIdx.x) - first, last - first + 1 + (pl.res_blocks ? 1 : 0), run, &flag, warp, lane);

@@ -32,12 +32,37 @@ def test_key_encoder_wait_runs_out_and_reports_timeout():
     _fresh_run_is_fine()
 
 
-@pytest.mark.parametrize("L,B,T,run_units", [
+DECODE_SHAPES = pytest.mark.parametrize("L,B,T,run_units", [
     (1, 1, 640, 1),      # stream kernel, nothing else in flight
     (1, 1, 640, 3),      # stream kernel, runs that cross slabs: the next unit's keys are in flight when the wait runs out
     (1, 1, 640, 0),      # small-call kernel, a unit per block: the wait behind the last unit
     (12, 4, 2029, 0),    # small-call kernel, four or five units per block, slabs of 13: the exit inside the walk
 ])
+
+
+@DECODE_SHAPES
+def test_cache_is_whole_after_a_decode_call_that_timed_out(L, B, T, run_units):
+    """Only the affected call's results are lost: its key and value rows are in the residual, and the next call over
+    the same cache is the oracle's (its status word keeps the first error)."""
+    import paper_2503_16257_b200 as P
+    from tests.test_gpu_launch_shapes import SampledRun
+    from workloads import make_step_inputs
+    run = SampledRun("tiny", L, B, T, 0.0, 4, sorted({(0, 0, 0), (L - 1, B - 1, 3), (L // 2, B // 2, 1)}))
+    run.cache.debug_set_decode_plan(run_units=run_units)
+    run.decode()
+    P.vidkv_debug_withhold_once(2)
+    run.decode(check=False)
+    assert run.cache.status() == -7
+    lay, row = run.cache.layout, run.cache.layer_state(0)["n_residual"] - 1
+    slabs = run.cache.cache[lay["slab_offset"]:].view(L * B * 4, lay["slab_stride"])
+    _, k, v = (torch.stack(t) for t in zip(*[make_step_inputs(run.wl, layer, 1, "cuda", T=T, B=B) for layer in range(L)]))
+    for rows, at in ((k, lay["kres_offset"]), (v, lay["vres_offset"])):
+        assert torch.equal(slabs[:, at + row * 256:at + (row + 1) * 256], rows.contiguous().view(torch.uint8).view(L * B * 4, 256))
+    run.decode()
+    run.decode()
+
+
+@DECODE_SHAPES
 def test_decode_wait_runs_out_and_reports_timeout(L, B, T, run_units):
     import paper_2503_16257_b200 as P
     from workloads import CONFIGS, make_layer_kv, make_step_inputs
