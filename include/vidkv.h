@@ -202,7 +202,8 @@ vidkv_status_t vidkv_cache_init(const vidkv_config_t* cfg, void* cache, size_t c
                                 vidkv_cache_t** handle);
 vidkv_status_t vidkv_cache_destroy(vidkv_cache_t* handle);
 
-/* Forget all tokens (host state only; the next quantize calls overwrite the buffers). */
+/* Forget all tokens (host state only; the next quantize calls overwrite the buffers, and the first
+ * key quantization among them clears the arrival counters in the workspace). */
 vidkv_status_t vidkv_cache_reset(vidkv_cache_t* handle, void* stream);
 
 /* Sec. 3.3(2) / Eq. 7: the cross-modal scores I = X_v X_t^T from hidden states, summed over

@@ -120,6 +120,7 @@ struct vidkv_cache {
   int dbg_run_units = 0;        // test hook: forced run length of the stream kernels (0 = choose)
   int mm_parity = 0;            // which min / max buffer the next key quantization accumulates into
   int64_t mm_dirty[2] = {0, 0}; // words of each buffer written since it was last re-armed
+  bool clear_counters = false;  // the next prompt's first key quantization clears the decode kernel's arrival counters
   std::vector<LayerInfo> layers;
 };
 
@@ -232,6 +233,8 @@ vidkv_status_t vidkv_cache_reset(vidkv_cache_t* h, void* stream) {
   if (!h) return VIDKV_ERR_INVALID_ARG;
   h->sel_set = false; h->sel_T = 0; h->n_prot = 0;
   h->layers.assign(h->cfg.L, LayerInfo());
+  // every decode call leaves the counters zero, unless two calls overlapped against the rules: a new prompt starts clean
+  h->clear_counters = true;
   return VIDKV_OK;
 }
 
@@ -348,13 +351,18 @@ vidkv_status_t vidkv_quantize_keys_layers(vidkv_cache_t* h, int32_t layer_begin,
   const int r = static_cast<int>(T % kG);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   KSrc src{K, stride_b, stride_h, stride_t, h->cfg.H_kv};
+  int32_t* const counters = reinterpret_cast<int32_t*>(h->workspace + h->ws.counters_off);
+  if (h->clear_counters && T_q == 0 && cudaMemsetAsync(counters, 0, static_cast<size_t>(h->ws.counter_words) * 4, s) != cudaSuccess)
+    return VIDKV_ERR_CUDA;
   if (T_q > 0) {
     const MinMaxBuffers mm = next_minmax(h, static_cast<int64_t>(n_layers) * h->cfg.B * h->cfg.H_kv);
-    if (launch_quantize_keys(h->cfg.in_dtype, src, T_q, r, h->cv, layer_begin, n_layers, 0, 0, mm, s) != cudaSuccess)
+    if (launch_quantize_keys(h->cfg.in_dtype, src, T_q, r, h->cv, layer_begin, n_layers, 0, 0, mm, counters,
+                             h->clear_counters ? h->ws.counter_words : 0, s) != cudaSuccess)
       return VIDKV_ERR_CUDA;
   } else if (launch_copy_to_residual(src, r, h->cv, layer_begin, n_layers, false, s) != cudaSuccess) {
     return VIDKV_ERR_CUDA;
   }
+  h->clear_counters = false;
   for (int l = layer_begin; l < layer_begin + n_layers; ++l) {
     LayerInfo& li = h->layers[l];
     li.k_done = true; li.T = T; li.T_q0 = T_q; li.n_res = r; li.n_flush = 0;
@@ -458,7 +466,7 @@ static vidkv_status_t decode_impl(vidkv_cache_t* h, int32_t layer_begin, int32_t
     const MinMaxBuffers mm = next_minmax(h, static_cast<int64_t>(n_layers) * h->cfg.B * h->cfg.H_kv);
     const int chunk = 1 + static_cast<int>(first.n_flush);
     const int64_t kgroup0 = first.T_q0 / kG + (kR / kG) * first.n_flush;
-    if (launch_quantize_keys(dt, ksrc, kR, 0, h->cv, layer_begin, n_layers, chunk, kgroup0, mm, s) != cudaSuccess)
+    if (launch_quantize_keys(dt, ksrc, kR, 0, h->cv, layer_begin, n_layers, chunk, kgroup0, mm, nullptr, 0, s) != cudaSuccess)
       return VIDKV_ERR_CUDA;
     const int64_t n_rest = first.T_q0 - h->n_prot;
     const int64_t tgroup0 = (n_rest + kG - 1) / kG + (kR / kG) * first.n_flush;

@@ -67,9 +67,11 @@ cudaError_t launch_init_workspace(uint32_t* minmax, int64_t n_words, int32_t* co
 // Algorithm 3 on `T_tokens` tokens (a multiple of 32) of every slab of layers
 // [layer0, layer0 + n_layers): writes chunk `chunk` of the chunk table and the key groups
 // starting at group index kgroup0.
-// n_res rows that follow (0..31) are copied to the residual.
+// n_res rows that follow (0..31) are copied to the residual.  n_counters > 0: clears the decode kernel's arrival counters on
+// the way.
 cudaError_t launch_quantize_keys(int dtype, const KSrc& src, int64_t T_tokens, int n_res, const CacheView& cv, int layer0,
-                                 int n_layers, int chunk, int64_t kgroup0, const MinMaxBuffers& mm, cudaStream_t stream);
+                                 int n_layers, int chunk, int64_t kgroup0, const MinMaxBuffers& mm, int32_t* counters, int64_t n_counters,
+                                 cudaStream_t stream);
 
 // Channel split and encode pass of Algorithm 3 for `n_slabs` slabs whose channel ranges are in mm.cur; launched behind the
 // range pass.  Writes the chunk table entry `chunk` too, and re-arms mm.next.

@@ -30,12 +30,16 @@ template <> struct Pair2<__nv_bfloat16> {
 
 template <typename T>
 __global__ void __launch_bounds__(256) k_range_kernel(KSrc src, int64_t T_tokens, int tokens_per_block, int splits, int n_res,
-                                                      CacheView cv, int layer0, uint32_t* __restrict__ minmax) {
+                                                      CacheView cv, int layer0, uint32_t* __restrict__ minmax,
+                                                      int32_t* __restrict__ counters, int64_t n_counters) {
   using P = Pair2<T>;
   using V = typename P::V;
   const int slab = blockIdx.y;
   pdl_wait();
   pdl_release();                                           // the encode pass may set itself up beside this one
+  for (int64_t i = (static_cast<int64_t>(blockIdx.y) * gridDim.x + blockIdx.x) * 256 + threadIdx.x; i < n_counters;
+       i += static_cast<int64_t>(gridDim.x) * gridDim.y * 256)
+    counters[i] = 0;
   if (static_cast<int>(blockIdx.x) == splits) {            // one more block per slab for the tokens that stay as they are
     copy_residual_rows(src, T_tokens, n_res, cv, layer0, slab, cv.kres_offset);
     return;
@@ -140,7 +144,8 @@ __global__ void __launch_bounds__(kD) k_select_kernel(const uint32_t* __restrict
 // ---------------------------------------------------------------------------------
 template <typename T>
 static cudaError_t launch_keys_t(const KSrc& src, int64_t T_tokens, int n_res, const CacheView& cv, int layer0, int n_layers,
-                                 int chunk, int64_t kgroup0, const MinMaxBuffers& mm, cudaStream_t stream) {
+                                 int chunk, int64_t kgroup0, const MinMaxBuffers& mm, int32_t* counters, int64_t n_counters,
+                                 cudaStream_t stream) {
   uint32_t* minmax = mm.cur;
   const int slabs_per_layer = cv.B * cv.H_kv;
   const int n_slabs = slabs_per_layer * n_layers;
@@ -149,7 +154,7 @@ static cudaError_t launch_keys_t(const KSrc& src, int64_t T_tokens, int n_res, c
   int tokens_per_block = 512;
   const int64_t splits = (T_tokens + tokens_per_block - 1) / tokens_per_block;
   if ((e = launch_dependent(k_range_kernel<T>, dim3(static_cast<unsigned>(splits + (n_res > 0)), n_slabs), dim3(256), 0, stream, src,
-                            T_tokens, tokens_per_block, static_cast<int>(splits), n_res, cv, layer0, minmax)))
+                            T_tokens, tokens_per_block, static_cast<int>(splits), n_res, cv, layer0, minmax, counters, n_counters)))
     return e;
   count_launches(1);
   const int dt = std::is_same<T, __half>::value ? VIDKV_F16 : VIDKV_BF16;
@@ -179,10 +184,11 @@ cudaError_t launch_init_workspace(uint32_t* minmax, int64_t n_words, int32_t* co
 }
 
 cudaError_t launch_quantize_keys(int dtype, const KSrc& src, int64_t T_tokens, int n_res, const CacheView& cv, int layer0,
-                                 int n_layers, int chunk, int64_t kgroup0, const MinMaxBuffers& mm, cudaStream_t stream) {
+                                 int n_layers, int chunk, int64_t kgroup0, const MinMaxBuffers& mm, int32_t* counters, int64_t n_counters,
+                                 cudaStream_t stream) {
   if (dtype == VIDKV_F16)
-    return launch_keys_t<__half>(src, T_tokens, n_res, cv, layer0, n_layers, chunk, kgroup0, mm, stream);
-  return launch_keys_t<__nv_bfloat16>(src, T_tokens, n_res, cv, layer0, n_layers, chunk, kgroup0, mm, stream);
+    return launch_keys_t<__half>(src, T_tokens, n_res, cv, layer0, n_layers, chunk, kgroup0, mm, counters, n_counters, stream);
+  return launch_keys_t<__nv_bfloat16>(src, T_tokens, n_res, cv, layer0, n_layers, chunk, kgroup0, mm, counters, n_counters, stream);
 }
 
 }  // namespace vidkv

@@ -236,6 +236,38 @@ def test_small_calls_in_one_launch(name, L, B, T, p, steps, check_from):
     assert run.cache.status() == 0
 
 
+@pytest.mark.parametrize("T", [2029, 20])
+def test_a_new_prompt_starts_from_cleared_arrival_counters(T):
+    """Two calls that overlap on one handle, against the rules, may leave arrival counters of the small-call kernel off
+    zero, and every later call would then join too early or never.  vidkv_cache_reset and the next prompt recover."""
+    import paper_2503_16257_b200 as P
+    wl = CONFIGS["tiny"]
+    cfg = P.VidKVConfig(B=1, L=2, max_prefill_tokens=2048, max_new_tokens=4, out_dtype=P.VIDKV_F32)
+    kv = [[x[:, :, :T].contiguous() for x in make_layer_kv(wl, layer, "cuda", T=2048, B=1)] for layer in range(2)]
+
+    def answer(c):
+        for layer, (K, V) in enumerate(kv):
+            c.quantize_keys(layer, K)
+            c.quantize_values(layer, V)
+        out = torch.empty((2, 1, 28, 128), dtype=torch.float32, device="cuda")
+        q, k, v = (torch.stack(t) for t in zip(*[make_step_inputs(wl, layer, 0, "cuda", T=2048, B=1) for layer in range(2)]))
+        c.decode_attention(0, 2, q, k, v, out)
+        return out
+
+    want = answer(P.VidKVCache(cfg))
+    c = P.VidKVCache(cfg)
+    answer(c)
+    # the counters lie behind the channel ranges, the partial records and the query images (each from a 256-byte boundary)
+    up = lambda n: -(-n // 256) * 256  # noqa: E731
+    records = P.vidkv_debug_decode_plan(cfg, 2048, 0, 1, 0, 2)["records_capacity"]
+    at = up(2 * 8 * 256 * 4) + up(records * 130 * 4) + up(8 * c.layout["max_chunks"] * 25 * 32 * 4)
+    words = c.workspace[at:at + 4 * (records // 8 // 7 + 12 * 8 + 64)].view(torch.int32)
+    assert not words.any()
+    words.fill_(1)
+    c.reset()
+    assert torch.equal(answer(c), want) and not words.any()
+
+
 # ------------------------------------------------------------------ one call, cut in different ways
 @pytest.mark.parametrize("name,T,B,L,p,k_ratio,one_bit", [
     ("tiny", 2029, 2, 2, 0.0, 0.5, "fft"), ("qwen", 2003, 2, 1, 0.0, 0.5, "fft"), ("tiny", 2029, 2, 2, 0.2, 0.5, "fft"),
