@@ -411,7 +411,7 @@ __global__ void __launch_bounds__(kSelThreads) select_tokens_kernel(const float*
                                                                     int32_t* idx_rest, int64_t stride_prot,
                                                                     int64_t stride_rest, int32_t* counts,
                                                                     int64_t expect_count) {
-  __shared__ int hist[3][kSelBins];
+  __shared__ __align__(8) int hist[3][kSelBins];   // read two bins at a time
   __shared__ int64_t s_warp[32];
   __shared__ int64_t s_block;                  // (keys at the threshold) << 32 | (keys above it) in this block's words
   __shared__ uint32_t s_bin, s_need;
