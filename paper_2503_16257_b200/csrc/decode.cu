@@ -84,6 +84,7 @@ DecodePlan plan_decode(const LayerState& st, int64_t n_slabs, bool stp, bool gen
   const int64_t most = !stp ? kMaxBlockUnits : partial ? kMaxBlockUnitsStpPartial : kMaxBlockUnitsStp;
   if (p.n_units == 0 || (per_block <= most && force_run_units == 0 && (!partial || run == 1))) {
     p.n_blocks = static_cast<int32_t>(p.n_units < blocks ? p.n_units : blocks);
+    p.records = (p.n_blocks + n_slabs) * kMaxRep;
     p.res_blocks = st.n_res > 0 && per_block <= 1 ? static_cast<int32_t>(n_slabs) : 0;
     p.counters_per_slab = static_cast<int32_t>(join_counters(most_parts(p.n_blocks) + (p.res_blocks > 0)));
   }

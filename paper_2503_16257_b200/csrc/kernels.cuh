@@ -154,7 +154,7 @@ struct DecodePlan {
   int64_t n_units;
   int32_t slab_parts;      // most runs that can touch one slab
   int32_t n_chunks;        // chunk-table entries the query preparation covers (0: nothing quantized)
-  int64_t records;         // records of one query head: (n_runs + n_slabs) * 8
+  int64_t records;         // records of one query head: (n_runs + n_slabs) * 8, or (n_blocks + n_slabs) * 8 in the block kernel
   int32_t n_blocks;
   int32_t res_blocks;      // blocks that attend to a slab's residual alone: n_slabs or 0 (the slab's last block does it)
   int32_t counters_per_slab;   // arrival counters of the merge tree

@@ -95,11 +95,18 @@ extern "C" vidkv_status_t vidkv_attend_noalloc(const vidkv_config_t* cfg, const 
   a.append_row = -1;
   a.plan = plan_decode(a.st, n_slabs, n_protected > 0, cv.kf.general != 0, device_sm_count(), 0);
   // the array holds the partial records, then (256-byte aligned) the per-chunk query images
-  const int64_t prep_at = (a.plan.records * kRecordFloats * 4 + 255) / 256 * 256;
-  const int64_t prep_bytes = static_cast<int64_t>(decode_prep_bytes(n_slabs, a.plan.n_chunks));
-  if (prep_at + prep_bytes > static_cast<int64_t>(kStaticPartialFloats * sizeof(float)) ||
-      n_slabs * a.plan.counters_per_slab > kStaticCounters)
-    return VIDKV_ERR_CAPACITY;
+  int64_t prep_at = 0;
+  auto fits = [&]() {
+    prep_at = (a.plan.records * kRecordFloats * 4 + 255) / 256 * 256;
+    const int64_t prep_bytes = static_cast<int64_t>(decode_prep_bytes(n_slabs, a.plan.n_chunks));
+    return prep_at + prep_bytes <= static_cast<int64_t>(kStaticPartialFloats * sizeof(float)) &&
+           n_slabs * a.plan.counters_per_slab <= kStaticCounters;
+  };
+  if (!fits()) {
+    // as few runs as have the same longest one: fewer records
+    a.plan = plan_decode(a.st, n_slabs, n_protected > 0, cv.kf.general != 0, device_sm_count(), a.plan.run_units);
+    if (!fits()) return VIDKV_ERR_CAPACITY;
+  }
   StaticScratch scratch;
   const vidkv_status_t sp = static_scratch(&scratch);
   if (sp != VIDKV_OK) return sp;

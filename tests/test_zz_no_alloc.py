@@ -83,3 +83,28 @@ def test_attend_noalloc_matches_the_oracle(p):
         P.vidkv_attend_noalloc(pair.cfg, pair.cache.cache, 992, 0, st["n_residual"], st["n_protected"], 0, L, q, out)
         torch.cuda.synchronize()
         assert np.abs(out.cpu().numpy().astype(np.float64) - ref).max() <= TOL_ABS
+
+
+@pytest.mark.parametrize("L,B,T", [
+    (28, 13, 320),      # 1456 slabs of two units: the small-call kernel
+    (28, 12, 640),      # 1344 slabs of four units: runs of four units in the stream kernel
+])
+def test_attend_noalloc_takes_what_its_array_holds(L, B, T):
+    """The 16 MiB hold a record per run and slab and 3200 bytes per (slab, chunk) here when runs are as few as their
+    longest one allows, 15.5 to 16.8 MB, though not with every warp of the device taking part.  Against the triples of the
+    same cache (another rounding reference of the probabilities, so TOL_ABS)."""
+    import paper_2503_16257_b200 as P
+    from tests.helpers import TOL_ABS
+    cfg = P.VidKVConfig(B=B, L=L, max_prefill_tokens=T, max_new_tokens=1, out_dtype=P.VIDKV_F32)
+    cache = P.VidKVCache(cfg)
+    gen = torch.Generator(device="cuda").manual_seed(1)
+    X = torch.randn((2, L, B, 4, T, 128), generator=gen, device="cuda").to(torch.float16)
+    cache.quantize_keys_layers(0, X[0])
+    cache.quantize_values_layers(0, X[1])
+    q = torch.randn((L, B, 28, 128), generator=gen, device="cuda").to(torch.float16)
+    part = torch.empty((1, L, B, 28, 130), dtype=torch.float32, device="cuda")
+    cache.decode_attention_partial(0, L, q, None, None, part[0])
+    want, out = torch.empty((L, B, 28, 128), device="cuda"), torch.empty((L, B, 28, 128), device="cuda")
+    P.vidkv_merge_partials(part, want)
+    P.vidkv_attend_noalloc(cfg, cache.cache, T, 0, 0, 0, 0, L, q, out)
+    assert float((out - want).abs().max()) <= TOL_ABS
