@@ -127,6 +127,16 @@ size_t merge_smem_bytes(int n_pad) {
   return static_cast<size_t>(2) * n_pad * kMergeRow + sizeof(float) * 8 * n_pad + sizeof(__half) * 8 * (n_pad + 8) + 3 * 8 * sizeof(float);
 }
 
+// Shared memory asked for so that no multiprocessor takes more than its share of the n_slabs merge blocks.
+constexpr size_t kMaxSmem = 226 * 1024;       // a block's largest, less the kilobyte that every block costs besides
+static size_t spread_smem(size_t needed, int n_slabs) {
+  const int sms = device_sm_count();
+  if (sms < 1) return needed;
+  const size_t share = (kMaxSmem + 1024) / static_cast<size_t>((n_slabs + sms - 1) / sms);
+  const size_t smem = share > 2048 ? (share - 1024) / 1024 * 1024 : 0;
+  return smem > needed ? smem : needed;
+}
+
 template <typename T>
 __global__ void __launch_bounds__(kD) decode_merge_kernel(DecodeArgs a, int n_res, int n_pad) {
   extern __shared__ __align__(16) uint8_t msm[];
@@ -364,12 +374,12 @@ cudaError_t launch_decode(const DecodeArgs& a_in, cudaStream_t stream) {
   count_launches(1);
   const int n_res = a.st.n_res;
   const int n_pad = (n_res + 15) / 16 * 16;
-  const size_t smem = merge_smem_bytes(n_pad);
+  const size_t smem = spread_smem(merge_smem_bytes(n_pad), n_slabs);
   static bool attr_set[64] = {};
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   if (!attr_set[dev]) {
-    const int most = static_cast<int>(merge_smem_bytes(kR));
+    const int most = static_cast<int>(kMaxSmem);
     if ((e = cudaFuncSetAttribute(decode_merge_kernel<__half>, cudaFuncAttributeMaxDynamicSharedMemorySize, most))) return e;
     if ((e = cudaFuncSetAttribute(decode_merge_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, most))) return e;
     attr_set[dev] = true;
