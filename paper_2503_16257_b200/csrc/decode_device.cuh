@@ -29,7 +29,23 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t b
                "l"(src), "r"(bytes), "r"(b)
                : "memory");
 }
-// Bounded wait of one lane for the phase with the given parity; false if it never completed.
+// Bounded wait for the phase with the given parity by a whole warp; false if it never completed.  All lanes get one
+// answer: a copy that lands just as the polls run out may be seen by some of them only, and what follows a wait (matrix
+// products, shuffles) needs the warp together.
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
+  const uint32_t b = smem_u32(bar);
+  for (uint32_t i = 0; i < kWaitLimit; ++i) {
+    uint32_t ok;
+    asm volatile(
+        "{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2; vote.sync.all.pred p, p, 0xffffffff; selp.u32 %0, 1, 0, p; }"
+        : "=r"(ok)
+        : "r"(b), "r"(parity)
+        : "memory");
+    if (ok) return true;
+  }
+  return false;
+}
+// The same by one lane.
 __device__ __forceinline__ bool mbar_wait_lane(uint64_t* bar, uint32_t parity) {
   const uint32_t b = smem_u32(bar);
   for (uint32_t i = 0; i < kWaitLimit; ++i) {
@@ -43,9 +59,6 @@ __device__ __forceinline__ bool mbar_wait_lane(uint64_t* bar, uint32_t parity) {
   }
   return false;
 }
-// The same by a whole warp, with one answer for all lanes: a copy that lands just as the polls run out may be seen by some
-// of them only, and what follows a wait (matrix products, shuffles) needs the warp together.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) { return __all_sync(0xffffffffu, mbar_wait_lane(bar, parity)); }
 
 }  // namespace
 }  // namespace vidkv
