@@ -13,8 +13,7 @@
 //   scores    warp g scores key group g of the unit: mma.sync.m16n8k16 with rows = query heads
 //             (exact binary16 pair hi + lo), columns = tokens, the codes expanded in registers;
 //   softmax   the unit's maxima per head meet in shared memory; the probabilities against them go to shared memory as
-//             binary16.  The running maximum moves (and the running output is rescaled) only when a unit
-//             exceeds it by more than kStaleLog2; a unit's sums join with the weight 2^(its maximum - running one);
+//             binary16, and the running output is brought to the unit's maximum before its P V joins;
 //   P V       warps 0-3 own 32 channels each: the ternary plane is peeled digit by digit into
 //             5 + trit and multiplied with the probabilities, the per-(group, channel) scales fold
 //             the group accumulators into the warp's running output, eight registers a lane.
@@ -299,8 +298,8 @@ __device__ __forceinline__ void make_images(uint32_t* img, const KeyFmt& kf, con
 // Running softmax of the block's part of one slab.  m (head lane / 4) is the same in every warp; o and l belong
 // to warps 0-3: o[4 i + c] = channel 32 w + 4 (lane / 4) + 2 i + c / 2, head 2 (lane % 4) + c % 2.
 struct Running {
-  float m;
-  float exact;         // what m would be if it followed every unit's maximum (for the triples of a token shard)
+  float m;             // reference: o and l are in units of 2^m
+  float exact;         // the largest unit maximum so far
   float l[2];
   float o[8];
   __device__ __forceinline__ void reset() {
@@ -313,22 +312,23 @@ struct Running {
 #pragma unroll
     for (int j = 0; j < 8; j += 2) { o[j] *= fa; o[j + 1] *= fb; }
   }
-  // Sums that are kept in units of another maximum: `weight` = 2^(that maximum - m) of head lane / 4.
-  __device__ __forceinline__ void add(const float (&po)[8], const float (&pl)[2], float weight, int r) {
-    const float wa = __shfl_sync(0xffffffffu, weight, 8 * r), wb = __shfl_sync(0xffffffffu, weight, 8 * r + 4);
-    l[0] = fmaf(wa, pl[0], l[0]); l[1] = fmaf(wb, pl[1], l[1]);
-#pragma unroll
-    for (int j = 0; j < 8; j += 2) { o[j] = fmaf(wa, po[j], o[j]); o[j + 1] = fmaf(wb, po[j + 1], o[j + 1]); }
+  // Reference of tokens whose largest base-2 logit is mu: their own maximum (kRefLag: see there).  Returns the factor that
+  // brings the sums so far to it.
+  __device__ __forceinline__ float refer_to(float mu) {
+    exact = fmaxf(exact, mu);
+    const float ref = fmaxf(mu, exact - kRefLag), f = ex2_approx(m - ref);    // 0 at the start of a slab (m = -inf)
+    m = ref;
+    return f;
   }
 };
 
 // P V of one staged ternary supergroup for the 32 channels of warp w (two MMA row blocks: fragment i covers channels
 // 32 w + 4 hd + 2 i + {0, 1} in rows hd, hd + 8).  P(g, nt) = probabilities of head hd at the supergroup's tokens
 // 32 g + 8 nt + 2 r, + 1 (binary16 pair); ps[g] = -5 * (sum of the group's probabilities) of heads 2 r, 2 r + 1, twice:
-// the accumulator fragment P V starts from.  Adds to o and l.
+// the accumulator fragment P V starts from.
 template <typename PFrag>
-__device__ __forceinline__ void pv_ternary(const uint8_t* vbuf, int w, PFrag P, const float4 (&ps)[kSGGroups], float (&out)[8], float (&l)[2],
-                                           int hd, int r) {
+__device__ __forceinline__ void pv_ternary(const uint8_t* vbuf, int w, PFrag P, const float4 (&ps)[kSGGroups], Running& run, int hd,
+                                           int r) {
   uint32_t W[2][8];
 #pragma unroll
   for (int kt = 0; kt < 2; ++kt) {
@@ -371,12 +371,12 @@ __device__ __forceinline__ void pv_ternary(const uint8_t* vbuf, int w, PFrag P, 
     const uint2 sc2 = *reinterpret_cast<const uint2*>(vbuf + kSG_Scales + g * (kD * 2) + (32 * w + 4 * hd) * 2);
     const float2 sa = __half22float2(*reinterpret_cast<const __half2*>(&sc2.x));
     const float2 sb = __half22float2(*reinterpret_cast<const __half2*>(&sc2.y));
-    out[0] = fmaf(sa.x, acc[0][0], out[0]); out[1] = fmaf(sa.x, acc[0][1], out[1]);
-    out[2] = fmaf(sa.y, acc[0][2], out[2]); out[3] = fmaf(sa.y, acc[0][3], out[3]);
-    out[4] = fmaf(sb.x, acc[1][0], out[4]); out[5] = fmaf(sb.x, acc[1][1], out[5]);
-    out[6] = fmaf(sb.y, acc[1][2], out[6]); out[7] = fmaf(sb.y, acc[1][3], out[7]);
-    l[0] = fmaf(-0.2f, ps[g].x, l[0]);
-    l[1] = fmaf(-0.2f, ps[g].y, l[1]);
+    run.o[0] = fmaf(sa.x, acc[0][0], run.o[0]); run.o[1] = fmaf(sa.x, acc[0][1], run.o[1]);
+    run.o[2] = fmaf(sa.y, acc[0][2], run.o[2]); run.o[3] = fmaf(sa.y, acc[0][3], run.o[3]);
+    run.o[4] = fmaf(sb.x, acc[1][0], run.o[4]); run.o[5] = fmaf(sb.x, acc[1][1], run.o[5]);
+    run.o[6] = fmaf(sb.y, acc[1][2], run.o[6]); run.o[7] = fmaf(sb.y, acc[1][3], run.o[7]);
+    run.l[0] = fmaf(-0.2f, ps[g].x, run.l[0]);
+    run.l[1] = fmaf(-0.2f, ps[g].y, run.l[1]);
   }
 }
 
@@ -424,12 +424,12 @@ __device__ __forceinline__ void pv_protected(const uint8_t* pg, int w, const uin
   run.o[6] += sb.y * acc[1][2] + zb.y * sp0; run.o[7] += sb.y * acc[1][3] + zb.y * sp1;
 }
 
-// The running maximum follows a maximum `mu` (base-2 logit of head lane / 4) that exceeds it by more than kStaleLog2:
-// true if some head's moved, with the factors of heads 2 r, 2 r + 1 and of the lane's own head.
-__device__ __forceinline__ bool move_maximum(float mu, bool integral, int r, float& m, float& fa, float& fb, float& f) {
+// The integral running maximum follows a maximum `mu` (base-2 logit of head lane / 4) that exceeds it by more than
+// kStaleLog2: true if some head's moved, with the factors of heads 2 r, 2 r + 1 and of the lane's own head.
+__device__ __forceinline__ bool move_maximum(float mu, int r, float& m, float& fa, float& fb, float& f) {
   const bool up = mu > m + kStaleLog2;                      // always true at the start of a slab (m = -inf)
   if (!__any_sync(0xffffffffu, up)) return false;
-  const float m_new = up ? (integral ? ceilf(mu) : mu) : m;
+  const float m_new = up ? ceilf(mu) : m;
   f = ex2_approx(m - m_new);                                // 1 for heads whose maximum stays
   m = m_new;
   fa = __shfl_sync(0xffffffffu, f, 8 * r);
@@ -480,17 +480,15 @@ __device__ __forceinline__ void add_residual(const DecodeArgs& a, const uint8_t*
   for (int t = r; t < n_res; t += 4) mu = fmaxf(mu, Sx[hd * kResS + t]);
   mu = fmaxf(mu, __shfl_xor_sync(0xffffffffu, mu, 1));
   mu = fmaxf(mu, __shfl_xor_sync(0xffffffffu, mu, 2));
-  float fa, fb, f;
-  run.exact = fmaxf(run.exact, mu);
-  if (move_maximum(mu, false, r, run.m, fa, fb, f)) run.scale(fa, fb);
-  const float weight = ex2_approx(mu - run.m);             // the residual's own maximum is its probabilities' reference
+  const float f = run.refer_to(mu);
+  run.scale(__shfl_sync(0xffffffffu, f, 8 * r), __shfl_sync(0xffffffffu, f, 8 * r + 4));
   const int n_pad = (n_res + 15) & ~15;
   for (int t = 8 * r + 32 * warp; warp < 4 && t < n_pad; t += kR) {
     uint32_t w[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const int t0 = t + 2 * j;
-      w[j] = pack_half2(t0 < n_res ? ex2_approx(Sx[hd * kResS + t0] - mu) : 0.0f, t0 + 1 < n_res ? ex2_approx(Sx[hd * kResS + t0 + 1] - mu) : 0.0f);
+      w[j] = pack_half2(t0 < n_res ? ex2_approx(Sx[hd * kResS + t0] - run.m) : 0.0f, t0 + 1 < n_res ? ex2_approx(Sx[hd * kResS + t0 + 1] - run.m) : 0.0f);
     }
     *reinterpret_cast<uint4*>(Px + hd * kResP + t) = make_uint4(w[0], w[1], w[2], w[3]);
   }
@@ -519,9 +517,10 @@ __device__ __forceinline__ void add_residual(const DecodeArgs& a, const uint8_t*
       mma_f16(acc[1], prmt(v[0].y, v[1].y, 0x5410u), prmt(v[0].y, v[1].y, 0x7632u), prmt(v[2].y, v[3].y, 0x5410u),
               prmt(v[2].y, v[3].y, 0x7632u), b0, b1);
     }
-    const float o[8] = {acc[0][0], acc[0][1], acc[0][2], acc[0][3], acc[1][0], acc[1][1], acc[1][2], acc[1][3]};
-    const float l[2] = {-0.2f * ps[0], -0.2f * ps[1]};
-    run.add(o, l, weight, r);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) run.o[j] += acc[j >> 2][j & 3];
+    run.l[0] = fmaf(-0.2f, ps[0], run.l[0]);
+    run.l[1] = fmaf(-0.2f, ps[1], run.l[1]);
   }
 }
 
@@ -747,7 +746,7 @@ __global__ void __launch_bounds__(kUnitThreads, GEN && STP ? kBlockGenStpPerSM :
       int img_chunk[2] = {-1, -1};                           // chunk c's images are in slot c % 2
       const uint32_t *ew = nullptr, *ep = nullptr;
       int u_hi = 0, p_hi = 0;                                // STP: stream positions written so far
-      float unit_weight = 0.0f;                              // otherwise: 2^(maximum of the unit whose P V is due - m)
+      float unit_factor = 0.0f;                              // otherwise: brings the sums to the reference of the unit whose P V is due
       auto request = [&]() {                                 // copies whose buffers are free (after a barrier; whole block)
         if (producer) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         while (sg_req < sg_end && sg_req < sg_next + 2) {
@@ -788,12 +787,9 @@ __global__ void __launch_bounds__(kUnitThreads, GEN && STP ? kBlockGenStpPerSM :
         float4 ps[kSGGroups];
 #pragma unroll
         for (int g = 0; g < kSGGroups; ++g) ps[g] = psum[unit & 1][g][r];
-        float o[8], l[2] = {0.0f, 0.0f};
-#pragma unroll
-        for (int j = 0; j < 8; ++j) o[j] = 0.0f;
+        run.scale(__shfl_sync(0xffffffffu, unit_factor, 8 * r), __shfl_sync(0xffffffffu, unit_factor, 8 * r + 4));
         pv_ternary(sm + S::v_at + (unit & 1) * kVBufBytes, warp,
-                   [&](int g, int nt) { return *reinterpret_cast<const uint32_t*>(prow + g * (kG * 2) + nt * 16); }, ps, o, l, hd, r);
-        run.add(o, l, unit_weight, r);
+                   [&](int g, int nt) { return *reinterpret_cast<const uint32_t*>(prow + g * (kG * 2) + nt * 16); }, ps, run, hd, r);
       };
       auto multiply_streams = [&](int u_done, int p_done) {
         const uint8_t* trow = sm + S::prob_at + hd * kRingRow + 4 * r;
@@ -812,7 +808,7 @@ __global__ void __launch_bounds__(kUnitThreads, GEN && STP ? kBlockGenStpPerSM :
                 mma_f16(c, kMinus5, kMinus5, kMinus5, kMinus5, P(g, 2), P(g, 3));
                 ps[g] = make_float4(c[0], c[1], c[2], c[3]);
               }
-              pv_ternary(sm + S::v_at + (vcnt & 1) * kVBufBytes, warp, P, ps, run.o, run.l, hd, r);
+              pv_ternary(sm + S::v_at + (vcnt & 1) * kVBufBytes, warp, P, ps, run, hd, r);
             }
           }
           ++sg_next; ++vcnt;
@@ -888,11 +884,16 @@ __global__ void __launch_bounds__(kUnitThreads, GEN && STP ? kBlockGenStpPerSM :
         if (STP) request();
         // ---- probabilities against the running maximum
         float fa, fb, f;
+        bool moved = false;
         const float4 ga = *reinterpret_cast<const float4*>(&gmax[i & 1][hd][0]);
         const float mu = fmaxf(fmaxf(fmaxf(ga.x, ga.y), fmaxf(ga.z, ga.w)), gmax[i & 1][hd][4]) * sl2;   // sl2 > 0
-        run.exact = fmaxf(run.exact, STP ? ceilf(mu) : mu);
-        const bool moved = move_maximum(mu, STP, r, run.m, fa, fb, f);
-        const float off = fmaf(cst, sl2, STP ? -run.m : -mu);
+        if (STP) {
+          run.exact = fmaxf(run.exact, ceilf(mu));
+          moved = move_maximum(mu, r, run.m, fa, fb, f);
+        } else {
+          f = run.refer_to(mu);
+        }
+        const float off = fmaf(cst, sl2, -run.m);
         if (!STP) {
           uint8_t* prow = sm + S::prob_at + ((i & 1) * 8 + hd) * kPRowBytes + warp * (kG * 2) + 4 * r;
           uint32_t P[4] = {0u, 0u, 0u, 0u};
@@ -908,8 +909,7 @@ __global__ void __launch_bounds__(kUnitThreads, GEN && STP ? kBlockGenStpPerSM :
           mma_f16(c, kMinus5, kMinus5, kMinus5, kMinus5, P[2], P[3]);
           if (hd == 0) psum[i & 1][warp][r] = make_float4(c[0], c[1], c[2], c[3]);
           if (k > k_begin) multiply(i - 1);
-          if (moved) run.scale(fa, fb);
-          unit_weight = ex2_approx(mu - run.m);
+          unit_factor = f;
         } else {
           const int u_old = u_hi, p_old = p_hi;
           p_hi = p_new;

@@ -12,6 +12,8 @@ constexpr int kGenKBufBytes = kSGGroups * kMaxKGroupBytes;    // the same for th
 constexpr int kVBufBytes = kSGBytes;                          // 5376: a ternary supergroup
 constexpr uint32_t kWaitLimit = 1u << 19;                     // mbarrier polls before a warp gives up (about a second)
 constexpr float kStaleLog2 = 6.0f;                            // the running maximum may lag a unit's maximum by this much
+constexpr float kRefLag = 60.0f;                              // a unit's reference is no further below the largest maximum (its sums
+                                                              // are then nothing beside the others'), so that running sums stay below 2^95
 constexpr uint32_t kMinus5 = 0xc500c500u;                     // binary16 pair (-5.0, -5.0)
 constexpr uint32_t kMinus4 = 0xc400c400u;                     // binary16 pair (-4.0, -4.0)
 

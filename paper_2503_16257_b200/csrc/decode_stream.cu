@@ -35,8 +35,10 @@ namespace {
 constexpr int kTotBytes = 4 * 2 * 32 * 16;             // 4096: the warp's running output (128 channels x 8 heads, float)
 constexpr int kWarpBufBytes = kKBufBytes + kVBufBytes + kTotBytes;   // 15232 per warp
 
-// Per-lane state of the running softmax of one slab (the running output itself is in shared memory).
+// Per-lane state of the running softmax of one slab (the running output itself is in shared memory).  m: the reference
+// that the running sums are in units of; top: the largest unit maximum so far.
 struct Running {
+  float top;
   float l[2];           // sums of the probabilities of heads 2 r, 2 r + 1
   float m;              // running maximum (base-2 logit) of head hd
 };
@@ -206,10 +208,10 @@ __device__ __forceinline__ void score_group_general(const uint8_t* kg, const Key
 // head hd at stream tokens 32 g + 8 nt + 2 r, + 1 (binary16 pairs) and ps[g] the accumulator
 // fragment -5 * (sum of those probabilities) of heads 2 r, 2 r + 1.  32 channels (two MMA row
 // blocks) at a time: fragment i of block w covers channels 32 w + 4 hd + 2 i + {0, 1} in rows hd,
-// hd + 8.  Adds into the warp's running output; WEIGHTED: times wa (heads 2 r) and wb (heads 2 r + 1).
-template <int NG, bool WEIGHTED>
+// hd + 8.  Adds into the warp's running output, which RESCALE multiplies by fa (heads 2 r) and fb (heads 2 r + 1) first.
+template <int NG, bool RESCALE>
 __device__ __forceinline__ void pv_ternary(const uint8_t* vbuf, float* totbuf, const uint32_t (&P)[NG][4],
-                                           const float (&ps)[NG][4], float wa, float wb, int lane, int hd, int r) {
+                                           const float (&ps)[NG][4], float fa, float fb, int lane, int hd, int r) {
 #pragma unroll 1
   for (int w = 0; w < 4; ++w) {
     float acc[NG][2][4];
@@ -250,8 +252,11 @@ __device__ __forceinline__ void pv_ternary(const uint8_t* vbuf, float* totbuf, c
       }
     }
     float4* tp = reinterpret_cast<float4*>(totbuf) + (2 * w) * 32 + lane;
-    float4 t0 = make_float4(0.0f, 0.0f, 0.0f, 0.0f), t1 = t0;
-    if (!WEIGHTED) { t0 = tp[0]; t1 = tp[32]; }
+    float4 t0 = tp[0], t1 = tp[32];
+    if (RESCALE) {
+      t0.x *= fa; t0.y *= fb; t0.z *= fa; t0.w *= fb;
+      t1.x *= fa; t1.y *= fb; t1.z *= fa; t1.w *= fb;
+    }
 #pragma unroll
     for (int g = 0; g < NG; ++g) {
       const uint2 sc2 = *reinterpret_cast<const uint2*>(vbuf + kSG_Scales + g * (kD * 2) + (32 * w + 4 * hd) * 2);
@@ -262,11 +267,6 @@ __device__ __forceinline__ void pv_ternary(const uint8_t* vbuf, float* totbuf, c
       t1.x += sb.x * acc[g][1][0]; t1.y += sb.x * acc[g][1][1];
       t1.z += sb.y * acc[g][1][2]; t1.w += sb.y * acc[g][1][3];
     }
-    if (WEIGHTED) {
-      const float4 u0 = tp[0], u1 = tp[32];
-      t0.x = fmaf(wa, t0.x, u0.x); t0.y = fmaf(wb, t0.y, u0.y); t0.z = fmaf(wa, t0.z, u0.z); t0.w = fmaf(wb, t0.w, u0.w);
-      t1.x = fmaf(wa, t1.x, u1.x); t1.y = fmaf(wb, t1.y, u1.y); t1.z = fmaf(wa, t1.z, u1.z); t1.w = fmaf(wb, t1.w, u1.w);
-    }
     tp[0] = t0;
     tp[32] = t1;
   }
@@ -276,9 +276,10 @@ __device__ __forceinline__ void pv_ternary(const uint8_t* vbuf, float* totbuf, c
 // Returns false if a copy never arrived.
 // SHARD (the call leaves triples): the probabilities are taken against the running maximum, which is part of the result
 // and fixes the cut.  Otherwise against the unit's own maximum: where their binary16 rounding falls depends on the unit
-// alone, not on where the warp's run began, and the largest one is exact; the unit's sums join the running ones with the
-// weight 2^(mu - m).  Off by 3.3e-5 of the outputs' norm on 64 slabs x 12544 tokens, where the running maximum gives
-// 1.14e-4 and another cut moves the outputs by 1.5e-4.  The weights cost 1.3 % of a step (a token shard's 2 %).
+// alone, not on where the warp's run began, and the largest one is exact; the running sums are brought to the unit's
+// reference first.  Off by 3.3e-5 of the outputs' norm on 64 slabs x 12544 tokens, where the running maximum gives
+// 1.14e-4 and another cut moves the outputs by 1.5e-4; 32 steps of 1792 slabs x 79 units take 25.89 ms that way, 25.61 ms
+// against the running maximum.
 template <int NG, bool GEN, bool SHARD>
 __device__ __forceinline__ bool process_unit(const KeyFmt& kf, const uint32_t*& ppc, uint8_t* kbuf, uint8_t* vbuf, float* totbuf, uint64_t* kbar, uint64_t* vbar,
                                              uint32_t& kpar, uint32_t& vpar, int lane, int hd, int r,
@@ -331,36 +332,37 @@ __device__ __forceinline__ bool process_unit(const KeyFmt& kf, const uint32_t*& 
   mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
   mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
   const float mu = mx * sl2;                                // sl2 > 0
-  {
+  float fa = 1.0f, fb = 1.0f;
+  if (!SHARD) {
+    run.top = fmaxf(run.top, mu);
+    const float ref = fmaxf(mu, run.top - kRefLag);
+    const float f = ex2_approx(run.m - ref);                // 0 for the first unit (run.m = -inf)
+    run.m = ref;
+    fa = __shfl_sync(0xffffffffu, f, 8 * r);
+    fb = __shfl_sync(0xffffffffu, f, 8 * r + 4);
+    run.l[0] *= fa; run.l[1] *= fb;
+  } else {
     const bool up = mu > run.m + kStaleLog2;                // always true for the first unit (run.m = -inf)
     if (__any_sync(0xffffffffu, up)) {
       const float m_new = up ? mu : run.m;
       const float f = ex2_approx(run.m - m_new);            // 1 for heads whose maximum stays
       run.m = m_new;
-      const float fa = __shfl_sync(0xffffffffu, f, 8 * r), fb = __shfl_sync(0xffffffffu, f, 8 * r + 4);
+      const float ga = __shfl_sync(0xffffffffu, f, 8 * r), gb = __shfl_sync(0xffffffffu, f, 8 * r + 4);
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
         float4* t = reinterpret_cast<float4*>(totbuf) + j * 32 + lane;
         float4 v = *t;
-        v.x *= fa; v.y *= fb; v.z *= fa; v.w *= fb;
+        v.x *= ga; v.y *= gb; v.z *= ga; v.w *= gb;
         *t = v;
       }
-      run.l[0] *= fa; run.l[1] *= fb;
+      run.l[0] *= ga; run.l[1] *= gb;
     }
-  }
-  const float ref = SHARD ? run.m : mu;
-  float wa = 1.0f, wb = 1.0f;
-  if (!SHARD) {
-    const float wgt = ex2_approx(mu - run.m);
-    wa = __shfl_sync(0xffffffffu, wgt, 8 * r);
-    wb = __shfl_sync(0xffffffffu, wgt, 8 * r + 4);
   }
   uint32_t P[NG][4];
   float ps[NG][4];
-  float sum0 = 0.0f, sum1 = 0.0f;
 #pragma unroll
   for (int g = 0; g < NG; ++g) {
-    const float off = fmaf(reinterpret_cast<const float*>(kbuf + g * kgb)[256 + lane], sl2, -ref);
+    const float off = fmaf(reinterpret_cast<const float*>(kbuf + g * kgb)[256 + lane], sl2, -run.m);
 #pragma unroll
     for (int nt = 0; nt < 4; ++nt) {
       const float2 v = reinterpret_cast<const float2*>(kbuf + g * kgb)[nt * 32 + lane];
@@ -372,16 +374,8 @@ __device__ __forceinline__ bool process_unit(const KeyFmt& kf, const uint32_t*& 
     ps[g][0] = 0.0f; ps[g][1] = 0.0f; ps[g][2] = 0.0f; ps[g][3] = 0.0f;
     mma_f16(ps[g], kMinus5, kMinus5, kMinus5, kMinus5, P[g][0], P[g][1]);
     mma_f16(ps[g], kMinus5, kMinus5, kMinus5, kMinus5, P[g][2], P[g][3]);
-    if (SHARD) {
-      run.l[0] = fmaf(-0.2f, ps[g][0], run.l[0]);
-      run.l[1] = fmaf(-0.2f, ps[g][1], run.l[1]);
-    } else {
-      sum0 += ps[g][0]; sum1 += ps[g][1];
-    }
-  }
-  if (!SHARD) {
-    run.l[0] = fmaf(-0.2f * wa, sum0, run.l[0]);
-    run.l[1] = fmaf(-0.2f * wb, sum1, run.l[1]);
+    run.l[0] = fmaf(-0.2f, ps[g][0], run.l[0]);
+    run.l[1] = fmaf(-0.2f, ps[g][1], run.l[1]);
   }
   __syncwarp();                                             // the scores are in registers: the key buffer is free
   if (more && lane == 0) {
@@ -395,7 +389,7 @@ __device__ __forceinline__ bool process_unit(const KeyFmt& kf, const uint32_t*& 
     return false;
   }
   vpar ^= 1u;
-  pv_ternary<NG, !SHARD>(vbuf, totbuf, P, ps, wa, wb, lane, hd, r);
+  pv_ternary<NG, !SHARD>(vbuf, totbuf, P, ps, fa, fb, lane, hd, r);
   __syncwarp();
   if (more && lane == 0) {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -483,7 +477,7 @@ __global__ void __launch_bounds__(kStreamWarps * 32, kStreamCtasPerSM) decode_st
   pdl_release();
   uint32_t kpar = 0u, vpar = 0u;
   Running run;
-  run.l[0] = 0.0f; run.l[1] = 0.0f; run.m = -INFINITY;
+  run.l[0] = 0.0f; run.l[1] = 0.0f; run.m = -INFINITY; run.top = -INFINITY;
   uint32_t qa[8], qha[8], qhb[8];
   const uint32_t* ppc = nullptr;
   int cur_chunk = -1, cur_slab = -1;
@@ -499,7 +493,7 @@ __global__ void __launch_bounds__(kStreamWarps * 32, kStreamCtasPerSM) decode_st
 #pragma unroll
       for (int j = 0; j < 8; ++j) reinterpret_cast<float4*>(totbuf)[j * 32 + lane] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
       run.l[0] = 0.0f; run.l[1] = 0.0f;
-      run.m = -INFINITY;
+      run.m = -INFINITY; run.top = -INFINITY;
       prep_slab = a.prep + static_cast<int64_t>(slab) * pl.n_chunks * (kPrepWords * 32) + lane;
       sl2 = __uint_as_float(__ldg(prep_slab + 24 * 32));
     }
