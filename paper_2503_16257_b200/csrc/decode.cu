@@ -166,25 +166,30 @@ __global__ void __launch_bounds__(kD) decode_merge_kernel(DecodeArgs a, int n_re
   const float* rec = a.partials + (slab + first_run) * (kMaxRep * kRecordFloats);
   pdl_wait();                                              // the partial records come from the attention kernel before
   const int64_t q0 = (static_cast<int64_t>(lb) * cv.H_q + h * rep) * kD;
-  // ---- the records' maxima, sums and this lane's output fragments are fetched first, so that their
-  // latency passes behind the staging of the residual (the first kRecAhead records; more are read later)
+  // ---- the records' maxima and sums (lane j: record j, for the heads warp and warp + 4) and this lane's output fragments
+  // of the first kRecAhead records are fetched first, so that their latency passes behind the residual
+  float2 head_ml[2];
+#pragma unroll
+  for (int x = 0; x < 2; ++x) {
+    const int k = warp + 4 * x;
+    head_ml[x] = make_float2(-INFINITY, 0.0f);
+    if (k < rep && lane < n_parts) head_ml[x] = __ldg(reinterpret_cast<const float2*>(rec + (lane * kMaxRep + k) * kRecordFloats));
+  }
   constexpr int kRecAhead = 3;
-  float rec_m[kRecAhead], rec_l[kRecAhead];
+  float rec_m[kRecAhead];
   float2 rec_o[kRecAhead][4];
 #pragma unroll
   for (int jp = 0; jp < kRecAhead; ++jp) {
-    rec_m[jp] = -INFINITY; rec_l[jp] = 0.0f;
+    rec_m[jp] = -INFINITY;
 #pragma unroll
     for (int j = 0; j < 4; ++j) rec_o[jp][j] = make_float2(0.0f, 0.0f);
     if (jp < n_parts && hd < rep) {
       const float* pr = rec + (jp * kMaxRep + hd) * kRecordFloats;
       rec_m[jp] = __ldg(pr);
-      rec_l[jp] = __ldg(pr + 1);
 #pragma unroll
       for (int j = 0; j < 4; ++j) rec_o[jp][j] = __ldg(reinterpret_cast<const float2*>(pr + 2 + 32 * warp + 8 * j + 2 * r));
     }
   }
-  (void)rec_l;
   if (n_pad > 0) {
     // ---- stage the residual rows (16-byte pieces, all loads of a thread independent)
     const uint4* ksrc = reinterpret_cast<const uint4*>(slab_ptr + cv.kres_offset);
@@ -236,11 +241,13 @@ __global__ void __launch_bounds__(kD) decode_merge_kernel(DecodeArgs a, int n_re
     __syncthreads();
   }
   // ---- maxima and denominators: warp w takes heads w and w + 4
-  for (int k = warp; k < kMaxRep; k += kD / 32) {
-    float m = -INFINITY, m_res = -INFINITY;
+#pragma unroll
+  for (int x = 0; x < 2; ++x) {
+    const int k = warp + 4 * x;
+    float m = head_ml[x].x, m_res = -INFINITY;
     if (k < rep) {
       for (int t = lane; t < n_res; t += 32) m_res = fmaxf(m_res, S[k * n_pad + t]);
-      for (int j = lane; j < n_parts; j += 32) m = fmaxf(m, __ldg(rec + (j * kMaxRep + k) * kRecordFloats));
+      for (int j = lane + 32; j < n_parts; j += 32) m = fmaxf(m, __ldg(rec + (j * kMaxRep + k) * kRecordFloats));
     }
 #pragma unroll
     for (int o = 16; o; o >>= 1) {
@@ -257,11 +264,13 @@ __global__ void __launch_bounds__(kD) decode_merge_kernel(DecodeArgs a, int n_re
       l += __half2float(ph);
     }
     l *= w_res;
-    if (k < rep)
-      for (int j = lane; j < n_parts; j += 32) {
+    if (k < rep) {
+      l += head_ml[x].y * exp2f(head_ml[x].x - m);          // 0 for a record that does not exist
+      for (int j = lane + 32; j < n_parts; j += 32) {
         const float* pr = rec + (j * kMaxRep + k) * kRecordFloats;
         l += pr[1] * exp2f(pr[0] - m);
       }
+    }
 #pragma unroll
     for (int o = 16; o; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
     if (lane == 0) { Mh[k] = m; Lh[k] = l; Wh[k] = w_res; }
