@@ -2,6 +2,7 @@
 // work (plan_decode), the launch sequence, and the last kernel of a step, which merges the
 // partial records of the attention kernels by log-sum-exp and, for caches without protected
 // tokens, attends to the FP16 / BF16 residual itself.
+#include <numeric>
 #include <type_traits>
 
 #include "decode_common.cuh"
@@ -11,17 +12,16 @@ namespace vidkv {
 namespace {
 
 constexpr int kMaxSMs = 256;        // multiprocessor count the sizing formulas assume at most
-constexpr int kMinRunUnits = 1;     // with fewer units than warps every unit gets its own warp (shortest critical path)
 // Units per block up to which a call goes to the block kernel.  It has one launch, short parts and a parallel merge
 // where the stream kernel has three launches and a warp per run, but takes half as many instructions again per unit
 // (every warp of the block pays the unit's loop).  Measured (us per call, block / stream kernel): 160 units of 4 slabs
-// 15.8 / 25.1, 2560 units of 16 slabs 33 / 59, 4480 units of 448 slabs (8 a block) 47 / 47, 8960 units of 112 slabs 75 / 77;
-// with protected tokens 160 units 21.9 / 31.2, 1792 units of 448 slabs (4 a block) 37 / 41, 2240 units of 224 slabs 50 / 43.
+// 15.7 / 25.8, 1184 of 16 22.9 / 36.6, 4032 of 112 (7 a block) 40.0 / 43.1, 4032 of 448 43.2 / 43.4, 4480 of 448 (8 a block) 47 / 47;
+// with protected tokens 160 of 4 21.5 / 31.0, 1152 of 64 (2 a block) 31.2 / 32.9, 1344 of 448 (3) 30.0 / 39.5, 1760 of 32 (4) 40.5 / 43.2,
+// 1568 of 224 (4) 39.9 / 39.1.  Where every unit has a warp of its own in the stream kernel, three a block are too many there
+// (1120 of 224 33.8 / 30.9), except for the general key formats (1120 of 112, 4 a block, 35.9 / 37.0).
 constexpr int kMaxBlockUnits = 7;
-constexpr int kMaxBlockUnitsStp = 3;
-// A token shard's call with protected tokens (exact maxima, see DecodePlan::equal_units): 1152 units of 64 slabs, two a block,
-// took 275 us for eight calls against 269 with runs.
-constexpr int kMaxBlockUnitsStpPartial = 1;
+constexpr int kMaxBlockUnitsStp = 4;
+constexpr int kMaxBlockUnitsStpRun1 = 2;
 
 }  // namespace
 
@@ -53,7 +53,7 @@ DecodePlan plan_decode(const LayerState& st, int64_t n_slabs, bool stp, bool gen
   const int sms = sm_count < 1 ? 1 : (sm_count > kMaxSMs ? kMaxSMs : sm_count);
   const int64_t warps = static_cast<int64_t>(sms) * (stp ? kStreamStpCtasPerSM : kStreamCtasPerSM) * kStreamWarps;
   int64_t run = (p.n_units + warps - 1) / warps;
-  if (run < kMinRunUnits) run = kMinRunUnits;
+  if (run < 1) run = 1;                                    // nothing quantized
   if (force_run_units > 0) run = force_run_units;
   p.run_units = static_cast<int32_t>(run);
   if (partial) p.equal_units = p.run_units;
@@ -80,10 +80,19 @@ DecodePlan plan_decode(const LayerState& st, int64_t n_slabs, bool stp, bool gen
   p.slab_parts = static_cast<int32_t>(most_parts(p.n_runs));
   p.records = (p.n_runs + n_slabs) * kMaxRep;
   const int64_t blocks = static_cast<int64_t>(sms) * (stp && general ? kBlockGenStpPerSM : kBlocksPerSM);
-  const int64_t per_block = (p.n_units + blocks - 1) / blocks;
-  const int64_t most = !stp ? kMaxBlockUnits : partial ? kMaxBlockUnitsStpPartial : kMaxBlockUnitsStp;
+  int64_t per_block = (p.n_units + blocks - 1) / blocks;
+  // A block that goes on in the next slab pays for query images, rings and join twice: where the proportional cut makes such
+  // blocks (slab s then begins d units * slabs / blocks after a block does, d running through the multiples of
+  // gcd(blocks, slabs)), every slab gets its own blocks, if it can without a longer stretch.  us, straddling / not: 64 slabs
+  // of 14 units 28.9 / 21.8, 448 of 3 28.2 / 21.0; with protected tokens 42.3 / 31.7 and 45.2 / 30.0.
+  int64_t even_blocks = 0;
+  if (p.n_units > 0 && p.n_units - std::gcd(blocks, n_slabs) * p.units_per_slab >= blocks) {
+    const int64_t share = blocks / n_slabs, even = share > 0 ? (p.units_per_slab + share - 1) / share : INT32_MAX;
+    if (stp || even <= per_block) { per_block = even; even_blocks = n_slabs * (share < p.units_per_slab ? share : p.units_per_slab); }
+  }
+  const int64_t most = !stp ? kMaxBlockUnits : general || run > 1 ? kMaxBlockUnitsStp : kMaxBlockUnitsStpRun1;
   if (p.n_units == 0 || (per_block <= most && force_run_units == 0 && (!partial || run == 1))) {
-    p.n_blocks = static_cast<int32_t>(p.n_units < blocks ? p.n_units : blocks);
+    p.n_blocks = static_cast<int32_t>(even_blocks > 0 ? even_blocks : p.n_units < blocks ? p.n_units : blocks);
     p.records = (p.n_blocks + n_slabs) * kMaxRep;
     p.res_blocks = st.n_res > 0 && per_block <= 1 ? static_cast<int32_t>(n_slabs) : 0;
     p.counters_per_slab = static_cast<int32_t>(join_counters(most_parts(p.n_blocks) + (p.res_blocks > 0)));
