@@ -29,7 +29,7 @@ template <> struct Pair2<__nv_bfloat16> {
 };
 
 template <typename T>
-__global__ void __launch_bounds__(256) k_range_kernel(KSrc src, int64_t T_tokens, int tokens_per_block, int splits, int n_res,
+__global__ void __launch_bounds__(256, 5) k_range_kernel(KSrc src, int64_t T_tokens, int tokens_per_block, int splits, int n_res,
                                                       CacheView cv, int layer0, uint32_t* __restrict__ minmax,
                                                       int32_t* __restrict__ counters, int64_t n_counters) {
   using P = Pair2<T>;
@@ -37,9 +37,10 @@ __global__ void __launch_bounds__(256) k_range_kernel(KSrc src, int64_t T_tokens
   const int slab = blockIdx.y;
   pdl_wait();
   pdl_release();                                           // the encode pass may set itself up beside this one
-  for (int64_t i = (static_cast<int64_t>(blockIdx.y) * gridDim.x + blockIdx.x) * 256 + threadIdx.x; i < n_counters;
-       i += static_cast<int64_t>(gridDim.x) * gridDim.y * 256)
-    counters[i] = 0;
+  if (n_counters > 0)
+    for (int64_t i = (static_cast<int64_t>(blockIdx.y) * gridDim.x + blockIdx.x) * 256 + threadIdx.x; i < n_counters;
+         i += static_cast<int64_t>(gridDim.x) * gridDim.y * 256)
+      counters[i] = 0;
   if (static_cast<int>(blockIdx.x) == splits) {            // one more block per slab for the tokens that stay as they are
     copy_residual_rows(src, T_tokens, n_res, cv, layer0, slab, cv.kres_offset);
     return;
