@@ -56,12 +56,18 @@ class SampledRun:
                     self.slabs[(sl, b, h)] = sc
             del K, V
 
-    def decode(self, check=True):
+    def decode(self, check=True, triples=False):
+        """triples: through the call that leaves (maximum, sum, output) triples, and their merge."""
         wl, L, B = self.wl, self.L, self.B
         q, k, v = (torch.stack(t) for t in zip(*[make_step_inputs(wl, layer, self.step, "cuda", T=self.T, B=B)
                                                   for layer in range(L)]))
         out = torch.empty((L, B, self.cfg.H_q, 128), dtype=torch.float32, device="cuda")
-        self.cache.decode_attention(0, L, q, k, v, out)
+        if triples:
+            part = torch.empty((1, L, B, self.cfg.H_q, 130), dtype=torch.float32, device="cuda")
+            self.cache.decode_attention_partial(0, L, q, k, v, part[0])
+            self.P.vidkv_merge_partials(part, out)
+        else:
+            self.cache.decode_attention(0, L, q, k, v, out)
         out = out.cpu().numpy().astype(np.float64)
         rep = self.cfg.H_q // self.cfg.H_kv
         worst = 0.0
@@ -219,20 +225,24 @@ def test_seeded_random_shapes_and_run_lengths(name, T, B, L, p, run_units, steps
 # ------------------------------------------------------------------ the one-launch kernel of small calls
 @pytest.mark.parametrize("name,L,B,T,p,steps,check_from", [
     ("tiny", 1, 1, 160, 0.0, 2, 0),          # one unit and a residual block per slab
-    ("qwen", 1, 1, 36000, 0.0, 2, 0),        # 900 units: two to a block, 113 parts and three levels of joins per slab
-    ("tiny", 12, 4, 2029, 0.0, 100, 96),     # 13 units per slab, five to a block, slabs shared by blocks; across a flush
-    ("tiny", 28, 4, 330, 0.0, 3, 0),         # slabs of three units, the last one a single group
+    ("qwen", 1, 1, 36000, 0.0, 2, 0),        # 225 units per slab, one or two to a block: about 148 parts, three levels of joins
+    ("tiny", 12, 4, 2029, 0.0, 118, 113),    # 13 units per slab, five to a block, slabs shared by blocks; across a flush
+    ("tiny", 28, 4, 362, 0.0, 3, 0),         # slabs of three units, the last one a single group; three to a block
+    ("tiny", 4, 4, 2285, 0.0, 2, 0),         # 64 slabs of 14 units and a group: blocks end with their slabs
     ("qwen", 1, 1, 163, 0.5, 2, 0),          # protected tokens: one unit per slab
-    ("tiny", 8, 4, 2029, 0.2, 100, 96),      # three units to a block; across a flush
+    ("tiny", 8, 4, 2029, 0.2, 118, 113),     # three or four units to a block, blocks end with their slabs; across a flush
+    ("qwen", 4, 4, 2285, 0.3, 2, 0),         # bfloat16
     ("llava", 1, 2, 26000, 0.93, 2, 0),      # long protected stream, 1304 units
 ])
 def test_small_calls_in_one_launch(name, L, B, T, p, steps, check_from):
-    """Calls of up to seven units (three with protected tokens) per block: block and slab boundaries inside and on unit
-    boundaries, the residual with a block of its own and with the slab's last block, every depth of the merge tree."""
+    """Calls of up to seven units (four with protected tokens) per block: block and slab boundaries inside and on unit
+    boundaries, the residual with a block of its own and with the slab's last block, every depth of the merge tree;
+    the step behind the last one leaves triples."""
     samples = sorted({(0, 0, 0), (L - 1, B - 1, 3), (L // 2, B // 2, 1)})
-    run = SampledRun(name, L, B, T, p, steps, samples)
+    run = SampledRun(name, L, B, T, p, steps + 1, samples)
     for s in range(steps):
         run.decode(check=s >= check_from)
+    run.decode(triples=True)
     assert run.cache.status() == 0
 
 
