@@ -245,7 +245,8 @@ vidkv_status_t vidkv_select_tokens(vidkv_cache_t* handle, const float* saliency,
  * E [B, T] (uint8, nonzero = protected; every batch element must protect the same
  * number of tokens, all below T - T % G).  n_protected >= 0 states that number: the call is
  * then asynchronous like the others, and a row of E that protects a different number sets
- * VIDKV_ERR_INVALID_ARG in the cache's status word (vidkv_cache_status).  n_protected == -1
+ * VIDKV_ERR_INVALID_ARG in the cache's status word (vidkv_cache_status); the row then goes on with its
+ * first n_protected tokens, or with unprotected ones added in token order.  n_protected == -1
  * lets the library count: it then reads the counts back and synchronises the stream once. */
 vidkv_status_t vidkv_set_token_mask(vidkv_cache_t* handle, const uint8_t* E, int64_t T, int64_t n_protected,
                                     void* stream);

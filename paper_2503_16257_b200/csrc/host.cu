@@ -307,6 +307,7 @@ vidkv_status_t vidkv_set_token_mask(vidkv_cache_t* h, const uint8_t* E, int64_t 
   int32_t* ip = reinterpret_cast<int32_t*>(h->workspace + h->ws.idx_prot_off);
   int32_t* ir = reinterpret_cast<int32_t*>(h->workspace + h->ws.idx_rest_off);
   int32_t* dc = reinterpret_cast<int32_t*>(h->workspace + h->ws.counts_off);
+  h->sel_set = false;                            // the selection of before is overwritten, whatever becomes of this one
   if (launch_mask_to_selection(E, T, T_q, h->cv, ip, ir, h->L.max_prot, h->cfg.max_prefill_tokens, dc, n_protected, s) !=
       cudaSuccess)
     return VIDKV_ERR_CUDA;

@@ -455,6 +455,7 @@ __global__ void __launch_bounds__(kSelThreads) select_tokens_kernel(const float*
       pmask |= (bins - 1) << shift;
     }
   }
+  int stray = 0;                               // the row of a mask protects more (1) or fewer (-1) tokens than stated
   // gt / eq bits of token group w, the same in every lane
   auto word_bits = [&](int64_t w, uint32_t& gt, uint32_t& eq) {
     const int64_t t = w * kG + lane;
@@ -465,76 +466,94 @@ __global__ void __launch_bounds__(kSelThreads) select_tokens_kernel(const float*
         g = key > thr; e = key == thr;
       }
     } else {
-      g = __ldg(mask + b * mask_stride + t) != 0;
+      const bool marked = __ldg(mask + b * mask_stride + t) != 0;
+      g = marked && stray <= 0;
+      e = stray > 0 ? marked : stray < 0 && !marked;
     }
     gt = __ballot_sync(0xffffffffu, g); eq = __ballot_sync(0xffffffffu, e);
   };
-  int64_t carry = 0;                           // (at) << 32 | (above) before the next stretch of words
-  if (n_blocks > 1) {
-    int64_t mine = 0;
+#pragma unroll 1
+  for (bool again = true; again;) {
+    int64_t carry = 0;                           // (at) << 32 | (above) before the next stretch of words
+    if (n_blocks > 1) {
+      int64_t mine = 0;
 #pragma unroll 8
-    for (int64_t w = w_begin + warp; w < w_end; w += 32) {
-      uint32_t gt, eq;
-      word_bits(w, gt, eq);
-      mine += static_cast<int64_t>(__popc(gt)) | (static_cast<int64_t>(__popc(eq)) << 32);
+      for (int64_t w = w_begin + warp; w < w_end; w += 32) {
+        uint32_t gt, eq;
+        word_bits(w, gt, eq);
+        mine += static_cast<int64_t>(__popc(gt)) | (static_cast<int64_t>(__popc(eq)) << 32);
+      }
+      if (lane == 0) s_warp[warp] = mine;
+      __syncthreads();
+      if (tid == 0) {
+        int64_t sum = 0;
+        for (int i = 0; i < 32; ++i) sum += s_warp[i];
+        s_block = sum;
+      }
+      cluster.sync();
+      for (int r = 0; r < rank; ++r) carry += *cluster.map_shared_rank(&s_block, r);
     }
-    if (lane == 0) s_warp[warp] = mine;
-    __syncthreads();
-    if (tid == 0) {
-      int64_t sum = 0;
-      for (int i = 0; i < 32; ++i) sum += s_warp[i];
-      s_block = sum;
-    }
-    cluster.sync();
-    for (int r = 0; r < rank; ++r) carry += *cluster.map_shared_rank(&s_block, r);
-  }
-  uint32_t* e_words = const_cast<uint32_t*>(cv.e_words(b));
-  uint32_t* e_prefix = const_cast<uint32_t*>(cv.e_prefix(b));
-  for (int64_t base = w_begin; base < w_end; base += kSelThreads) {
-    // up to 1024 words at a time: every warp takes per_warp consecutive ones, lane i keeps word i
-    const int n = static_cast<int>(min(static_cast<int64_t>(kSelThreads), w_end - base));
-    const int per_warp = (n + 31) / 32;
-    const int n_own = max(0, min(per_warp, n - warp * per_warp));
-    const int64_t w0 = base + warp * per_warp;
-    uint32_t gt = 0, eq = 0;
+    uint32_t* e_words = const_cast<uint32_t*>(cv.e_words(b));
+    uint32_t* e_prefix = const_cast<uint32_t*>(cv.e_prefix(b));
+    for (int64_t base = w_begin; base < w_end; base += kSelThreads) {
+      // up to 1024 words at a time: every warp takes per_warp consecutive ones, lane i keeps word i
+      const int n = static_cast<int>(min(static_cast<int64_t>(kSelThreads), w_end - base));
+      const int per_warp = (n + 31) / 32;
+      const int n_own = max(0, min(per_warp, n - warp * per_warp));
+      const int64_t w0 = base + warp * per_warp;
+      uint32_t gt = 0, eq = 0;
 #pragma unroll 8
-    for (int i = 0; i < n_own; ++i) {
-      uint32_t g, e;
-      word_bits(w0 + i, g, e);
-      if (lane == i) { gt = g; eq = e; }
-    }
-    int64_t total;
-    const int64_t before = carry + block_exclusive_scan(static_cast<int64_t>(__popc(gt)) | (static_cast<int64_t>(__popc(eq)) << 32), s_warp, &total);
-    carry += total;
-    const int64_t eq_before = before >> 32;
-    int take = static_cast<int>(need) - static_cast<int>(min(eq_before, static_cast<int64_t>(need)));
-    const int prot = static_cast<int>((before & 0xffffffff) + (static_cast<int64_t>(need) - take));
-    uint32_t word = gt;
-    for (uint32_t rem = eq; rem && take > 0; rem &= rem - 1, --take) word |= rem & (0u - rem);
-    if (lane < n_own) {
-      e_words[w0 + lane] = word;
-      e_prefix[w0 + lane] = static_cast<uint32_t>(prot);
-    }
+      for (int i = 0; i < n_own; ++i) {
+        uint32_t g, e;
+        word_bits(w0 + i, g, e);
+        if (lane == i) { gt = g; eq = e; }
+      }
+      int64_t total;
+      const int64_t before = carry + block_exclusive_scan(static_cast<int64_t>(__popc(gt)) | (static_cast<int64_t>(__popc(eq)) << 32), s_warp, &total);
+      carry += total;
+      const int64_t eq_before = before >> 32;
+      int take = static_cast<int>(need) - static_cast<int>(min(eq_before, static_cast<int64_t>(need)));
+      const int prot = static_cast<int>((before & 0xffffffff) + (static_cast<int64_t>(need) - take));
+      uint32_t word = gt;
+      for (uint32_t rem = eq; rem && take > 0; rem &= rem - 1, --take) word |= rem & (0u - rem);
+      if (lane < n_own) {
+        e_words[w0 + lane] = word;
+        e_prefix[w0 + lane] = static_cast<uint32_t>(prot);
+      }
 #pragma unroll 4
-    for (int i = 0; i < n_own; ++i) {
-      const uint32_t bits = __shfl_sync(0xffffffffu, word, i);
-      const int64_t t = (w0 + i) * kG + lane;
-      const int64_t pk = __shfl_sync(0xffffffffu, prot, i) + __popc(bits & ((1u << lane) - 1u));
-      if ((bits >> lane) & 1u) {
-        if (pk < stride_prot) idx_prot[b * stride_prot + pk] = static_cast<int32_t>(t);
-      } else {
-        idx_rest[b * stride_rest + (t - pk)] = static_cast<int32_t>(t);
+      for (int i = 0; i < n_own; ++i) {
+        const uint32_t bits = __shfl_sync(0xffffffffu, word, i);
+        const int64_t t = (w0 + i) * kG + lane;
+        const int64_t pk = __shfl_sync(0xffffffffu, prot, i) + __popc(bits & ((1u << lane) - 1u));
+        if ((bits >> lane) & 1u) {
+          if (pk < stride_prot) idx_prot[b * stride_prot + pk] = static_cast<int32_t>(t);
+        } else {
+          idx_rest[b * stride_rest + (t - pk)] = static_cast<int32_t>(t);
+        }
       }
     }
-  }
-  if (rank == n_blocks - 1 && tid == 0) {
-    const int n = static_cast<int>((carry & 0xffffffff) + min(carry >> 32, static_cast<int64_t>(need)));
-    e_prefix[W] = static_cast<uint32_t>(n);
-    e_words[W] = 0;
-    if (counts) counts[b] = n;
-    // a mask whose row does not protect the number of tokens the caller stated
-    if (expect_count >= 0 && n != expect_count)
-      atomicCAS(reinterpret_cast<int*>(cv.base + kHdrStatus), VIDKV_OK, VIDKV_ERR_INVALID_ARG);
+    if (rank == n_blocks - 1 && tid == 0) {
+      const int n = static_cast<int>((carry & 0xffffffff) + min(carry >> 32, static_cast<int64_t>(need)));
+      e_prefix[W] = static_cast<uint32_t>(n);
+      e_words[W] = 0;
+      if (counts) counts[b] = n;
+      s_block = n;
+    }
+    // A mask whose row does not protect the number of tokens that the caller stated: reported, and the row is done once more
+    // with its first `expect_count` tokens, or with unprotected ones added in token order, so that the lists and the mask hold
+    // what the quantizer and the attention kernels count on.
+    again = false;
+    if (expect_count >= 0 && stray == 0) {
+      cluster.sync();
+      const int64_t n = *cluster.map_shared_rank(&s_block, n_blocks - 1);
+      cluster.sync();
+      if (n != expect_count) {
+        if (rank == 0 && tid == 0) atomicCAS(reinterpret_cast<int*>(cv.base + kHdrStatus), VIDKV_OK, VIDKV_ERR_INVALID_ARG);
+        stray = n > expect_count ? 1 : -1;
+        need = static_cast<uint32_t>(stray > 0 ? expect_count : expect_count - n);
+        again = true;
+      }
+    }
   }
   if (n_blocks > 1) cluster.sync();            // the other blocks may still read this one's shared memory
 }

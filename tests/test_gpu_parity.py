@@ -718,6 +718,45 @@ def test_token_mask_entry_point_matches_saliency_selection():
     assert d.status() == -1
 
 
+@pytest.mark.parametrize("T", [320, 16384 + 40])          # one block a row, a cluster a row
+def test_mask_rows_that_miss_the_stated_count_stay_consistent(T):
+    """A stated count that a row of the mask does not hold is reported in the status word, and nothing behind it reads
+    gather lists that were never written: the row keeps its first tokens or is filled up in token order."""
+    import paper_2503_16257_b200 as P
+    from workloads import make_layer_kv, make_step_inputs
+    wl, n, Tq = CONFIGS["tiny"], 51, T - T % 32
+    r = np.random.default_rng(T)
+    E = np.zeros((3, T), dtype=np.uint8)
+    for b, count in enumerate((n, n + 9, n - 12)):
+        E[b, r.choice(Tq, count, replace=False)] = 1
+    want = E.copy()
+    want[1, np.nonzero(E[1])[0][n:]] = 0
+    want[2, np.nonzero(E[2, :Tq] == 0)[0][:12]] = 1
+    cfg = P.VidKVConfig(B=3, L=1, max_prefill_tokens=T, max_new_tokens=2, p_ratio=0.2, out_dtype=P.VIDKV_F32)
+    K, V = make_layer_kv(wl, 0, "cuda", T=T, B=3)
+    q, k, v = (x[None] for x in make_step_inputs(wl, 0, 0, "cuda", T=T, B=3))
+    outs = []
+    for mask, stated, status in ((want, n, 0), (E, n, -1)):
+        c = P.VidKVCache(cfg)
+        c.set_token_mask(torch.from_numpy(mask).cuda(), T, n_protected=stated)
+        assert c.status() == status
+        c.quantize_keys(0, K)
+        c.quantize_values(0, V)
+        out = torch.empty((1, 3, 28, 128), dtype=torch.float32, device="cuda")
+        c.decode_attention(0, 1, q, k, v, out)
+        assert (c.get_selection(0, T)[1].cpu().numpy() == want).all()
+        outs.append(out)
+    assert torch.equal(outs[0], outs[1]) and torch.isfinite(outs[0]).all()
+    # a mask that the library was to count and refused leaves no selection behind
+    c = P.VidKVCache(cfg)
+    c.set_token_mask(torch.from_numpy(want).cuda(), T)
+    with pytest.raises(P.VidKVError):
+        c.set_token_mask(torch.from_numpy(E).cuda(), T)
+    with pytest.raises(P.VidKVError) as e:
+        c.quantize_values(0, V)
+    assert e.value.status == -5
+
+
 def test_saliency_ties_take_lower_index():
     import paper_2503_16257_b200 as P
     T = 64
