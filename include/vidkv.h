@@ -294,9 +294,10 @@ vidkv_status_t vidkv_decode_attention(vidkv_cache_t* handle, int32_t layer_begin
  * shards, each held by its own cache (its own device), because Softmax(q K^T) V over the whole
  * sequence follows from per-shard (maximum, sum, unnormalised output) triples.
  * vidkv_decode_attention_partial is vidkv_decode_attention for one shard:
- *   partial [n_layers, B, H_q, 130] float32 device: per query head the largest base-2 logit
- *           m = max_t (q . k_t) * softmax_scale * log2(e), l = sum_t 2^(logit_t - m) and
- *           o[128] = sum_t 2^(logit_t - m) v_t over the shard's tokens (packed cache + residual);
+ *   partial [n_layers, B, H_q, 130] float32 device: per query head a reference m, l = sum_t 2^(logit_t - m) and
+ *           o[128] = sum_t 2^(logit_t - m) v_t over the shard's tokens (packed cache + residual), with
+ *           logit_t = (q . k_t) * softmax_scale * log2(e).  m is within 7 of the largest logit: the maximum
+ *           that the walk over the tokens has kept, rounded up to an integer where tokens are protected;
  *   k_new, v_new: the shard that owns the newest token passes them (appended first, residual
  *           flushed when full, exactly as in vidkv_decode_attention); the other shards pass NULL
  *           for both and are attended to as they stand (STATE if such a shard holds no token).
@@ -381,7 +382,7 @@ vidkv_status_t vidkv_attend_noalloc(const vidkv_config_t* cfg, const void* cache
                                     float softmax_scale, void* stream);
 
 /* Test hooks (no counterpart in the paper; the results of a decode call do not depend on them
- * beyond floating-point summation order).  Algorithm 1 "Decoding" leaves the evaluation order of
+ * beyond floating-point summation order; the reference m of a triple does).  Algorithm 1 "Decoding" leaves the evaluation order of
  * Eq. 3 open; the library cuts a decode call into work like this: the quantized tokens of all
  * slabs of the call form one sequence of 160-token units, and every warp of the launch walks a
  * run of at most `run_units` consecutive units (crossing slab boundaries where its run does) and leaves

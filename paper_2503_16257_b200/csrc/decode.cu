@@ -15,7 +15,7 @@ constexpr int kMaxSMs = 256;        // multiprocessor count the sizing formulas 
 // Units per block up to which a call goes to the block kernel.  It has one launch, short parts and a parallel merge
 // where the stream kernel has three launches and a warp per run, but takes half as many instructions again per unit
 // (every warp of the block pays the unit's loop).  Measured (us per call, block / stream kernel): 160 units of 4 slabs
-// 15.7 / 25.8, 1184 of 16 22.9 / 36.6, 4032 of 112 (7 a block) 40.0 / 43.1, 4032 of 448 43.2 / 43.4, 4480 of 448 (8 a block) 47 / 47;
+// 15.7 / 25.8, 1184 of 16 22.9 / 36.6, 4032 of 112 (7 a block) 40.0 / 43.1, 4032 of 448 43.2 / 43.4, 4480 of 448 (8 a block) 46.5 / 42.7;
 // with protected tokens 160 of 4 21.5 / 31.0, 1152 of 64 (2 a block) 31.2 / 32.9, 1344 of 448 (3) 30.0 / 39.5, 1760 of 32 (4) 40.5 / 43.2,
 // 1568 of 224 (4) 39.9 / 39.1.  Where every unit has a warp of its own in the stream kernel, three a block are too many there
 // (1120 of 224 33.8 / 30.9), except for the general key formats (1120 of 112, 4 a block, 35.9 / 37.0).
@@ -64,9 +64,9 @@ DecodePlan plan_decode(const LayerState& st, int64_t n_slabs, bool stp, bool gen
     // With protected tokens a run pays for every slab that it enters and for the supergroup and the protected group that it
     // shares with its neighbour at a cut inside a slab.  Where a slab divides evenly into its share of the warps (at most half
     // a key group per run left over), every slab gets that many runs and none straddles two.  us per step, all warps /
-    // evenly: 112 slabs of 6400 tokens 59.5 / 59.0, of 16000 109.1 / 107.2, 168 of 9000 98.3 / 92.4, 224 of 6400 (k = 0.75)
-    // 117.4 / 112.3; uneven shares lose: 64 slabs of 12544 (4.4 units a run) 64.8 / 69.2, 112 of 12544 (7.8) 90.4 / 92.9.
-    // Without protected tokens they lose too: 112 slabs of 12819 70.3 / 77.0.
+    // evenly: 112 slabs of 6400 tokens 53.1 / 53.1, of 16000 101.0 / 101.2, 168 of 9000 93.3 / 87.0, 224 of 6400 (k = 0.75)
+    // 111.3 / 107.8; uneven shares lose (measured before the merge blocks spread, which takes 5 us off either): 64 slabs of
+    // 12544 (4.4 units a run) 64.8 / 69.2, 112 of 12544 (7.8) 90.4 / 92.9, without protected tokens 112 of 12819 70.3 / 77.0.
     const int64_t share = warps / n_slabs, groups = T_qt / kG;
     if (groups >= share * kSGGroups && groups % (share * kSGGroups) <= share / 2 && n_slabs * share * run >= p.n_units)
       runs = n_slabs * share;
@@ -136,7 +136,10 @@ size_t merge_smem_bytes(int n_pad) {
   return static_cast<size_t>(2) * n_pad * kMergeRow + sizeof(float) * 8 * n_pad + sizeof(__half) * 8 * (n_pad + 8) + 3 * 8 * sizeof(float);
 }
 
-// Shared memory asked for so that no multiprocessor takes more than its share of the n_slabs merge blocks.
+// Shared memory asked for so that no multiprocessor takes more than its share of the n_slabs merge blocks: left alone they
+// gather on the multiprocessors that the stream kernel frees first and share one path to L2 while others idle.  us a call,
+// gathered / spread: triples of 4 slabs x 600 units 125.8 / 79.8, protected 16 x 74 54.5 / 41.4, 112 x 40 57.9 / 53.7; asking
+// for 100 KB or 56 KB at most instead: 4 x 600 94.6 / 175.7.
 constexpr size_t kMaxSmem = 226 * 1024;       // a block's largest, less the kilobyte that every block costs besides
 static size_t spread_smem(size_t needed, int n_slabs) {
   const int sms = device_sm_count();

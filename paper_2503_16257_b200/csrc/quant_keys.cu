@@ -100,10 +100,8 @@ __global__ void __launch_bounds__(256, 5) k_range_kernel(KSrc src, int64_t T_tok
 
 // ---------------------------------------------------------------------------------
 // Channel selection for the general key formats (the default format's encoder does it itself).  One block of 128 threads
-// per slab.  rank(c) = number of channels
-// that come before c in (range descending, index ascending) order; the first 64 are
-// the anomalous ones.  Writes the chunk-table entry: 64 anomalous ids ascending, then
-// 64 normal ids ascending.
+// per slab.  rank(c) = number of channels that come before c in (range descending, index ascending) order; the first n2 are
+// the anomalous ones.  Writes the chunk-table entry: n2 anomalous ids ascending, then the normal ids ascending.
 // ---------------------------------------------------------------------------------
 __global__ void __launch_bounds__(kD) k_select_kernel(const uint32_t* __restrict__ minmax, CacheView cv,
                                                       int layer0, int slabs_per_layer, int chunk,
