@@ -33,7 +33,7 @@ FALLBACK_HBM_GBS = 6650.0         # earlier measurement on this machine, used if ME
 # profiles/decode_stream_stp_kernel_batched_4layers_p02.txt (p > 0): a 4-layer cut of the batched workload
 # (3 211 264 cached token-heads per launch), scaled to the launch by the token-heads it processes
 # (traffic is proportional to them).
-NCU_TRAFFIC_BYTES_PER_TOKEN_HEAD = {"decode_stream_kernel": 71.75, "decode_stream_stp_kernel": 79.28}
+NCU_TRAFFIC_BYTES_PER_TOKEN_HEAD = {"decode_stream_kernel": 71.79, "decode_stream_stp_kernel": 79.45}
 
 
 KERNEL_TIMING_STRIDE = 4
