@@ -12,7 +12,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libvidkv.so")
 SOURCES = ["host.cu", "quant_keys.cu", "quant_keys_enc.cu", "quant_keys_general.cu", "quant_values.cu", "decode.cu", "decode_prep.cu", "decode_block.cu", "decode_stream.cu", "dequant.cu", "export.cu", "noalloc.cu", "saliency.cu", "chan_metrics.cu"]
-HEADERS = ["common.cuh", "quant_common.cuh", "kernels.cuh", "decode_common.cuh", "decode_device.cuh", os.path.join("..", "..", "include", "vidkv.h")]
+HEADERS = ["common.cuh", "quant_common.cuh", "kernels.cuh", "decode_common.cuh", "decode_device.cuh", "decode_score.cuh", os.path.join("..", "..", "include", "vidkv.h")]
 
 
 def _nvcc() -> str:

@@ -49,25 +49,6 @@ __device__ __forceinline__ void cp_async16(void* smem_dst, const void* gmem_src)
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-__device__ __forceinline__ uint32_t hmul2_u(uint32_t a, uint32_t b) {
-  uint32_t d;
-  asm("mul.rn.f16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
-  return d;
-}
-// a * b + c on two binary16 lanes (one rounding)
-__device__ __forceinline__ uint32_t hfma2_u(uint32_t a, uint32_t b, uint32_t c) {
-  uint32_t d;
-  asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
-  return d;
-}
-// a * b - c on two binary16 lanes (one rounding)
-__device__ __forceinline__ uint32_t hfms2_u(uint32_t a, uint32_t b, uint32_t c) {
-  uint32_t d;
-  const __half2 x = __hfma2(*reinterpret_cast<const __half2*>(&a), *reinterpret_cast<const __half2*>(&b),
-                            __hneg2(*reinterpret_cast<const __half2*>(&c)));
-  d = *reinterpret_cast<const uint32_t*>(&x);
-  return d;
-}
 __device__ __forceinline__ uint32_t mad_u32(uint32_t a, uint32_t b, uint32_t c) {
   uint32_t d;
   asm("mad.lo.u32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
@@ -92,12 +73,6 @@ __device__ __forceinline__ uint32_t field_or(uint32_t x, uint32_t c) {
   asm("lop3.b32 %0, %1, 0x03000300, %2, 0xEA;" : "=r"(d) : "r"(x), "r"(c));
   return d;
 }
-// c with the sign of each binary16 lane flipped where that lane's bit 15 of x is 0.
-__device__ __forceinline__ uint32_t signed_by(uint32_t x, uint32_t c) {
-  uint32_t d;
-  asm("lop3.b32 %0, %1, 0x80008000, %2, 0xA6;" : "=r"(d) : "r"(x), "r"(c));
-  return d;
-}
 constexpr uint32_t kFour = 0x44004400u;   // binary16 pair (4.0, 4.0)
 
 __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
@@ -109,12 +84,10 @@ __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
 // 2^k as a float, |k| <= 126
 __device__ __forceinline__ float pow2i(int k) { return __uint_as_float(static_cast<uint32_t>(127 + k) << 23); }
 
-// Query normalisation.  The score operands q_j s_j and Q_f s_f are binary16 numbers, so a large
-// query entry times a large key scale would overflow although the score itself is an ordinary
-// float.  Every query head is therefore multiplied by the power of two 2^(-e - kQShift), e =
-// floor(log2(max_c |q_c|)), which puts its largest entry into [1/8, 1/4): no product of a scaled
-// entry (or of a spectrum coefficient, at most 16 times the largest entry) with a binary16 scale
-// below 16376 leaves the binary16 range.  Scores are linear in q, so the softmax multiplies by the
+// Query normalisation.  The query goes to the tensor cores as binary16, its transform as a leading part and a remainder.  Every query
+// head is therefore multiplied by the power of two 2^(-e - kQShift), e = floor(log2(max_c |q_c|)), which puts its largest entry into
+// [1/8, 1/4) and its largest spectrum coefficient below 4 (at most 16 times the largest entry), well inside the binary16 range.  Scores
+// are linear in q, so the softmax multiplies by the
 // inverse power of two; both factors are exact.  head_exponent returns e (0 for a head that is all
 // zero or holds no finite maximum); the NSUB lanes sub = 0..NSUB-1 share the 128 entries of the row,
 // and all 32 lanes of the warp must call it.

@@ -20,10 +20,10 @@ size_t decode_prep_bytes(int64_t n_slabs, int64_t n_chunks) {
 // ---------------------------------------------------------------------------------
 // Query preparation: one warp per (chunk, slab).  Writes, per lane, the 24 register images the
 // attention kernel needs for this chunk's channel split:
-//   words  0.. 7  binary16 pairs of q at the anomalous slots (16 r + 2 i, 16 r + 2 i + 1)
-//   words  8..15  leading binary16 part of the transformed query Q at the spectrum
-//                 columns (16 r + 2 i, 16 r + 2 i + 1)
-//   words 16..23  binary16 remainder Q - leading part
+//   words  j < 8  binary16 pairs of q at the anomalous slots (8 j + 2 r, 8 j + 2 r + 1)
+//   words  8 + j  leading binary16 part of the transformed query Q at the spectrum
+//                 columns (c, c + 1), c = 16 (j / 2) + 14 - 8 (j % 2) - 2 r
+//   words 16 + j  binary16 remainder Q - leading part
 //   word  24      float: softmax scale * log2 e * 2^(e + kQShift), which turns a score of this
 //                 normalised query into a base-2 logit
 // for head lane / 4 (zero when that head does not exist) and r = lane % 4, all of the query
@@ -60,14 +60,10 @@ __global__ void __launch_bounds__(kPrepThreads) decode_prep_kernel(DecodeArgs a,
   }
   uint32_t* out = a.prep + (static_cast<int64_t>(slab) * n_chunks + chunk) * (kPrepWords * 32) + lane;
   // anomalous slots
-  {
-    const uint4 p0 = __ldg(reinterpret_cast<const uint4*>(perm + 16 * r));
-    const uint32_t pw[4] = {p0.x, p0.y, p0.z, p0.w};
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const uint32_t two = pw[i >> 1] >> (16 * (i & 1));
-      out[i * 32] = pack_half2(q_at(two & 0xffu), q_at((two >> 8) & 0xffu));
-    }
+  for (int j = 0; j < 8; ++j) {
+    const uint32_t two = __ldg(reinterpret_cast<const uint16_t*>(perm + 8 * j + 2 * r));
+    out[j * 32] = pack_half2(q_at(two & 0xffu), q_at(two >> 8));
   }
   // transformed query: A = q at the normal channels (rows 8-15 unused), B = matrix fragments
   uint32_t af[4][2];
@@ -90,14 +86,16 @@ __global__ void __launch_bounds__(kPrepThreads) decode_prep_kernel(DecodeArgs a,
       mma_f16(acc[nt], af[ks][0], 0u, af[ks][1], 0u, bw.z, bw.w);
     }
   }
-  // lane (hd, r) now holds Q of head hd at columns 16 r + 2 nt + {0, 1}
+  // lane (hd, r) now holds Q of head hd at columns 16 r + 2 nt + {0, 1}: word 2 r + (nt < 4) of lane (hd, 3 - nt % 4)
+  uint32_t* outQ = out + (8 + 2 * r) * 32 + 3 - r;
 #pragma unroll
   for (int nt = 0; nt < 8; ++nt) {
     const float w0 = (r == 0 && nt == 0) ? 1.0f : 2.0f;            // columns 0 and 1 are not doubled
     const float x0 = acc[nt][0] * w0, x1 = acc[nt][1] * w0;
     const __half h0 = __float2half_rn(x0), h1 = __float2half_rn(x1);
-    out[(8 + nt) * 32] = pack_half2(__half2float(h0), __half2float(h1));
-    out[(16 + nt) * 32] = pack_half2(x0 - __half2float(h0), x1 - __half2float(h1));
+    uint32_t* o = outQ + (nt < 4 ? 32 : 0) - (nt & 3);
+    o[0] = pack_half2(__half2float(h0), __half2float(h1));
+    o[8 * 32] = pack_half2(x0 - __half2float(h0), x1 - __half2float(h1));
   }
   // factor that turns a score in the normalised units into a base-2 logit
   out[24 * 32] = __float_as_uint(a.scale * 1.4426950408889634f * pow2i(qe + kQShift));
@@ -106,8 +104,8 @@ __global__ void __launch_bounds__(kPrepThreads) decode_prep_kernel(DecodeArgs a,
 // ---------------------------------------------------------------------------------
 // The same for the general key formats (KeyFmt): one warp per (chunk, slab); per lane (head hd = lane / 4,
 // r = lane % 4), all of the normalised query:
-//   words 0 .. n2/8 - 1         binary16 pairs of q at the two-bit slots 32 (w / 4) + 8 r + 2 (w % 4), + 1
-//   then n1/8 words             plain mode: pairs of q at the one-bit channels with the same index rule;
+//   words w < n2/8              binary16 pairs of q at the two-bit slots 8 w + 2 r, + 1
+//   then n1/8 words             plain mode: pairs of q at the one-bit channels 8 w + 6 - 2 r, + 1;
 //                               Eq. 5: leading binary16 part of the transformed query Q at those columns,
 //   then (Eq. 5) n1/8 words     binary16 remainder Q - leading part
 //   word 24                     the factor that turns a score into a base-2 logit
@@ -141,13 +139,13 @@ __global__ void __launch_bounds__(kPrepThreads) decode_prep_general_kernel(Decod
   }
   uint32_t* out = a.prep + (static_cast<int64_t>(slab) * n_chunks + chunk) * (kPrepWords * 32) + lane;
   for (int w = 0; w < n2 / 8; ++w) {
-    const int j = 32 * (w >> 2) + 8 * r + 2 * (w & 3);
+    const int j = 8 * w + 2 * r;
     out[w * 32] = pack_half2(q_at(perm[j]), q_at(perm[j + 1]));
   }
   const int w1 = n2 / 8;
   if (cv.kf.plain) {
     for (int w = 0; w < n1 / 8; ++w) {
-      const int i = 32 * (w >> 2) + 8 * r + 2 * (w & 3);
+      const int i = 8 * w + 6 - 2 * r;
       out[(w1 + w) * 32] = pack_half2(q_at(perm[n2 + i]), q_at(perm[n2 + i + 1]));
     }
   } else {
@@ -161,11 +159,12 @@ __global__ void __launch_bounds__(kPrepThreads) decode_prep_general_kernel(Decod
       x[0] = fmaf(qv, wa.x, x[0]); x[1] = fmaf(qv, wa.y, x[1]); x[2] = fmaf(qv, wa.z, x[2]); x[3] = fmaf(qv, wa.w, x[3]);
       x[4] = fmaf(qv, wb.x, x[4]); x[5] = fmaf(qv, wb.y, x[5]); x[6] = fmaf(qv, wb.z, x[6]); x[7] = fmaf(qv, wb.w, x[7]);
     }
+    uint32_t* outQ = out + (w1 + r) * 32 + 3 - r;            // columns 8 r + 2 w, + 1: word r of lane (hd, 3 - w)
 #pragma unroll
     for (int w = 0; w < 4; ++w) {
       const __half h0 = __float2half_rn(x[2 * w]), h1 = __float2half_rn(x[2 * w + 1]);
-      out[(w1 + w) * 32] = pack_half2(__half2float(h0), __half2float(h1));
-      out[(w1 + 4 + w) * 32] = pack_half2(x[2 * w] - __half2float(h0), x[2 * w + 1] - __half2float(h1));
+      outQ[-w] = pack_half2(__half2float(h0), __half2float(h1));
+      outQ[4 * 32 - w] = pack_half2(x[2 * w] - __half2float(h0), x[2 * w + 1] - __half2float(h1));
     }
   }
   out[24 * 32] = __float_as_uint(a.scale * 1.4426950408889634f * pow2i(qe + kQShift));

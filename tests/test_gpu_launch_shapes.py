@@ -357,3 +357,19 @@ def test_flushes_after_a_prompt_with_nothing_to_quantize(T):
                 assert np.abs(again[0, 0].cpu().numpy().astype(np.float64) - r2).max() <= TOL_ABS
     assert cache.layer_state(0) == dict(n_quantized=256, n_residual=T + steps - 256, n_chunks=2, n_protected=0)
     assert cache.status() == 0
+
+
+@pytest.mark.parametrize("run_units", [0, 1, 3])
+@pytest.mark.parametrize("T,p,steps", [(352, 0.0, 2), (416, 0.2, 2), (1664, 0.3, 130)])
+def test_cache_memory_that_nobody_has_written_does_not_count(run_units, T, p, steps):
+    """Cache memory full of NaN patterns before the prompt: the last unit of a slab, the last supergroup of a ternary
+    stream and (a flush later) its gap have groups that do not exist, whose codes and scales nobody has written."""
+    pair = Pair(CONFIGS["tiny"], T, B=1, L=1, p=p, max_new=steps)
+    pair.cache.cache[256:] = 255                             # all but the header
+    pair.prefill()
+    pair.cache.debug_set_decode_plan(run_units=run_units)
+    for s in range(steps):
+        out, ref = pair.decode()
+        if s < 2 or s >= 126:
+            assert np.abs(out - ref).max() <= TOL_ABS, s
+    assert pair.cache.status() == 0
