@@ -176,34 +176,12 @@ __global__ void __launch_bounds__(kD) decode_merge_kernel(DecodeArgs a, int n_re
     }
   }
   const float* rec = a.partials + (slab + first_run) * (kMaxRep * kRecordFloats);
-  pdl_wait();                                              // the partial records come from the attention kernel before
   const int64_t q0 = (static_cast<int64_t>(lb) * cv.H_q + h * rep) * kD;
-  // ---- the records' maxima and sums (lane j: record j, for the heads warp and warp + 4) and this lane's output fragments
-  // of the first kRecAhead records are fetched first, so that their latency passes behind the residual
-  float2 head_ml[2];
-#pragma unroll
-  for (int x = 0; x < 2; ++x) {
-    const int k = warp + 4 * x;
-    head_ml[x] = make_float2(-INFINITY, 0.0f);
-    if (k < rep && lane < n_parts) head_ml[x] = __ldg(reinterpret_cast<const float2*>(rec + (lane * kMaxRep + k) * kRecordFloats));
-  }
-  constexpr int kRecAhead = 3;
-  float rec_m[kRecAhead];
-  float2 rec_o[kRecAhead][4];
-#pragma unroll
-  for (int jp = 0; jp < kRecAhead; ++jp) {
-    rec_m[jp] = -INFINITY;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) rec_o[jp][j] = make_float2(0.0f, 0.0f);
-    if (jp < n_parts && hd < rep) {
-      const float* pr = rec + (jp * kMaxRep + hd) * kRecordFloats;
-      rec_m[jp] = __ldg(pr);
-#pragma unroll
-      for (int j = 0; j < 4; ++j) rec_o[jp][j] = __ldg(reinterpret_cast<const float2*>(pr + 2 + 32 * warp + 8 * j + 2 * r));
-    }
-  }
   if (n_pad > 0) {
-    // ---- stage the residual rows (16-byte pieces, all loads of a thread independent)
+    // ---- stage the residual rows (16-byte pieces, all loads of a thread independent).  Up to the records nothing here comes from the
+    // attention kernel before, so it goes on while that kernel's last blocks still run: the rows, the appended one among them, are
+    // older than the preparation kernel, for which that kernel waited before it let this one start.  (Behind the wait the residual took
+    // 3-5 us of a step.)
     const uint4* ksrc = reinterpret_cast<const uint4*>(slab_ptr + cv.kres_offset);
     const uint4* vsrc = reinterpret_cast<const uint4*>(slab_ptr + cv.vres_offset);
     constexpr bool kConvert = !std::is_same<T, __half>::value;          // bfloat16 values -> binary16 (exact for the admitted inputs)
@@ -252,40 +230,23 @@ __global__ void __launch_bounds__(kD) decode_merge_kernel(DecodeArgs a, int n_re
     }
     __syncthreads();
   }
-  // ---- maxima and denominators: warp w takes heads w and w + 4
+  // ---- the residual's maxima and probabilities: warp w takes heads w and w + 4
+  float m_res[2], l_res[2];
 #pragma unroll
   for (int x = 0; x < 2; ++x) {
     const int k = warp + 4 * x;
-    float m = head_ml[x].x, m_res = -INFINITY;
-    if (k < rep) {
-      for (int t = lane; t < n_res; t += 32) m_res = fmaxf(m_res, S[k * n_pad + t]);
-      for (int j = lane + 32; j < n_parts; j += 32) m = fmaxf(m, __ldg(rec + (j * kMaxRep + k) * kRecordFloats));
-    }
+    m_res[x] = -INFINITY;
+    if (k < rep)
+      for (int t = lane; t < n_res; t += 32) m_res[x] = fmaxf(m_res[x], S[k * n_pad + t]);
 #pragma unroll
-    for (int o = 16; o; o >>= 1) {
-      m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-      m_res = fmaxf(m_res, __shfl_xor_sync(0xffffffffu, m_res, o));
-    }
-    m = fmaxf(m, m_res);
-    const float w_res = k < rep && n_res > 0 ? exp2f(m_res - m) : 0.0f;
-    float l = 0.0f;
+    for (int o = 16; o; o >>= 1) m_res[x] = fmaxf(m_res[x], __shfl_xor_sync(0xffffffffu, m_res[x], o));
+    l_res[x] = 0.0f;                                       // this lane's tokens
     for (int t = lane; t < n_pad; t += 32) {
       __half ph = __float2half_rn(0.0f);
-      if (k < rep && t < n_res) ph = __float2half_rn(exp2f(S[k * n_pad + t] - m_res));
+      if (k < rep && t < n_res) ph = __float2half_rn(exp2f(S[k * n_pad + t] - m_res[x]));
       Ph[k * PS + t] = ph;
-      l += __half2float(ph);
+      l_res[x] += __half2float(ph);
     }
-    l *= w_res;
-    if (k < rep) {
-      l += head_ml[x].y * exp2f(head_ml[x].x - m);          // 0 for a record that does not exist
-      for (int j = lane + 32; j < n_parts; j += 32) {
-        const float* pr = rec + (j * kMaxRep + k) * kRecordFloats;
-        l += pr[1] * exp2f(pr[0] - m);
-      }
-    }
-#pragma unroll
-    for (int o = 16; o; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
-    if (lane == 0) { Mh[k] = m; Lh[k] = l; Wh[k] = w_res; }
   }
   __syncthreads();
   // ---- P V_r: warp w owns channels 32 w .. 32 w + 31 as four 8-channel tiles
@@ -303,6 +264,55 @@ __global__ void __launch_bounds__(kD) decode_merge_kernel(DecodeArgs a, int n_re
       mma_f16(acc[j], a0, 0u, a2, 0u, b0, b1);
     }
   }
+  // ---- the records: maxima and sums (lane j: record j, for the heads warp and warp + 4) and this lane's output fragments
+  // of the first kRecAhead of them in one round of loads
+  pdl_wait();
+  float2 head_ml[2];
+#pragma unroll
+  for (int x = 0; x < 2; ++x) {
+    const int k = warp + 4 * x;
+    head_ml[x] = make_float2(-INFINITY, 0.0f);
+    if (k < rep && lane < n_parts) head_ml[x] = __ldg(reinterpret_cast<const float2*>(rec + (lane * kMaxRep + k) * kRecordFloats));
+  }
+  constexpr int kRecAhead = 3;
+  float rec_m[kRecAhead];
+  float2 rec_o[kRecAhead][4];
+#pragma unroll
+  for (int jp = 0; jp < kRecAhead; ++jp) {
+    rec_m[jp] = -INFINITY;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) rec_o[jp][j] = make_float2(0.0f, 0.0f);
+    if (jp < n_parts && hd < rep) {
+      const float* pr = rec + (jp * kMaxRep + hd) * kRecordFloats;
+      rec_m[jp] = __ldg(pr);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) rec_o[jp][j] = __ldg(reinterpret_cast<const float2*>(pr + 2 + 32 * warp + 8 * j + 2 * r));
+    }
+  }
+  // ---- maxima and denominators over all parts
+#pragma unroll
+  for (int x = 0; x < 2; ++x) {
+    const int k = warp + 4 * x;
+    float m = head_ml[x].x;
+    if (k < rep)
+      for (int j = lane + 32; j < n_parts; j += 32) m = fmaxf(m, __ldg(rec + (j * kMaxRep + k) * kRecordFloats));
+#pragma unroll
+    for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    m = fmaxf(m, m_res[x]);
+    const float w_res = k < rep && n_res > 0 ? exp2f(m_res[x] - m) : 0.0f;
+    float l = l_res[x] * w_res;
+    if (k < rep) {
+      l += head_ml[x].y * exp2f(head_ml[x].x - m);          // 0 for a record that does not exist
+      for (int j = lane + 32; j < n_parts; j += 32) {
+        const float* pr = rec + (j * kMaxRep + k) * kRecordFloats;
+        l += pr[1] * exp2f(pr[0] - m);
+      }
+    }
+#pragma unroll
+    for (int o = 16; o; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+    if (lane == 0) { Mh[k] = m; Lh[k] = l; Wh[k] = w_res; }
+  }
+  __syncthreads();
   // ---- join the records: lane (hd, r) holds head hd, channels 32 w + 8 j + 2 r, + 1
   if (hd < rep) {
     const float M = Mh[hd], inv = 1.0f / Lh[hd], w_res = Wh[hd];
