@@ -169,21 +169,34 @@ __device__ __forceinline__ void make_images(uint32_t* img, const ImageSource& sr
     }
   } else {
     const int n2 = kf.n2, n1 = kD - n2, w1 = n2 / 8, n_pairs = kf.plain ? kD / 8 : w1;
-#pragma unroll 1
-    for (int w = warp; w < n_pairs; w += kUnitWarps) {
-      const int j = w < w1 ? 8 * w + 2 * r : n2 + 8 * (w - w1) + 6 - 2 * r;
-      put(w, lane, pack_half2(q_at(perm[j]), q_at(perm[j + 1])));
+    constexpr int kTurns = (16 + kUnitWarps - 1) / kUnitWarps;
+    uint32_t two[kTurns];
+#pragma unroll
+    for (int turn = 0; turn < kTurns; ++turn) {
+      const int w = warp + turn * kUnitWarps;
+      two[turn] = w < n_pairs ? __ldg(reinterpret_cast<const uint16_t*>(perm + (w < w1 ? 8 * w + 2 * r : 8 * w + 6 - 2 * r))) : 0u;
+    }
+#pragma unroll
+    for (int turn = 0; turn < kTurns; ++turn) {
+      const int w = warp + turn * kUnitWarps;
+      if (w < n_pairs) put(w, lane, pack_half2(q_at(two[turn] & 0xffu), q_at(two[turn] >> 8)));
     }
     if (!kf.plain && n1 > 0 && warp == kUnitWarps - 1) {
-      // n1 = 32: lane r owns the columns 8 r .. 8 r + 7
-      float x[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+      // n1 = 32: lane r owns the columns 8 r .. 8 r + 7; sums of eight channels each, added in the order of decode_prep_general_kernel
+      float x[8];
       const float4* wt = reinterpret_cast<const float4*>(dft.w32) + 2 * r;
-#pragma unroll 4
-      for (int c = 0; c < 32; ++c) {
-        const float qv = q_at(perm[n2 + c]);
-        const float4 wa = __ldg(wt + 8 * c), wb = __ldg(wt + 8 * c + 1);
-        x[0] = fmaf(qv, wa.x, x[0]); x[1] = fmaf(qv, wa.y, x[1]); x[2] = fmaf(qv, wa.z, x[2]); x[3] = fmaf(qv, wa.w, x[3]);
-        x[4] = fmaf(qv, wb.x, x[4]); x[5] = fmaf(qv, wb.y, x[5]); x[6] = fmaf(qv, wb.z, x[6]); x[7] = fmaf(qv, wb.w, x[7]);
+#pragma unroll 1
+      for (int part = 0; part < 4; ++part) {
+        float y[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll
+        for (int c = 8 * part, i = 0; i < 8; ++c, ++i) {
+          const float qv = q_at(perm[n2 + c]);
+          const float4 wa = __ldg(wt + 8 * c), wb = __ldg(wt + 8 * c + 1);
+          y[0] = fmaf(qv, wa.x, y[0]); y[1] = fmaf(qv, wa.y, y[1]); y[2] = fmaf(qv, wa.z, y[2]); y[3] = fmaf(qv, wa.w, y[3]);
+          y[4] = fmaf(qv, wb.x, y[4]); y[5] = fmaf(qv, wb.y, y[5]); y[6] = fmaf(qv, wb.z, y[6]); y[7] = fmaf(qv, wb.w, y[7]);
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) x[i] = part == 0 ? y[i] : x[i] + y[i];
       }
 #pragma unroll
       for (int w = 0; w < 4; ++w) {
