@@ -183,7 +183,7 @@ __device__ __forceinline__ void scale_output(float* totbuf, float fa, float fb, 
   }
 }
 
-// P V of one staged ternary supergroup of ng groups (FULL: five; the others' probabilities are zero): for its groups, P[g][nt] holds the probabilities of
+// P V of one staged ternary supergroup, its first ng groups (FULL: five; the others' probabilities are zero): P[g][nt] holds the probabilities of
 // head hd at stream tokens 32 g + 8 nt + 2 r, + 1 (binary16 pairs) and ps[g] the accumulator
 // fragment -5 * (sum of those probabilities) of heads 2 r, 2 r + 1.  32 channels (two MMA row
 // blocks) at a time: fragment i of block w covers channels 32 w + 4 hd + 2 i + {0, 1} in rows hd,
@@ -531,8 +531,7 @@ __global__ void __launch_bounds__(kStreamWarps * 32, kStreamStpCtasPerSM) decode
   const int64_t u_begin = pl.run_begin(run_id);
   const int64_t u_end = run_id < pl.n_runs ? pl.run_begin(run_id + 1) : u_begin;
   if (u_begin >= u_end) return;
-  const KeyFmt& kf = a.cv.kf;
-  const int kgb = GEN ? kf.group_bytes : kKGroupBytes;
+  const int kgb = GEN ? cv.kf.group_bytes : kKGroupBytes;
   constexpr int kbuf_bytes = GEN ? kGenKBufBytes : kKBufBytes;
   uint8_t* kbuf = smem_raw + warp * (kStpWarpBytes - kKBufBytes + kbuf_bytes);
   uint8_t* vbuf = kbuf + kbuf_bytes;
@@ -555,21 +554,16 @@ __global__ void __launch_bounds__(kStreamWarps * 32, kStreamStpCtasPerSM) decode
   const int T_q0 = static_cast<int>(a.st.T_q0), T_qt = T_q0 + static_cast<int>(a.st.n_flush) * kR;
   const int n_groups = T_qt / kG;
   const int n_prot = static_cast<int>(a.n_prot), n_rest = T_q0 - n_prot;
-  const int u_fl0 = (n_rest + kG - 1) / kG * kG;                                          // flushed tokens start here
-  const int tg_total = (n_rest + kG - 1) / kG + (kR / kG) * static_cast<int>(a.st.n_flush);   // ternary groups that exist
-  const int sg_total = (tg_total + kSGGroups - 1) / kSGGroups;
-  const int pg_total = (n_prot + kG - 1) / kG;
-  const uint8_t* slab0 = cv.base + cv.slab_offset + static_cast<int64_t>(a.layer0) * cv.B * cv.H_kv * cv.slab_stride;
+  const int u_fl0 = (n_rest + kG - 1) / kG * kG;            // stream position where the flushed tokens start
   int slab = static_cast<int>(u_begin / S);
   int k = static_cast<int>(u_begin - static_cast<int64_t>(slab) * S);
-  auto groups_of = [&](int kk) -> int {
-    const int left = n_groups - kk * kSGGroups;
-    return left < kSGGroups ? left : kSGGroups;
+  const uint8_t* slab_ptr = cv.base + cv.slab_offset + (static_cast<int64_t>(a.layer0) * cv.B * cv.H_kv + slab) * cv.slab_stride;
+  auto load_keys = [&](const uint8_t* slab_at, int kk) {    // one lane
+    bulk_load(kbuf, slab_at + cv.kgroup_offset + static_cast<int64_t>(kk) * (kSGGroups * kgb), min(kSGGroups, n_groups - kk * kSGGroups) * kgb, kbar);
   };
-  auto key_src = [&](int sl, int kk) -> const uint8_t* {
-    return slab0 + static_cast<int64_t>(sl) * cv.slab_stride + cv.kgroup_offset + static_cast<int64_t>(kk) * (kSGGroups * kgb);
-  };
-  if (lane == 0) bulk_load(kbuf, key_src(slab, k), groups_of(k) * kgb, kbar);
+  auto load_supergroup = [&](int sg) { bulk_load(vbuf, slab_ptr + cv.tern_offset + static_cast<int64_t>(sg) * kVBufBytes, kVBufBytes, vbar); };
+  auto load_protected = [&](int pg) { bulk_load(pbuf, slab_ptr + cv.prot_offset + static_cast<int64_t>(pg) * kPGBytes, kPGBytes, pbar); };
+  if (lane == 0) load_keys(slab_ptr, k);
   pdl_wait();                                              // the prepared query (and nothing else so far) comes from the kernel before
   pdl_release();
   const uint32_t lt_mask = (1u << lane) - 1u;              // lanes (= tokens of a group) before this one
@@ -578,49 +572,48 @@ __global__ void __launch_bounds__(kStreamWarps * 32, kStreamStpCtasPerSM) decode
   Running run;
   run.reset();
   Query<GEN> qy;
-  int cur_chunk = -1, cur_slab = -1;
+  int cur_chunk = -1;
   const uint32_t* ew = nullptr;
   const uint32_t* ep = nullptr;
-  const uint8_t* slab_ptr = nullptr;
-  int sg_next = 0, pg_next = 0;
+  // the part of the slab's value streams that the run's units fill ends before supergroup sg_end and protected group pg_end: nothing is
+  // fetched for a neighbour
+  int sg_next = 0, pg_next = 0, sg_end = 0, pg_end = 0;
   float sl2[2] = {0.0f, 0.0f};
-  bool ok = true;
+  bool ok = true, entering = true;
 #pragma unroll 1
-  for (int64_t u = u_begin; u < u_end && ok; ++u) {
+  for (int left = static_cast<int>(u_end - u_begin); left > 0; --left) {
     const int t_unit = k * kStreamUnitTokens;
-    if (slab != cur_slab) {
-      if (cur_slab >= 0) write_record(a, cur_slab, run_id, lane, hd, r, run, totbuf);
-      cur_slab = slab;
+    if (entering) {
       cur_chunk = -1;
-      slab_ptr = slab0 + static_cast<int64_t>(slab) * cv.slab_stride;
       const int b = (slab / cv.H_kv) % cv.B;
       ew = cv.e_words(b);
       ep = cv.e_prefix(b);
+      // where the run enters and leaves the two value streams
+      auto streams_at = [&](int t, int& u, int& p) {
+        if (t <= T_q0) { p = static_cast<int>(__ldg(ep + t / kG)); u = t - p; }
+        else { p = n_prot; u = u_fl0 + (t - T_q0); }
+      };
+      int t_begin, p_begin, t_stop, p_stop;
+      streams_at(t_unit, t_begin, p_begin);
+      streams_at(left < S - k ? (k + left) * kStreamUnitTokens : T_qt, t_stop, p_stop);
+      sg_next = t_begin / kStreamUnitTokens; sg_end = (t_stop + kStreamUnitTokens - 1) / kStreamUnitTokens;
+      pg_next = p_begin / kG; pg_end = (p_stop + kG - 1) / kG;
       // zero the running output and both rings
       for (int i = lane; i < (kTotBytes + kRingBytes) / 16; i += 32)
         reinterpret_cast<uint4*>(totbuf)[i] = make_uint4(0u, 0u, 0u, 0u);
       run.reset();
       head_factors(prep_words(a, slab, lane), lane, r, sl2);
-      // where the run enters the two value streams
-      int pp0, uu0;
-      if (t_unit <= T_q0) { pp0 = static_cast<int>(__ldg(ep + t_unit / kG)); uu0 = t_unit - pp0; }
-      else { pp0 = n_prot; uu0 = u_fl0 + (t_unit - T_q0); }
-      sg_next = uu0 / kStreamUnitTokens;
-      pg_next = pp0 / kG;
       __syncwarp();
+      v_pending = sg_next < sg_end;
+      p_pending = pg_next < pg_end;
       if (lane == 0) {
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        if (sg_next < sg_total) bulk_load(vbuf, slab_ptr + cv.tern_offset + static_cast<int64_t>(sg_next) * kVBufBytes, kVBufBytes, vbar);
-        if (pg_next < pg_total) bulk_load(pbuf, slab_ptr + cv.prot_offset + static_cast<int64_t>(pg_next) * kPGBytes, kPGBytes, pbar);
+        if (v_pending) load_supergroup(sg_next);
+        if (p_pending) load_protected(pg_next);
       }
-      v_pending = sg_next < sg_total;
-      p_pending = pg_next < pg_total;
     }
-    const int ng = groups_of(k);
-    int nslab = slab, nk = k + 1;
-    if (nk == S) { nk = 0; ++nslab; }
-    const bool more = u + 1 < u_end;
-    const bool last_of_slab = !more || nslab != slab;      // the run leaves this slab after this unit
+    const int ng = min(kSGGroups, n_groups - k * kSGGroups);
+    const bool last = k + 1 == S, more = left > 1, last_of_slab = !more || last;   // the run leaves this slab after this unit
     // the E words and prefix counts of the unit's groups (lane g: group g; lane ng: the prefix count at the
     // unit's end) are fetched now and picked up with shuffles after the scores, their latency hidden behind them
     uint32_t e_word_l = 0u;
@@ -661,6 +654,8 @@ __global__ void __launch_bounds__(kStreamWarps * 32, kStreamStpCtasPerSM) decode
     // ---- probabilities, scattered into stream order.  Where a token goes depends on the token
     // alone, so lane j works out the entry of the group's token j and the lanes pick up the entries of
     // their own four tokens with shuffles.
+    const int base0 = __shfl_sync(0xffffffffu, e_base_l, 0);   // protected tokens before the unit
+    const int t_at = (t_unit - base0) % kTRing, p_at = base0 % kPRing;
 #pragma unroll 1
     for (int g = 0; g < ng; ++g) {
       uint32_t P[4];
@@ -671,7 +666,10 @@ __global__ void __launch_bounds__(kStreamWarps * 32, kStreamStpCtasPerSM) decode
       if (tg < T_q0) {
         const int below = __popc(word & lt_mask);
         const bool prot = (word >> lane) & 1u;
-        const int dst = (prot ? kTRing + (base + below) % kPRing : (tg - base + lane - below) % kTRing) * kEntry;
+        int at = prot ? p_at + (base - base0) + below : t_at + g * kG - (base - base0) + lane - below;   // less than one turn ahead
+        const int turn = prot ? kPRing : kTRing;
+        at -= at >= turn ? turn : 0;
+        const int dst = (prot ? kTRing + at : at) * kEntry;
 #pragma unroll
         for (int nt = 0; nt < 4; ++nt) *reinterpret_cast<uint32_t*>(rings + __shfl_sync(0xffffffffu, dst, 8 * nt + hd) + 4 * r) = P[nt];
       } else {
@@ -684,7 +682,7 @@ __global__ void __launch_bounds__(kStreamWarps * 32, kStreamStpCtasPerSM) decode
     __syncwarp();
     if (more && lane == 0) {
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      bulk_load(kbuf, key_src(nslab, nk), groups_of(nk) * kgb, kbar);
+      load_keys(slab_ptr + (last ? cv.slab_stride : 0), last ? 0 : k + 1);
     }
     // ---- how far the two streams are complete now
     const int t_end = t_unit + ng * kG;
@@ -693,13 +691,12 @@ __global__ void __launch_bounds__(kStreamWarps * 32, kStreamStpCtasPerSM) decode
     else { pp_hi = n_prot; u_hi = u_fl0 + (t_end - T_q0); }
     if (last_of_slab) {
       // what is left of the last supergroup / group belongs to a neighbour (or to nobody): zeros
-      const int sg_end = (u_hi + kStreamUnitTokens - 1) / kStreamUnitTokens * kStreamUnitTokens;
-      zero_ring_range(rings, kTRing, u_hi, sg_end, lane);
-      zero_ring_range(rings + kTRing * kEntry, kPRing, pp_hi, (pp_hi + kG - 1) / kG * kG, lane);
+      zero_ring_range(rings, kTRing, u_hi, sg_end * kStreamUnitTokens, lane);
+      zero_ring_range(rings + kTRing * kEntry, kPRing, pp_hi, pg_end * kG, lane);
       __syncwarp();
     }
     // ---- ternary supergroups whose positions are all written
-    while (ok && (last_of_slab ? sg_next * kStreamUnitTokens < u_hi : (sg_next + 1) * kStreamUnitTokens <= u_hi)) {
+    while (last_of_slab ? sg_next < sg_end : (sg_next + 1) * kStreamUnitTokens <= u_hi) {
       if (!mbar_wait(vbar, vpar)) { ok = false; break; }
       vpar ^= 1u;
       v_pending = false;
@@ -715,19 +712,20 @@ __global__ void __launch_bounds__(kStreamWarps * 32, kStreamStpCtasPerSM) decode
         run.l[0] = fmaf(-0.2f, ps[g][0], run.l[0]);
         run.l[1] = fmaf(-0.2f, ps[g][1], run.l[1]);
       }
-      pv_ternary<false, false>(vbuf, totbuf, tg_total - sg_next * kSGGroups, P, ps, 1.0f, 1.0f, lane, hd, r);
+      // groups without positions of this run may not exist.  (Leaving their products out, and those before the run's first position, takes
+      // branches between the groups: 848 -> 926 us a step of 16 users, 47.3 -> 49.4 of one clip.)
+      const int n_used = last_of_slab ? (u_hi - sg_next * kStreamUnitTokens + kG - 1) / kG : kSGGroups;
+      pv_ternary<false, false>(vbuf, totbuf, n_used, P, ps, 1.0f, 1.0f, lane, hd, r);
       ++sg_next;
       __syncwarp();
-      if (sg_next < sg_total) {
-        if (lane == 0) {
-          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-          bulk_load(vbuf, slab_ptr + cv.tern_offset + static_cast<int64_t>(sg_next) * kVBufBytes, kVBufBytes, vbar);
-        }
-        v_pending = true;
+      v_pending = sg_next < sg_end;
+      if (v_pending && lane == 0) {
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        load_supergroup(sg_next);
       }
     }
     // ---- protected groups whose positions are all written
-    while (ok && (last_of_slab ? pg_next * kG < pp_hi : (pg_next + 1) * kG <= pp_hi)) {
+    while (ok && (last_of_slab ? pg_next < pg_end : (pg_next + 1) * kG <= pp_hi)) {
       if (!mbar_wait(pbar, ppar)) { ok = false; break; }
       ppar ^= 1u;
       p_pending = false;
@@ -736,20 +734,21 @@ __global__ void __launch_bounds__(kStreamWarps * 32, kStreamStpCtasPerSM) decode
       pv_protected(pbuf, totbuf, P4, run.l, lane, hd, r);
       ++pg_next;
       __syncwarp();
-      if (pg_next < pg_total) {
-        if (lane == 0) {
-          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-          bulk_load(pbuf, slab_ptr + cv.prot_offset + static_cast<int64_t>(pg_next) * kPGBytes, kPGBytes, pbar);
-        }
-        p_pending = true;
+      p_pending = pg_next < pg_end;
+      if (p_pending && lane == 0) {
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        load_protected(pg_next);
       }
     }
-    if (last_of_slab && ok) {
-      // copies fetched ahead for a neighbour's part of the streams: let them land, the buffers are reused
-      if (v_pending) { ok = mbar_wait(vbar, vpar); vpar ^= 1u; v_pending = false; }
-      if (ok && p_pending) { ok = mbar_wait(pbar, ppar); ppar ^= 1u; p_pending = false; }
+    if (!ok) break;
+    entering = last;
+    if (last_of_slab) write_record(a, slab, run_id, lane, hd, r, run, totbuf);
+    ++k;
+    if (last) {
+      k = 0;
+      ++slab;
+      slab_ptr += cv.slab_stride;
     }
-    slab = nslab; k = nk;
   }
   if (!ok) {
     // a copy never arrived: report it, and let the others that are in flight land before the warp leaves
@@ -757,9 +756,7 @@ __global__ void __launch_bounds__(kStreamWarps * 32, kStreamStpCtasPerSM) decode
     if (k_pending) mbar_wait(kbar, kpar);
     if (v_pending) mbar_wait(vbar, vpar);
     if (p_pending) mbar_wait(pbar, ppar);
-    return;
   }
-  write_record(a, cur_slab, run_id, lane, hd, r, run, totbuf);
 }
 
 cudaError_t launch_decode_stream_stp(const DecodeArgs& a, cudaStream_t stream) {
