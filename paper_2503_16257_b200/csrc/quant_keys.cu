@@ -150,7 +150,11 @@ static cudaError_t launch_keys_t(const KSrc& src, int64_t T_tokens, int n_res, c
   const int n_slabs = slabs_per_layer * n_layers;
   if (T_tokens <= 0 || n_slabs <= 0) return cudaSuccess;
   cudaError_t e;
+  // Tokens a block: 512, fewer where that leaves multiprocessors without two blocks (the pass is latency then: 4 slabs of 6307 tokens
+  // in 52 blocks, four rounds of loads each, 6.2 us).
   int tokens_per_block = 512;
+  const int64_t enough = 2 * device_sm_count();
+  while (tokens_per_block > 64 && (T_tokens + tokens_per_block - 1) / tokens_per_block * n_slabs < enough) tokens_per_block /= 2;
   const int64_t splits = (T_tokens + tokens_per_block - 1) / tokens_per_block;
   if ((e = launch_dependent(k_range_kernel<T>, dim3(static_cast<unsigned>(splits + (n_res > 0)), n_slabs), dim3(256), 0, stream, src,
                             T_tokens, tokens_per_block, static_cast<int>(splits), n_res, cv, layer0, minmax, counters, n_counters)))

@@ -323,6 +323,13 @@ __global__ void __launch_bounds__(kEncThreads, 2) k_encode_kernel(KSrc src, int6
   // memory, operand A is built and the half's accumulators of the tile before have been read (one arrival per warp).
   // Every wait is bounded; whoever runs out of patience sets the fault flag and waits and arrives no more.
   if (loader && tile_begin < tile_end) { load_next(0); load_next(1); }   // the keys are complete: the range pass has waited for them
+  constexpr int kAVec = (32768 + 16384 * (Enc<T>::kParts - 1)) / 16;
+  auto clear_operand = [&]() {
+#pragma unroll 4
+    for (int i = tid; i < kAVec; i += 256) reinterpret_cast<uint4*>(a_ex)[i] = make_uint4(0u, 0u, 0u, 0u);
+  };
+  bool cleared = true;                                       // operand A, for the block's first slab while the ranges still come in
+  if (warp != 8) clear_operand();
   pdl_wait();                                                // the ranges
   if (warp == 8) {
     uint32_t parity = 0;
@@ -415,9 +422,8 @@ __global__ void __launch_bounds__(kEncThreads, 2) k_encode_kernel(KSrc src, int6
           if (ti == 0) slab_ptr[cv.chunk_table_offset + static_cast<int64_t>(chunk) * kChunkBytes + at] = static_cast<uint8_t>(c);
         }
       }
-      constexpr int kAVec = (32768 + 16384 * (Enc<T>::kParts - 1)) / 16;
-#pragma unroll 4
-      for (int i = tid; i < kAVec; i += 256) reinterpret_cast<uint4*>(a_ex)[i] = make_uint4(0u, 0u, 0u, 0u);
+      if (!cleared) clear_operand();
+      cleared = false;
       asm volatile("bar.sync 1, 256;" ::: "memory");
       if (tid < kNA) {
         const int c = perm[tid];
