@@ -2,6 +2,7 @@
 // work (plan_decode), the launch sequence, and the last kernel of a step, which merges the
 // partial records of the attention kernels by log-sum-exp and, for caches without protected
 // tokens, attends to the FP16 / BF16 residual itself.
+#include <algorithm>
 #include <numeric>
 #include <type_traits>
 
@@ -12,16 +13,28 @@ namespace vidkv {
 namespace {
 
 constexpr int kMaxSMs = 256;        // multiprocessor count the sizing formulas assume at most
-// Units per block up to which a call goes to the block kernel.  It has one launch, short parts and a parallel merge
-// where the stream kernel has three launches and a warp per run, but takes half as many instructions again per unit
-// (every warp of the block pays the unit's loop).  Measured (us per call, block / stream kernel): 160 units of 4 slabs
-// 15.7 / 25.8, 1184 of 16 22.9 / 36.6, 4032 of 112 (7 a block) 40.0 / 43.1, 4032 of 448 43.2 / 43.4, 4480 of 448 (8 a block) 46.5 / 42.7;
-// with protected tokens 160 of 4 21.5 / 31.0, 1152 of 64 (2 a block) 31.2 / 32.9, 1344 of 448 (3) 30.0 / 39.5, 1760 of 32 (4) 40.5 / 43.2,
-// 1568 of 224 (4) 39.9 / 39.1.  Where every unit has a warp of its own in the stream kernel, three a block are too many there
-// (1120 of 224 33.8 / 30.9), except for the general key formats (1120 of 112, 4 a block, 35.9 / 37.0).
-constexpr int kMaxBlockUnits = 7;
-constexpr int kMaxBlockUnitsStp = 4;
-constexpr int kMaxBlockUnitsStpRun1 = 2;
+// Work up to which a call goes to the block kernel: units of its longest block times the blocks that share a multiprocessor.  It has
+// one launch and a parallel merge where the stream kernel has three launches, a warp per run and one merge block per slab, but takes
+// half as many instructions again per unit (every warp of the block pays the unit's loop).  So the line rises with the units of a
+// slab: few and long slabs leave the stream kernel's merge with hundreds of records a block.  Measured, us per call (half
+// of the channels two-bit), block / stream kernel, at the work in brackets:
+//   slabs of up to 8 units  448 slabs of 3 (12) 22.9 / 25.2, 448 of 5 (16) 35.5 / 32.3, 224 of 8 (16) 27.5 / 23.6, 448 of 8 (24) 44.0 / 36.1
+//   longer                  64 of 14 (9) 19.9 / 21.1, 168 of 12 (16) 28.7 / 29.4, 96 of 24 (16) 28.8 / 29.3, 112 of 22 (20) 32.0 / 29.3,
+//                           64 of 40 (18) 33.1 / 31.2, 56 of 50 (20) 34.2 / 31.4, 32 of 70 (16) 29.7 / 35.3, 32 of 100 (24) 37.4 / 37.4,
+//                           32 of 140 (32) 45.8 / 44.3, 16 of 79 (9) 21.7 / 31.6, 16 of 200 (24) 37.4 / 46.2, 16 of 400 (45) 58.0 / 60.1,
+//                           8 of 600 (33) 50.0 / 70.1, 4 of 160 (6) 19.7 / 39.6, 4 of 900 (27) 42.0 / 99.1, 4 of 1225 (36) 50.3 / 104.4
+//   of 9 to 19, no block in two slabs  128 of 18 (18) 29.0 / 30.4, 192 of 13 (20) 32.4 / 30.6 (kept here: the tests of the bounded waits
+//                           hold the kernel to this shape); with blocks in two slabs 224 of 11 (20) 32.9 / 29.7
+//   with protected tokens   112 slabs of 4 (6) 22.7 / 24.7, 224 of 8 (24) 41.8 / 33.2, 112 of 10 (12) 31.3 / 27.3, 64 of 14 (9) 28.7 / 27.1,
+//                           64 of 28 (15) 37.1 / 33.5, 32 of 40 (12) 32.4 / 35.3, 32 of 70 (18) 41.4 / 38.5, 16 of 79 (9) 28.9 / 41.6,
+//                           16 of 140 (18) 41.1 / 44.4, 16 of 200 (24) 50.2 / 51.6, 16 of 400 (45) 79.5 / 70.3, 4 of 600 (15) 44.0 / 80.6
+static int64_t most_block_work(int64_t units_per_slab, bool stp, bool straddles) {
+  const int64_t S = units_per_slab;
+  if (stp) return std::min<int64_t>(6 + S / 6, 40);
+  if (S < 9) return 14;
+  if (S < 20 && !straddles) return 20;
+  return std::min(std::max<int64_t>(14 + S / 10, 16), int64_t{40});
+}
 
 }  // namespace
 
@@ -79,22 +92,50 @@ DecodePlan plan_decode(const LayerState& st, int64_t n_slabs, bool stp, bool gen
   };
   p.slab_parts = static_cast<int32_t>(most_parts(p.n_runs));
   p.records = (p.n_runs + n_slabs) * kMaxRep;
-  const int64_t blocks = static_cast<int64_t>(sms) * (stp && general ? kBlockGenStpPerSM : kBlocksPerSM);
-  int64_t per_block = (p.n_units + blocks - 1) / blocks;
-  // A block that goes on in the next slab pays for query images, rings and join twice: where the proportional cut makes such
-  // blocks (slab s then begins d units * slabs / blocks after a block does, d running through the multiples of
-  // gcd(blocks, slabs)), every slab gets its own blocks, if it can without a longer stretch.  us, straddling / not: 64 slabs
-  // of 14 units 28.9 / 21.8, 448 of 3 28.2 / 21.0; with protected tokens 42.3 / 31.7 and 45.2 / 30.0.
-  int64_t even_blocks = 0;
-  if (p.n_units > 0 && p.n_units - std::gcd(blocks, n_slabs) * p.units_per_slab >= blocks) {
-    const int64_t share = blocks / n_slabs, even = share > 0 ? (p.units_per_slab + share - 1) / share : INT32_MAX;
-    if (stp || even <= per_block) { per_block = even; even_blocks = n_slabs * (share < p.units_per_slab ? share : p.units_per_slab); }
+  // The block kernel's cut for `per_sm` blocks on each multiprocessor.
+  struct BlockCut { int64_t blocks, longest, even; bool straddles; };
+  const auto cut_for = [&](int per_sm) -> BlockCut {
+    BlockCut c = {static_cast<int64_t>(sms) * per_sm, 0, 0, false};
+    c.longest = (p.n_units + c.blocks - 1) / c.blocks;
+    // A block that goes on in the next slab pays for query images, rings and join twice: where the proportional cut makes such
+    // blocks (slab s then begins d units * slabs / blocks after a block does, d running through the multiples of
+    // gcd(blocks, slabs)), every slab gets its own blocks, if it can without a longer stretch.  us, straddling / not: 64 slabs
+    // of 14 units 28.9 / 21.8, 448 of 3 28.2 / 21.0; with protected tokens 42.3 / 31.7 and 45.2 / 30.0.
+    c.straddles = p.n_units > 0 && p.n_units - std::gcd(c.blocks, n_slabs) * p.units_per_slab >= c.blocks;
+    if (c.straddles) {
+      const int64_t share = c.blocks / n_slabs, even = share > 0 ? (p.units_per_slab + share - 1) / share : INT32_MAX;
+      if (stp || even <= c.longest) {
+        c.longest = even;
+        c.even = n_slabs * (share < p.units_per_slab ? share : p.units_per_slab);
+        c.straddles = false;
+      }
+    }
+    return c;
+  };
+  // Without protected tokens there are two variants: three blocks on a multiprocessor with 128 registers a thread, or four with 96, which
+  // keep some of the loop's state in local memory.  Three, unless that makes the longest stretch more than a unit longer, has
+  // blocks that go on in the next slab (worth two units) where four have none, or leaves one of the one-unit blocks and residuals of a
+  // short call waiting for another to end.  us a call, four / three: 16 slabs of 79 units 24.2 / 20.9, 64 of 14 (2 and 3 units
+  // a block) 21.5 / 19.2, 4 of 160 21.5 / 19.4; but 112 of 10 (2; 3 with blocks in two slabs) 20.5 / 23.7, 32 of 40 24.9 / 27.1, 128 of 3 and
+  // their residuals 12.9 / 14.1, 112 of 20 (4; 6) 28.2 / 29.3.  The general key formats' loop has more of that state, and three blocks are better
+  // wherever every slab has a block: 112 of 20 33.4 / 31.6, 16 of 200 (6; 8) 44.7 / 40.6, 128 of 3 13.4 / 13.0; 448 of 3 25.8 / 26.9.
+  // With protected tokens four would not fit in the registers at all (128 slabs of 3 20.7 / 16.2).
+  BlockCut cut = cut_for(kBlocksPerSM);
+  p.blocks_per_sm = kBlocksPerSM;
+  if (!stp) {
+    const BlockCut more = cut_for(kMoreBlocksPerSM);
+    bool fewer = n_slabs <= cut.blocks;
+    if (fewer && !general) {
+      if (more.longest <= 1) fewer = p.n_units + (st.n_res > 0 ? n_slabs : 0) <= cut.blocks;
+      else fewer = cut.longest + 2 * cut.straddles <= more.longest + 2 * more.straddles + 1;
+    }
+    if (!fewer) { cut = more; p.blocks_per_sm = kMoreBlocksPerSM; }
   }
-  const int64_t most = !stp ? kMaxBlockUnits : general || run > 1 ? kMaxBlockUnitsStp : kMaxBlockUnitsStpRun1;
-  if (p.n_units == 0 || (per_block <= most && force_run_units == 0 && (!partial || run == 1))) {
-    p.n_blocks = static_cast<int32_t>(even_blocks > 0 ? even_blocks : p.n_units < blocks ? p.n_units : blocks);
+  const bool block = cut.longest * p.blocks_per_sm <= most_block_work(p.units_per_slab, stp, cut.straddles);
+  if (p.n_units == 0 || (block && force_run_units == 0 && (!partial || run == 1))) {
+    p.n_blocks = static_cast<int32_t>(cut.even > 0 ? cut.even : p.n_units < cut.blocks ? p.n_units : cut.blocks);
     p.records = (p.n_blocks + n_slabs) * kMaxRep;
-    p.res_blocks = st.n_res > 0 && per_block <= 1 ? static_cast<int32_t>(n_slabs) : 0;
+    p.res_blocks = st.n_res > 0 && cut.longest <= 1 ? static_cast<int32_t>(n_slabs) : 0;
     p.counters_per_slab = static_cast<int32_t>(join_counters(most_parts(p.n_blocks) + (p.res_blocks > 0)));
   }
   return p;

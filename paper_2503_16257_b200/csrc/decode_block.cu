@@ -1,5 +1,5 @@
-// Decode attention over the packed cache (Algorithm 1 "Decoding", Eq. 3) in one launch, for calls of a few thousand
-// 160-token units (five 32-token key groups) at most; plan_decode holds the rule.
+// Decode attention over the packed cache (Algorithm 1 "Decoding", Eq. 3) in one launch, for small calls (up to some 5000
+// 160-token units of five 32-token key groups where the slabs are few and long); most_block_work holds the rule.
 //
 // What bounds such a call is latency: launches, dependent loads, a unit's serial work and the merge of the partial
 // results.  6400 tokens, a unit a block (11.4 us from the first block's start to the last one's end): query images 2.2,
@@ -43,10 +43,10 @@ namespace {
 
 constexpr int kUnitWarps = 5;
 constexpr int kUnitThreads = kUnitWarps * 32;
-constexpr int kImgBytes = 24 * 32 * 4;                        // query images of one chunk
+constexpr int kImgBytes = 40 * 32 * 4;                        // query images of one chunk
 constexpr int kTRing = 512, kPRing = 512;                     // ring positions: an unfinished supergroup (group), two units and the gap
                                                               // before the flushed tokens
-constexpr int kPBufs = 6;                                     // staged protected groups
+constexpr int kPBufs = 5;                                     // staged protected groups (as many as leave room for four blocks)
 constexpr int kResS = 132, kResP = 136;                       // row lengths of the residual's scores and probabilities
 constexpr int kResScratch = 8 * kResS * 4 + 8 * kResP * 2;    // 6400
 
@@ -62,6 +62,18 @@ template <bool GEN, bool STP> struct Smem {
   static constexpr int bytes = prob_at + prob_bytes;
 };
 
+// The query as score_blocks takes it, from the images in shared memory, four words a load.
+struct ImageQuery {
+  const uint32_t* img;
+  __device__ __forceinline__ uint4 words(int j) const { return *reinterpret_cast<const uint4*>(img + 128 * j); }
+  __device__ __forceinline__ uint4 pairs(int f) const { return words(f); }
+  __device__ __forceinline__ void spectrum(int f, int par, uint32_t (&h)[4], uint32_t (&l)[4]) const {
+    const uint4 a = words(2 + 2 * f + par), b = words(6 + 2 * f + par);
+    h[0] = a.x; h[1] = a.y; h[2] = a.z; h[3] = a.w;
+    l[0] = b.x; l[1] = b.y; l[2] = b.z; l[3] = b.w;
+  }
+};
+
 // Scores of one key group (t as in score_group) and the group's constants of heads 2 r, 2 r + 1.  img: this lane's query words of the
 // group's chunk, four words a 16-byte load, 32 loads apart.
 template <bool GEN>
@@ -73,20 +85,12 @@ __device__ __forceinline__ void score(uint8_t* kg, const KeyFmt& kf, int lane, i
   } else {
     GroupBytes gb;
     gb.fetch(kg, lane);
-    uint32_t x[24];
-#pragma unroll
-    for (int j = 0; j < 6; ++j) {
-      const uint4 v = *reinterpret_cast<const uint4*>(img + 128 * j);
-      x[4 * j] = v.x; x[4 * j + 1] = v.y; x[4 * j + 2] = v.z; x[4 * j + 3] = v.w;
-    }
-    group_constants(kg, 1, g, r, [&](int j) { return x[j]; }, cst);
+    const ImageQuery q{img};
+    group_constants(kg, 1, g, r, q, cst);
     __syncwarp();
     put_scales(gb, gb, kg, lane);
     __syncwarp();
-    // i = (2 f + par) 4 + y: word 4 f + y, its high half for par = 0
-    score_group(gb, kg, r, [&](int j) { return x[j]; },
-                [&](int i) { const uint32_t w = x[8 + (i >> 3) * 4 + (i & 3)]; return (i & 4) ? sign_pair_lo(w) : sign_pair_hi(w); },
-                [&](int i) { const uint32_t w = x[16 + (i >> 3) * 4 + (i & 3)]; return (i & 4) ? sign_pair_lo(w) : sign_pair_hi(w); }, t);
+    score_group(gb, kg, r, q, t);
   }
 }
 
@@ -94,9 +98,9 @@ __device__ __forceinline__ void score(uint8_t* kg, const KeyFmt& kf, int lane, i
 // Query images of one chunk's channel split, by the whole block: word i of lane (head hd = lane / 4,
 // r = lane % 4) at ((i / 4) * 32 + lane) * 4 + i % 4, so that four words are one 16-byte load:
 //   words  j < 8            binary16 pair of q at the anomalous slots 8 j + 2 r, + 1
-//   words  8 + j            leading binary16 part of the transformed query Q at the spectrum columns c, c + 1,
-//                           c = 16 (j / 2) + 14 - 8 (j % 2) - 2 r
-//   words 16 + j            binary16 remainder Q - leading part;
+//   words  8 + 4 (2 f + par) + i   (-Q, Q), leading binary16 part of the transformed query Q at the spectrum column
+//                           32 f + 16 (i / 2) + 15 - 8 (i % 2) - 2 r - par
+//   words 24 + 4 (2 f + par) + i   the same of the binary16 remainder Q - leading part;
 // zero for heads that do not
 // exist, all of the query normalised by its head's power of two (head_exponent).  Q_f = sum_c q_c W[c, f] with W the
 // weights with which spectrum column f enters channel c of the inverse orthonormal 64-point transform of a Hermitian
@@ -158,14 +162,17 @@ __device__ __forceinline__ void make_images(uint32_t* img, const ImageSource& sr
         mma_f16(acc, af[ks][0], 0u, af[ks][1], 0u, bw.x, bw.y);
         mma_f16(acc, af[ks][0], 0u, af[ks][1], 0u, bw.z, bw.w);
       }
-      // lane (hd, r) now holds Q of head hd at columns 16 r + 2 nt + {0, 1}: word 2 r + (nt < 4) of lane (hd, 3 - nt % 4)
+      // lane (hd, r) now holds Q of head hd at columns 16 r + 2 nt + {0, 1}, which belong to lane (hd, 3 - nt % 4)
       const float w0 = (r == 0 && nt == 0) ? 1.0f : 2.0f;            // columns 0 and 1 are not doubled
       const float x0 = acc[0] * w0, x1 = acc[1] * w0;
       const __half h0 = __float2half_rn(x0), h1 = __float2half_rn(x1);
-      const int j = 2 * r + (nt < 4 ? 1 : 0), to = lane - r + 3 - (nt & 3);
+      const int at = 8 + (r >> 1) * 8 + 2 * (r & 1) + (nt < 4 ? 1 : 0), to = lane - r + 3 - (nt & 3);   // f = r / 2, i = 2 (r % 2) + (nt < 4)
       put(nt, lane, pack_half2(q_at(src.two[turn] & 0xffu), q_at(src.two[turn] >> 8)));
-      put(8 + j, to, pack_half2(__half2float(h0), __half2float(h1)));
-      put(16 + j, to, pack_half2(x0 - __half2float(h0), x1 - __half2float(h1)));
+      const uint32_t hi = pack_half2(__half2float(h0), __half2float(h1)), lo = pack_half2(x0 - __half2float(h0), x1 - __half2float(h1));
+      put(at, to, sign_pair_hi(hi));                                 // par = 0: the odd column of the pair
+      put(at + 4, to, sign_pair_lo(hi));
+      put(at + 16, to, sign_pair_hi(lo));
+      put(at + 20, to, sign_pair_lo(lo));
     }
   } else {
     const int n2 = kf.n2, n1 = kD - n2, w1 = n2 / 8, n_pairs = kf.plain ? kD / 8 : w1;
@@ -471,7 +478,10 @@ __device__ __forceinline__ void join_records(const float* rec, int64_t stride, i
   float4 oa[kJoin], ob[kJoin];
 #pragma unroll
   for (int j = 0; j < kJoin; ++j) {
-    const float* q = rec + (j < n ? j : 0) * stride + 16 + 2 * r * kD + 32 * w + 4 * hd;
+    oa[j] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    ob[j] = oa[j];
+    if (j >= n) continue;
+    const float* q = rec + j * stride + 16 + 2 * r * kD + 32 * w + 4 * hd;
     oa[j] = __ldcg(reinterpret_cast<const float4*>(q));
     ob[j] = __ldcg(reinterpret_cast<const float4*>(q + kD));
   }
@@ -576,8 +586,8 @@ __device__ __forceinline__ void zero_ring(uint8_t* ring, int ring_len, int pos_b
 
 }  // namespace
 
-template <bool GEN, bool STP, typename T>
-__global__ void __launch_bounds__(kUnitThreads, GEN && STP ? kBlockGenStpPerSM : kBlocksPerSM) decode_block_kernel(DecodeArgs a) {
+template <bool GEN, bool STP, int kPerSM, typename T>
+__global__ void __launch_bounds__(kUnitThreads, kPerSM) decode_block_kernel(DecodeArgs a) {
   using S = Smem<GEN, STP>;
   extern __shared__ __align__(128) uint8_t sm[];
   __shared__ __align__(8) uint64_t kbar[2], vbar[2], pbar[kPBufs];
@@ -945,7 +955,7 @@ __global__ void __launch_bounds__(kUnitThreads, GEN && STP ? kBlockGenStpPerSM :
   }
 }
 
-template <bool GEN, bool STP, typename T>
+template <bool GEN, bool STP, int kPerSM, typename T>
 static cudaError_t launch_block_t(const DecodeArgs& a, cudaStream_t stream) {
   constexpr int smem = Smem<GEN, STP>::bytes;
   static bool attr_set[64] = {};
@@ -954,23 +964,26 @@ static cudaError_t launch_block_t(const DecodeArgs& a, cudaStream_t stream) {
   if ((e = cudaGetDevice(&dev))) return e;
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   if (!attr_set[dev]) {
-    if ((e = cudaFuncSetAttribute(decode_block_kernel<GEN, STP, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem))) return e;
+    if ((e = cudaFuncSetAttribute(decode_block_kernel<GEN, STP, kPerSM, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem))) return e;
     attr_set[dev] = true;
   }
   count_launches(1);
-  return launch_dependent(decode_block_kernel<GEN, STP, T>, dim3(a.plan.n_blocks + a.plan.res_blocks), dim3(kUnitThreads), smem, stream, a);
+  return launch_dependent(decode_block_kernel<GEN, STP, kPerSM, T>, dim3(a.plan.n_blocks + a.plan.res_blocks), dim3(kUnitThreads), smem, stream, a);
+}
+
+template <bool GEN, typename T>
+static cudaError_t launch_block_as(const DecodeArgs& a, bool stp, bool more, cudaStream_t stream) {
+  if (stp) return launch_block_t<GEN, true, kBlocksPerSM, T>(a, stream);
+  return more ? launch_block_t<GEN, false, kMoreBlocksPerSM, T>(a, stream) : launch_block_t<GEN, false, kBlocksPerSM, T>(a, stream);
 }
 
 cudaError_t launch_decode_block(const DecodeArgs& a_in, cudaStream_t stream) {
   DecodeArgs a = a_in;
   const bool gen = a.cv.kf.general != 0, stp = a.n_prot > 0, half = a.in_dtype == VIDKV_F16;
   if (g_debug_withhold == 2) { a.withhold = stp ? 0 : 1; g_debug_withhold = 0; }
-  if (gen) {
-    if (stp) return half ? launch_block_t<true, true, __half>(a, stream) : launch_block_t<true, true, __nv_bfloat16>(a, stream);
-    return half ? launch_block_t<true, false, __half>(a, stream) : launch_block_t<true, false, __nv_bfloat16>(a, stream);
-  }
-  if (stp) return half ? launch_block_t<false, true, __half>(a, stream) : launch_block_t<false, true, __nv_bfloat16>(a, stream);
-  return half ? launch_block_t<false, false, __half>(a, stream) : launch_block_t<false, false, __nv_bfloat16>(a, stream);
+  const bool more = a.plan.blocks_per_sm == kMoreBlocksPerSM;
+  if (gen) return half ? launch_block_as<true, __half>(a, stp, more, stream) : launch_block_as<true, __nv_bfloat16>(a, stp, more, stream);
+  return half ? launch_block_as<false, __half>(a, stp, more, stream) : launch_block_as<false, __nv_bfloat16>(a, stp, more, stream);
 }
 
 }  // namespace vidkv

@@ -66,11 +66,11 @@ __device__ __forceinline__ void put_scales(const GroupBytes& a, const GroupBytes
 
 // Products of NT row blocks: block m's codes are we[m] (even slots: the low half-words' tokens in rows 0-7, the high ones' in rows 8-15),
 // odd slots wo[m], signs bits[m]; kg: where put_scales left the operands.  t = a0 + 2 a1.
-// q(j): binary16 pair of q at slots 8 j + 2 r, + 1 of head g (lane = 4 g + r).  qh(i), ql(i), i = (2 f + par) 4 + x: (-Q, Q) at
-// spectrum column 32 f + 16 (x / 2) + 15 - 8 (x % 2) - 2 r - par.
-template <int NT, typename Q, typename QH, typename QL>
-__device__ __forceinline__ void score_blocks(const uint32_t (&we)[NT], const uint32_t (&wo)[NT], const uint32_t (&bits)[NT], const uint8_t* kg, int r, Q q,
-                                             QH qh, QL ql, float (&t)[NT][4]) {
+// The query: q.pairs(f)[i] = binary16 pair of q at slots 8 (4 f + i) + 2 r, + 1 of head g (lane = 4 g + r); q.spectrum(f, par, h, l): (-Q, Q) at
+// spectrum column 32 f + 16 (i / 2) + 15 - 8 (i % 2) - 2 r - par, leading part h[i] and remainder l[i].
+template <int NT, typename Q>
+__device__ __forceinline__ void score_blocks(const uint32_t (&we)[NT], const uint32_t (&wo)[NT], const uint32_t (&bits)[NT], const uint8_t* kg, int r,
+                                             const Q& q, float (&t)[NT][4]) {
   const uint8_t* ap = kg + 16 * r;
   float a0[NT][4], a1[NT][4];       // weight 1, weight 2
 #pragma unroll
@@ -88,12 +88,10 @@ __device__ __forceinline__ void score_blocks(const uint32_t (&we)[NT], const uin
 #pragma unroll
     for (int f = 0; f < 2; ++f) {
       uint32_t b[4], h[4], l[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        b[i] = par ? row_pair_hi(q(4 * f + i)) : row_pair_lo(q(4 * f + i));
-        h[i] = qh((2 * f + par) * 4 + i);
-        l[i] = ql((2 * f + par) * 4 + i);
-      }
+      const uint4 qp = q.pairs(f);
+      b[0] = par ? row_pair_hi(qp.x) : row_pair_lo(qp.x); b[1] = par ? row_pair_hi(qp.y) : row_pair_lo(qp.y);
+      b[2] = par ? row_pair_hi(qp.z) : row_pair_lo(qp.z); b[3] = par ? row_pair_hi(qp.w) : row_pair_lo(qp.w);
+      q.spectrum(f, par, h, l);
       const uint4 s2 = *reinterpret_cast<const uint4*>(ap + 128 * f + 64 * par), s1 = *reinterpret_cast<const uint4*>(ap + 256 + 128 * f + 64 * par);
 #pragma unroll
       for (int m = 0; m < NT; ++m) {
@@ -124,15 +122,15 @@ __device__ __forceinline__ void score_blocks(const uint32_t (&we)[NT], const uin
 }
 // Scores without their group's constant, in the units of the normalised query: t[m] = tokens 16 m + g (heads 2 r, 2 r + 1) and
 // 16 m + 8 + g of one group ...
-template <typename Q, typename QH, typename QL>
-__device__ __forceinline__ void score_group(const GroupBytes& a, const uint8_t* kg, int r, Q q, QH qh, QL ql, float (&t)[2][4]) {
+template <typename Q>
+__device__ __forceinline__ void score_group(const GroupBytes& a, const uint8_t* kg, int r, const Q& q, float (&t)[2][4]) {
   const uint32_t we[2] = {prmt(a.c2.x, a.c2.y, 0x5410u), prmt(a.c2.z, a.c2.w, 0x5410u)}, wo[2] = {prmt(a.c2.x, a.c2.y, 0x7632u), prmt(a.c2.z, a.c2.w, 0x7632u)};
   const uint32_t bits[2] = {a.c1.x, a.c1.y};
-  score_blocks<2>(we, wo, bits, kg, r, q, qh, ql, t);
+  score_blocks<2>(we, wo, bits, kg, r, q, t);
 }
 // ... and of two.
-template <typename Q, typename QH, typename QL>
-__device__ __forceinline__ void score_groups(const GroupBytes& a, const GroupBytes& b, const uint8_t* kg, int r, Q q, QH qh, QL ql, float (&ta)[2][4],
+template <typename Q>
+__device__ __forceinline__ void score_groups(const GroupBytes& a, const GroupBytes& b, const uint8_t* kg, int r, const Q& q, float (&ta)[2][4],
                                              float (&tb)[2][4]) {
   const uint32_t wa[4] = {a.c2.x, a.c2.y, a.c2.z, a.c2.w}, wb[4] = {b.c2.x, b.c2.y, b.c2.z, b.c2.w};
   uint32_t we[4], wo[4];
@@ -140,7 +138,7 @@ __device__ __forceinline__ void score_groups(const GroupBytes& a, const GroupByt
   for (int m = 0; m < 4; ++m) { we[m] = prmt(wa[m], wb[m], 0x5410u); wo[m] = prmt(wa[m], wb[m], 0x7632u); }
   const uint32_t bits[4] = {prmt(a.c1.x, b.c1.x, 0x5410u), prmt(a.c1.x, b.c1.x, 0x7632u), prmt(a.c1.y, b.c1.y, 0x5410u), prmt(a.c1.y, b.c1.y, 0x7632u)};
   float t[4][4];
-  score_blocks<4>(we, wo, bits, kg, r, q, qh, ql, t);
+  score_blocks<4>(we, wo, bits, kg, r, q, t);
 #pragma unroll
   for (int m = 0; m < 4; ++m)
 #pragma unroll
@@ -149,12 +147,16 @@ __device__ __forceinline__ void score_groups(const GroupBytes& a, const GroupByt
 
 // The constants sum q z of up to eight groups at once: c[0], c[1] = those of group min(g, n - 1) and heads 2 r, 2 r + 1.
 template <typename Q>
-__device__ __forceinline__ void group_constants(const uint8_t* kbuf, int n, int g, int r, Q q, float (&c)[2]) {
+__device__ __forceinline__ void group_constants(const uint8_t* kbuf, int n, int g, int r, const Q& q, float (&c)[2]) {
   const uint8_t* z = kbuf + min(g, n - 1) * kKGroupBytes + kKG_Z2 + 4 * r;
   float d[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+  auto word = [&](int at) { return *reinterpret_cast<const uint32_t*>(z + at); };
 #pragma unroll
-  for (int ks = 0; ks < 4; ++ks)
-    mma_f16(d, *reinterpret_cast<const uint32_t*>(z + 32 * ks), 0u, *reinterpret_cast<const uint32_t*>(z + 32 * ks + 16), 0u, q(2 * ks), q(2 * ks + 1));
+  for (int f = 0; f < 2; ++f) {
+    const uint4 qp = q.pairs(f);
+    mma_f16(d, word(64 * f), 0u, word(64 * f + 16), 0u, qp.x, qp.y);
+    mma_f16(d, word(64 * f + 32), 0u, word(64 * f + 48), 0u, qp.z, qp.w);
+  }
   c[0] = d[0]; c[1] = d[1];
 }
 

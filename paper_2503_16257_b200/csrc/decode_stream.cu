@@ -43,7 +43,12 @@ struct Running {
 // What a lane keeps of one chunk's prepared query.
 template <bool GEN> struct Query;
 template <> struct Query<false> {
-  uint32_t q[8], qh[16], ql[16];      // as score_group takes them
+  uint32_t q[8], qh[16], ql[16];      // as score_blocks takes them: words 4 f + i and (2 f + par) 4 + i
+  __device__ __forceinline__ uint4 pairs(int f) const { return make_uint4(q[4 * f], q[4 * f + 1], q[4 * f + 2], q[4 * f + 3]); }
+  __device__ __forceinline__ void spectrum(int f, int par, uint32_t (&h)[4], uint32_t (&l)[4]) const {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) { h[i] = qh[(2 * f + par) * 4 + i]; l[i] = ql[(2 * f + par) * 4 + i]; }
+  }
   __device__ __forceinline__ void load(const uint32_t* pp) {
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
@@ -55,7 +60,7 @@ template <> struct Query<false> {
     }
   }
   __device__ __forceinline__ void constants(const uint8_t* kbuf, const KeyFmt&, int n, int g, int r, float (&c)[2]) const {
-    group_constants(kbuf, n, g, r, [&](int j) { return q[j]; }, c);
+    group_constants(kbuf, n, g, r, *this, c);
   }
   __device__ __forceinline__ void score(uint8_t* ga, uint8_t* gb, const KeyFmt&, int lane, int r, float (&ta)[2][4], float (&tb)[2][4]) const {
     GroupBytes a, b;
@@ -64,7 +69,7 @@ template <> struct Query<false> {
     __syncwarp();
     put_scales(a, b, ga, lane);
     __syncwarp();
-    score_groups(a, b, ga, r, [&](int j) { return q[j]; }, [&](int j) { return qh[j]; }, [&](int j) { return ql[j]; }, ta, tb);
+    score_groups(a, b, ga, r, *this, ta, tb);
   }
   __device__ __forceinline__ void score(uint8_t* ga, const KeyFmt&, int lane, int r, float (&t)[2][4]) const {
     GroupBytes a;
@@ -72,7 +77,7 @@ template <> struct Query<false> {
     __syncwarp();
     put_scales(a, a, ga, lane);
     __syncwarp();
-    score_group(a, ga, r, [&](int j) { return q[j]; }, [&](int j) { return qh[j]; }, [&](int j) { return ql[j]; }, t);
+    score_group(a, ga, r, *this, t);
   }
 };
 template <> struct Query<true> {

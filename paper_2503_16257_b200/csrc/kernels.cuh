@@ -131,9 +131,8 @@ constexpr int kStreamWarps = 4;         // warps per CTA of the stream kernel
 constexpr int kStreamCtasPerSM = 3;     // its CTAs per multiprocessor (register bound)
 constexpr int kStreamStpCtasPerSM = 2;  // the same for the variant with protected tokens (shared-memory bound)
 constexpr int kPrepWords = 25;          // 32-bit words per lane per (slab, chunk) of prepared query
-constexpr int kBlocksPerSM = 4;         // blocks of the block kernel per multiprocessor (96 registers x 160 threads;
-                                        // 56 KB of shared memory with protected tokens)
-constexpr int kBlockGenStpPerSM = 3;    // general key formats with protected tokens: 60 KB
+constexpr int kBlocksPerSM = 3;         // blocks of the block kernel per multiprocessor: 128 registers x 160 threads
+constexpr int kMoreBlocksPerSM = 4;     // its variant for calls that are better off with more blocks (96 registers; no protected tokens)
 constexpr int kRecordFloats = 130; // one partial record: running maximum (base-2 logits), sum, out[128]
 constexpr int kPartFloats = kMaxRep * kRecordFloats;   // the block kernel's record of a part of a slab: m [8], l [8], out [8][128]
 constexpr int kJoin = 8;           // records joined at a node of the block kernel's merge tree
@@ -156,6 +155,7 @@ struct DecodePlan {
   int32_t n_chunks;        // chunk-table entries the query preparation covers (0: nothing quantized)
   int64_t records;         // records of one query head: (n_runs + n_slabs) * 8, or (n_blocks + n_slabs) * 8 in the block kernel
   int32_t n_blocks;
+  int32_t blocks_per_sm;   // the block kernel's variant: kBlocksPerSM or kMoreBlocksPerSM
   int32_t res_blocks;      // blocks that attend to a slab's residual alone: n_slabs or 0 (the slab's last block does it)
   int32_t counters_per_slab;   // arrival counters of the merge tree
   int32_t equal_units;     // > 0: runs of exactly this many units (the last one shorter) instead of a proportional share

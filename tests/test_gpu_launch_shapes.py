@@ -373,3 +373,40 @@ def test_cache_memory_that_nobody_has_written_does_not_count(run_units, T, p, st
         if s < 2 or s >= 126:
             assert np.abs(out - ref).max() <= TOL_ABS, s
     assert pair.cache.status() == 0
+
+
+@pytest.mark.parametrize("name,L,B,T,p,k_ratio,one_bit", [
+    ("tiny", 27, 1, 362, 0.0, 0.5, "fft"),         # 108 slabs of three units and their residuals: 432 blocks, three to a multiprocessor
+    ("tiny", 28, 1, 362, 0.0, 0.5, "fft"),         # 448 blocks: four
+    ("qwen", 28, 4, 362, 0.0, 0.75, "minmax"),     # more slabs than blocks at three to a multiprocessor
+    ("tiny", 1, 4, 11300, 0.0, 0.75, "minmax"),    # 16 slabs of 71 units, two or three to a block
+    ("tiny", 1, 1, 196000, 0.0, 0.5, "fft"),       # the longest slab: 1225 units, 111 parts
+    ("llava", 1, 4, 22400, 0.2, 0.5, "fft"),       # protected tokens, 140 units, five or six to a block
+])
+def test_block_kernel_at_the_edges_of_its_variants(name, L, B, T, p, k_ratio, one_bit):
+    """The small-call kernel against the stream kernel with runs of 40 units, over the same cache.  They differ by the order of
+    float32 sums: chains of at most 40 units of 5 groups, 31 records and the residual, 250 x 2^-24 = 1.5e-5 of the norm."""
+    import paper_2503_16257_b200 as P
+    wl = CONFIGS[name]
+    cfg = P.VidKVConfig(B=B, L=L, max_prefill_tokens=T, max_new_tokens=4, p_ratio=p, k_ratio=k_ratio,
+                        key_1bit_mode=P.VIDKV_KEY1BIT_PLAIN_MINMAX if one_bit == "minmax" else P.VIDKV_KEY1BIT_FFT_SIGN,
+                        in_dtype=P.VIDKV_F16 if wl.dtype == "fp16" else P.VIDKV_BF16, out_dtype=P.VIDKV_F32)
+    q, k, v = (torch.stack(t) for t in zip(*[make_step_inputs(wl, layer, 0, "cuda", T=T, B=B) for layer in range(L)]))
+    outs = []
+    for run_units, launches in ((0, 1), (40, 3)):
+        c = P.VidKVCache(cfg)
+        if p > 0:
+            l_v = min(wl.l_v, T - T % 32)
+            c.select_tokens(make_saliency(wl, "cpu", l_v=l_v, B=B).cuda(), 0, l_v, T)
+        for layer in range(L):
+            K, V = make_layer_kv(wl, layer, "cuda", T=T, B=B)
+            c.quantize_keys(layer, K)
+            c.quantize_values(layer, V)
+        c.debug_set_decode_plan(run_units=run_units)
+        out = torch.empty((L, B, 28, 128), dtype=torch.float32, device="cuda")
+        before = P.vidkv_launch_count()
+        c.decode_attention(0, L, q, k, v, out)
+        assert P.vidkv_launch_count() - before == launches
+        assert c.status() == 0
+        outs.append(out.double())
+    assert float((outs[0] - outs[1]).norm() / outs[1].norm()) <= 1.5e-5
