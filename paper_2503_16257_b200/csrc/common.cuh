@@ -139,6 +139,9 @@ __device__ __forceinline__ float ordered_float(uint32_t u) {
 // b = sum d_g * 3^(4-g); the stored byte is ceil(256 * b / 243), which lets a decoder
 // peel digits with multiply / shift and no division.
 __host__ __device__ __forceinline__ uint32_t trit_byte_encode(uint32_t b) { return (256u * b + 242u) / 243u; }
+// the same in bits 24-31, for b <= 242: floor(2^32 / 243) falls short of 2^32 / 243 by less than half, so by less than 110 in
+// 242 times as much, and the fractions of 256 b / 243 are 0 or at least 1 / 243 = 69042 of 2^24
+__device__ __forceinline__ uint32_t trit_byte_top(uint32_t b) { return b * 17674762u + 16777215u; }
 __host__ __device__ __forceinline__ uint32_t trit_byte_decode(uint32_t q) { return (q * 243u) >> 8; }
 // Byte plane of a ternary supergroup (4096 bytes = 32 stream tokens x 128 channels), laid out
 // for the tensor-core decoder: token j = 2 m + parity, pair m = 8 kt + 4 u + r; channel

@@ -13,18 +13,23 @@ namespace cg = cooperative_groups;
 __device__ __forceinline__ __half2 as_half2(uint32_t v) { return *reinterpret_cast<const __half2*>(&v); }
 
 // ---------------------------------------------------------------------------------
-// 1.58Quant (Eq. 6) of one supergroup = 5 groups x 32 stream tokens x 128 channels by a block of 256 threads.
+// 1.58Quant (Eq. 6) of one supergroup = 5 groups x 32 stream tokens x 128 channels by a block of 320 threads.
 // Stream position u of the unprotected tokens maps to token idx_rest[u] (identity when
 // no token is protected).
 //   stage   the 160 x 128 tile is copied to shared memory as it is (cp.async, 16 bytes a piece);
-//   pass 1  s = Mean |v| per (group, channel): thread = (channel pair, quarter of the group's
-//           tokens), float32 partial sums combined in a fixed order;
-//   pass 2  thread = one 32-bit word of the byte plane = (token pair, channel pair): the
-//           comparisons |v| > alpha run on two channels at a time against the smallest
+//   pass 1  s = Mean |v| per (group, channel), float32, and the threshold: thread = (group, channel pair), so nothing
+//           has to meet in shared memory but the threshold;
+//   pass 2  thread = two 32-bit words of the byte plane = (token pair, four channels):
+//           the comparisons |v| > alpha run on two channels at a time against the smallest
 //           representable number above alpha = gamma * s, the five digits of a byte are
-//           chained in binary16 (exact, <= 242), and the byte code comes from a 243-entry table.
+//           chained in binary16 (exact, <= 242), and the byte code is the top byte of one multiply-add.
+// What bounds it is the copies' latency, covered by the blocks that share a multiprocessor: five of them (45 KB, 32 registers; a
+// list of token positions costs a second latency).  With 256 threads, partial sums in shared memory, a table of byte codes and four
+// blocks, 64 slabs of 12544 tokens took 55.2 us and 73.1 with a fifth of the tokens protected; now 46.3 (205 MB in and
+// 53 out, 5.6 TB/s) and 56.6.  The new pass 2 alone gave 51.8 and 72.0.
 // ---------------------------------------------------------------------------------
 constexpr int kSGTokens = kSGGroups * kG;   // 160
+constexpr int kVThreads = kSGGroups * kD / 2;  // 320: a channel pair of a group each
 constexpr int kVRowBytes = 272;             // 256 bytes of data + padding: rows four apart land 16 banks apart
 
 template <typename T> struct Simd2;
@@ -34,8 +39,8 @@ template <> struct Simd2<__half> {
     const __half2 r = __hge2(*reinterpret_cast<const __half2*>(&a), *reinterpret_cast<const __half2*>(&b));
     return *reinterpret_cast<const uint32_t*>(&r);
   }
-  static __device__ __forceinline__ uint32_t gt(uint32_t a, uint32_t b) {
-    const __half2 r = __hgt2(*reinterpret_cast<const __half2*>(&a), *reinterpret_cast<const __half2*>(&b));
+  static __device__ __forceinline__ uint32_t above_minus(uint32_t a, uint32_t b) {      // a > -b
+    const __half2 r = __hgt2(*reinterpret_cast<const __half2*>(&a), __hneg2(*reinterpret_cast<const __half2*>(&b)));
     return *reinterpret_cast<const uint32_t*>(&r);
   }
   // smallest element value strictly above x >= 0
@@ -49,8 +54,8 @@ template <> struct Simd2<__nv_bfloat16> {
     const __nv_bfloat162 r = __hge2(*reinterpret_cast<const __nv_bfloat162*>(&a), *reinterpret_cast<const __nv_bfloat162*>(&b));
     return *reinterpret_cast<const uint32_t*>(&r) & 0x3c003c00u;
   }
-  static __device__ __forceinline__ uint32_t gt(uint32_t a, uint32_t b) {
-    const __nv_bfloat162 r = __hgt2(*reinterpret_cast<const __nv_bfloat162*>(&a), *reinterpret_cast<const __nv_bfloat162*>(&b));
+  static __device__ __forceinline__ uint32_t above_minus(uint32_t a, uint32_t b) {
+    const __nv_bfloat162 r = __hgt2(*reinterpret_cast<const __nv_bfloat162*>(&a), __hneg2(*reinterpret_cast<const __nv_bfloat162*>(&b)));
     return *reinterpret_cast<const uint32_t*>(&r) & 0x3c003c00u;
   }
   static __device__ __forceinline__ uint16_t above(float x) {
@@ -64,15 +69,12 @@ __device__ __forceinline__ void cp_async16_v(void* smem_dst, const void* gmem_sr
 }
 
 // NZ: the stored scale is the mean of |v| over the non-zero codes instead of Mean |v| (one more
-// sweep over the staged tile; needs kSGGroups * 4 * kD more floats of shared memory).
+// sweep over the staged tile).
 template <typename T, bool NZ>
 __device__ __forceinline__ void ternary_supergroup(uint8_t* vsm, KSrc src, int64_t n_rest, CacheView cv, int layer0,
                                                    SelView sel, float gamma) {
   uint8_t* tile = vsm;                                                         // [160][kVRowBytes]
-  float* part = reinterpret_cast<float*>(tile + kSGTokens * kVRowBytes);       // [5][4][128]
-  uint32_t* thr = reinterpret_cast<uint32_t*>(part + kSGGroups * 4 * kD);      // [5][64] threshold pairs
-  uint8_t* lut = reinterpret_cast<uint8_t*>(thr + kSGGroups * 64);             // [256]
-  float* cnt = reinterpret_cast<float*>(lut + 256);                            // [5][4][128], NZ only
+  uint32_t* thr = reinterpret_cast<uint32_t*>(tile + kSGTokens * kVRowBytes);  // [5][64] threshold pairs
   const int tid = threadIdx.x;
   const int slab = blockIdx.y;                              // over the layers of the call, then b, then h
   const int lb = slab / cv.H_kv, h = slab % cv.H_kv;
@@ -83,145 +85,138 @@ __device__ __forceinline__ void ternary_supergroup(uint8_t* vsm, KSrc src, int64
   const int32_t* idx = sel.idx_rest ? sel.idx_rest + b * sel.stride_rest : nullptr;
   // ---- stage (rows past the end of the stream are zero: their trits come out 0)
   {
-    // thread = 16-byte piece (tid % 16) of rows tid / 16 + 16 k.  The stream positions of all its
+    // thread = 16-byte piece (tid % 16) of rows tid / 16 + 20 k.  The stream positions of all its
     // rows are fetched first, so that the gather list costs one memory latency, not one per row.
-    constexpr int kRowsPerThread = kSGTokens * 16 / 256;
+    constexpr int kRowsPerThread = kSGTokens * 16 / kVThreads;
     const int row0 = tid >> 4, piece = tid & 15;
-    int64_t tok[kRowsPerThread];
+    int tok[kRowsPerThread];                                // positions fit 32 bits, as the index lists do
 #pragma unroll
     for (int k = 0; k < kRowsPerThread; ++k) {
-      const int row = row0 + 16 * k;
-      tok[k] = row < n_rows ? (idx ? static_cast<int64_t>(__ldg(idx + u0 + row)) : (u0 + row)) : -1;
+      const int row = row0 + kVThreads / 16 * k;
+      tok[k] = row < n_rows ? (idx ? __ldg(idx + u0 + row) : static_cast<int>(u0) + row) : -1;
     }
 #pragma unroll
     for (int k = 0; k < kRowsPerThread; ++k) {
-      uint8_t* dst = tile + (row0 + 16 * k) * kVRowBytes + piece * 16;
-      if (tok[k] >= 0) cp_async16_v(dst, reinterpret_cast<const uint8_t*>(base + tok[k] * src.stride_t) + piece * 16);
+      uint8_t* dst = tile + (row0 + kVThreads / 16 * k) * kVRowBytes + piece * 16;
+      if (tok[k] >= 0) cp_async16_v(dst, reinterpret_cast<const uint8_t*>(base + static_cast<int64_t>(tok[k]) * src.stride_t) + piece * 16);
       else *reinterpret_cast<uint4*>(dst) = make_uint4(0u, 0u, 0u, 0u);
     }
   }
   asm volatile("cp.async.commit_group;" ::: "memory");
-  if (tid < 243) lut[tid] = static_cast<uint8_t>(trit_byte_encode(tid));
   asm volatile("cp.async.wait_group 0;" ::: "memory");
   __syncthreads();
   uint8_t* sg = cv.slab(layer, b, h) + cv.tern_offset + static_cast<int64_t>(blockIdx.x) * kSGBytes;
-  // ---- pass 1: partial sums of |v| over 8 tokens
+  // ---- pass 1: thread = (group, channel pair); the sum of 32 tokens is the sum of four sums of eight
   {
-    const int cp = tid & 63, q = tid >> 6;
+    const int g = tid >> 6, cp = tid & 63;
+    const int n = max(0, min(kG, n_rows - g * kG));
+    const uint8_t* rp = tile + g * (kG * kVRowBytes) + cp * 4;
+    float sum[2] = {0.0f, 0.0f};
 #pragma unroll
-    for (int g = 0; g < kSGGroups; ++g) {
+    for (int q = 0; q < 4; ++q) {
       float a0 = 0.0f, a1 = 0.0f;
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
-        const uint32_t w = *reinterpret_cast<const uint32_t*>(tile + (g * kG + q * 8 + j) * kVRowBytes + cp * 4);
-        const float2 f = Elem<T>::to_float2(w);
+        const float2 f = Elem<T>::to_float2(*reinterpret_cast<const uint32_t*>(rp + (q * 8 + j) * kVRowBytes));
         a0 += fabsf(f.x); a1 += fabsf(f.y);
       }
-      *reinterpret_cast<float2*>(part + (g * 4 + q) * kD + 2 * cp) = make_float2(a0, a1);
+      sum[0] = q ? sum[0] + a0 : a0;
+      sum[1] = q ? sum[1] + a1 : a1;
     }
-  }
-  __syncthreads();
-  for (int item = tid; item < kSGGroups * kD; item += 256) {
-    const int c = item & (kD - 1), g = item >> 7;
-    const int n = max(0, min(kG, n_rows - g * kG));
-    uint16_t a = 1u;                                   // empty group: every v is 0, nothing exceeds it
+    uint32_t A = 0x00010001u;                          // empty group: every v is 0, nothing exceeds it
     if (n > 0) {
-      const float* pp = part + g * 4 * kD + c;
-      const float sum = ((pp[0] + pp[kD]) + pp[2 * kD]) + pp[3 * kD];
-      const uint16_t sh = f2h_bits(__fdiv_rn(sum, static_cast<float>(n)));
-      if (!NZ) reinterpret_cast<uint16_t*>(sg + kSG_Scales)[g * kD + c] = sh;
-      a = Simd2<T>::above(__fmul_rn(gamma, h2f(sh)));
+      const uint16_t s0 = f2h_bits(__fdiv_rn(sum[0], static_cast<float>(n))), s1 = f2h_bits(__fdiv_rn(sum[1], static_cast<float>(n)));
+      if (!NZ) reinterpret_cast<uint32_t*>(sg + kSG_Scales)[tid] = s0 | static_cast<uint32_t>(s1) << 16;
+      A = Simd2<T>::above(__fmul_rn(gamma, h2f(s0))) | static_cast<uint32_t>(Simd2<T>::above(__fmul_rn(gamma, h2f(s1)))) << 16;
     }
-    reinterpret_cast<uint16_t*>(thr)[item] = a;
+    thr[tid] = A;
+    if (NZ && n > 0) {
+      // ---- sums and counts of |v| over the elements whose code is not 0 (v >= A or v <= -A)
+      const uint32_t one = 0x3c003c00u;
+      float count[2] = {0.0f, 0.0f};
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        float a0 = 0.0f, a1 = 0.0f;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const uint32_t w = *reinterpret_cast<const uint32_t*>(rp + (q * 8 + j) * kVRowBytes);
+          const __half2 nz = __hsub2(__hadd2(as_half2(Simd2<T>::ge(w, A)), as_half2(one)), as_half2(Simd2<T>::above_minus(w, A)));
+          const float2 m = __half22float2(nz), f = Elem<T>::to_float2(w);
+          a0 = fmaf(m.x, fabsf(f.x), a0); a1 = fmaf(m.y, fabsf(f.y), a1);
+          count[0] += m.x; count[1] += m.y;
+        }
+        sum[0] = q ? sum[0] + a0 : a0;
+        sum[1] = q ? sum[1] + a1 : a1;
+      }
+      uint32_t sh = 0u;
+#pragma unroll
+      for (int j = 0; j < 2; ++j)
+        if (count[j] > 0.0f) sh |= static_cast<uint32_t>(f2h_bits(__fdiv_rn(sum[j], count[j]))) << (16 * j);
+      reinterpret_cast<uint32_t*>(sg + kSG_Scales)[tid] = sh;
+    }
   }
   __syncthreads();
-  if (NZ) {
-    // ---- sums and counts of |v| over the elements whose code is not 0 (v >= A or v <= -A)
-    const int cp = tid & 63, q = tid >> 6;
-    const uint32_t one = 0x3c003c00u;
-#pragma unroll
-    for (int g = 0; g < kSGGroups; ++g) {
-      const uint32_t A = thr[g * 64 + cp], nA = A ^ 0x80008000u;
-      float a0 = 0.0f, a1 = 0.0f, c0 = 0.0f, c1 = 0.0f;
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const uint32_t w = *reinterpret_cast<const uint32_t*>(tile + (g * kG + q * 8 + j) * kVRowBytes + cp * 4);
-        const __half2 nz = __hsub2(__hadd2(as_half2(Simd2<T>::ge(w, A)), as_half2(one)), as_half2(Simd2<T>::gt(w, nA)));
-        const float2 m = __half22float2(nz), f = Elem<T>::to_float2(w);
-        a0 = fmaf(m.x, fabsf(f.x), a0); a1 = fmaf(m.y, fabsf(f.y), a1);
-        c0 += m.x; c1 += m.y;
-      }
-      *reinterpret_cast<float2*>(part + (g * 4 + q) * kD + 2 * cp) = make_float2(a0, a1);
-      *reinterpret_cast<float2*>(cnt + (g * 4 + q) * kD + 2 * cp) = make_float2(c0, c1);
-    }
-    __syncthreads();
-    for (int item = tid; item < kSGGroups * kD; item += 256) {
-      const int c = item & (kD - 1), g = item >> 7;
-      if (n_rows - g * kG > 0) {
-        const float* pp = part + g * 4 * kD + c;
-        const float* pc = cnt + g * 4 * kD + c;
-        const float sum = ((pp[0] + pp[kD]) + pp[2 * kD]) + pp[3 * kD];
-        const float n_nz = ((pc[0] + pc[kD]) + pc[2 * kD]) + pc[3 * kD];
-        reinterpret_cast<uint16_t*>(sg + kSG_Scales)[g * kD + c] = n_nz > 0.0f ? f2h_bits(__fdiv_rn(sum, n_nz)) : static_cast<uint16_t>(0);
-      }
-    }
-  }
-  // ---- pass 2: one word of the plane per thread and step
-#pragma unroll
-  for (int wi = 0; wi < kG * kD / 4 / 256; ++wi) {
-    // bits 4 and 5 of the word index trade places: a warp then reads 16 words of each of two rows
-    // that lie four rows apart (conflict-free with the 272-byte row stride) and still writes
-    // whole 64-byte pieces of the plane
-    const int w0 = tid + 256 * wi;
-    const int wd = (w0 & ~0x30) | ((w0 & 0x10) << 1) | ((w0 & 0x20) >> 1);
-    const int cp = 16 * ((wd >> 6) & 3) + 2 * ((wd >> 1) & 7) + (wd & 1);
-    const int m = 8 * ((wd >> 9) & 1) + 4 * ((wd >> 8) & 1) + ((wd >> 4) & 3);
-    uint32_t b0 = 0u, b1 = 0u;                        // binary16 pairs (even channel, odd channel) of tokens 2m, 2m+1
+  // ---- pass 2: two words of the plane (four channels) per thread and step
+#pragma unroll 1
+  for (int i = tid; i < kG * kD / 8; i += kVThreads) {
+    // bits 3 and 4 of the pair's index trade places: a half warp then reads 64 bytes of each of two rows that lie four rows
+    // apart (conflict-free with the 272-byte row stride) and still writes whole 64-byte pieces of the plane
+    const int pair = (i & ~0x18) | ((i & 0x08) << 1) | ((i & 0x10) >> 1);
+    const int cp = 16 * ((pair >> 5) & 3) + 2 * (pair & 7);
+    const int m = 4 * (pair >> 7) + ((pair >> 3) & 3);
+    uint32_t b0[2] = {0u, 0u}, b1[2] = {0u, 0u};      // binary16 pairs (even channel, odd channel) of tokens 2m, 2m+1
     const uint32_t three = 0x42004200u;
     const uint8_t* rp0 = tile + (2 * m) * kVRowBytes + cp * 4;
-    const uint32_t* thp = thr + cp;
 #pragma unroll
     for (int g = 0; g < kSGGroups; ++g) {
-      const uint32_t A = thp[g * 64], nA = A ^ 0x80008000u;
       const uint8_t* rp = rp0 + g * (kG * kVRowBytes);
-      const uint32_t v0 = *reinterpret_cast<const uint32_t*>(rp);
-      const uint32_t v1 = *reinterpret_cast<const uint32_t*>(rp + kVRowBytes);
-      // digit = [v > alpha] + [v >= -alpha] = [v >= A] + [v > -A]
-      const __half2 d0 = __hadd2(as_half2(Simd2<T>::ge(v0, A)), as_half2(Simd2<T>::gt(v0, nA)));
-      const __half2 d1 = __hadd2(as_half2(Simd2<T>::ge(v1, A)), as_half2(Simd2<T>::gt(v1, nA)));
-      const __half2 t0 = __hfma2(as_half2(b0), *reinterpret_cast<const __half2*>(&three), d0);
-      const __half2 t1 = __hfma2(as_half2(b1), *reinterpret_cast<const __half2*>(&three), d1);
-      b0 = *reinterpret_cast<const uint32_t*>(&t0);
-      b1 = *reinterpret_cast<const uint32_t*>(&t1);
+      const uint2 t = *reinterpret_cast<const uint2*>(thr + g * 64 + cp);
+      const uint32_t A[2] = {t.x, t.y};
+      const uint2 r0 = *reinterpret_cast<const uint2*>(rp), r1 = *reinterpret_cast<const uint2*>(rp + kVRowBytes);
+      const uint32_t v0[2] = {r0.x, r0.y}, v1[2] = {r1.x, r1.y};
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        // digit = [v > alpha] + [v >= -alpha] = [v >= A] + [v > -A]
+        const __half2 d0 = __hadd2(as_half2(Simd2<T>::ge(v0[j], A[j])), as_half2(Simd2<T>::above_minus(v0[j], A[j])));
+        const __half2 d1 = __hadd2(as_half2(Simd2<T>::ge(v1[j], A[j])), as_half2(Simd2<T>::above_minus(v1[j], A[j])));
+        const __half2 t0 = __hfma2(as_half2(b0[j]), *reinterpret_cast<const __half2*>(&three), d0);
+        const __half2 t1 = __hfma2(as_half2(b1[j]), *reinterpret_cast<const __half2*>(&three), d1);
+        b0[j] = *reinterpret_cast<const uint32_t*>(&t0);
+        b1[j] = *reinterpret_cast<const uint32_t*>(&t1);
+      }
     }
-    // 1024 + b puts the integer b into the low mantissa bits
-    const uint32_t k1024 = 0x64006400u;
-    const __half2 e0 = __hadd2(as_half2(b0), *reinterpret_cast<const __half2*>(&k1024));
-    const __half2 e1 = __hadd2(as_half2(b1), *reinterpret_cast<const __half2*>(&k1024));
-    const uint32_t x0 = *reinterpret_cast<const uint32_t*>(&e0), x1 = *reinterpret_cast<const uint32_t*>(&e1);
-    // word bytes: (even ch, tok 2m), (even ch, tok 2m+1), (odd ch, tok 2m), (odd ch, tok 2m+1)
-    const uint32_t word = static_cast<uint32_t>(lut[x0 & 0xffu]) | (static_cast<uint32_t>(lut[x1 & 0xffu]) << 8) |
-                          (static_cast<uint32_t>(lut[(x0 >> 16) & 0xffu]) << 16) |
-                          (static_cast<uint32_t>(lut[(x1 >> 16) & 0xffu]) << 24);
-    reinterpret_cast<uint32_t*>(sg)[wd] = word;
+    uint32_t word[2];
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      // 1024 + b puts the integer b into the low mantissa bits
+      const uint32_t k1024 = 0x64006400u;
+      const __half2 e0 = __hadd2(as_half2(b0[j]), *reinterpret_cast<const __half2*>(&k1024));
+      const __half2 e1 = __hadd2(as_half2(b1[j]), *reinterpret_cast<const __half2*>(&k1024));
+      const uint32_t x0 = *reinterpret_cast<const uint32_t*>(&e0), x1 = *reinterpret_cast<const uint32_t*>(&e1);
+      // word bytes: (even ch, tok 2m), (even ch, tok 2m+1), (odd ch, tok 2m), (odd ch, tok 2m+1)
+      const uint32_t even = __byte_perm(trit_byte_top(x0 & 0xffu), trit_byte_top(x1 & 0xffu), 0x0073);
+      const uint32_t odd = __byte_perm(trit_byte_top((x0 >> 16) & 0xffu), trit_byte_top((x1 >> 16) & 0xffu), 0x0073);
+      word[j] = __byte_perm(even, odd, 0x5410);
+    }
+    reinterpret_cast<uint2*>(sg)[pair] = make_uint2(word[0], word[1]);
   }
 }
 
 // ---------------------------------------------------------------------------------
-// 2-bit GQuant (Eq. 4) of groups of up to 32 protected tokens: 128 threads per group, two groups per block.
+// 2-bit GQuant (Eq. 4) of groups of up to 32 protected tokens: 128 threads per group, two groups per block (its last two warps idle).
 //
 // code(v) = clamp(rint((v - z) / s), 0, 3) does not decrease with v, so it equals the number of
 // k in {1, 2, 3} with v >= X_k, X_k the smallest value of the input type whose code reaches k (code_cut).
 // The elements are compared with X_k two channels at a time; the comparisons' ones times 4^e, on top of 1024, put the
-// fields of a code byte into the low bits of two binary16 lanes.  2508 protected and 10036 other tokens of 64 slabs take 78
-// us; three threshold searches with divisions per channel, conversions and float comparisons per element took 95.
+// fields of a code byte into the low bits of two binary16 lanes.  2508 protected and 10036 other tokens of 64 slabs took 78 us
+// when it came in (57 now); three threshold searches with divisions per channel, conversions and float comparisons per element took 95.
 // ---------------------------------------------------------------------------------
 constexpr int kPRow = 144;                  // elements per staged row: rows two apart land 16 banks apart
 constexpr int kProtectSmem = 2 * (kG * kPRow * 2 + 3 * kD * 2);
 
 template <typename T>
 __device__ __forceinline__ void protect_groups(uint8_t* vsm, const KSrc& src, int block, const CacheView& cv, int layer0, const SelView& sel) {
-  const int half = threadIdx.x >> 7, tid = threadIdx.x & 127;
+  const int half = threadIdx.x >> 7, tid = threadIdx.x & 127;                           // half 2: the block's last two warps, idle
   uint16_t* tile = reinterpret_cast<uint16_t*>(vsm) + half * kG * kPRow;                    // [32][kPRow]
   uint16_t* s_thr = reinterpret_cast<uint16_t*>(vsm + 2 * kG * kPRow * 2) + half * 3 * kD;     // [3][128]
   const int slab = blockIdx.y;
@@ -230,9 +225,9 @@ __device__ __forceinline__ void protect_groups(uint8_t* vsm, const KSrc& src, in
   const T* base = reinterpret_cast<const T*>(src.ptr) + static_cast<int64_t>(lb) * src.stride_b + h * src.stride_h;
   const int64_t pgroup = 2 * static_cast<int64_t>(block) + half;
   const int64_t p0 = pgroup * kG;
-  const int n_rows = static_cast<int>(min(static_cast<int64_t>(kG), sel.n_prot - p0));       // <= 0: nothing left for this half
+  const int n_rows = half > 1 ? 0 : static_cast<int>(min(static_cast<int64_t>(kG), sel.n_prot - p0));   // <= 0: nothing left for this half
   const int32_t* idx = sel.idx_prot + b * sel.stride_prot;
-  {
+  if (half <= 1) {
     const int lane16 = tid & 15, row = tid >> 4;
     int tok[kG / 8];
 #pragma unroll
@@ -299,7 +294,7 @@ __device__ __forceinline__ void protect_groups(uint8_t* vsm, const KSrc& src, in
 // 12544 tokens took 745 us, without 720.
 // ---------------------------------------------------------------------------------
 template <typename T, bool NZ>
-__global__ void __launch_bounds__(256) v_quantize_kernel(KSrc src, int64_t T_q, int64_t n_rest, int n_res, CacheView cv, int layer0, SelView sel,
+__global__ void __launch_bounds__(kVThreads, 5) v_quantize_kernel(KSrc src, int64_t T_q, int64_t n_rest, int n_res, CacheView cv, int layer0, SelView sel,
                                                          float gamma, int ternary_blocks, int protect_blocks) {
   extern __shared__ __align__(16) uint8_t vsm[];
   pdl_wait();
@@ -567,8 +562,7 @@ static cudaError_t quantize_values_t(const KSrc& src, int64_t T_q, int n_res, co
   const int n_slabs = n_layers * cv.B * cv.H_kv;
   const int ternary_blocks = static_cast<int>((T_q - sel.n_prot + kSGTokens - 1) / kSGTokens);
   const int protect_blocks = static_cast<int>((sel.n_prot + 2 * kG - 1) / (2 * kG));
-  constexpr size_t smem = kSGTokens * kVRowBytes + sizeof(float) * kSGGroups * 4 * kD + sizeof(uint32_t) * kSGGroups * 64 + 256 +
-                          (NZ ? sizeof(float) * kSGGroups * 4 * kD : 0);
+  constexpr size_t smem = kSGTokens * kVRowBytes + sizeof(uint32_t) * kSGGroups * 64;
   static_assert(smem >= kProtectSmem, "the protected groups live in the ternary tile's shared memory");
   static bool attr_set_dev[64] = {};   // function attributes are per device (and per instantiation)
   int dev = 0;
@@ -581,7 +575,7 @@ static cudaError_t quantize_values_t(const KSrc& src, int64_t T_q, int n_res, co
   }
   count_launches(1);
   return launch_dependent(v_quantize_kernel<T, NZ>, dim3(static_cast<unsigned>(ternary_blocks + protect_blocks + (n_res > 0)), n_slabs),
-                          dim3(256), smem, stream, src, T_q, T_q - sel.n_prot, n_res, cv, layer, sel, gamma, ternary_blocks, protect_blocks);
+                          dim3(kVThreads), smem, stream, src, T_q, T_q - sel.n_prot, n_res, cv, layer, sel, gamma, ternary_blocks, protect_blocks);
 }
 
 cudaError_t launch_quantize_values(int dtype, const KSrc& src, int64_t T_q, int n_res, const CacheView& cv, int layer, int n_layers,
