@@ -103,8 +103,14 @@ extern "C" vidkv_status_t vidkv_attend_noalloc(const vidkv_config_t* cfg, const 
            n_slabs * a.plan.counters_per_slab <= kStaticCounters;
   };
   if (!fits()) {
-    // as few runs as have the same longest one: fewer records
-    a.plan = plan_decode(a.st, n_slabs, n_protected > 0, cv.kf.general != 0, device_sm_count(), a.plan.run_units);
+    // as few runs as have the same longest one: fewer records.  Calls of few units may have longer runs, so that what the block
+    // kernel's few records (one per block and slab) would have room for has room here as well: up to 7 units (4 with protected tokens).
+    const int most = n_protected > 0 ? 4 : 7;
+    int run = a.plan.run_units;
+    const bool few = a.plan.n_units <= static_cast<int64_t>(most) * kMoreBlocksPerSM * device_sm_count();
+    do {
+      a.plan = plan_decode(a.st, n_slabs, n_protected > 0, cv.kf.general != 0, device_sm_count(), run);
+    } while (!fits() && few && ++run <= most);
     if (!fits()) return VIDKV_ERR_CAPACITY;
   }
   StaticScratch scratch;

@@ -410,3 +410,27 @@ def test_block_kernel_at_the_edges_of_its_variants(name, L, B, T, p, k_ratio, on
         assert c.status() == 0
         outs.append(out.double())
     assert float((outs[0] - outs[1]).norm() / outs[1].norm()) <= 1.5e-5
+
+
+def test_attention_without_a_workspace_takes_longer_runs_where_its_scratch_is_short():
+    """448 slabs of six units over eight chunks: the query images leave room for 1276 records, runs of one or two units would
+    leave 1792 and more.  The same attention as the call with a workspace, but for the order of float32 sums (1.5e-5, above)."""
+    import paper_2503_16257_b200 as P
+    L, B, steps = 28, 4, 7 * 128 + 1
+    cfg = P.VidKVConfig(B=B, L=L, max_prefill_tokens=64, max_new_tokens=steps, p_ratio=0.0, out_dtype=P.VIDKV_F32)
+    c = P.VidKVCache(cfg)
+    g = torch.Generator(device="cuda").manual_seed(11)
+    K, V = (torch.randn((B, 4, 64, 128), device="cuda", generator=g).half() for _ in range(2))
+    for layer in range(L):
+        c.quantize_keys(layer, K)
+        c.quantize_values(layer, V)
+    q = torch.randn((L, B, 28, 128), device="cuda", generator=g).half()
+    rows = torch.randn((2, 16, L, B, 4, 128), device="cuda", generator=g).half()
+    out, again = (torch.empty((L, B, 28, 128), dtype=torch.float32, device="cuda") for _ in range(2))
+    for s in range(steps):
+        c.decode_attention(0, L, q, rows[0, s % 16], rows[1, s % 16], out)
+    st = c.layer_state(0)
+    assert (st["n_quantized"], st["n_residual"]) == (64 + 7 * 128, 1)
+    P.vidkv_attend_noalloc(cfg, c.cache, 64, 7, 1, 0, 0, L, q, again)
+    assert c.status() == 0
+    assert float((again.double() - out.double()).norm() / out.double().norm()) <= 1.5e-5
