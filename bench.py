@@ -27,13 +27,13 @@ if ROOT not in sys.path:
     sys.path.insert(0, ROOT)
 
 NOMINAL_HBM_GBS = 8000.0          # the 8 TB/s the targets are quoted against
-FALLBACK_HBM_GBS = 6650.0         # earlier measurement on this machine, used if MEASURED_PEAKS.json is absent
+FALLBACK_HBM_GBS = 6650.0         # an earlier measurement, used if there is no measured one
 # DRAM bytes per cached token per KV head moved by one launch of the decode attention kernel, from the
 # ncu captures summarised in profiles/decode_stream_kernel_batched_4layers.txt (p = 0) and
 # profiles/decode_stream_stp_kernel_batched_4layers_p02.txt (p > 0): a 4-layer cut of the batched workload
 # (3 211 264 cached token-heads per launch), scaled to the launch by the token-heads it processes
 # (traffic is proportional to them).
-NCU_TRAFFIC_BYTES_PER_TOKEN_HEAD = {"decode_stream_kernel": 71.79, "decode_stream_stp_kernel": 79.45}
+NCU_TRAFFIC_BYTES_PER_TOKEN_HEAD = {"decode_stream_kernel": 71.70, "decode_stream_stp_kernel": 77.73}
 
 
 KERNEL_TIMING_STRIDE = 4

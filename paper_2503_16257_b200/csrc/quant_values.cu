@@ -23,8 +23,8 @@ __device__ __forceinline__ __half2 as_half2(uint32_t v) { return *reinterpret_ca
 //           the comparisons |v| > alpha run on two channels at a time against the smallest
 //           representable number above alpha = gamma * s, the five digits of a byte are
 //           chained in binary16 (exact, <= 242), and the byte code is the top byte of one multiply-add.
-// What bounds it is the copies' latency, covered by the blocks that share a multiprocessor: five of them (45 KB, 32 registers; a
-// list of token positions costs a second latency).  With 256 threads, partial sums in shared memory, a table of byte codes and four
+// What bounds it is instructions (7613 a block, 73 % of what the multiprocessors issue) beside the copies' latency, which the blocks that
+// share a multiprocessor cover: five of them (45 KB, 32 registers; a list of token positions costs a second latency).  With 256 threads, partial sums in shared memory, a table of byte codes and four
 // blocks, 64 slabs of 12544 tokens took 55.2 us and 73.1 with a fifth of the tokens protected; now 46.3 (205 MB in and
 // 53 out, 5.6 TB/s) and 56.6.  The new pass 2 alone gave 51.8 and 72.0.
 // ---------------------------------------------------------------------------------
