@@ -22,11 +22,12 @@ __device__ __forceinline__ __half2 as_half2(uint32_t v) { return *reinterpret_ca
 //   pass 2  thread = two 32-bit words of the byte plane = (token pair, four channels):
 //           the comparisons |v| > alpha run on two channels at a time against the smallest
 //           representable number above alpha = gamma * s, the five digits of a byte are
-//           chained in binary16 (exact, <= 242), and the byte code is the top byte of one multiply-add.
+//           summed in binary16 (exact, 1024 to 1266), and the byte code is the top byte of one multiply-add.
 // What bounds it is instructions (7613 a block, 73 % of what the multiprocessors issue) beside the copies' latency, which the blocks that
 // share a multiprocessor cover: five of them (45 KB, 32 registers; a list of token positions costs a second latency).  With 256 threads, partial sums in shared memory, a table of byte codes and four
-// blocks, 64 slabs of 12544 tokens took 55.2 us and 73.1 with a fifth of the tokens protected; now 46.3 (205 MB in and
-// 53 out, 5.6 TB/s) and 56.6.  The new pass 2 alone gave 51.8 and 72.0.
+// blocks, 64 slabs of 12544 tokens took 55.2 us and 73.1 with a fifth of the tokens protected; now 44.1 (205 MB in and
+// 53 out, 5.9 TB/s) and 55.1.  The 64-bit pass 2 alone gave 51.8 and 72.0, five blocks 46.3 and 56.6, digits with their weights in one
+// multiply-add a comparison and no division for full groups the rest.
 // ---------------------------------------------------------------------------------
 constexpr int kSGTokens = kSGGroups * kG;   // 160
 constexpr int kVThreads = kSGGroups * kD / 2;  // 320: a channel pair of a group each
@@ -125,7 +126,10 @@ __device__ __forceinline__ void ternary_supergroup(uint8_t* vsm, KSrc src, int64
     }
     uint32_t A = 0x00010001u;                          // empty group: every v is 0, nothing exceeds it
     if (n > 0) {
-      const uint16_t s0 = f2h_bits(__fdiv_rn(sum[0], static_cast<float>(n))), s1 = f2h_bits(__fdiv_rn(sum[1], static_cast<float>(n)));
+      // a full group's quotient by 32 is the product with 2^-5, to the bit
+      const float m0 = n == kG ? sum[0] * (1.0f / kG) : __fdiv_rn(sum[0], static_cast<float>(n));
+      const float m1 = n == kG ? sum[1] * (1.0f / kG) : __fdiv_rn(sum[1], static_cast<float>(n));
+      const uint16_t s0 = f2h_bits(m0), s1 = f2h_bits(m1);
       if (!NZ) reinterpret_cast<uint32_t*>(sg + kSG_Scales)[tid] = s0 | static_cast<uint32_t>(s1) << 16;
       A = Simd2<T>::above(__fmul_rn(gamma, h2f(s0))) | static_cast<uint32_t>(Simd2<T>::above(__fmul_rn(gamma, h2f(s1)))) << 16;
     }
@@ -164,8 +168,9 @@ __device__ __forceinline__ void ternary_supergroup(uint8_t* vsm, KSrc src, int64
     const int pair = (i & ~0x18) | ((i & 0x08) << 1) | ((i & 0x10) >> 1);
     const int cp = 16 * ((pair >> 5) & 3) + 2 * (pair & 7);
     const int m = 4 * (pair >> 7) + ((pair >> 3) & 3);
-    uint32_t b0[2] = {0u, 0u}, b1[2] = {0u, 0u};      // binary16 pairs (even channel, odd channel) of tokens 2m, 2m+1
-    const uint32_t three = 0x42004200u;
+    // binary16 pairs (even channel, odd channel) of tokens 2m, 2m+1; 1024 + b puts the integer b into the low mantissa bits
+    uint32_t b0[2] = {0x64006400u, 0x64006400u}, b1[2] = {0x64006400u, 0x64006400u};
+    constexpr uint32_t weights[kSGGroups] = {0x55105510u, 0x4ec04ec0u, 0x48804880u, 0x42004200u, 0x3c003c00u};   // 81, 27, 9, 3, 1
     const uint8_t* rp0 = tile + (2 * m) * kVRowBytes + cp * 4;
 #pragma unroll
     for (int g = 0; g < kSGGroups; ++g) {
@@ -177,10 +182,9 @@ __device__ __forceinline__ void ternary_supergroup(uint8_t* vsm, KSrc src, int64
 #pragma unroll
       for (int j = 0; j < 2; ++j) {
         // digit = [v > alpha] + [v >= -alpha] = [v >= A] + [v > -A]
-        const __half2 d0 = __hadd2(as_half2(Simd2<T>::ge(v0[j], A[j])), as_half2(Simd2<T>::above_minus(v0[j], A[j])));
-        const __half2 d1 = __hadd2(as_half2(Simd2<T>::ge(v1[j], A[j])), as_half2(Simd2<T>::above_minus(v1[j], A[j])));
-        const __half2 t0 = __hfma2(as_half2(b0[j]), *reinterpret_cast<const __half2*>(&three), d0);
-        const __half2 t1 = __hfma2(as_half2(b1[j]), *reinterpret_cast<const __half2*>(&three), d1);
+        const __half2 w = as_half2(weights[g]);
+        const __half2 t0 = __hfma2(as_half2(Simd2<T>::above_minus(v0[j], A[j])), w, __hfma2(as_half2(Simd2<T>::ge(v0[j], A[j])), w, as_half2(b0[j])));
+        const __half2 t1 = __hfma2(as_half2(Simd2<T>::above_minus(v1[j], A[j])), w, __hfma2(as_half2(Simd2<T>::ge(v1[j], A[j])), w, as_half2(b1[j])));
         b0[j] = *reinterpret_cast<const uint32_t*>(&t0);
         b1[j] = *reinterpret_cast<const uint32_t*>(&t1);
       }
@@ -188,11 +192,7 @@ __device__ __forceinline__ void ternary_supergroup(uint8_t* vsm, KSrc src, int64
     uint32_t word[2];
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
-      // 1024 + b puts the integer b into the low mantissa bits
-      const uint32_t k1024 = 0x64006400u;
-      const __half2 e0 = __hadd2(as_half2(b0[j]), *reinterpret_cast<const __half2*>(&k1024));
-      const __half2 e1 = __hadd2(as_half2(b1[j]), *reinterpret_cast<const __half2*>(&k1024));
-      const uint32_t x0 = *reinterpret_cast<const uint32_t*>(&e0), x1 = *reinterpret_cast<const uint32_t*>(&e1);
+      const uint32_t x0 = b0[j], x1 = b1[j];
       // word bytes: (even ch, tok 2m), (even ch, tok 2m+1), (odd ch, tok 2m), (odd ch, tok 2m+1)
       const uint32_t even = __byte_perm(trit_byte_top(x0 & 0xffu), trit_byte_top(x1 & 0xffu), 0x0073);
       const uint32_t odd = __byte_perm(trit_byte_top((x0 >> 16) & 0xffu), trit_byte_top((x1 >> 16) & 0xffu), 0x0073);
@@ -209,7 +209,7 @@ __device__ __forceinline__ void ternary_supergroup(uint8_t* vsm, KSrc src, int64
 // k in {1, 2, 3} with v >= X_k, X_k the smallest value of the input type whose code reaches k (code_cut).
 // The elements are compared with X_k two channels at a time; the comparisons' ones times 4^e, on top of 1024, put the
 // fields of a code byte into the low bits of two binary16 lanes.  2508 protected and 10036 other tokens of 64 slabs took 78 us
-// when it came in (57 now); three threshold searches with divisions per channel, conversions and float comparisons per element took 95.
+// when it came in (55 now); three threshold searches with divisions per channel, conversions and float comparisons per element took 95.
 // ---------------------------------------------------------------------------------
 constexpr int kPRow = 144;                  // elements per staged row: rows two apart land 16 banks apart
 constexpr int kProtectSmem = 2 * (kG * kPRow * 2 + 3 * kD * 2);
