@@ -23,7 +23,7 @@ __device__ __forceinline__ __half2 as_half2(uint32_t v) { return *reinterpret_ca
 //           the comparisons |v| > alpha run on two channels at a time against the smallest
 //           representable number above alpha = gamma * s, the five digits of a byte are
 //           summed in binary16 (exact, 1024 to 1266), and the byte code is the top byte of one multiply-add.
-// What bounds it is instructions (7613 a block, 73 % of what the multiprocessors issue) beside the copies' latency, which the blocks that
+// What bounds it is instructions (7396 a block; SM throughput 72 %) beside the copies' latency, which the blocks that
 // share a multiprocessor cover: five of them (45 KB, 32 registers; a list of token positions costs a second latency).  With 256 threads, partial sums in shared memory, a table of byte codes and four
 // blocks, 64 slabs of 12544 tokens took 55.2 us and 73.1 with a fifth of the tokens protected; now 44.1 (205 MB in and
 // 53 out, 5.9 TB/s) and 55.1.  The 64-bit pass 2 alone gave 51.8 and 72.0, five blocks 46.3 and 56.6, digits with their weights in one
