@@ -125,13 +125,15 @@ DecodePlan plan_decode(const LayerState& st, int64_t n_slabs, bool stp, bool gen
   if (!stp) {
     const BlockCut more = cut_for(kMoreBlocksPerSM);
     bool fewer = n_slabs <= cut.blocks;
+    if (general && cut.straddles && !more.straddles && more.longest * kMoreBlocksPerSM < cut.longest * kBlocksPerSM) fewer = false;
     if (fewer && !general) {
       if (more.longest <= 1) fewer = p.n_units + (st.n_res > 0 ? n_slabs : 0) <= cut.blocks;
       else fewer = cut.longest + 2 * cut.straddles <= more.longest + 2 * more.straddles + 1;
     }
     if (!fewer) { cut = more; p.blocks_per_sm = kMoreBlocksPerSM; }
   }
-  const bool block = cut.longest * p.blocks_per_sm <= most_block_work(p.units_per_slab, stp, cut.straddles);
+  const int64_t work = cut.longest * p.blocks_per_sm + (general && !stp && (cut.straddles || p.blocks_per_sm == kMoreBlocksPerSM) ? 3 : 0);
+  const bool block = work <= most_block_work(p.units_per_slab, stp, cut.straddles);
   if (p.n_units == 0 || (block && force_run_units == 0 && (!partial || run == 1))) {
     p.n_blocks = static_cast<int32_t>(cut.even > 0 ? cut.even : p.n_units < cut.blocks ? p.n_units : cut.blocks);
     p.records = (p.n_blocks + n_slabs) * kMaxRep;

@@ -74,12 +74,18 @@ struct ImageQuery {
   }
 };
 
+struct ImageWords {                                          // the same for the general formats
+  const uint32_t* img;
+  __device__ __forceinline__ uint32_t operator()(int j) const { return img[(j >> 2) * 128 + (j & 3)]; }
+  __device__ __forceinline__ uint4 four(int j) const { return *reinterpret_cast<const uint4*>(img + 32 * j); }
+};
+
 // Scores of one key group (t as in score_group) and the group's constants of heads 2 r, 2 r + 1.  img: this lane's query words of the
 // group's chunk, four words a 16-byte load, 32 loads apart.
 template <bool GEN>
 __device__ __forceinline__ void score(uint8_t* kg, const KeyFmt& kf, int lane, int g, int r, const uint32_t* img, float (&t)[2][4], float (&cst)[2]) {
   if constexpr (GEN) {
-    auto word = [&](int j) { return img[(j >> 2) * 128 + (j & 3)]; };
+    const ImageWords word{img};
     group_constants_general(kg, kf, 1, g, r, word, cst);
     score_group_general(kg, kf, lane, r, word, t);
   } else {

@@ -160,7 +160,7 @@ __device__ __forceinline__ void group_constants(const uint8_t* kbuf, int n, int 
   c[0] = d[0]; c[1] = d[1];
 }
 
-// The same for the general layout (KeyFmt), one group (ga) or two.  word(j): this lane's query words of the groups' chunk: n2 / 8 pairs of q at slots
+// The same for the general layout (KeyFmt), one group (ga) or two.  word(j): this lane's query words of the groups' chunk, word.four(j) four of them from a multiple of four on: n2 / 8 pairs of q at slots
 // 8 j + 2 r, + 1; then pairs at the one-bit columns 8 j + 6 - 2 r, + 1: of q in plain mode, of Q's leading part and then of
 // its remainder for Eq. 5.
 template <bool TWO, typename Word>
@@ -186,12 +186,12 @@ __device__ __forceinline__ void score_general(const uint8_t* ga, const uint8_t* 
   };
 #pragma unroll 1
   for (int b = 0; b < n2b; ++b) {
-    uint32_t q[4], lo[NT], hi[NT];
+    uint4 q;
+    uint32_t lo[NT], hi[NT];
     uint4 sa, sb;
     const int at = kf.off_s2 + 64 * b + 8 * (r & 1);
     scales(at, sel2, sa.x, sa.y); scales(at + 16, sel2, sa.z, sa.w); scales(at + 32, sel2, sb.x, sb.y); scales(at + 48, sel2, sb.z, sb.w);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) q[j] = word(4 * b + j);
+    q = word.four(4 * b);
     const uint2 ca = *reinterpret_cast<const uint2*>(ga + 256 * b + lane * 8);
     uint32_t w[NT];
     if constexpr (TWO) {
@@ -203,23 +203,23 @@ __device__ __forceinline__ void score_general(const uint8_t* ga, const uint8_t* 
 #pragma unroll
     for (int m = 0; m < NT; ++m) { lo[m] = bits_meta(w[m]); hi[m] = bits_meta(w[m] >> 1); }
 #pragma unroll
-    for (int m = 0; m < NT; ++m) mma_sp<0>(a0[m], sa, row_pair_lo(q[0]), row_pair_hi(q[0]), row_pair_lo(q[1]), row_pair_hi(q[1]), lo[m]);
+    for (int m = 0; m < NT; ++m) mma_sp<0>(a0[m], sa, row_pair_lo(q.x), row_pair_hi(q.x), row_pair_lo(q.y), row_pair_hi(q.y), lo[m]);
 #pragma unroll
-    for (int m = 0; m < NT; ++m) mma_sp<0>(a1[m], sa, row_pair_lo(q[0]), row_pair_hi(q[0]), row_pair_lo(q[1]), row_pair_hi(q[1]), hi[m]);
+    for (int m = 0; m < NT; ++m) mma_sp<0>(a1[m], sa, row_pair_lo(q.x), row_pair_hi(q.x), row_pair_lo(q.y), row_pair_hi(q.y), hi[m]);
 #pragma unroll
-    for (int m = 0; m < NT; ++m) mma_sp<1>(a0[m], sb, row_pair_lo(q[2]), row_pair_hi(q[2]), row_pair_lo(q[3]), row_pair_hi(q[3]), lo[m]);
+    for (int m = 0; m < NT; ++m) mma_sp<1>(a0[m], sb, row_pair_lo(q.z), row_pair_hi(q.z), row_pair_lo(q.w), row_pair_hi(q.w), lo[m]);
 #pragma unroll
-    for (int m = 0; m < NT; ++m) mma_sp<1>(a1[m], sb, row_pair_lo(q[2]), row_pair_hi(q[2]), row_pair_lo(q[3]), row_pair_hi(q[3]), hi[m]);
+    for (int m = 0; m < NT; ++m) mma_sp<1>(a1[m], sb, row_pair_lo(q.z), row_pair_hi(q.z), row_pair_lo(q.w), row_pair_hi(q.w), hi[m]);
   }
   const int w1 = kf.n2 >> 3, nw1 = (kD - kf.n2) >> 3;
 #pragma unroll 1
   for (int b = 0; b < n1b; ++b) {
-    uint32_t q[4], e[NT];
+    uint4 q;
+    uint32_t e[NT];
     uint4 sa, sb;
     const int at = kf.off_s1 + 64 * b + 8 - 8 * (r & 1);
     scales(at, sel1, sa.x, sa.y); scales(at + 16, sel1, sa.z, sa.w); scales(at + 32, sel1, sb.x, sb.y); scales(at + 48, sel1, sb.z, sb.w);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) q[j] = word(w1 + 4 * b + j);
+    q = word.four(w1 + 4 * b);
     const uint32_t ca = *reinterpret_cast<const uint32_t*>(ga + kf.off_bits1 + 128 * b + lane * 4);
     const uint32_t cb = TWO ? *reinterpret_cast<const uint32_t*>(gb + kf.off_bits1 + 128 * b + lane * 4) : 0u;
 #pragma unroll
@@ -230,20 +230,17 @@ __device__ __forceinline__ void score_general(const uint8_t* ga, const uint8_t* 
     }
     if (kf.plain) {
 #pragma unroll
-      for (int m = 0; m < NT; ++m) mma_sp<0>(a0[m], sa, row_pair_hi(q[0]), row_pair_lo(q[0]), row_pair_hi(q[1]), row_pair_lo(q[1]), e[m]);
+      for (int m = 0; m < NT; ++m) mma_sp<0>(a0[m], sa, row_pair_hi(q.x), row_pair_lo(q.x), row_pair_hi(q.y), row_pair_lo(q.y), e[m]);
 #pragma unroll
-      for (int m = 0; m < NT; ++m) mma_sp<1>(a0[m], sb, row_pair_hi(q[2]), row_pair_lo(q[2]), row_pair_hi(q[3]), row_pair_lo(q[3]), e[m]);
+      for (int m = 0; m < NT; ++m) mma_sp<1>(a0[m], sb, row_pair_hi(q.z), row_pair_lo(q.z), row_pair_hi(q.w), row_pair_lo(q.w), e[m]);
     } else {
 #pragma unroll
       for (int piece = 0; piece < 2; ++piece) {
 #pragma unroll
-        for (int m = 0; m < NT; ++m) mma_sp<0>(a0[m], sa, sign_pair_hi(q[0]), sign_pair_lo(q[0]), sign_pair_hi(q[1]), sign_pair_lo(q[1]), e[m]);
+        for (int m = 0; m < NT; ++m) mma_sp<0>(a0[m], sa, sign_pair_hi(q.x), sign_pair_lo(q.x), sign_pair_hi(q.y), sign_pair_lo(q.y), e[m]);
 #pragma unroll
-        for (int m = 0; m < NT; ++m) mma_sp<1>(a0[m], sb, sign_pair_hi(q[2]), sign_pair_lo(q[2]), sign_pair_hi(q[3]), sign_pair_lo(q[3]), e[m]);
-        if (piece == 0) {
-#pragma unroll
-          for (int j = 0; j < 4; ++j) q[j] = word(w1 + nw1 + 4 * b + j);
-        }
+        for (int m = 0; m < NT; ++m) mma_sp<1>(a0[m], sb, sign_pair_hi(q.z), sign_pair_lo(q.z), sign_pair_hi(q.w), sign_pair_lo(q.w), e[m]);
+        if (piece == 0) q = word.four(w1 + nw1 + 4 * b);
       }
     }
   }

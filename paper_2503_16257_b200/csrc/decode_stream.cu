@@ -81,16 +81,21 @@ template <> struct Query<false> {
   }
 };
 template <> struct Query<true> {
+  struct Words {
+    const uint32_t* p;
+    __device__ __forceinline__ uint32_t operator()(int j) const { return __ldg(p + j * 32); }
+    __device__ __forceinline__ uint4 four(int j) const { return make_uint4((*this)(j), (*this)(j + 1), (*this)(j + 2), (*this)(j + 3)); }
+  };
   const uint32_t* p;                  // the words stay in global memory (L1): five formats share one instantiation
   __device__ __forceinline__ void load(const uint32_t* pp) { p = pp; }
   __device__ __forceinline__ void constants(const uint8_t* kbuf, const KeyFmt& kf, int n, int g, int r, float (&c)[2]) const {
-    group_constants_general(kbuf, kf, n, g, r, [&](int j) { return __ldg(p + j * 32); }, c);
+    group_constants_general(kbuf, kf, n, g, r, Words{p}, c);
   }
   __device__ __forceinline__ void score(uint8_t* ga, uint8_t* gb, const KeyFmt& kf, int lane, int r, float (&ta)[2][4], float (&tb)[2][4]) const {
-    score_groups_general(ga, gb, kf, lane, r, [&](int j) { return __ldg(p + j * 32); }, ta, tb);
+    score_groups_general(ga, gb, kf, lane, r, Words{p}, ta, tb);
   }
   __device__ __forceinline__ void score(uint8_t* ga, const KeyFmt& kf, int lane, int r, float (&t)[2][4]) const {
-    score_group_general(ga, kf, lane, r, [&](int j) { return __ldg(p + j * 32); }, t);
+    score_group_general(ga, kf, lane, r, Words{p}, t);
   }
 };
 
