@@ -310,12 +310,13 @@ __global__ void __launch_bounds__(kD) decode_merge_kernel(DecodeArgs a, int n_re
   // ---- the records: maxima and sums (lane j: record j, for the heads warp and warp + 4) and this lane's output fragments
   // of the first kRecAhead of them in one round of loads
   pdl_wait();
+  rec = behind_wait(rec);
   float2 head_ml[2];
 #pragma unroll
   for (int x = 0; x < 2; ++x) {
     const int k = warp + 4 * x;
     head_ml[x] = make_float2(-INFINITY, 0.0f);
-    if (k < rep && lane < n_parts) head_ml[x] = __ldg(reinterpret_cast<const float2*>(rec + (lane * kMaxRep + k) * kRecordFloats));
+    if (k < rep && lane < n_parts) head_ml[x] = *reinterpret_cast<const float2*>(rec + (lane * kMaxRep + k) * kRecordFloats);
   }
   constexpr int kRecAhead = 3;
   float rec_m[kRecAhead];
@@ -327,9 +328,9 @@ __global__ void __launch_bounds__(kD) decode_merge_kernel(DecodeArgs a, int n_re
     for (int j = 0; j < 4; ++j) rec_o[jp][j] = make_float2(0.0f, 0.0f);
     if (jp < n_parts && hd < rep) {
       const float* pr = rec + (jp * kMaxRep + hd) * kRecordFloats;
-      rec_m[jp] = __ldg(pr);
+      rec_m[jp] = *pr;
 #pragma unroll
-      for (int j = 0; j < 4; ++j) rec_o[jp][j] = __ldg(reinterpret_cast<const float2*>(pr + 2 + 32 * warp + 8 * j + 2 * r));
+      for (int j = 0; j < 4; ++j) rec_o[jp][j] = *reinterpret_cast<const float2*>(pr + 2 + 32 * warp + 8 * j + 2 * r);
     }
   }
   // ---- maxima and denominators over all parts
@@ -338,7 +339,7 @@ __global__ void __launch_bounds__(kD) decode_merge_kernel(DecodeArgs a, int n_re
     const int k = warp + 4 * x;
     float m = head_ml[x].x;
     if (k < rep)
-      for (int j = lane + 32; j < n_parts; j += 32) m = fmaxf(m, __ldg(rec + (j * kMaxRep + k) * kRecordFloats));
+      for (int j = lane + 32; j < n_parts; j += 32) m = fmaxf(m, load_settled(rec + (j * kMaxRep + k) * kRecordFloats));
 #pragma unroll
     for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
     m = fmaxf(m, m_res[x]);

@@ -130,15 +130,15 @@ struct ImageSource {
     const int r = lane & 3;
 #pragma unroll
     for (int ks = 0; ks < 4; ++ks) {
-      pa[ks] = __ldg(reinterpret_cast<const uint16_t*>(perm + kNA + 16 * ks + 2 * r));
-      pb[ks] = __ldg(reinterpret_cast<const uint16_t*>(perm + kNA + 16 * ks + 2 * r + 8));
+      pa[ks] = *reinterpret_cast<const uint16_t*>(perm + kNA + 16 * ks + 2 * r);
+      pb[ks] = *reinterpret_cast<const uint16_t*>(perm + kNA + 16 * ks + 2 * r + 8);
     }
 #pragma unroll
     for (int turn = 0; turn < kTurns; ++turn) {
       const int nt = min(warp + turn * kUnitWarps, 7);
-      two[turn] = __ldg(reinterpret_cast<const uint16_t*>(perm + 8 * nt + 2 * r));
+      two[turn] = *reinterpret_cast<const uint16_t*>(perm + 8 * nt + 2 * r);
 #pragma unroll
-      for (int ks = 0; ks < 4; ++ks) bw[turn][ks] = __ldg(reinterpret_cast<const uint4*>(dft.frag + ((ks * 8 + nt) * 32 + lane) * 4));
+      for (int ks = 0; ks < 4; ++ks) bw[turn][ks] = *reinterpret_cast<const uint4*>(dft.frag + ((ks * 8 + nt) * 32 + lane) * 4);
     }
   }
 };
@@ -187,7 +187,7 @@ __device__ __forceinline__ void make_images(uint32_t* img, const ImageSource& sr
 #pragma unroll
     for (int turn = 0; turn < kTurns; ++turn) {
       const int w = warp + turn * kUnitWarps;
-      two[turn] = w < n_pairs ? __ldg(reinterpret_cast<const uint16_t*>(perm + (w < w1 ? 8 * w + 2 * r : 8 * w + 6 - 2 * r))) : 0u;
+      two[turn] = w < n_pairs ? *reinterpret_cast<const uint16_t*>(perm + (w < w1 ? 8 * w + 2 * r : 8 * w + 6 - 2 * r)) : 0u;
     }
 #pragma unroll
     for (int turn = 0; turn < kTurns; ++turn) {
@@ -204,7 +204,7 @@ __device__ __forceinline__ void make_images(uint32_t* img, const ImageSource& sr
 #pragma unroll
         for (int c = 8 * part, i = 0; i < 8; ++c, ++i) {
           const float qv = q_at(perm[n2 + c]);
-          const float4 wa = __ldg(wt + 8 * c), wb = __ldg(wt + 8 * c + 1);
+          const float4 wa = wt[8 * c], wb = wt[8 * c + 1];
           y[0] = fmaf(qv, wa.x, y[0]); y[1] = fmaf(qv, wa.y, y[1]); y[2] = fmaf(qv, wa.z, y[2]); y[3] = fmaf(qv, wa.w, y[3]);
           y[4] = fmaf(qv, wb.x, y[4]); y[5] = fmaf(qv, wb.y, y[5]); y[6] = fmaf(qv, wb.z, y[6]); y[7] = fmaf(qv, wb.w, y[7]);
         }
@@ -373,7 +373,7 @@ __device__ __forceinline__ bool move_maximum(const float (&mu)[2], float (&m)[2]
 __device__ __forceinline__ void append_row(const DecodeArgs& a, int slab, uint8_t* slab_ptr, int lane) {
   if (a.append_row < 0) return;
   const uint4* srcp = reinterpret_cast<const uint4*>(lane < 16 ? a.k_new : a.v_new) + static_cast<int64_t>(slab) * 16 + (lane & 15);
-  reinterpret_cast<uint4*>(slab_ptr + (lane < 16 ? a.cv.kres_offset : a.cv.vres_offset))[a.append_row * 16 + (lane & 15)] = __ldg(srcp);
+  reinterpret_cast<uint4*>(slab_ptr + (lane < 16 ? a.cv.kres_offset : a.cv.vres_offset))[a.append_row * 16 + (lane & 15)] = *srcp;
 }
 
 // The slab's residual rows (n_res of them, the step's new row among them: append_row by warp 0 first) in the input type: scores on the tensor
@@ -389,7 +389,7 @@ __device__ __forceinline__ void add_residual(const DecodeArgs& a, const uint8_t*
   __half* Px = reinterpret_cast<__half*>(scratch + 8 * kResS * 4);
   uint4 qn[4];
 #pragma unroll
-  for (int j = 0; j < 4; ++j) qn[j] = live ? __ldg(reinterpret_cast<const uint4*>(qrow + 32 * j + 8 * r)) : make_uint4(0u, 0u, 0u, 0u);
+  for (int j = 0; j < 4; ++j) qn[j] = live ? *reinterpret_cast<const uint4*>(qrow + 32 * j + 8 * r) : make_uint4(0u, 0u, 0u, 0u);
   __syncthreads();                                         // the row is there, and nobody uses the scratch memory any more
   const uint8_t* kr = slab_ptr + cv.kres_offset;
   const float sl2 = a.scale * 1.4426950408889634f;
@@ -723,7 +723,7 @@ __global__ void __launch_bounds__(kUnitThreads, kPerSM) decode_block_kernel(Deco
         ep = cv.e_prefix(b);
         // where this block enters and leaves the two value streams
         auto stream_at = [&](int t, int& u, int& p) {
-          if (t <= T_q0) { p = static_cast<int>(__ldg(ep + t / kG)); u = t - p; }
+          if (t <= T_q0) { p = static_cast<int>(ep[t / kG]); u = t - p; }
           else { p = n_prot; u = u_fl0 + (t - T_q0); }
         };
         int ue, pe;
@@ -794,8 +794,8 @@ __global__ void __launch_bounds__(kUnitThreads, kPerSM) decode_block_kernel(Deco
         const int tg = (g_first + warp) * kG;                // first token of the warp's group
         const int t_end = (g_first + ng) * kG;
         if (STP) {
-          if (warp < ng && tg < T_q0) { e_word = __ldg(ew + g_first + warp); e_base = static_cast<int>(__ldg(ep + g_first + warp)); }
-          p_new = t_end <= T_q0 ? static_cast<int>(__ldg(ep + t_end / kG)) : n_prot;
+          if (warp < ng && tg < T_q0) { e_word = ew[g_first + warp]; e_base = static_cast<int>(ep[g_first + warp]); }
+          p_new = t_end <= T_q0 ? static_cast<int>(ep[t_end / kG]) : n_prot;
         }
         // ---- images of the chunks this unit touches (two at most; what they replace was last read before a barrier)
         {

@@ -99,7 +99,7 @@ __device__ __forceinline__ int head_exponent(const T* qrow, int sub, bool live) 
     const uint2* p = reinterpret_cast<const uint2*>(qrow + sub * (kD / NSUB));
 #pragma unroll
     for (int i = 0; i < kD / NSUB / 4; ++i) {
-      const uint2 v = __ldg(p + i);
+      const uint2 v = p[i];
       const float2 a = Elem<T>::to_float2(v.x), b = Elem<T>::to_float2(v.y);
       m = fmaxf(m, fmaxf(fmaxf(fabsf(a.x), fabsf(a.y)), fmaxf(fabsf(b.x), fabsf(b.y))));
     }

@@ -52,8 +52,8 @@ template <> struct Query<false> {
   __device__ __forceinline__ void load(const uint32_t* pp) {
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
-      q[j] = __ldg(pp + j * 32);
-      const uint32_t h = __ldg(pp + (8 + j) * 32), l = __ldg(pp + (16 + j) * 32);
+      q[j] = pp[j * 32];
+      const uint32_t h = pp[(8 + j) * 32], l = pp[(16 + j) * 32];
       const int at = (j >> 2) * 8 + (j & 3);
       qh[at] = sign_pair_hi(h); qh[at + 4] = sign_pair_lo(h);
       ql[at] = sign_pair_hi(l); ql[at + 4] = sign_pair_lo(l);
@@ -83,7 +83,7 @@ template <> struct Query<false> {
 template <> struct Query<true> {
   struct Words {
     const uint32_t* p;
-    __device__ __forceinline__ uint32_t operator()(int j) const { return __ldg(p + j * 32); }
+    __device__ __forceinline__ uint32_t operator()(int j) const { return p[j * 32]; }
     __device__ __forceinline__ uint4 four(int j) const { return make_uint4((*this)(j), (*this)(j + 1), (*this)(j + 2), (*this)(j + 3)); }
   };
   const uint32_t* p;                  // the words stay in global memory (L1): five formats share one instantiation
@@ -163,8 +163,8 @@ __device__ __forceinline__ void score_unit(const DecodeArgs& a, int slab, uint8_
 // The factors of heads 2 r, 2 r + 1 that turn a score in the units of the normalised query into a base-2 logit (word 24 of lane 4 h
 // holds head h's; prep_slab points at the lane's own words).
 __device__ __forceinline__ void head_factors(const uint32_t* prep_slab, int lane, int r, float (&sl2)[2]) {
-  sl2[0] = __uint_as_float(__ldg(prep_slab + 24 * 32 - lane + 8 * r));
-  sl2[1] = __uint_as_float(__ldg(prep_slab + 24 * 32 - lane + 8 * r + 4));
+  sl2[0] = __uint_as_float(prep_slab[24 * 32 - lane + 8 * r]);
+  sl2[1] = __uint_as_float(prep_slab[24 * 32 - lane + 8 * r + 4]);
 }
 
 // Probabilities of group gi: P[nt] = binary16 pair of heads 2 r, 2 r + 1 and token 8 nt + g.
@@ -600,7 +600,7 @@ __global__ void __launch_bounds__(kStreamWarps * 32, kStreamStpCtasPerSM) decode
       ep = cv.e_prefix(b);
       // where the run enters and leaves the two value streams
       auto streams_at = [&](int t, int& u, int& p) {
-        if (t <= T_q0) { p = static_cast<int>(__ldg(ep + t / kG)); u = t - p; }
+        if (t <= T_q0) { p = static_cast<int>(ep[t / kG]); u = t - p; }
         else { p = n_prot; u = u_fl0 + (t - T_q0); }
       };
       int t_begin, p_begin, t_stop, p_stop;
@@ -631,8 +631,8 @@ __global__ void __launch_bounds__(kStreamWarps * 32, kStreamStpCtasPerSM) decode
     {
       const int gl = t_unit / kG + lane;
       if (lane <= ng && gl * kG <= T_q0) {
-        e_base_l = static_cast<int>(__ldg(ep + gl));
-        if (lane < ng && gl * kG < T_q0) e_word_l = __ldg(ew + gl);
+        e_base_l = static_cast<int>(ep[gl]);
+        if (lane < ng && gl * kG < T_q0) e_word_l = ew[gl];
       }
     }
     // ---- scores of the unit's groups into the key buffer (raw scores, then the group's constant)

@@ -8,8 +8,21 @@ namespace vidkv {
 // Programmatic dependent launch: a kernel launched with the stream-serialization attribute may start
 // while the kernel before it still runs; pdl_wait() returns once that kernel has completed and its
 // writes are visible (a no-op for an ordinary launch), pdl_release() lets the kernel after this one start.
+// Behind the wait, global memory is read through ordinary loads.  A read-only load (__ldg) is for data that nobody writes while
+// the kernel runs, which what the kernel before leaves is not, and nothing but its address keeps the compiler from moving it ahead of the wait.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// For a chain of such loads that should all be under way at once: a pointer that is known from here (behind the wait) on, and a load
+// through it that the compiler may schedule as freely as a read-only one (nobody writes the data any more until the kernel ends).
+__device__ __forceinline__ const float* behind_wait(const float* p) {
+  asm volatile("" : "+l"(p)::"memory");
+  return p;
+}
+__device__ __forceinline__ float load_settled(const float* p) {
+  float v;
+  asm("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  return v;
+}
 // Launch `kernel` so that it may overlap the tail of the previous kernel on `stream` (it must call pdl_wait()
 // before touching anything that kernel writes).
 template <typename... KArgs, typename... Args>
@@ -39,8 +52,14 @@ __device__ __forceinline__ void copy_residual_rows(const KSrc& src, int64_t t_be
   const int lb = slab / cv.H_kv, h = slab % cv.H_kv;
   const uint16_t* base = static_cast<const uint16_t*>(src.ptr) + static_cast<int64_t>(lb) * src.stride_b + h * src.stride_h;
   uint4* dst = reinterpret_cast<uint4*>(cv.slab(layer0 + lb / cv.B, lb % cv.B, h) + res_offset);
-  for (int i = threadIdx.x; i < n_tok * 16; i += blockDim.x)
-    dst[i] = __ldg(reinterpret_cast<const uint4*>(base + (t_begin + (i >> 4)) * src.stride_t) + (i & 15));
+  auto piece = [&](int i) { return reinterpret_cast<const uint4*>(base + (t_begin + (i >> 4)) * src.stride_t)[i & 15]; };
+  const int n = n_tok * 16, step = blockDim.x;
+  for (int i = threadIdx.x; i < n; i += 2 * step) {         // two loads under way per thread
+    const bool two = i + step < n;
+    const uint4 a = piece(i), b = two ? piece(i + step) : a;
+    dst[i] = a;
+    if (two) dst[i + step] = b;
+  }
 }
 
 // Token-selection data handed to the value quantizer (NULL lists = no protection).

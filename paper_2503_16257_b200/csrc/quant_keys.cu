@@ -54,7 +54,7 @@ __global__ void __launch_bounds__(256, 5) k_range_kernel(KSrc src, int64_t T_tok
   bool any = false;
   int64_t t = t0 + row;
   if (t < t1) {
-    const uint4 v = __ldg(reinterpret_cast<const uint4*>(base + t * src.stride_t) + lane16);
+    const uint4 v = reinterpret_cast<const uint4*>(base + t * src.stride_t)[lane16];
     const V* pv = reinterpret_cast<const V*>(&v);
 #pragma unroll
     for (int i = 0; i < 4; ++i) { mn[i] = pv[i]; mx[i] = pv[i]; }
@@ -64,7 +64,7 @@ __global__ void __launch_bounds__(256, 5) k_range_kernel(KSrc src, int64_t T_tok
   for (; t + 48 < t1; t += 64) {                       // four rows in flight per thread
     uint4 v[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) v[k] = __ldg(reinterpret_cast<const uint4*>(base + (t + 16 * k) * src.stride_t) + lane16);
+    for (int k = 0; k < 4; ++k) v[k] = reinterpret_cast<const uint4*>(base + (t + 16 * k) * src.stride_t)[lane16];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       const V* pv = reinterpret_cast<const V*>(&v[k]);
@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(256, 5) k_range_kernel(KSrc src, int64_t T_tok
     }
   }
   for (; t < t1; t += 16) {
-    const uint4 v = __ldg(reinterpret_cast<const uint4*>(base + t * src.stride_t) + lane16);
+    const uint4 v = reinterpret_cast<const uint4*>(base + t * src.stride_t)[lane16];
     const V* pv = reinterpret_cast<const V*>(&v);
 #pragma unroll
     for (int i = 0; i < 4; ++i) { mn[i] = P::mn(mn[i], pv[i]); mx[i] = P::mx(mx[i], pv[i]); }

@@ -389,7 +389,7 @@ __global__ void __launch_bounds__(kEncThreads, 2) k_encode_kernel(KSrc src, int6
       for (int part = 0; part < Enc<T>::kParts; ++part)
 #pragma unroll
         for (int j = 0; j < 2; ++j)
-          wv[part][j] = __ldg(reinterpret_cast<const uint4*>(g_dft_w + (Enc<T>::kTab + part) * 4096) + tid + 256 * j);
+          wv[part][j] = reinterpret_cast<const uint4*>(g_dft_w + (Enc<T>::kTab + part) * 4096)[tid + 256 * j];
       // TopK (Algorithm 3): rank(c) = channels before c in (range descending, index ascending) order, two threads per
       // channel; the first 64 are the anomalous ones.  Every block does it for the slabs it meets, about 0.5 us, where a
       // kernel of its own took 3 us and a launch gap per call.

@@ -94,7 +94,7 @@ __device__ __forceinline__ void ternary_supergroup(uint8_t* vsm, KSrc src, int64
 #pragma unroll
     for (int k = 0; k < kRowsPerThread; ++k) {
       const int row = row0 + kVThreads / 16 * k;
-      tok[k] = row < n_rows ? (idx ? __ldg(idx + u0 + row) : static_cast<int>(u0) + row) : -1;
+      tok[k] = row < n_rows ? (idx ? idx[u0 + row] : static_cast<int>(u0) + row) : -1;
     }
 #pragma unroll
     for (int k = 0; k < kRowsPerThread; ++k) {
@@ -231,13 +231,15 @@ __device__ __forceinline__ void protect_groups(uint8_t* vsm, const KSrc& src, in
     const int lane16 = tid & 15, row = tid >> 4;
     int tok[kG / 8];
 #pragma unroll
-    for (int k = 0; k < kG / 8; ++k) tok[k] = row + 8 * k < n_rows ? __ldg(idx + p0 + row + 8 * k) : -1;
+    for (int k = 0; k < kG / 8; ++k) tok[k] = row + 8 * k < n_rows ? idx[p0 + row + 8 * k] : -1;
+    uint4 v[kG / 8];
 #pragma unroll
     for (int k = 0; k < kG / 8; ++k) {
-      uint4 v = make_uint4(0, 0, 0, 0);
-      if (tok[k] >= 0) v = __ldg(reinterpret_cast<const uint4*>(base + static_cast<int64_t>(tok[k]) * src.stride_t) + lane16);
-      reinterpret_cast<uint4*>(tile + (row + 8 * k) * kPRow)[lane16] = v;
+      v[k] = make_uint4(0, 0, 0, 0);
+      if (tok[k] >= 0) v[k] = reinterpret_cast<const uint4*>(base + static_cast<int64_t>(tok[k]) * src.stride_t)[lane16];
     }
+#pragma unroll
+    for (int k = 0; k < kG / 8; ++k) reinterpret_cast<uint4*>(tile + (row + 8 * k) * kPRow)[lane16] = v[k];
   }
   __syncthreads();
   uint8_t* pg = cv.slab(layer, b, h) + cv.prot_offset + pgroup * kPGBytes;
