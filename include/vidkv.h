@@ -389,7 +389,8 @@ vidkv_status_t vidkv_attend_noalloc(const vidkv_config_t* cfg, const void* cache
  * one partial result per slab it touches; calls of a few thousand units at most take another
  * kernel, whose blocks walk stretches of units together.
  * vidkv_debug_set_decode_plan forces run_units (>= 1), and with it the first of the two kernels, for later
- * vidkv_decode_attention calls on this handle; 0 leaves the choice to the library.  A forced plan that needs more partial records
+ * vidkv_decode_attention calls on this handle; -1 forces the second (calls of up to two million units, and
+ * triples of calls whose every run is one unit); 0 leaves the choice to the library.  A forced plan that needs more partial records
  * than the workspace holds makes the decode call return VIDKV_ERR_CAPACITY.
  * vidkv_debug_decode_plan (host only) reports the plan for given token counts on a device with
  * sm_count multiprocessors: plan_out[8] = { units per slab, run_units, runs (= warps),

@@ -347,7 +347,8 @@ class VidKVCache:
         _check("vidkv_set_profile_events", self.lib.vidkv_set_profile_events(self.handle, a, b))
 
     def debug_set_decode_plan(self, run_units: int = 0):
-        """Test hook: force the run length (160-token units per warp) of later decode calls; 0 = choose."""
+        """Test hook: force the run length (160-token units per warp) of later decode calls; -1 = the
+        small-call kernel, 0 = choose."""
         _check("vidkv_debug_set_decode_plan", self.lib.vidkv_debug_set_decode_plan(self.handle, run_units))
 
     def status(self) -> int:

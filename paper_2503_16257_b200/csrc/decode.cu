@@ -13,6 +13,7 @@ namespace vidkv {
 namespace {
 
 constexpr int kMaxSMs = 256;        // multiprocessor count the sizing formulas assume at most
+constexpr int64_t kMostForcedUnits = 1 << 21;   // the block kernel multiplies units by blocks in 32 bits
 // Work up to which a call goes to the block kernel: units of its longest block times the blocks that share a multiprocessor.  It has
 // one launch and a parallel merge where the stream kernel has three launches, a warp per run and one merge block per slab, but takes
 // half as many instructions again per unit (every warp of the block pays the unit's loop).  So the line rises with the units of a
@@ -134,7 +135,7 @@ DecodePlan plan_decode(const LayerState& st, int64_t n_slabs, bool stp, bool gen
   }
   const int64_t work = cut.longest * p.blocks_per_sm + (general && !stp && (cut.straddles || p.blocks_per_sm == kMoreBlocksPerSM) ? 3 : 0);
   const bool block = work <= most_block_work(p.units_per_slab, stp, cut.straddles);
-  if (p.n_units == 0 || (block && force_run_units == 0 && (!partial || run == 1))) {
+  if (p.n_units == 0 || ((block || (force_run_units < 0 && p.n_units < kMostForcedUnits)) && force_run_units <= 0 && (!partial || run == 1))) {
     p.n_blocks = static_cast<int32_t>(cut.even > 0 ? cut.even : p.n_units < cut.blocks ? p.n_units : cut.blocks);
     p.records = (p.n_blocks + n_slabs) * kMaxRep;
     p.res_blocks = st.n_res > 0 && cut.longest <= 1 ? static_cast<int32_t>(n_slabs) : 0;

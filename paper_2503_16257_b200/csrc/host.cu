@@ -117,7 +117,7 @@ struct vidkv_cache {
   uint8_t* workspace;
   bool sel_set;
   int64_t sel_T, n_prot;
-  int dbg_run_units = 0;        // test hook: forced run length of the stream kernels (0 = choose)
+  int dbg_run_units = 0;        // test hook: forced run length of the stream kernels (0 = choose, -1 = the small-call kernel)
   int mm_parity = 0;            // which min / max buffer the next key quantization accumulates into
   int64_t mm_dirty[2] = {0, 0}; // words of each buffer written since it was last re-armed
   bool clear_counters = false;  // the next prompt's first key quantization clears the decode kernel's arrival counters
@@ -519,7 +519,7 @@ vidkv_status_t vidkv_debug_withhold_once(int32_t what) {
 }
 
 vidkv_status_t vidkv_debug_set_decode_plan(vidkv_cache_t* h, int32_t run_units) {
-  if (!h || run_units < 0) return VIDKV_ERR_INVALID_ARG;
+  if (!h || run_units < -1) return VIDKV_ERR_INVALID_ARG;
   h->dbg_run_units = run_units;
   return VIDKV_OK;
 }
@@ -531,7 +531,7 @@ vidkv_status_t vidkv_debug_decode_plan(const vidkv_config_t* cfg, int64_t n_pref
   const vidkv_status_t st = check_config(cfg);
   if (st != VIDKV_OK) return st;
   if (n_layers < 1 || n_layers > cfg->L || n_prefill_quantized < 0 || n_prefill_quantized % kG || n_flushed_chunks < 0 ||
-      n_residual < 0 || n_residual > kR || n_protected < 0 || sm_count < 1 || run_units < 0)
+      n_residual < 0 || n_residual > kR || n_protected < 0 || sm_count < 1 || run_units < -1)
     return VIDKV_ERR_INVALID_ARG;
   Layout L;
   compute_layout(*cfg, &L);

@@ -186,7 +186,7 @@ struct DecodePlan {
 };
 // stp: the cache holds protected tokens (the stream kernel for them keeps fewer warps per multiprocessor).
 // general: a key format other than the default.
-// force_run_units: 0 = choose; otherwise the test hook's value (always the stream kernel).
+// force_run_units: 0 = choose; otherwise the test hook's value: > 0 the stream kernel with runs of that many units, -1 the block kernel.
 // partial: the call leaves (maximum, sum, unnormalised output) triples.  Their maximum is the one the walk has kept, which
 // need not be the largest logit, so it depends on how the units are cut: such calls keep runs of equal length, and take the
 // block kernel only where every run is one unit (its maximum is then exact however blocks share the units).

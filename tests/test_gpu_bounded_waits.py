@@ -36,7 +36,7 @@ DECODE_SHAPES = pytest.mark.parametrize("L,B,T,run_units", [
     (1, 1, 640, 1),      # stream kernel, nothing else in flight
     (1, 1, 640, 3),      # stream kernel, runs that cross slabs: the next unit's keys are in flight when the wait runs out
     (1, 1, 640, 0),      # small-call kernel, a unit per block: the wait behind the last unit
-    (12, 4, 2029, 0),    # small-call kernel, four or five units per block, slabs of 13: the exit inside the walk
+    (12, 4, 2029, -1),   # small-call kernel, four or five units per block, slabs of 13: the exit inside the walk
 ])
 
 
@@ -80,6 +80,6 @@ def test_decode_wait_runs_out_and_reports_timeout(L, B, T, run_units):
     before = P.vidkv_launch_count()
     P.vidkv_debug_withhold_once(2)
     cache.decode_attention(0, L, q, k, v, out)
-    assert P.vidkv_launch_count() - before == (3 if run_units else 1)      # the kernel that the case is about
+    assert P.vidkv_launch_count() - before == (3 if run_units > 0 else 1)      # the kernel that the case is about
     assert cache.status() == -7
     _fresh_run_is_fine()

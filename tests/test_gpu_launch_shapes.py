@@ -235,13 +235,15 @@ def test_seeded_random_shapes_and_run_lengths(name, T, B, L, p, run_units, steps
     ("llava", 1, 2, 26000, 0.93, 2, 0),      # long protected stream, 1304 units
 ])
 def test_small_calls_in_one_launch(name, L, B, T, p, steps, check_from):
-    """Calls of up to seven units (four with protected tokens) per block: block and slab boundaries inside and on unit
-    boundaries, the residual with a block of its own and with the slab's last block, every depth of the merge tree;
-    the step behind the last one leaves triples."""
+    """Block and slab boundaries inside and on unit boundaries, the residual with a block of its own and with the slab's last
+    block, every depth of the merge tree; the step behind the last one leaves triples."""
     samples = sorted({(0, 0, 0), (L - 1, B - 1, 3), (L // 2, B // 2, 1)})
     run = SampledRun(name, L, B, T, p, steps + 1, samples)
+    run.cache.debug_set_decode_plan(run_units=-1)            # whichever kernel would be faster here
     for s in range(steps):
+        before = run.P.vidkv_launch_count()
         run.decode(check=s >= check_from)
+        assert run.P.vidkv_launch_count() - before == 1 or run.cache.layer_state(0)["n_residual"] == 0   # (a flush has its own)
     run.decode(triples=True)
     assert run.cache.status() == 0
 
