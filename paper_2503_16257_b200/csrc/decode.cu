@@ -2,7 +2,7 @@
 // work (plan_decode), the launch sequence, and the last kernel of a step, which merges the
 // partial records of the attention kernels by log-sum-exp and, for caches without protected
 // tokens, attends to the FP16 / BF16 residual itself.
-#include <algorithm>
+#include <cmath>
 #include <numeric>
 #include <type_traits>
 
@@ -14,28 +14,46 @@ namespace {
 
 constexpr int kMaxSMs = 256;        // multiprocessor count the sizing formulas assume at most
 constexpr int64_t kMostForcedUnits = 1 << 21;   // the block kernel multiplies units by blocks in 32 bits
-// Work up to which a call goes to the block kernel: units of its longest block times the blocks that share a multiprocessor.  It has
-// one launch and a parallel merge where the stream kernel has three launches, a warp per run and one merge block per slab, but takes
-// half as many instructions again per unit (every warp of the block pays the unit's loop).  So the line rises with the units of a
-// slab: few and long slabs leave the stream kernel's merge with hundreds of records a block.  Measured, us per call (half
-// of the channels two-bit), block / stream kernel, at the work in brackets:
-//   slabs of up to 8 units  448 slabs of 3 (12) 22.9 / 25.2, 448 of 5 (16) 35.5 / 32.3, 224 of 8 (16) 27.5 / 23.6, 448 of 8 (24) 44.0 / 36.1
-//   longer                  64 of 14 (9) 19.9 / 21.1, 168 of 12 (16) 28.7 / 29.4, 96 of 24 (16) 28.8 / 29.3, 112 of 22 (20) 32.0 / 29.3,
-//                           64 of 40 (18) 33.1 / 31.2, 56 of 50 (20) 34.2 / 31.4, 32 of 70 (16) 29.7 / 35.3, 32 of 100 (24) 37.4 / 37.4,
-//                           32 of 140 (32) 45.8 / 44.3, 16 of 79 (9) 21.7 / 31.6, 16 of 200 (24) 37.4 / 46.2, 16 of 400 (45) 58.0 / 60.1,
-//                           8 of 600 (33) 50.0 / 70.1, 4 of 160 (6) 19.7 / 39.6, 4 of 900 (27) 42.0 / 99.1, 4 of 1225 (36) 50.3 / 104.4
-//   of 9 to 19, no block in two slabs  128 of 18 (18) 29.0 / 30.4, 192 of 13 (20) 32.4 / 30.6 (kept here: the tests of the bounded waits
-//                           hold the kernel to this shape); with blocks in two slabs 224 of 11 (20) 32.9 / 29.7
-//   with protected tokens   112 slabs of 4 (6) 22.7 / 24.7, 224 of 8 (24) 41.8 / 33.2, 112 of 10 (12) 31.3 / 27.3, 64 of 14 (9) 28.7 / 27.1,
-//                           64 of 28 (15) 37.1 / 33.5, 32 of 40 (12) 32.4 / 35.3, 32 of 70 (18) 41.4 / 38.5, 16 of 79 (9) 28.9 / 41.6,
-//                           16 of 140 (18) 41.1 / 44.4, 16 of 200 (24) 50.2 / 51.6, 16 of 400 (45) 79.5 / 70.3, 4 of 600 (15) 44.0 / 80.6
-static int64_t most_block_work(int64_t units_per_slab, bool stp, bool straddles) {
-  const int64_t S = units_per_slab;
-  if (stp) return std::min<int64_t>(6 + S / 6, 40);
-  if (S < 9) return 14;
-  if (S < 20 && !straddles) return 20;
-  return std::min(std::max<int64_t>(14 + S / 10, 16), int64_t{40});
-}
+// What the choice between the attention kernels goes by: estimated microseconds of a call, linear in what it is made of.  The block kernel
+// has one launch and a parallel merge; the stream kernel has three launches, a merge block per slab that reads the slab's records one behind the
+// other, and a third fewer instructions per unit.  The block kernel comes with three blocks on a multiprocessor and 128 registers a thread, or
+// with four and 96 (which keep some of the loop's state in local memory); not for general key formats with protected tokens, where four
+// are slower throughout.  The coefficients are least-squares fits to 650 measured calls of 4 to 1120 slabs and 1 to 1800 units a slab, the ones
+// near the line weighted most, and moved within a few percent so that the choice is the faster kernel there: over those calls it costs 0.2 % more than the
+// fastest of the three, 6.4 % at most.  us, three blocks / four / stream:
+//   half of the channels two-bit  112 slabs of 2 units 10.8 / 13.0 / 15.8, 448 of 3 26.1 / 22.3 / 25.1, 448 of 4 29.0 / 26.5 / 26.3, 448 of 8 40.9 / 43.6 / 35.1,
+//     224 of 8 28.4 / 28.3 / 24.6, 112 of 20 29.7 / 28.0 / 28.7, 192 of 13 32.5 / 31.8 / 28.9, 176 of 13 31.2 / 32.5 / 28.8, 128 of 18 28.8 / 32.6 / 29.3,
+//     32 of 140 44.8 / 44.9 / 43.3, 16 of 79 20.8 / 24.5 / 30.8, 16 of 400 56.2 / 57.3 / 59.2, 4 of 1225 47.8 / 49.6 / 103.5
+//   k = 0.75, plain one-bit code  112 of 2 10.3 / 13.0 / 18.4, 448 of 2 22.5 / 19.6 / 24.2, 448 of 3 26.2 / 25.3 / 25.3, 112 of 10 22.9 / 21.5 / 24.6, 112 of 20 30.7 / 32.2 / 31.9,
+//     96 of 24 31.5 / 32.3 / 32.7, 192 of 13 34.0 / 36.9 / 32.6, 16 of 200 39.2 / 42.8 / 48.2, 16 of 400 65.5 / 70.7 / 68.3
+//   k = 0.75, Eq. 5 (longer preparation in every block)  112 of 2 12.9 / 15.9 / 18.5, 448 of 3 31.5 / 28.0 / 26.4, 112 of 14 31.3 / 29.3 / 26.4, 32 of 40 31.3 / 29.3 / 28.8
+//   a fifth of the tokens protected, half of the channels two-bit  112 of 4 22.4 / 21.8 / 24.5, 224 of 4 27.1 / 29.7 / 25.2, 448 of 2 - / 26.3 / 26.8, 560 of 3 - / 33.0 / 36.8,
+//     592 of 4 - / 40.1 / 34.9, 64 of 14 27.2 / 32.1 / 26.6, 32 of 40 32.6 / - / 33.5, 16 of 300 64.8 / - / 61.2, 8 of 600 61.7 / - / 71.8
+//   the same, k = 0.75, plain     224 of 4 29.0 / 41.3 / 27.5, 64 of 14 27.8 / 42.8 / 28.6, 16 of 200 55.8 / - / 55.3, 16 of 300 74.3 / - / 69.7
+struct BlockCost {
+  double base;
+  double unit;      // a unit of the longest stretch
+  double load;      // a unit per multiprocessor
+  double entry;     // a slab that a block enters behind its first
+  double join;      // a level of the merge tree
+  double slab;      // a hundred slabs
+};
+struct StreamCost {
+  double base;
+  double unit;      // a unit of the longest run
+  double load;      // a unit per warp of the device
+  double record;    // a record of a slab
+  double slab;      // a hundred slabs
+};
+struct CallCost { BlockCost three, four; StreamCost stream; };
+// [protected tokens][format: default, general without Eq. 5, general with it]
+constexpr CallCost kCallCost[2][3] = {
+    {{{7.83, 2.16, 0.30, 3.49, 1.91, 0.46}, {9.93, 3.38, 0.16, 4.53, 1.36, 0.29}, {12.76, 2.28, 6.67, 0.16, 0.97}},
+     {{6.02, 2.42, 0.45, 2.74, 2.27, 0.71}, {8.08, 4.67, 0.20, 3.74, 1.12, 0.40}, {12.88, 5.17, 4.26, 0.18, 0.90}},
+     {{9.28, 2.47, 0.45, 4.72, 1.96, 0.43}, {10.88, 4.62, 0.23, 4.61, 1.25, 0.36}, {13.47, 5.41, 4.23, 0.20, 0.95}}},
+    {{{12.20, 3.77, 0.15, 0.0, 2.02, -0.38}, {17.03, 4.68, 0.31, 0.0, 1.66, -0.28}, {15.93, 5.20, 2.22, 0.18, 0.86}},
+     {{9.81, 4.83, 0.10, 0.0, 2.54, -0.25}, {}, {16.80, 7.04, 2.08, 0.18, 0.65}},
+     {{12.74, 4.63, 0.18, 0.0, 2.33, -0.29}, {}, {17.19, 7.43, 1.84, 0.19, 0.82}}}};
 
 }  // namespace
 
@@ -58,7 +76,7 @@ static int64_t join_counters(int64_t n) {
   return c;
 }
 
-DecodePlan plan_decode(const LayerState& st, int64_t n_slabs, bool stp, bool general, int sm_count, int force_run_units, bool partial) {
+DecodePlan plan_decode(const LayerState& st, int64_t n_slabs, bool stp, const KeyFmt& kf, int sm_count, int force_run_units, bool partial) {
   DecodePlan p = {};
   const int64_t T_qt = st.T_q0 + st.n_flush * kR;
   p.n_chunks = T_qt > 0 ? 1 + static_cast<int32_t>(st.n_flush) : 0;
@@ -93,48 +111,44 @@ DecodePlan plan_decode(const LayerState& st, int64_t n_slabs, bool stp, bool gen
   };
   p.slab_parts = static_cast<int32_t>(most_parts(p.n_runs));
   p.records = (p.n_runs + n_slabs) * kMaxRep;
-  // The block kernel's cut for `per_sm` blocks on each multiprocessor.
-  struct BlockCut { int64_t blocks, longest, even; bool straddles; };
-  const auto cut_for = [&](int per_sm) -> BlockCut {
-    BlockCut c = {static_cast<int64_t>(sms) * per_sm, 0, 0, false};
-    c.longest = (p.n_units + c.blocks - 1) / c.blocks;
+  // The block kernel's cut for `per_sm` blocks on each multiprocessor, and its estimated time.
+  struct BlockCut { int64_t blocks, longest, even; bool straddles; double us; };
+  const CallCost& cost = kCallCost[stp][kf.general == 0 ? 0 : kf.plain || kf.n1() == 0 ? 1 : 2];
+  const auto cut_for = [&](int per_sm, const BlockCost& c) -> BlockCut {
+    BlockCut cut = {static_cast<int64_t>(sms) * per_sm, 0, 0, false, 0.0};
+    cut.longest = (p.n_units + cut.blocks - 1) / cut.blocks;
     // A block that goes on in the next slab pays for query images, rings and join twice: where the proportional cut makes such
     // blocks (slab s then begins d units * slabs / blocks after a block does, d running through the multiples of
     // gcd(blocks, slabs)), every slab gets its own blocks, if it can without a longer stretch.  us, straddling / not: 64 slabs
     // of 14 units 28.9 / 21.8, 448 of 3 28.2 / 21.0; with protected tokens 42.3 / 31.7 and 45.2 / 30.0.
-    c.straddles = p.n_units > 0 && p.n_units - std::gcd(c.blocks, n_slabs) * p.units_per_slab >= c.blocks;
-    if (c.straddles) {
-      const int64_t share = c.blocks / n_slabs, even = share > 0 ? (p.units_per_slab + share - 1) / share : INT32_MAX;
-      if (stp || even <= c.longest) {
-        c.longest = even;
-        c.even = n_slabs * (share < p.units_per_slab ? share : p.units_per_slab);
-        c.straddles = false;
+    cut.straddles = p.n_units > 0 && p.n_units - std::gcd(cut.blocks, n_slabs) * p.units_per_slab >= cut.blocks;
+    bool apart = true;                                     // with protected tokens blocks never share slabs' ends
+    if (cut.straddles) {
+      const int64_t share = cut.blocks / n_slabs, even = share > 0 ? (p.units_per_slab + share - 1) / share : 0;
+      apart = share > 0;
+      if (share > 0 && (stp || even <= cut.longest)) {
+        cut.longest = even;
+        cut.even = n_slabs * (share < p.units_per_slab ? share : p.units_per_slab);
+        cut.straddles = false;
       }
     }
-    return c;
+    if (p.n_units == 0) return cut;
+    const int64_t entered = cut.straddles ? (cut.longest - 1 + p.units_per_slab - 1) / p.units_per_slab : 0;
+    int levels = 0;
+    for (int64_t parts = (p.units_per_slab + cut.longest - 1) / cut.longest; parts > 1; parts = (parts + kJoin - 1) / kJoin) ++levels;
+    cut.us = c.base + c.unit * cut.longest + c.load * p.n_units / sms + c.entry * entered + c.join * levels + c.slab * 0.01 * n_slabs;
+    if (stp && !apart) cut.us = INFINITY;
+    return cut;
   };
-  // Without protected tokens there are two variants: three blocks on a multiprocessor with 128 registers a thread, or four with 96, which
-  // keep some of the loop's state in local memory.  Three, unless that makes the longest stretch more than a unit longer, has
-  // blocks that go on in the next slab (worth two units) where four have none, or leaves one of the one-unit blocks and residuals of a
-  // short call waiting for another to end.  us a call, four / three: 16 slabs of 79 units 24.2 / 20.9, 64 of 14 (2 and 3 units
-  // a block) 21.5 / 19.2, 4 of 160 21.5 / 19.4; but 112 of 10 (2; 3 with blocks in two slabs) 20.5 / 23.7, 32 of 40 24.9 / 27.1, 128 of 3 and
-  // their residuals 12.9 / 14.1, 112 of 20 (4; 6) 28.2 / 29.3.  The general key formats' loop has more of that state, and three blocks are better
-  // wherever every slab has a block: 112 of 20 33.4 / 31.6, 16 of 200 (6; 8) 44.7 / 40.6, 128 of 3 13.4 / 13.0; 448 of 3 25.8 / 26.9.
-  // With protected tokens four would not fit in the registers at all (128 slabs of 3 20.7 / 16.2).
-  BlockCut cut = cut_for(kBlocksPerSM);
+  BlockCut cut = cut_for(kBlocksPerSM, cost.three);
   p.blocks_per_sm = kBlocksPerSM;
-  if (!stp) {
-    const BlockCut more = cut_for(kMoreBlocksPerSM);
-    bool fewer = n_slabs <= cut.blocks;
-    if (general && cut.straddles && !more.straddles && more.longest * kMoreBlocksPerSM < cut.longest * kBlocksPerSM) fewer = false;
-    if (fewer && !general) {
-      if (more.longest <= 1) fewer = p.n_units + (st.n_res > 0 ? n_slabs : 0) <= cut.blocks;
-      else fewer = cut.longest + 2 * cut.straddles <= more.longest + 2 * more.straddles + 1;
-    }
-    if (!fewer) { cut = more; p.blocks_per_sm = kMoreBlocksPerSM; }
+  if (!stp || !kf.general) {
+    const BlockCut more = cut_for(kMoreBlocksPerSM, cost.four);
+    if (more.us < cut.us) { cut = more; p.blocks_per_sm = kMoreBlocksPerSM; }
   }
-  const int64_t work = cut.longest * p.blocks_per_sm + (general && !stp && (cut.straddles || p.blocks_per_sm == kMoreBlocksPerSM) ? 3 : 0);
-  const bool block = work <= most_block_work(p.units_per_slab, stp, cut.straddles);
+  const StreamCost& sc = cost.stream;
+  const double stream_us = sc.base + sc.unit * run + sc.load * p.n_units / warps + sc.record * p.units_per_slab / run + sc.slab * 0.01 * n_slabs;
+  const bool block = cut.us < stream_us;
   if (p.n_units == 0 || ((block || (force_run_units < 0 && p.n_units < kMostForcedUnits)) && force_run_units <= 0 && (!partial || run == 1))) {
     p.n_blocks = static_cast<int32_t>(cut.even > 0 ? cut.even : p.n_units < cut.blocks ? p.n_units : cut.blocks);
     p.records = (p.n_blocks + n_slabs) * kMaxRep;

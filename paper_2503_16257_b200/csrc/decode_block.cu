@@ -1,5 +1,5 @@
-// Decode attention over the packed cache (Algorithm 1 "Decoding", Eq. 3) in one launch, for small calls (up to some 5000
-// 160-token units of five 32-token key groups where the slabs are few and long); most_block_work holds the rule.
+// Decode attention over the packed cache (Algorithm 1 "Decoding", Eq. 3) in one launch, for small calls (up to some 10000
+// 160-token units of five 32-token key groups where the slabs are few and long); plan_decode has the rule.
 //
 // What bounds such a call is latency: launches, dependent loads, a unit's serial work and the merge of the partial
 // results.  6400 tokens, a unit a block (11.4 us from the first block's start to the last one's end): query images 2.2,
@@ -46,7 +46,8 @@ constexpr int kUnitThreads = kUnitWarps * 32;
 constexpr int kImgBytes = 40 * 32 * 4;                        // query images of one chunk
 constexpr int kTRing = 512, kPRing = 512;                     // ring positions: an unfinished supergroup (group), two units and the gap
                                                               // before the flushed tokens
-constexpr int kPBufs = 5;                                     // staged protected groups (as many as leave room for four blocks)
+constexpr int kPBufs = 5;                                     // staged protected groups: as many as a unit can fill, or the rings would run over; with
+                                                              // them four blocks share a multiprocessor's memory
 constexpr int kResS = 132, kResP = 136;                       // row lengths of the residual's scores and probabilities
 constexpr int kResScratch = 8 * kResS * 4 + 8 * kResP * 2;    // 6400
 
@@ -979,6 +980,9 @@ static cudaError_t launch_block_t(const DecodeArgs& a, cudaStream_t stream) {
 
 template <bool GEN, typename T>
 static cudaError_t launch_block_as(const DecodeArgs& a, bool stp, bool more, cudaStream_t stream) {
+  if constexpr (!GEN) {
+    if (stp && more) return launch_block_t<GEN, true, kMoreBlocksPerSM, T>(a, stream);
+  }
   if (stp) return launch_block_t<GEN, true, kBlocksPerSM, T>(a, stream);
   return more ? launch_block_t<GEN, false, kMoreBlocksPerSM, T>(a, stream) : launch_block_t<GEN, false, kBlocksPerSM, T>(a, stream);
 }

@@ -454,7 +454,7 @@ static vidkv_status_t decode_impl(vidkv_cache_t* h, int32_t layer_begin, int32_t
   a.withhold = 0;
   a.st.T_q0 = first.T_q0; a.st.n_flush = first.n_flush; a.st.n_res = first.n_res + (append ? 1 : 0);
   const int64_t n_slabs = static_cast<int64_t>(n_layers) * h->cfg.B * h->cfg.H_kv;
-  a.plan = plan_decode(a.st, n_slabs, h->n_prot > 0, h->cv.kf.general != 0, device_sm_count(), h->dbg_run_units, partial != nullptr);
+  a.plan = plan_decode(a.st, n_slabs, h->n_prot > 0, h->cv.kf, device_sm_count(), h->dbg_run_units, partial != nullptr);
   if (a.plan.records > h->ws.partial_entries || n_slabs * a.plan.counters_per_slab > h->ws.counter_words) return VIDKV_ERR_CAPACITY;
   if (launch_decode(a, s) != cudaSuccess) return VIDKV_ERR_CUDA;
   if (!append) return VIDKV_OK;
@@ -540,7 +540,7 @@ vidkv_status_t vidkv_debug_decode_plan(const vidkv_config_t* cfg, int64_t n_pref
   LayerState ls;
   ls.T_q0 = n_prefill_quantized; ls.n_flush = n_flushed_chunks; ls.n_res = n_residual;
   const DecodePlan p = plan_decode(ls, static_cast<int64_t>(n_layers) * cfg->B * cfg->H_kv, n_protected > 0,
-                                   key_fmt_of_config(*cfg).general != 0, sm_count, run_units);
+                                   key_fmt_of_config(*cfg), sm_count, run_units);
   plan_out[0] = p.units_per_slab; plan_out[1] = p.run_units; plan_out[2] = p.n_runs; plan_out[3] = p.slab_parts;
   plan_out[4] = p.records; plan_out[5] = w.partial_entries; plan_out[6] = p.n_chunks; plan_out[7] = p.n_units;
   return VIDKV_OK;

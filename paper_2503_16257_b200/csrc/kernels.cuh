@@ -151,7 +151,7 @@ constexpr int kStreamCtasPerSM = 3;     // its CTAs per multiprocessor (register
 constexpr int kStreamStpCtasPerSM = 2;  // the same for the variant with protected tokens (shared-memory bound)
 constexpr int kPrepWords = 25;          // 32-bit words per lane per (slab, chunk) of prepared query
 constexpr int kBlocksPerSM = 3;         // blocks of the block kernel per multiprocessor: 128 registers x 160 threads
-constexpr int kMoreBlocksPerSM = 4;     // its variant for calls that are better off with more blocks (96 registers; no protected tokens)
+constexpr int kMoreBlocksPerSM = 4;     // its variant for calls that are better off with more blocks (96 registers)
 constexpr int kRecordFloats = 130; // one partial record: running maximum (base-2 logits), sum, out[128]
 constexpr int kPartFloats = kMaxRep * kRecordFloats;   // the block kernel's record of a part of a slab: m [8], l [8], out [8][128]
 constexpr int kJoin = 8;           // records joined at a node of the block kernel's merge tree
@@ -185,12 +185,11 @@ struct DecodePlan {
   __host__ __device__ int64_t run_of(int64_t u) const { return equal_units > 0 ? u / equal_units : ((u + 1) * n_runs - 1) / n_units; }
 };
 // stp: the cache holds protected tokens (the stream kernel for them keeps fewer warps per multiprocessor).
-// general: a key format other than the default.
 // force_run_units: 0 = choose; otherwise the test hook's value: > 0 the stream kernel with runs of that many units, -1 the block kernel.
 // partial: the call leaves (maximum, sum, unnormalised output) triples.  Their maximum is the one the walk has kept, which
 // need not be the largest logit, so it depends on how the units are cut: such calls keep runs of equal length, and take the
 // block kernel only where every run is one unit (its maximum is then exact however blocks share the units).
-DecodePlan plan_decode(const LayerState& st, int64_t n_slabs, bool stp, bool general, int sm_count, int force_run_units,
+DecodePlan plan_decode(const LayerState& st, int64_t n_slabs, bool stp, const KeyFmt& kf, int sm_count, int force_run_units,
                        bool partial = false);
 // Arrival counters any call that needs at most `records` records on at most max_slabs slabs uses.
 int64_t max_decode_counters(int64_t max_slabs, int64_t records);

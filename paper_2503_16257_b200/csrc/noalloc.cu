@@ -93,7 +93,7 @@ extern "C" vidkv_status_t vidkv_attend_noalloc(const vidkv_config_t* cfg, const 
   a.partial_out = nullptr;
   const int64_t n_slabs = static_cast<int64_t>(n_layers) * cfg->B * cfg->H_kv;
   a.append_row = -1;
-  a.plan = plan_decode(a.st, n_slabs, n_protected > 0, cv.kf.general != 0, device_sm_count(), 0);
+  a.plan = plan_decode(a.st, n_slabs, n_protected > 0, cv.kf, device_sm_count(), 0);
   // the array holds the partial records, then (256-byte aligned) the per-chunk query images
   int64_t prep_at = 0;
   auto fits = [&]() {
@@ -109,7 +109,7 @@ extern "C" vidkv_status_t vidkv_attend_noalloc(const vidkv_config_t* cfg, const 
     int run = a.plan.run_units;
     const bool few = a.plan.n_units <= static_cast<int64_t>(most) * kMoreBlocksPerSM * device_sm_count();
     do {
-      a.plan = plan_decode(a.st, n_slabs, n_protected > 0, cv.kf.general != 0, device_sm_count(), run);
+      a.plan = plan_decode(a.st, n_slabs, n_protected > 0, cv.kf, device_sm_count(), run);
     } while (!fits() && few && ++run <= most);
     if (!fits()) return VIDKV_ERR_CAPACITY;
   }

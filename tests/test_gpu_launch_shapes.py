@@ -381,6 +381,8 @@ def test_cache_memory_that_nobody_has_written_does_not_count(run_units, T, p, st
     ("tiny", 27, 1, 362, 0.0, 0.5, "fft"),         # 108 slabs of three units and their residuals: 432 blocks, three to a multiprocessor
     ("tiny", 28, 1, 362, 0.0, 0.5, "fft"),         # 448 blocks: four
     ("qwen", 28, 4, 362, 0.0, 0.75, "minmax"),     # more slabs than blocks at three to a multiprocessor
+    ("qwen", 28, 4, 330, 0.0, 0.75, "minmax"),     # the same of two units: four blocks on a multiprocessor for the general formats
+    ("llava", 28, 5, 362, 0.2, 0.5, "fft"),        # the same with protected tokens
     ("tiny", 1, 4, 11300, 0.0, 0.75, "minmax"),    # 16 slabs of 71 units, two or three to a block
     ("tiny", 1, 1, 196000, 0.0, 0.5, "fft"),       # the longest slab: 1225 units, 111 parts
     ("llava", 1, 4, 22400, 0.2, 0.5, "fft"),       # protected tokens, 140 units, five or six to a block
