@@ -24,6 +24,8 @@ static __device__ __align__(256) float g_static_partials[kStaticPartialFloats];
 constexpr int kStaticCounters = 4096;
 static __device__ int32_t g_static_counters[kStaticCounters];
 
+constexpr int kFewUnits = 7, kFewUnitsStp = 4;   // see where runs are made longer; without / with protected tokens
+
 constexpr int kMaxDevices = 64;
 struct StaticScratch {
   float* partials;
@@ -103,14 +105,18 @@ extern "C" vidkv_status_t vidkv_attend_noalloc(const vidkv_config_t* cfg, const 
            n_slabs * a.plan.counters_per_slab <= kStaticCounters;
   };
   if (!fits()) {
-    // as few runs as have the same longest one: fewer records.  Calls of few units may have longer runs, so that what the block
-    // kernel's few records (one per block and slab) would have room for has room here as well: up to 7 units (4 with protected tokens).
-    const int most = n_protected > 0 ? 4 : 7;
-    int run = a.plan.run_units;
-    const bool few = a.plan.n_units <= static_cast<int64_t>(most) * kMoreBlocksPerSM * device_sm_count();
-    do {
-      a.plan = plan_decode(a.st, n_slabs, n_protected > 0, cv.kf, device_sm_count(), run);
-    } while (!fits() && few && ++run <= most);
+    // Fewer records: the shortest runs whose records have room beside the query images, at least as few as have the same longest one.  What
+    // longer runs would save is bounded, and so is what is taken: calls of up to kFewUnits (kFewUnitsStp) units for each of four blocks
+    // a multiprocessor, with runs of up to as many units; everything beyond is refused (use fewer layers per call), whichever kernel
+    // the plan would have chosen.
+    const int most = n_protected > 0 ? kFewUnitsStp : kFewUnits;
+    const bool few = a.plan.n_units <= static_cast<int64_t>(most) * 4 * device_sm_count();
+    const int64_t room = static_cast<int64_t>(kStaticPartialFloats * sizeof(float)) - static_cast<int64_t>(decode_prep_bytes(n_slabs, a.plan.n_chunks));
+    const int64_t runs = room / 256 * 256 / static_cast<int64_t>(kPartFloats * sizeof(float)) - n_slabs;
+    int64_t run = a.plan.run_units;
+    if (few && runs > 0 && run * runs < a.plan.n_units) run = (a.plan.n_units + runs - 1) / runs;
+    if (run > a.plan.run_units && run > most) return VIDKV_ERR_CAPACITY;
+    a.plan = plan_decode(a.st, n_slabs, n_protected > 0, cv.kf, device_sm_count(), static_cast<int>(run));
     if (!fits()) return VIDKV_ERR_CAPACITY;
   }
   StaticScratch scratch;
