@@ -14,22 +14,27 @@ namespace {
 
 constexpr int kMaxSMs = 256;        // multiprocessor count the sizing formulas assume at most
 constexpr int64_t kMostForcedUnits = 1 << 21;   // the block kernel multiplies units by blocks in 32 bits
-// What the choice between the attention kernels goes by: estimated microseconds of a call, linear in what it is made of.  The block kernel
-// has one launch and a parallel merge; the stream kernel has three launches, a merge block per slab that reads the slab's records one behind the
-// other, and a third fewer instructions per unit.  The block kernel comes with three blocks on a multiprocessor and 128 registers a thread, or
-// with four and 96 (which keep some of the loop's state in local memory); not for general key formats with protected tokens, where four
-// are slower throughout.  The coefficients are least-squares fits to 650 measured calls of 4 to 1120 slabs and 1 to 1800 units a slab, the ones
-// near the line weighted most, and moved within a few percent so that the choice is the faster kernel there: over those calls it costs 0.2 % more than the
-// fastest of the three, 6.4 % at most.  us, three blocks / four / stream:
-//   half of the channels two-bit  112 slabs of 2 units 10.8 / 13.0 / 15.8, 448 of 3 26.1 / 22.3 / 25.1, 448 of 4 29.0 / 26.5 / 26.3, 448 of 8 40.9 / 43.6 / 35.1,
-//     224 of 8 28.4 / 28.3 / 24.6, 112 of 20 29.7 / 28.0 / 28.7, 192 of 13 32.5 / 31.8 / 28.9, 176 of 13 31.2 / 32.5 / 28.8, 128 of 18 28.8 / 32.6 / 29.3,
-//     32 of 140 44.8 / 44.9 / 43.3, 16 of 79 20.8 / 24.5 / 30.8, 16 of 400 56.2 / 57.3 / 59.2, 4 of 1225 47.8 / 49.6 / 103.5
-//   k = 0.75, plain one-bit code  112 of 2 10.3 / 13.0 / 18.4, 448 of 2 22.5 / 19.6 / 24.2, 448 of 3 26.2 / 25.3 / 25.3, 112 of 10 22.9 / 21.5 / 24.6, 112 of 20 30.7 / 32.2 / 31.9,
-//     96 of 24 31.5 / 32.3 / 32.7, 192 of 13 34.0 / 36.9 / 32.6, 16 of 200 39.2 / 42.8 / 48.2, 16 of 400 65.5 / 70.7 / 68.3
-//   k = 0.75, Eq. 5 (longer preparation in every block)  112 of 2 12.9 / 15.9 / 18.5, 448 of 3 31.5 / 28.0 / 26.4, 112 of 14 31.3 / 29.3 / 26.4, 32 of 40 31.3 / 29.3 / 28.8
-//   a fifth of the tokens protected, half of the channels two-bit  112 of 4 22.4 / 21.8 / 24.5, 224 of 4 27.1 / 29.7 / 25.2, 448 of 2 - / 26.3 / 26.8, 560 of 3 - / 33.0 / 36.8,
-//     592 of 4 - / 40.1 / 34.9, 64 of 14 27.2 / 32.1 / 26.6, 32 of 40 32.6 / - / 33.5, 16 of 300 64.8 / - / 61.2, 8 of 600 61.7 / - / 71.8
-//   the same, k = 0.75, plain     224 of 4 29.0 / 41.3 / 27.5, 64 of 14 27.8 / 42.8 / 28.6, 16 of 200 55.8 / - / 55.3, 16 of 300 74.3 / - / 69.7
+// What the choice between the attention kernels goes by: estimated microseconds of a call, linear in what it is made of.  The block
+// kernel has one launch and a parallel merge; the stream kernel has three launches, a merge block per slab that reads the slab's records one
+// behind the other, and a third fewer instructions per unit.  The block kernel comes with three blocks on a multiprocessor and 128 registers
+// a thread, or with four and 96 (which keep some of the loop's state in local memory); not for general key formats with protected tokens,
+// where four are slower throughout.  The coefficients are least-squares fits to 648 measured calls of 4 to 1120 slabs and 1 to 1800 units a
+// slab, the ones near the line weighted most, and moved within a few percent so that the choice is the faster kernel there: over those
+// calls it costs 0.2 % more than the fastest of the three, 6.4 % at most.  us, three blocks / four / stream:
+//   half of the channels two-bit (slabs of units): 112 of 2 10.9 / 13.1 / 15.5, 448 of 3 26.1 / 22.3 / 25.1, 448 of 4 29.0 / 26.5 / 26.3,
+//     448 of 8 40.9 / 43.4 / 35.1, 224 of 8 28.3 / 28.1 / 24.6, 112 of 20 29.5 / 27.9 / 28.6, 192 of 13 32.3 / 31.6 / 29.0,
+//     176 of 13 31.1 / 32.8 / 28.7, 128 of 18 28.7 / 32.6 / 29.2, 32 of 140 44.7 / 44.2 / 43.5, 16 of 79 20.9 / 24.4 / 30.9,
+//     16 of 400 56.5 / 56.6 / 59.9, 4 of 1225 48.1 / 49.0 / 104.0
+//   k = 0.75, plain one-bit code: 112 of 2 10.4 / 12.9 / 18.4, 448 of 2 22.5 / 19.6 / 24.2, 448 of 3 26.2 / 25.3 / 25.3,
+//     112 of 10 22.9 / 21.4 / 24.6, 112 of 20 30.6 / 32.1 / 32.1, 96 of 24 31.5 / 32.2 / 32.7, 192 of 13 34.1 / 36.9 / 32.8,
+//     16 of 200 39.5 / 42.7 / 48.4, 16 of 400 66.0 / 70.6 / 68.6
+//   k = 0.75, Eq. 5 (longer preparation in every block): 112 of 2 13.2 / 15.7 / 18.5, 448 of 3 31.5 / 27.9 / 26.4,
+//     112 of 14 31.8 / 29.3 / 26.7, 32 of 40 31.4 / 29.4 / 28.8
+//   a fifth of the tokens protected, half of the channels two-bit: 112 of 4 22.3 / 21.8 / 24.6, 224 of 4 27.1 / 29.7 / 25.1,
+//     448 of 2 - / 26.3 / 26.6, 560 of 3 - / 33.0 / 37.1, 592 of 4 - / 40.1 / 34.9, 64 of 14 27.2 / 32.1 / 26.6, 32 of 40 32.6 / - / 33.7,
+//     16 of 300 64.7 / - / 61.5, 8 of 600 61.8 / - / 71.9
+//   the same with k = 0.75, plain, three blocks / stream: 224 of 4 29.0 / 27.5, 64 of 14 27.8 / 28.6, 16 of 200 55.7 / 55.3,
+//     16 of 300 74.0 / 69.7
 struct BlockCost {
   double base;
   double unit;      // a unit of the longest stretch

@@ -46,8 +46,8 @@ constexpr int kUnitThreads = kUnitWarps * 32;
 constexpr int kImgBytes = 40 * 32 * 4;                        // query images of one chunk
 constexpr int kTRing = 512, kPRing = 512;                     // ring positions: an unfinished supergroup (group), two units and the gap
                                                               // before the flushed tokens
-constexpr int kPBufs = 5;                                     // staged protected groups: as many as a unit can fill, or the rings would run over; with
-                                                              // them four blocks share a multiprocessor's memory
+constexpr int kPBufs = 5;                                     // staged protected groups: as many as a unit can fill, or the rings would run
+                                                              // over; four blocks share a multiprocessor's memory with them
 constexpr int kResS = 132, kResP = 136;                       // row lengths of the residual's scores and probabilities
 constexpr int kResScratch = 8 * kResS * 4 + 8 * kResP * 2;    // 6400
 

@@ -102,8 +102,8 @@ __global__ void __launch_bounds__(kPrepThreads) decode_prep_kernel(DecodeArgs a,
 }
 
 // ---------------------------------------------------------------------------------
-// The same for the general key formats (KeyFmt): one warp per (chunk, slab); per lane (head hd = lane / 4,
-// r = lane % 4), all of the normalised query:
+// The same for the general key formats (KeyFmt): a block of four warps per (chunk, slab), each a quarter of the pair words and of the sums
+// over the normal channels, which meet in shared memory; per lane (head hd = lane / 4, r = lane % 4), all of the normalised query:
 //   words w < n2/8              binary16 pairs of q at the two-bit slots 8 w + 2 r, + 1
 //   then n1/8 words             plain mode: pairs of q at the one-bit channels 8 w + 6 - 2 r, + 1;
 //                               Eq. 5: leading binary16 part of the transformed query Q at those columns,

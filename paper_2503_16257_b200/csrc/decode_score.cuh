@@ -160,9 +160,9 @@ __device__ __forceinline__ void group_constants(const uint8_t* kbuf, int n, int 
   c[0] = d[0]; c[1] = d[1];
 }
 
-// The same for the general layout (KeyFmt), one group (ga) or two.  word(j): this lane's query words of the groups' chunk, word.four(j) four of them from a multiple of four on: n2 / 8 pairs of q at slots
-// 8 j + 2 r, + 1; then pairs at the one-bit columns 8 j + 6 - 2 r, + 1: of q in plain mode, of Q's leading part and then of
-// its remainder for Eq. 5.
+// The same for the general layout (KeyFmt), one group (ga) or two.  word(j): this lane's query words of the groups' chunk, word.four(j)
+// four of them from a multiple of four on: n2 / 8 pairs of q at slots 8 j + 2 r, + 1; then pairs at the one-bit columns 8 j + 6 - 2 r, + 1:
+// of q in plain mode, of Q's leading part and then of its remainder for Eq. 5.
 template <bool TWO, typename Word>
 __device__ __forceinline__ void score_general(const uint8_t* ga, const uint8_t* gb, const KeyFmt& kf, int lane, int r, Word word, float (&t)[TWO ? 4 : 2][4]) {
   constexpr int NT = TWO ? 4 : 2;

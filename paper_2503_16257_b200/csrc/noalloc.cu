@@ -111,7 +111,8 @@ extern "C" vidkv_status_t vidkv_attend_noalloc(const vidkv_config_t* cfg, const 
     // the plan would have chosen.
     const int most = n_protected > 0 ? kFewUnitsStp : kFewUnits;
     const bool few = a.plan.n_units <= static_cast<int64_t>(most) * 4 * device_sm_count();
-    const int64_t room = static_cast<int64_t>(kStaticPartialFloats * sizeof(float)) - static_cast<int64_t>(decode_prep_bytes(n_slabs, a.plan.n_chunks));
+    const int64_t images = static_cast<int64_t>(decode_prep_bytes(n_slabs, a.plan.n_chunks));
+    const int64_t room = static_cast<int64_t>(kStaticPartialFloats * sizeof(float)) - images;
     const int64_t runs = room / 256 * 256 / static_cast<int64_t>(kPartFloats * sizeof(float)) - n_slabs;
     int64_t run = a.plan.run_units;
     if (few && runs > 0 && run * runs < a.plan.n_units) run = (a.plan.n_units + runs - 1) / runs;
